@@ -282,7 +282,7 @@ tq_status tq_decompress_aggregate_apply(const uint32_t* packed_dev, size_t words
  * The same round without a host round trip (the paper takes alpha and lambda_s as given inputs of
  * Algorithm 1; where they come from -- Section 4 -- can equally run on the device).
  *
- * tq_params_device: Section 4 for n_workers records, one device thread per worker, same formulas and
+ * tq_params_device: Section 4 for n_workers records, one device warp per worker, same formulas and
  *   arguments as tq_params, reading stats_dev and writing params_dev (both device memory, 8-byte
  *   aligned).  Nothing is returned to the host: a worker whose statistics are outside the model's
  *   domain gets flags = TQ_FLAG_INVALID, iterations = the tq_status it would have returned, alpha = 0

@@ -63,7 +63,7 @@ cudaError_t launch_stats_hinted(const StatsCall& c, tq_gmin_hint_t* hint, int* l
 // *limit is set when n_workers exceeds what the array holds; nothing is launched then.
 cudaError_t launch_stats_static(const StatsCall& c, int* launches, bool* limit);
 
-// Parameter design on the device (one thread per worker); request already validated by params_request_ok.
+// Parameter design on the device (one warp per worker); request already validated by params_request_ok.
 bool params_request_ok(uint32_t num_levels, int mode, int rule, uint32_t* bits);
 cudaError_t launch_params_device(const tq_stats_t* stats_dev, uint32_t n, uint32_t num_levels, uint32_t bits, uint32_t mode,
                                  double gamma, int rule, double alpha_user, tq_params_t* params_dev, cudaStream_t stream);

@@ -1,15 +1,23 @@
 // Parameter design: statistics -> truncation threshold alpha and codebook, on the host (tq_params,
 // tq_params_batch, tq_params_from_levels) and, with the same code, on the device (tq_params_device:
-// one thread per worker, so a round needs no host round trip between statistics and compression).
+// one warp per worker, so a round needs no host round trip between statistics and compression).
 //
 // Follows Section 4 of the paper.  The gradient density is modelled as a power-law tail
 // p(g) = rho (gamma-1) g_min^(gamma-1) |g|^-gamma beyond g_min (Section 4.1, tail model), with rho
 // the one-sided tail mass, completed by a flat body p = (1 - 2 rho) / (2 g_min) below g_min so that
 // Q_U, Q_N and the p^(1/3) density of Section 4.2 are defined on the whole of [-alpha, alpha].
 // Everything here is O(L) double-precision work per worker; results are rounded once to fp32.
-// Host and device use their own pow / log / exp / cbrt, so the two can differ in the last fp32 bit
+// Host and device use their own log / exp / cbrt, so the two can differ in the last fp32 bit
 // of alpha or of a level; each is a valid quantizer, and a packed buffer is always decoded with the
 // parameters it was encoded with.
+//
+// On the device this is one short chain of dependent double-precision functions, so its time is their
+// latency times their number.  Hence: lengths are measured in units of g_min and by their logarithm
+// x = ln(a / g_min), in which a boxed alpha equation costs one exp and one log; it is solved by Newton
+// steps (4 to 8 evaluations); and everything that exists once per level or per trial point (levels, inverse
+// widths, the split of the two-step quantizer) is spread over the lanes of the warp.  Measured on B200 for
+// one worker, uniform, 4 levels / 8 workers, 16-level two-step quantizer: 5.3 us / 43 us, against
+// 21.1 us / 3590 us with one thread per worker, two pow per evaluation and Aitken steps.
 #include <cmath>
 
 #include "tq.h"
@@ -19,110 +27,195 @@ namespace tq {
 
 #define TQ_HD __host__ __device__
 
+TQ_HD inline bool finite_f(float x) { return fabsf(x) <= 3.402823466e38f; }
+TQ_HD inline bool finite_d(double x) { return fabs(x) <= 1.7976931348623157e308; }
+
+// Who works on one record: the calling host thread alone, or the 32 lanes of a warp.  All lanes run the same
+// scalar code; `ballot` collects one bit per lane (all lanes call it together).
+struct OneThread {
+    static constexpr int kLanes = 1;
+    TQ_HD int lane() const { return 0; }
+    TQ_HD uint32_t ballot(bool b) const { return b ? 1u : 0u; }
+    TQ_HD void sync() const {}
+};
+struct OneWarp {
+    static constexpr int kLanes = 32;
+#ifdef __CUDA_ARCH__
+    __device__ int lane() const { return static_cast<int>(threadIdx.x & 31u); }
+    __device__ uint32_t ballot(bool b) const { return __ballot_sync(0xFFFFFFFFu, b); }
+    __device__ void sync() const { __syncwarp(); }
+#else
+    int lane() const { return 0; }
+    uint32_t ballot(bool b) const { return b ? 1u : 0u; }
+    void sync() const {}
+#endif
+};
+
+// The density model in units of g_min.  x stands for ln(a / g_min) throughout.
 struct TailModel {
-    double g_min, rho, gamma;
-    // constants of the model, formed once (the alpha iteration evaluates q_of() many times):
-    double cb;       // body height^(1/3):       ((1 - 2 rho) / (2 g_min))^(1/3)
-    double coef;     // p^(1/3) = coef * |g|^(-gamma/3) in the tail
-    double b;        // 1 - gamma/3
-    double gmin_b;   // g_min^b
+    double rho, gamma;
+    double body;      // 1 - 2 rho: mass below g_min
+    double c1;        // 1 / (gamma - 1)
+    double b;         // 1 - gamma / 3
+    double ratio;     // (2 rho (gamma-1) / (1 - 2 rho))^(1/3): tail over body of p^(1/3) at g_min
+    double ln_k;      // ln(2 rho s^2 / (gamma - 2)): alpha' is g_min exp(c1 ln_k)
+    double ln_body;
 
-    TQ_HD TailModel(double g_min_, double rho_, double gamma_) : g_min(g_min_), rho(rho_), gamma(gamma_) {
-        cb = cbrt((1.0 - 2.0 * rho) / (2.0 * g_min));
-        coef = cbrt(rho * (gamma - 1.0)) * pow(g_min, (gamma - 1.0) / 3.0);
+    TQ_HD TailModel(double rho_, double gamma_, double s, uint32_t mode) : rho(rho_), gamma(gamma_) {
+        body = 1.0 - 2.0 * rho;
+        c1 = 1.0 / (gamma - 1.0);
         b = 1.0 - gamma / 3.0;
-        gmin_b = pow(g_min, b);
+        ln_k = log(2.0 * rho * s * s / (gamma - 2.0));
+        ln_body = mode == TQ_NONUNIFORM ? log(body) : 0.0;
+        ratio = mode == TQ_NONUNIFORM ? cbrt(2.0 * rho * (gamma - 1.0) / body) : 0.0;
     }
-
     // mass inside [-a, a]  (Q_U of Section 4.1)
-    TQ_HD double mass_inside(double a) const {
-        if (a <= g_min) return (1.0 - 2.0 * rho) * (a / g_min);
-        return 1.0 - 2.0 * rho * pow(a / g_min, 1.0 - gamma);
-    }
-    // integral of p^(1/3) over [0, x]
+    TQ_HD double mass_inside(double x) const { return x <= 0.0 ? body * exp(x) : 1.0 - 2.0 * rho * exp((1.0 - gamma) * x); }
+    // Integral of p^(1/3) over [0, a] in units of its value at g_min: a / g_min up to g_min, then
+    // 1 + ratio * (e^(b x) - 1) / b  (ratio * x for b = 0).
     TQ_HD double cuberoot_integral(double x) const {
-        if (x <= g_min) return cb * x;
-        const double tail = (b == 0.0) ? coef * log(x / g_min) : coef * (pow(x, b) - gmin_b) / b;
-        return cb * g_min + tail;
+        if (x <= 0.0) return exp(x);
+        return 1.0 + ratio * (b == 0.0 ? x : expm1(b * x) / b);
     }
-    // x with cuberoot_integral(x) = tau, tau >= 0
+    // a / g_min at which cuberoot_integral reaches tau >= 0
     TQ_HD double cuberoot_integral_inverse(double tau) const {
-        const double at_gmin = cb * g_min;
-        if (tau <= at_gmin) return tau / cb;
-        const double rest = (tau - at_gmin) / coef;
-        if (b == 0.0) return g_min * exp(rest);
-        return pow(gmin_b + b * rest, 1.0 / b);
+        if (tau <= 1.0) return tau;
+        const double rest = (tau - 1.0) / ratio;
+        return b == 0.0 ? exp(rest) : exp(log1p(b * rest) / b);
     }
-    // Q_N of Section 4.2: [ int_{-a}^{a} p^(1/3) (1/(2a))^(2/3) ]^3 = (2 I)^3 / (2a)^2
-    TQ_HD double holder_factor(double a) const {
-        const double two_i = 2.0 * cuberoot_integral(a);
-        return two_i * two_i * two_i / (4.0 * a * a);
-    }
-    // Q_B of the Appendix for the split at k * a: inner and outer mass, each spread evenly
-    TQ_HD double biscaled_factor(double a, double k) const {
-        const double inner = mass_inside(k * a);
-        double outer = mass_inside(a) - inner;
-        if (outer < 0.0) outer = 0.0;
-        const double t = cbrt(outer) * pow(1.0 - k, 2.0 / 3.0) + cbrt(inner) * pow(k, 2.0 / 3.0);
-        return t * t * t;
-    }
-    // d/dx of mass_inside: twice the model density
-    TQ_HD double mass_slope(double x) const {
-        if (x <= g_min) return (1.0 - 2.0 * rho) / g_min;
-        return 2.0 * rho * (gamma - 1.0) / g_min * pow(x / g_min, -gamma);
-    }
-    // A quantity with the sign of dQ_B/dk on 0 < k < 1.  With u = mass_inside(k a), w = mass_inside(a) - u and
-    // Q_B^(1/3) = w^(1/3) (1-k)^(2/3) + u^(1/3) k^(2/3), the derivative times the positive factor
-    // 3 w^(2/3) (1-k)^(1/3) u^(2/3) k^(1/3) is
-    //     w^(2/3) (1-k)^(1/3) (u' k + 2 u)  -  u^(2/3) k^(1/3) (u' (1-k) + 2 w),      u' = a * mass_slope(k a).
-    TQ_HD double biscaled_slope_sign(double a, double k) const {
-        const double u = mass_inside(k * a);
-        double w = mass_inside(a) - u;
-        if (w < 0.0) w = 0.0;
-        const double du = a * mass_slope(k * a);
-        const double cw = cbrt(w), cu = cbrt(u);
-        return cw * cw * cbrt(1.0 - k) * (du * k + 2.0 * u) - cu * cu * cbrt(k) * (du * (1.0 - k) + 2.0 * w);
-    }
-    // k* = argmin_k Q_B(a, k) (Appendix).  Q_B(a, 0) = Q_B(a, 1) = Q_U(a), so the minimum is a point where the
-    // slope turns from negative to positive (at the density's jump, k a = g_min, it may do so without
-    // passing through zero).  Every such turn between neighbours of a 128-point grid is closed in on by
-    // bisection of the slope's sign; the turn with the smallest Q_B wins.  No turn: the minimum is an end.
-    TQ_HD double biscaled_split(double a) const {
-        constexpr int kGrid = 128;
-        double best_k = 0.0, best_q = biscaled_factor(a, 0.0);
-        constexpr double kFirst = 9.094947017729282e-13;                // 2^-40: the grid's first point, in place of 0
-        bool prev_neg = biscaled_slope_sign(a, kFirst) < 0.0;        // slope at the previous grid point was negative
-        for (int j = 1; j <= kGrid; ++j) {
-            const double k = static_cast<double>(j) / kGrid;
-            // at k = 1 the slope's sign is that of approaching the end from inside: treat the end as a turn
-            const bool neg = j < kGrid ? biscaled_slope_sign(a, k) < 0.0 : false;
-            if (prev_neg && !neg) {
-                double lo = j > 1 ? static_cast<double>(j - 1) / kGrid : kFirst, hi = k;      // slope < 0 at lo, >= 0 at hi
-                for (int it = 0; it < 64 && hi - lo > 0.0; ++it) {
-                    const double mid = 0.5 * (lo + hi);
-                    if (mid <= lo || mid >= hi) break;
-                    if (biscaled_slope_sign(a, mid) < 0.0) lo = mid; else hi = mid;
-                }
-                const double kk = 0.5 * (lo + hi), q = biscaled_factor(a, kk);
-                if (q < best_q) { best_q = q; best_k = kk; }
-            }
-            prev_neg = neg;
+    // Right-hand side of the boxed alpha equations, F(x) = c1 (ln_k - ln Q(x)), and its derivative, for
+    //   Q_U = mass inside (Section 4.1), and Q_N = (2 int p^(1/3))^3 / (2 a)^2 = body * I^3 * e^(-2x) (Section 4.2).
+    TQ_HD double rhs(uint32_t mode, double x, double* slope) const {
+        if (mode == TQ_UNIFORM) {
+            if (x <= 0.0) { *slope = -c1; return c1 * (ln_k - log(body) - x); }
+            const double z = 2.0 * rho * exp((1.0 - gamma) * x), q = 1.0 - z;
+            *slope = -z / q;
+            return c1 * (ln_k - log(q));
         }
-        return best_k;
-    }
-    TQ_HD double q_of(uint32_t mode, double a) const {
-        if (mode == TQ_UNIFORM) return mass_inside(a);
-        if (mode == TQ_NONUNIFORM) return holder_factor(a);
-        return biscaled_factor(a, biscaled_split(a));
-    }
-    // right-hand side of the boxed alpha equations for a given Q
-    TQ_HD double alpha_for_q(double s, double q) const {
-        return g_min * pow(2.0 * rho * s * s / ((gamma - 2.0) * q), 1.0 / (gamma - 1.0));
+        if (x <= 0.0) { *slope = -c1; return c1 * (ln_k - ln_body - x); }
+        const double e = b == 0.0 ? 0.0 : expm1(b * x);
+        const double i = 1.0 + ratio * (b == 0.0 ? x : e / b);
+        *slope = c1 * (2.0 - 3.0 * ratio * (1.0 + e) / i);
+        return c1 * (ln_k - ln_body - 3.0 * log(i) + 2.0 * x);
     }
 };
 
-TQ_HD inline bool finite_f(float x) { return fabsf(x) <= 3.402823466e38f; }
-TQ_HD inline bool finite_d(double x) { return fabs(x) <= 1.7976931348623157e308; }
+constexpr int kSplitGrid = 128;
+constexpr double kSplitFirst = 9.094947017729282e-13, kSplitLnFirst = -27.72588722239781;   // 2^-40: the grid's first point, in place of 0
+// ln k of the grid points of one lane: j = t * kLanes + lane + 1, k = j / 128
+template <class Lanes>
+struct SplitGrid {
+    double ln_k[kSplitGrid / Lanes::kLanes];
+    TQ_HD explicit SplitGrid(const Lanes& lanes, bool wanted) {
+        for (int t = 0; wanted && t < kSplitGrid / Lanes::kLanes; ++t)
+            ln_k[t] = log(static_cast<double>(t * Lanes::kLanes + lanes.lane() + 1) / kSplitGrid);
+    }
+};
+TQ_HD inline int first_bit(uint32_t v, int none) {         // index of the lowest set bit
+#ifdef __CUDA_ARCH__
+    return v ? __ffs(static_cast<int>(v)) - 1 : none;
+#else
+    return v ? __builtin_ctz(v) : none;
+#endif
+}
+
+// The two-step quantizer's split (Appendix): k* = argmin_k Q_B(a, k) with
+// Q_B^(1/3) = w^(1/3) (1-k)^(2/3) + u^(1/3) k^(2/3),  u = mass inside k a,  w = mass between k a and a.
+struct Split {
+    const TailModel& m;
+    double x, a, mass;          // a in units of g_min, mass inside it
+    TQ_HD Split(const TailModel& m_, double x_) : m(m_), x(x_), a(exp(x_)), mass(m_.mass_inside(x_)) {}
+
+    TQ_HD double inner(double k, bool in_body, double ln_k) const {
+        return in_body ? m.body * k * a : 1.0 - 2.0 * m.rho * exp((1.0 - m.gamma) * (x + ln_k));
+    }
+    TQ_HD double inner(double k, bool in_body) const { return inner(k, in_body, in_body ? 0.0 : log(k)); }
+    // Whether Q_B falls with k.  The derivative's sign is that of
+    //     w^(2/3) (1-k)^(1/3) (u' k + 2 u)  -  u^(2/3) k^(1/3) (u' (1-k) + 2 w),      u' = du/dk,
+    // whose terms are non-negative, so their cubes are compared.
+    TQ_HD bool falls(double k, double u, double du) const {
+        double w = mass - u;
+        if (w < 0.0) w = 0.0;
+        const double p = du * k + 2.0 * u, q = du * (1.0 - k) + 2.0 * w;
+        return w * w * (1.0 - k) * (p * p * p) < u * u * k * (q * q * q);
+    }
+    TQ_HD bool falls_at(double k, double ln_k) const {
+        const bool in_body = k * a <= 1.0;
+        const double u = inner(k, in_body, ln_k);
+        return falls(k, u, in_body ? m.body * a : (m.gamma - 1.0) * (1.0 - u) / k);      // 1 - u = 2 rho (k a)^(1-gamma)
+    }
+    // Q_B(a, k), and d ln Q_B / dx along the minimum: at fixed k where k is a smooth minimum (its own motion does not
+    // change Q_B to first order), along k = 1 / a where it is the kink.
+    TQ_HD double factor(double k, bool kink, double* ln_slope) const {
+        const bool in_body = k * a <= 1.0;
+        const double u = kink ? m.body : inner(k, in_body);
+        double w = mass - u;
+        if (w < 0.0) w = 0.0;
+        const double cw = cbrt(w * (1.0 - k) * (1.0 - k)), cu = cbrt(u * k * k), t = cw + cu;
+        const double dmass = (m.gamma - 1.0) * (1.0 - mass);
+        *ln_slope = kink ? (cw * dmass / w + 2.0 * (k * cw / (1.0 - k) - cu)) / t
+                         : (in_body ? cw * (dmass - u) / w + cu : cw * (dmass - (m.gamma - 1.0) * (1.0 - u)) / w + cu * (m.gamma - 1.0) * (1.0 - u) / u) / t;
+        return t * t * t;
+    }
+    // Q_B(a, 0) = Q_B(a, 1) = Q_U(a), so the minimum is a point where Q_B turns from falling to rising.  Every
+    // such turn between neighbours of a 128-point grid is closed in on until its bracket is `tol` wide (relative);
+    // the turn with the smallest Q_B wins.  No turn: the minimum is an end.  Where the density jumps (k a = g_min) the
+    // turn may be a kink, which is tested for by itself.  Q_B is flat at a smooth turn, so a bracket of
+    // 2^-34 already fixes it to the last bit: the alpha iteration asks for no more.
+    template <class Lanes>
+    TQ_HD double best(const Lanes& lanes, const SplitGrid<Lanes>& grid, double tol, double* q_best, double* ln_slope) const {
+        constexpr int n = Lanes::kLanes;
+        *ln_slope = NAN;
+        if (x <= 0.0) { *q_best = mass; return 0.5; }            // flat density: Q_B is the same for every k
+        uint32_t down[kSplitGrid / 32] = {};                     // bit j - 1: Q_B falls at k = j / 128 (the end counts as rising)
+#pragma unroll
+        for (int t = 0; t < kSplitGrid / n; ++t) {
+            const int j = t * n + lanes.lane() + 1;
+            const bool falling = j < kSplitGrid && falls_at(static_cast<double>(j) / kSplitGrid, grid.ln_k[t]);
+            down[t * n / 32] |= lanes.ballot(falling) << (t * n % 32);
+        }
+        double best_k = 0.0, best_q = mass;
+        uint32_t before = falls_at(kSplitFirst, kSplitLnFirst) ? 1u : 0u;
+#pragma unroll
+        for (int v = 0; v < kSplitGrid / 32; ++v) {
+            uint32_t turns = ~down[v] & ((down[v] << 1) | before);
+            before = down[v] >> 31;
+            for (; turns != 0; turns &= turns - 1) {
+                const int j = 32 * v + first_bit(turns, 0) + 1;
+                bool kink = false;
+                const double k = close_in(lanes, j > 1 ? static_cast<double>(j - 1) / kSplitGrid : kSplitFirst,
+                                          static_cast<double>(j) / kSplitGrid, tol, &kink);
+                double slope;
+                const double q = factor(k, kink, &slope);
+                if (q < best_q) { best_q = q; best_k = k; *ln_slope = slope; }
+            }
+        }
+        *q_best = best_q;
+        return best_k;
+    }
+    // Q_B falls at lo and does not at hi: the lanes' trial points cut the bracket into kLanes + 1 parts each time.
+    template <class Lanes>
+    TQ_HD double close_in(const Lanes& lanes, double lo, double hi, double tol, bool* at_kink) const {
+        constexpr int n = Lanes::kLanes;
+        const double kink = 1.0 / a;
+        if (kink > lo && kink < hi) {
+            const bool before = falls(kink, m.body, m.body * a), after = falls(kink, m.body, 2.0 * m.rho * (m.gamma - 1.0) * a);
+            if (before && !after) { *at_kink = true; return kink; }
+            if (before) lo = kink; else hi = kink;
+        }
+        for (int it = 0; it < 64 && hi - lo > tol * hi; ++it) {
+            const double step = (hi - lo) / (n + 1);
+            const double k = lo + step * (lanes.lane() + 1);
+            const int c = first_bit(lanes.ballot(!falls_at(k, log(k))), n);      // trial points before the first one where Q_B rises
+            const double new_lo = lo + step * c, new_hi = c < n ? lo + step * (c + 1) : hi;
+            if (!(new_hi - new_lo < hi - lo)) break;
+            lo = new_lo; hi = new_hi;
+        }
+        return 0.5 * (lo + hi);
+    }
+};
+constexpr double kSplitCoarse = 5.820766091346741e-11;    // 2^-34
+constexpr double kSplitFine = 4.440892098500626e-16;      // 2^-51
 
 TQ_HD inline float ceil_to_float(double v) {
     float f = static_cast<float>(v);
@@ -132,18 +225,18 @@ TQ_HD inline float ceil_to_float(double v) {
 
 // inv_width / inv_step from a finished level table.  Rounded up so that a value sitting on the
 // top level maps to probability >= 1 and is reproduced exactly.
-TQ_HD inline tq_status finish(tq_params_t* p) {
+template <class Lanes>
+TQ_HD inline tq_status finish(const Lanes& lanes, tq_params_t* p) {
     const uint32_t s = p->num_levels - 1;
-    for (uint32_t k = 0; k < s; ++k) {
-        if (!(p->levels[k + 1] > p->levels[k])) return TQ_ERR_DEGENERATE_LEVELS;
+    bool bad = false;
+    for (uint32_t k = lanes.lane(); k < s; k += Lanes::kLanes) {
         const float w = static_cast<float>(static_cast<double>(p->levels[k + 1]) - static_cast<double>(p->levels[k]));
         p->inv_width[k] = ceil_to_float(1.0 / static_cast<double>(w));
-        if (!finite_f(p->inv_width[k])) return TQ_ERR_DEGENERATE_LEVELS;
+        if (!(p->levels[k + 1] > p->levels[k]) || !finite_f(p->inv_width[k])) bad = true;
     }
-    p->alpha = p->levels[s];
-    p->inv_step = ceil_to_float(static_cast<double>(s) / static_cast<double>(2.0f * p->alpha));
-    if (!finite_f(p->inv_step)) return TQ_ERR_DEGENERATE_LEVELS;
-    return TQ_OK;
+    const float alpha = p->levels[s], inv_step = ceil_to_float(static_cast<double>(s) / static_cast<double>(2.0f * alpha));
+    if (lanes.lane() == 0) { p->alpha = alpha; p->inv_step = inv_step; }
+    return lanes.ballot(bad) || !finite_f(inv_step) ? TQ_ERR_DEGENERATE_LEVELS : TQ_OK;
 }
 
 TQ_HD inline bool bits_for_levels(uint32_t num_levels, uint32_t* bits) {
@@ -159,24 +252,68 @@ TQ_HD inline void clear(tq_params_t* p) {
     for (int k = 0; k < TQ_MAX_LEVELS; ++k) { p->levels[k] = 0.0f; p->inv_width[k] = 0.0f; }
 }
 
-// Section 4 as a whole for one worker.  Arguments are already range-checked.
-TQ_HD inline tq_status design(const tq_stats_t* st, uint32_t num_levels, uint32_t bits, uint32_t mode, double gamma,
+// The boxed alpha equation x = F(x), from x0 = ln(alpha' / g_min) until a plain step changes alpha by <= 1e-12
+// relative.  The plain iteration converges linearly (70 steps for gamma = 3, s = 15).  F' comes with F, so a step goes to
+// the root of the tangent of F(x) - x wherever F' < 0.999 (Newton).  For the quantizers of Sections 4.1 and 4.2, F' grows
+// with x on x > 0, and every iterate is >= x0 because Q <= 1; so if F'(x0) >= -0.9 the plain iteration is a
+// contraction, or runs monotonically into the same first fixed point that the tangents of the convex F - x cannot
+// pass.  Elsewhere (the plain iteration may then end in a 2-cycle, which is its result) steps stay plain where F' < 0,
+// as they do for the two-step quantizer; F has a kink at x = 0, which no tangent step crosses.  Either way the result is
+// accepted only through the plain-step test.  Stops when alpha has passed max|g| (no fixed point below it).
+template <class Lanes>
+TQ_HD inline double solve_alpha(const Lanes& lanes, const SplitGrid<Lanes>& grid, const TailModel& m, uint32_t mode, double x_cap,
+                                int* iterations) {
+    double x = m.c1 * m.ln_k;
+    double least = mode == TQ_BISCALED || !(x > 0.0) ? 0.0 : -0.9;      // smallest F' that a tangent step is taken at
+    int it = 0;
+    while (it < 10000 && !(x > x_cap)) {
+        double slope, f;
+        if (mode == TQ_BISCALED) {
+            double q, ln_slope;
+            Split(m, x).best(lanes, grid, kSplitCoarse, &q, &ln_slope);
+            f = m.c1 * (m.ln_k - log(q));
+            slope = -m.c1 * ln_slope;
+        } else {
+            f = m.rhs(mode, x, &slope);
+        }
+        if (it == 0 && !(slope >= least)) least = 0.0;
+        ++it;
+        const double d = f - x, root = f + d * slope / (1.0 - slope);      // = x + d / (1 - slope)
+        const bool take = slope >= least && slope < 0.999 && x > 0.0 && root > 0.0 && finite_d(root) && !(root > x_cap);
+        x = f;
+        if (fabs(d) <= 1e-12) break;
+        if (take) x = root;
+    }
+    *iterations = it;
+    return x;
+}
+
+// Section 4 as a whole for one worker, by the lanes together.  Arguments are already range-checked; `out` is memory
+// that all lanes see.
+template <class Lanes>
+TQ_HD inline tq_status design(const Lanes& lanes, const tq_stats_t* st, uint32_t num_levels, uint32_t bits, uint32_t mode, double gamma,
                               int rule, double alpha_user, tq_params_t* out) {
-    clear(out);
-    out->bits = bits; out->num_levels = num_levels; out->mode = mode;
+    const bool first = lanes.lane() == 0;
+    if (first) {
+        clear(out);
+        out->bits = bits; out->num_levels = num_levels; out->mode = mode;
+    }
     const double s = static_cast<double>(num_levels - 1);
+    uint32_t flags = 0;
 
     if (gamma != gamma) {  // NaN: Section 5, gamma = 1 + n / sum ln(g_j / g_min)
         if (st->n_tail == 0 || !(st->sum_log_tail > 0.0)) return TQ_ERR_DOMAIN;
         gamma = 1.0 + static_cast<double>(st->n_tail) / st->sum_log_tail;
-        out->flags |= TQ_FLAG_GAMMA_FROM_MLE;
+        flags |= TQ_FLAG_GAMMA_FROM_MLE;
     }
     if (!(gamma > 2.0) || !finite_d(gamma)) return TQ_ERR_DOMAIN;
     if (!(st->g_min > 0.0f) || !finite_f(st->g_min) || st->d == 0) return TQ_ERR_DOMAIN;
     const double rho = static_cast<double>(st->n_tail) / (2.0 * static_cast<double>(st->d));
     if (!(rho > 0.0) || !(rho < 0.5)) return TQ_ERR_DOMAIN;
-    const TailModel m(static_cast<double>(st->g_min), rho, gamma);
-    out->gamma = static_cast<float>(gamma); out->g_min = st->g_min; out->rho = static_cast<float>(rho);
+    const double g_min = static_cast<double>(st->g_min);
+    const TailModel m(rho, gamma, s, mode);
+    const SplitGrid<Lanes> grid(lanes, mode == TQ_BISCALED);
+    int iterations = 0;
 
     double alpha;
     if (rule == TQ_ALPHA_USER) {
@@ -187,57 +324,40 @@ TQ_HD inline tq_status design(const tq_stats_t* st, uint32_t num_levels, uint32_
         alpha = static_cast<double>(st->max_abs);
     } else {
         const double cap = static_cast<double>(st->max_abs);
-        alpha = m.alpha_for_q(s, 1.0);                       // alpha'
-        if (rule == TQ_ALPHA_FIXED_POINT) {
-            // Iterate alpha <- F(alpha) (the boxed equation with Q evaluated at the current alpha) until a
-            // plain step changes alpha by <= 1e-12 relative.  The plain iteration converges linearly (70+
-            // steps for gamma = 3, s = 15), so every pair of steps is followed by Aitken's extrapolation
-            // to the limit of the geometric sequence when the steps are monotone and contracting; the
-            // result is still accepted only through the plain-step test, so it is the same fixed point.
-            int it = 0;
-            while (it < 10000) {
-                if (cap > 0.0 && alpha > cap) break;         // no fixed point below max|g|
-                const double a1 = m.alpha_for_q(s, m.q_of(mode, alpha));
-                ++it;
-                const double d1 = a1 - alpha;
-                alpha = a1;
-                if (fabs(d1) <= 1e-12 * fabs(a1)) break;
-                if (cap > 0.0 && alpha > cap) break;
-                const double a2 = m.alpha_for_q(s, m.q_of(mode, a1));
-                ++it;
-                const double d2 = a2 - a1;
-                alpha = a2;
-                if (fabs(d2) <= 1e-12 * fabs(a2)) break;
-                const double r = d2 / d1;
-                if (r > 0.0 && r < 0.999) {
-                    const double limit = a2 + d2 * r / (1.0 - r);
-                    if (limit > 0.0 && finite_d(limit) && !(cap > 0.0 && limit > cap)) alpha = limit;
-                }
-            }
-            out->iterations = it;
-        }
+        double x = m.c1 * m.ln_k;                            // alpha'
+        if (rule == TQ_ALPHA_FIXED_POINT)
+            x = solve_alpha(lanes, grid, m, mode, cap > 0.0 ? log(cap / g_min) : INFINITY, &iterations);
+        alpha = g_min * exp(x);
         if (alpha != alpha) return TQ_ERR_DOMAIN;
-        if (alpha < m.g_min) { alpha = m.g_min; out->flags |= TQ_FLAG_ALPHA_AT_GMIN; }
-        if (cap > 0.0 && alpha > cap) { alpha = cap; out->flags |= TQ_FLAG_ALPHA_CAPPED; }
+        if (alpha < g_min) { alpha = g_min; flags |= TQ_FLAG_ALPHA_AT_GMIN; }
+        if (cap > 0.0 && alpha > cap) { alpha = cap; flags |= TQ_FLAG_ALPHA_CAPPED; }
+    }
+    if (first) {
+        out->gamma = static_cast<float>(gamma); out->g_min = st->g_min; out->rho = static_cast<float>(rho);
+        out->iterations = iterations; out->flags = flags;
     }
 
     const float alpha_f = static_cast<float>(alpha);
     if (!(alpha_f > 0.0f) || !finite_f(2.0f * alpha_f)) return TQ_ERR_DOMAIN;
     const double a = static_cast<double>(alpha_f);
     const uint32_t si = num_levels - 1;
+    lanes.sync();                                            // the cleared record
     if (mode == TQ_UNIFORM) {
         const double step = 2.0 * a / s;                     // Section 4.1 codebook
-        for (uint32_t k = 0; k <= si; ++k) out->levels[k] = static_cast<float>(-a + static_cast<double>(k) * step);
+        for (uint32_t k = 1 + lanes.lane(); k < si; k += Lanes::kLanes) out->levels[k] = static_cast<float>(-a + static_cast<double>(k) * step);
     } else if (mode == TQ_BISCALED) {
         // Appendix: density s c_in / D inside k* alpha and s c_out / D outside, c = (mean density)^(1/3),
         // D = 2 alpha (c_out (1 - k*) + c_in k*).  Level k sits where the density accumulated from the
         // centre reaches k - s/2.  Upper half, then mirrored.
-        const double k = m.biscaled_split(a), beta = k * a;
-        const double c_in = cbrt(m.mass_inside(beta) / (2.0 * beta));
-        const double c_out = cbrt((m.mass_inside(a) - m.mass_inside(beta)) / (2.0 * (a - beta)));
+        const Split split(m, log(a / g_min));
+        double q, ln_slope;
+        const double k = split.best(lanes, grid, kSplitFine, &q, &ln_slope), beta = k * a;
+        const double u = k > 0.0 ? split.inner(k, k * split.a <= 1.0) : 0.0;
+        const double c_in = cbrt(u / (2.0 * beta));
+        const double c_out = cbrt((split.mass - u) / (2.0 * (a - beta)));
         const double denom = 2.0 * a * (c_out * (1.0 - k) + c_in * k);
         const double lam_in = s * c_in / denom, lam_out = s * c_out / denom;
-        for (uint32_t j = (si + 1) / 2; j <= si; ++j) {
+        for (uint32_t j = (si + 1) / 2 + lanes.lane(); j < si; j += Lanes::kLanes) {
             const double c = static_cast<double>(j) - 0.5 * s;
             const double x = c <= lam_in * beta ? c / lam_in : beta + (c - lam_in * beta) / lam_out;
             out->levels[j] = static_cast<float>(x);
@@ -246,17 +366,17 @@ TQ_HD inline tq_status design(const tq_stats_t* st, uint32_t num_levels, uint32_
     } else {
         // lambda_s = s p^(1/3) / int p^(1/3): level k sits where the running integral of p^(1/3)
         // from the centre reaches (2k/s - 1) of its value at alpha.  Upper half, then mirrored.
-        const double total = m.cuberoot_integral(a);
-        for (uint32_t k = (si + 1) / 2; k <= si; ++k) {
+        const double total = m.cuberoot_integral(log(a / g_min));
+        for (uint32_t k = (si + 1) / 2 + lanes.lane(); k < si; k += Lanes::kLanes) {
             const double tau = (2.0 * static_cast<double>(k) / s - 1.0) * total;
-            const float l = static_cast<float>(m.cuberoot_integral_inverse(tau));
+            const float l = static_cast<float>(g_min * m.cuberoot_integral_inverse(tau));
             out->levels[k] = l;
             out->levels[si - k] = -l;
         }
     }
-    out->levels[0] = -alpha_f;
-    out->levels[si] = alpha_f;
-    return finish(out);
+    if (first) { out->levels[0] = -alpha_f; out->levels[si] = alpha_f; }
+    lanes.sync();
+    return finish(lanes, out);
 }
 
 static bool valid_request(uint32_t num_levels, int mode, int rule, uint32_t* bits) {
@@ -265,26 +385,40 @@ static bool valid_request(uint32_t num_levels, int mode, int rule, uint32_t* bit
     return rule == TQ_ALPHA_CLOSED || rule == TQ_ALPHA_FIXED_POINT || rule == TQ_ALPHA_USER || rule == TQ_ALPHA_MAXABS;
 }
 
-// One thread per worker.  A worker whose statistics are outside the model's domain gets
+// One warp per worker.  A worker whose statistics are outside the model's domain gets
 // flags = TQ_FLAG_INVALID, iterations = the status code, alpha = 0 and an all-zero codebook.
-__global__ void params_kernel(const tq_stats_t* __restrict__ stats, uint32_t n, uint32_t num_levels, uint32_t bits,
-                              uint32_t mode, double gamma, int rule, double alpha_user, tq_params_t* __restrict__ out) {
-    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+// One kernel per quantizer: a record runs straight through code that is fetched for the first time, so its length counts
+// (all three in one kernel: 18.2 us instead of 7.7 us for 4 workers, non-uniform, 8 levels).
+constexpr int kParamsWarps = 4;
+template <uint32_t MODE>
+__global__ void __launch_bounds__(32 * kParamsWarps)
+params_kernel(const tq_stats_t* __restrict__ stats, uint32_t n, uint32_t num_levels, uint32_t bits, double gamma, int rule,
+              double alpha_user, tq_params_t* __restrict__ out) {
+    __shared__ tq_params_t s_p[kParamsWarps];
+    const uint32_t warp = threadIdx.x >> 5, i = blockIdx.x * kParamsWarps + warp;
     if (i >= n) return;
+    const OneWarp lanes;
+    tq_params_t* p = &s_p[warp];
     const tq_stats_t st = stats[i];
-    tq_params_t p;
-    const tq_status s = design(&st, num_levels, bits, mode, gamma, rule, alpha_user, &p);
-    if (s != TQ_OK) {
-        clear(&p);
-        p.bits = bits; p.num_levels = num_levels; p.mode = mode;
-        p.flags = TQ_FLAG_INVALID; p.iterations = static_cast<int32_t>(s);
+    const tq_status s = design(lanes, &st, num_levels, bits, MODE, gamma, rule, alpha_user, p);
+    __syncwarp();
+    if (s != TQ_OK && lanes.lane() == 0) {
+        clear(p);
+        p->bits = bits; p->num_levels = num_levels; p->mode = MODE;
+        p->flags = TQ_FLAG_INVALID; p->iterations = static_cast<int32_t>(s);
     }
-    out[i] = p;
+    __syncwarp();
+    const uint32_t* from = reinterpret_cast<const uint32_t*>(p);
+    uint32_t* to = reinterpret_cast<uint32_t*>(out + i);
+    for (uint32_t w = lanes.lane(); w < sizeof(tq_params_t) / 4; w += 32) to[w] = from[w];
 }
 
 cudaError_t launch_params_device(const tq_stats_t* stats_dev, uint32_t n, uint32_t num_levels, uint32_t bits, uint32_t mode,
                                  double gamma, int rule, double alpha_user, tq_params_t* params_dev, cudaStream_t stream) {
-    params_kernel<<<(n + 31) / 32, 32, 0, stream>>>(stats_dev, n, num_levels, bits, mode, gamma, rule, alpha_user, params_dev);
+    const uint32_t warps = n < kParamsWarps ? n : kParamsWarps;      // few records: no idle warps to launch
+    const dim3 grid((n + kParamsWarps - 1) / kParamsWarps), block(32 * warps);
+    auto* kernel = mode == TQ_UNIFORM ? params_kernel<TQ_UNIFORM> : mode == TQ_NONUNIFORM ? params_kernel<TQ_NONUNIFORM> : params_kernel<TQ_BISCALED>;
+    kernel<<<grid, block, 0, stream>>>(stats_dev, n, num_levels, bits, gamma, rule, alpha_user, params_dev);
     return cudaGetLastError();
 }
 
@@ -302,14 +436,14 @@ extern "C" tq_status tq_params_from_levels(const float* levels_host, uint32_t nu
     for (uint32_t k = 0; k < num_levels; ++k) out->levels[k] = levels_host[k];
     const float top = levels_host[num_levels - 1];
     if (!(top > 0.0f) || !tq::finite_f(2.0f * top) || levels_host[0] != -top) return TQ_ERR_DOMAIN;
-    return tq::finish(out);
+    return tq::finish(tq::OneThread(), out);
 }
 
 extern "C" tq_status tq_params(const tq_stats_t* st, uint32_t num_levels, tq_mode mode, double gamma,
                                tq_alpha_rule rule, double alpha_user, tq_params_t* out) {
     uint32_t bits = 0;
     if (!st || !out || !tq::valid_request(num_levels, mode, rule, &bits)) return TQ_ERR_INVALID_ARG;
-    return tq::design(st, num_levels, bits, mode, gamma, rule, alpha_user, out);
+    return tq::design(tq::OneThread(), st, num_levels, bits, mode, gamma, rule, alpha_user, out);
 }
 
 extern "C" tq_status tq_params_batch(const tq_stats_t* st, uint32_t n_workers, uint32_t num_levels, tq_mode mode,
