@@ -200,7 +200,7 @@ tq_status tq_compress_device_params(const void* grad_dev, tq_dtype dtype, uint64
     c.launches = &launched;
     const cudaError_t e = tq::launch_compress(c);
     if (e != cudaSuccess) return cuda_failed(e);
-    g_launches += static_cast<uint64_t>(launched);   // table mode: main kernel + the (usually empty) binary-search pass; bf16: + the decision-table kernel
+    g_launches += static_cast<uint64_t>(launched);   // bf16 table codebooks: the decision-table kernel and the one for the rows it leaves
     return TQ_OK;
 }
 

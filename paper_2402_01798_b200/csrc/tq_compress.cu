@@ -246,44 +246,16 @@ __device__ __forceinline__ float slot_as_float(const uint32_t (&rnd)[4], int e) 
     return __uint_as_float(__byte_perm(rnd[e >> 1], DN ? kSlotExpBits : kMagicBits, (e & 1) ? 0x7432u : 0x7410u));
 }
 
-template <int BITS, int SEARCH, bool BF16, bool TAIL>
-__device__ __forceinline__ void quantize_run(const Raw8<BF16> (&g)[4], uint32_t* prow, uint64_t run, uint64_t d, uint64_t words_out,
-                                             uint32_t worker, const RoundKeys& rk, const RunCtx& cx);
-
-// One run of 32 elements: load, quantize, pack, store.  TAIL = the last, possibly partial run of a row
-// (element-wise guarded loads, zero padding bits, guarded stores and the row's alignment padding).
-template <int BITS, int SEARCH, bool BF16, bool TAIL>
-__device__ __forceinline__ void compress_run(const char* row, uint32_t* prow, uint64_t run, uint64_t d, uint64_t words_out,
-                                             uint32_t worker, const RoundKeys& rk, const RunCtx& cx) {
-    constexpr size_t esz = BF16 ? 2 : 4;
-    const uint64_t j0 = run << 5;
-    Raw8<BF16> g[4];
-    if constexpr (!TAIL) {
-#pragma unroll
-        for (int grp = 0; grp < 4; ++grp) load8_raw<BF16>(row + (j0 + 8 * grp) * esz, g[grp]);
-    } else {
-#pragma unroll
-        for (int grp = 0; grp < 4; ++grp)
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const uint64_t j = j0 + 8 * grp + e;
-                set_elem<BF16>(g[grp], e, j < d ? load1<BF16>(row, j) : 0.0f);
-            }
-    }
-
-    quantize_run<BITS, SEARCH, BF16, TAIL>(g, prow, run, d, words_out, worker, rk, cx);
-}
-
-// The arithmetic of one run whose 32 elements are already in registers: quantize, pack, store.
-template <int BITS, int SEARCH, bool BF16, bool TAIL>
-__device__ __forceinline__ void quantize_run(const Raw8<BF16> (&g)[4], uint32_t* prow, uint64_t run, uint64_t d, uint64_t words_out,
-                                             uint32_t worker, const RoundKeys& rk, const RunCtx& cx) {
+// The arithmetic of one run of 32 elements that are already in registers: quantize, pack, store.
+template <int BITS, int SEARCH, bool BF16>
+__device__ __forceinline__ void quantize_run(const Raw8<BF16> (&g)[4], uint32_t* prow, uint64_t run, uint32_t worker,
+                                             const RoundKeys& rk, const RunCtx& cx) {
     const uint64_t j0 = run << 5;
     const uint32_t blk_lo = static_cast<uint32_t>(j0 >> 3);
     const PhiloxRun pr = philox_run(static_cast<uint32_t>(j0 >> 35), worker, rk);
     const f32x2 alpha2 = both(cx.alpha), inv_step2 = both(cx.inv_step), cell_scale2 = both(cx.cell_scale);
-    // whole runs of the scaled uniform path hand pack8 the codes as denormals (2- and 4-bit codes)
-    constexpr bool DN = SEARCH == kUniform && !TAIL && (BITS == 2 || BITS == 4);
+    // the scaled uniform path hands pack8 the codes as denormals (2- and 4-bit codes)
+    constexpr bool DN = SEARCH == kUniform && (BITS == 2 || BITS == 4);
     uint32_t chunk[4];   // the 8*BITS packed bits of each group
 #pragma unroll
     for (int grp = 0; grp < 4; ++grp) {
@@ -307,13 +279,6 @@ __device__ __forceinline__ void quantize_run(const Raw8<BF16> (&g)[4], uint32_t*
                 else code[h] = pair(code_binary<BITS>(g0, cx.alpha, cx.s_search, reinterpret_cast<const float2*>(cx.s_cell), rf0),
                                     code_binary<BITS>(g1, cx.alpha, cx.s_search, reinterpret_cast<const float2*>(cx.s_cell), rf1));
             }
-            if constexpr (TAIL) {                 // padding bits are zero
-                float c0, c1;
-                unpair(code[h], c0, c1);
-                if (j0 + 8 * grp + e >= d) c0 = 0.0f;
-                if (j0 + 8 * grp + e + 1 >= d) c1 = 0.0f;
-                code[h] = pair(c0, c1);
-            }
         }
         chunk[grp] = pack8<BITS, DN>(code);
     }
@@ -330,19 +295,61 @@ __device__ __forceinline__ void quantize_run(const Raw8<BF16> (&g)[4], uint32_t*
     if constexpr (BITS == 1) { w[0] = chunk[0] | (chunk[1] << 8) | (chunk[2] << 16) | (chunk[3] << 24); }
 
     uint32_t* dst = prow + run * BITS;
-    if constexpr (!TAIL) {   // every word of an interior run lies below words_out
-        if constexpr (BITS == 4) *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
-        if constexpr (BITS == 3) { dst[0] = w[0]; dst[1] = w[1]; dst[2] = w[2]; }
-        if constexpr (BITS == 2) *reinterpret_cast<uint2*>(dst) = make_uint2(w[0], w[1]);
-        if constexpr (BITS == 1) dst[0] = w[0];
-    } else {
-        // last run of the row: write its words that exist, then zero the alignment padding
-        const uint64_t first = run * BITS;
+    if constexpr (BITS == 4) *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
+    if constexpr (BITS == 3) { dst[0] = w[0]; dst[1] = w[1]; dst[2] = w[2]; }
+    if constexpr (BITS == 2) *reinterpret_cast<uint2*>(dst) = make_uint2(w[0], w[1]);
+    if constexpr (BITS == 1) dst[0] = w[0];
+}
+
+// One whole run: load, quantize, pack, store.
+template <int BITS, int SEARCH, bool BF16>
+__device__ __forceinline__ void compress_run(const char* row, uint32_t* prow, uint64_t run, uint32_t worker, const RoundKeys& rk,
+                                             const RunCtx& cx) {
+    constexpr size_t esz = BF16 ? 2 : 4;
+    Raw8<BF16> g[4];
 #pragma unroll
-        for (int i = 0; i < BITS; ++i)
-            if (first + i < words_out) dst[i] = w[i];
-        for (uint64_t k = first + BITS; k < words_out; ++k) prow[k] = 0u;
+    for (int grp = 0; grp < 4; ++grp) load8_raw<BF16>(row + ((run << 5) + 8 * grp) * esz, g[grp]);
+    quantize_run<BITS, SEARCH, BF16>(g, prow, run, worker, rk, cx);
+}
+
+// A row's last run, possibly partial, by one warp: a lane takes one element, with the decision in its plain form (clip,
+// interval, p, T, code = k + [r < T]); bits beyond the row's end and the padding words are zero.
+template <int BITS, bool UNIFORM, bool BF16>
+__device__ __forceinline__ void compress_last_run(const char* row, uint32_t* prow, uint64_t d, uint32_t worker, const RoundKeys& rk,
+                                                  const WorkerQ& q) {
+    constexpr int s = (1 << BITS) - 1;
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint64_t run = (d - 1) >> 5, j = (run << 5) + lane;
+    uint32_t code = 0;
+    if (j < d) {
+        const float t = fminf(fmaxf(load1<BF16>(row, j), -q.alpha), q.alpha);      // NaN -> -alpha
+        float k = 0.0f, p;
+        if constexpr (UNIFORM) {
+            const float x = __fmul_rn(__fadd_rn(t, q.alpha), q.inv_step);
+            k = fminf(floorf(x), static_cast<float>(s - 1));
+            p = __fsub_rn(x, k);
+        } else {
+            int i = 0;
+            for (int l = 1; l < s; ++l)
+                if (q.levels[l] <= t) i = l;
+            k = static_cast<float>(i);
+            p = __fmul_rn(__fsub_rn(t, q.levels[i]), q.inv_width[i]);
+        }
+        uint32_t rnd[4];
+        philox_block(static_cast<uint32_t>(j >> 3), philox_run(static_cast<uint32_t>(j >> 35), worker, rk), rk, rnd);
+        const uint32_t word = (lane & 4u) ? ((lane & 2u) ? rnd[3] : rnd[2]) : ((lane & 2u) ? rnd[1] : rnd[0]);
+        const uint32_t r = (lane & 1u) ? word >> 16 : word & 0xFFFFu;
+        code = static_cast<uint32_t>(k + rounds_up(p, __uint_as_float(kMagicBits | r)));
     }
+    const uint64_t at = static_cast<uint64_t>(code) << ((lane * BITS) & 31u);
+    const uint32_t w = (lane * BITS) >> 5;
+    const uint64_t first = run * BITS, words_out = (((d * BITS + 31) >> 5) + 3) & ~static_cast<uint64_t>(3);
+#pragma unroll
+    for (uint32_t i = 0; i < BITS; ++i) {
+        const uint32_t bits = __reduce_or_sync(0xFFFFFFFFu, (w == i ? static_cast<uint32_t>(at) : 0u) | (w + 1 == i ? static_cast<uint32_t>(at >> 32) : 0u));
+        if (lane == i && first + i < words_out) prow[first + i] = bits;
+    }
+    if (first + BITS + lane < words_out) prow[first + BITS + lane] = 0u;             // at most three words of padding
 }
 
 #ifndef TQ_COMPRESS_MIN_BLOCKS
@@ -380,52 +387,27 @@ __device__ __forceinline__ void build_tables(const WorkerQ& q, float2* s_grid, f
     if constexpr (!is_uniform(SEARCH)) __syncthreads();
 }
 
-// Per-block set-up of the shared tables for quantizer q, then the block's share of the runs of one row
-// (`row`: its first gradient element, `prow`: its first packed word).
-// s_grid must hold kMaxGridCells + 1 entries when SEARCH == kGrid.
-template <int BITS, int SEARCH, bool BF16>
-__device__ __forceinline__ void compress_row(const WorkerQ& q, float2* s_grid, float2* s_cell, float* s_search,
-                                             const char* __restrict__ row, uint64_t d, const RoundKeys& rk, uint32_t worker,
-                                             uint32_t* __restrict__ prow, uint64_t words_out) {
-    build_tables<BITS, SEARCH>(q, s_grid, s_cell, s_search);
-
-    const uint64_t n_runs = (d + 31) >> 5;
-    const RunCtx cx{q.alpha, q.inv_step, q.top, q.inv_2alpha, q.cell_scale, uniform_q<BITS>(q), reinterpret_cast<const char*>(s_grid),
-                    reinterpret_cast<const char*>(s_cell), s_search};
-    const uint64_t stride = static_cast<uint64_t>(gridDim.x) * kThreads;
-
-    uint64_t run = static_cast<uint64_t>(blockIdx.x) * kThreads + threadIdx.x;
-    const uint64_t interior = n_runs - 1;      // every run before the row's last one is full
-    for (; run < interior; run += stride)
-        compress_run<BITS, SEARCH, BF16, false>(row, prow, run, d, words_out, worker, rk, cx);
-    if (run == n_runs - 1)
-        compress_run<BITS, SEARCH, BF16, true>(row, prow, run, d, words_out, worker, rk, cx);
-}
-
-// The same for worker wi's row of a [N][grad_stride] block and its row of the [N][words_stride] output.
-template <int BITS, int SEARCH, bool BF16>
-__device__ __forceinline__ void compress_block(const WorkerQ& q, float2* s_grid, float2* s_cell, float* s_search,
-                                               const void* __restrict__ grad, uint64_t d, uint64_t grad_stride,
-                                               const RoundKeys& rk, uint32_t worker, uint32_t wi,
-                                               uint32_t* __restrict__ packed, uint64_t words_stride, uint64_t words_out) {
-    constexpr size_t esz = BF16 ? 2 : 4;
-    compress_row<BITS, SEARCH, BF16>(q, s_grid, s_cell, s_search,
-                                     static_cast<const char*>(grad) + static_cast<uint64_t>(wi) * grad_stride * esz, d, rk, worker,
-                                     packed + static_cast<uint64_t>(wi) * words_stride, words_out);
-}
-
 // Quantizers passed by value in the kernel's parameter space (host-side tq_params).
 template <int BITS, int SEARCH, bool BF16>
 __global__ void __launch_bounds__(kThreads, TQ_COMPRESS_MIN_BLOCKS)
 compress_kernel(const void* __restrict__ grad, uint64_t d, uint64_t grad_stride,
                 const __grid_constant__ CompressArgs args, const __grid_constant__ RoundKeys rk,
-                uint32_t first_worker, uint32_t* __restrict__ packed, uint64_t words_stride, uint64_t words_out) {
+                uint32_t first_worker, uint32_t* __restrict__ packed, uint64_t words_stride) {
     __shared__ __align__(16) float2 s_grid[SEARCH == kGrid ? kMaxGridCells + 1 : 1];
     __shared__ __align__(16) float2 s_cell[TQ_MAX_LEVELS];
     __shared__ float s_search[2 * TQ_MAX_LEVELS];
-    const uint32_t wi = blockIdx.y;
-    compress_block<BITS, SEARCH, BF16>(args.q[wi], s_grid, s_cell, s_search, grad, d, grad_stride, rk, first_worker + wi, wi,
-                                       packed, words_stride, words_out);
+    constexpr size_t esz = BF16 ? 2 : 4;
+    const WorkerQ& q = args.q[blockIdx.y];
+    const uint32_t worker = first_worker + blockIdx.y;
+    const char* row = static_cast<const char*>(grad) + static_cast<uint64_t>(blockIdx.y) * grad_stride * esz;
+    uint32_t* prow = packed + static_cast<uint64_t>(blockIdx.y) * words_stride;
+    build_tables<BITS, SEARCH>(q, s_grid, s_cell, s_search);
+    const RunCtx cx{q.alpha, q.inv_step, q.top, q.inv_2alpha, q.cell_scale, uniform_q<BITS>(q), reinterpret_cast<const char*>(s_grid),
+                    reinterpret_cast<const char*>(s_cell), s_search};
+    const uint64_t whole = (d - 1) >> 5, stride = static_cast<uint64_t>(gridDim.x) * kThreads;     // runs before the row's last one are whole
+    for (uint64_t run = static_cast<uint64_t>(blockIdx.x) * kThreads + threadIdx.x; run < whole; run += stride)
+        compress_run<BITS, SEARCH, BF16>(row, prow, run, worker, rk, cx);
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x < 32) compress_last_run<BITS, is_uniform(SEARCH), BF16>(row, prow, d, worker, rk, q);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -452,7 +434,7 @@ template <int BITS, bool BF16>
 __global__ void __launch_bounds__(kThreads, TQ_COMPRESS_MIN_BLOCKS)
 compress_tma_kernel(const __grid_constant__ CUtensorMap tmap, const void* __restrict__ grad, uint64_t d, uint64_t grad_stride,
                     const __grid_constant__ CompressArgs args, const __grid_constant__ RoundKeys rk,
-                    uint32_t first_worker, uint32_t* __restrict__ packed, uint64_t words_stride, uint64_t words_out) {
+                    uint32_t first_worker, uint32_t* __restrict__ packed, uint64_t words_stride) {
     constexpr uint32_t kRowBytes = 32 * (BF16 ? 2 : 4), kTileBytes = kThreads * kRowBytes;
     __shared__ __align__(16) float2 s_grid[kMaxGridCells + 1];
     __shared__ __align__(16) float2 s_cell[TQ_MAX_LEVELS];
@@ -506,16 +488,14 @@ compress_tma_kernel(const __grid_constant__ CUtensorMap tmap, const void* __rest
         // makes the give-up decision uniform.
         if (__syncthreads_or(!ok)) { expired = true; break; }
         if (threadIdx.x == 0 && tile + gridDim.x < n_tiles) issue(tile + gridDim.x);
-        if (run < interior) quantize_run<BITS, kGrid, BF16, false>(g, prow, run, d, words_out, first_worker + wi, rk, cx);
+        if (run < interior) quantize_run<BITS, kGrid, BF16>(g, prow, run, first_worker + wi, rk, cx);
     }
     if (expired) {
         atomicAdd(&g_compress_wait_expired, 1u);
         if (threadIdx.x == 0) mbar_wait(bar, parity ^ 1u);            // the copy that did not land in time
         return;
     }
-    // the row's last run, by the thread that the striding would have given it to
-    if ((interior / kThreads) % gridDim.x == blockIdx.x && interior % kThreads == threadIdx.x)
-        compress_run<BITS, kGrid, BF16, true>(row, prow, interior, d, words_out, first_worker + wi, rk, cx);
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x < 32) compress_last_run<BITS, false, BF16>(row, prow, d, first_worker + wi, rk, q);
 }
 
 cudaError_t read_compress_wait_expired(unsigned int* count) {
@@ -528,125 +508,127 @@ __device__ __forceinline__ uint32_t cell_index(float g, float alpha, float inv_2
 }
 
 // Quantizers read from device memory (tq_params_device): no host round trip before the launch.
-// Thread 0 turns worker wi's tq_params_t into the kernel's WorkerQ, including the choice of the lookup
-// grid.  Returns false when this block has nothing to do in a kernel of kind FALLBACK:
-//   FALLBACK = false (main kernel): uniform rows, rows with a lookup grid, and all-zero rows for workers
-//              marked invalid (alpha = 0);
-//   FALLBACK = true: only the rows whose levels no grid separates (binary search).  It is launched
-//              after the main kernel and its blocks return at once for every other row, so the rarely
-//              needed path costs one near-empty launch instead of registers in the main kernel.
+// The block turns a job's tq_params_t into the kernel's WorkerQ, including the choice of the lookup grid (the lanes of
+// the first warp try one resolution each).  Ends with a block barrier.
 template <int BITS, bool NONUNIFORM>
-__device__ __forceinline__ void load_worker(const tq_params_t* __restrict__ params, uint32_t wi, WorkerQ& s_q) {
-    if (threadIdx.x < TQ_MAX_LEVELS) {
-        s_q.levels[threadIdx.x] = params[wi].levels[threadIdx.x];
-        s_q.inv_width[threadIdx.x] = params[wi].inv_width[threadIdx.x];
-    }
-    __syncthreads();                 // the levels are in shared memory from here on
-    if (threadIdx.x == 0) {
-        const tq_params_t& p = params[wi];
-        const float alpha = p.alpha;
+__device__ __forceinline__ void load_worker(const tq_params_t& p, WorkerQ& s_q) {
+    if (threadIdx.x < 32) {
+        const uint32_t lane = threadIdx.x;
+        if (lane < TQ_MAX_LEVELS) {
+            s_q.levels[lane] = p.levels[lane];
+            s_q.inv_width[lane] = p.inv_width[lane];
+        }
+        __syncwarp();
+        const float alpha = p.alpha, inv_step = p.inv_step;
         const bool ok = alpha > 0.0f && p.bits == BITS && !(p.flags & TQ_FLAG_INVALID);
         const float inv_2alpha = ok ? __fdiv_rn(1.0f, __fmul_rn(2.0f, alpha)) : 0.0f;
-        s_q.alpha = ok ? alpha : 0.0f;
-        s_q.inv_step = p.inv_step;
-        s_q.inv_step_l = scaled_inv_step(p.inv_step, 1u << BITS);
-        s_q.top = static_cast<float>((1 << BITS) - 1);
-        s_q.inv_2alpha = inv_2alpha;
         uint32_t cells = 0;
-        if (NONUNIFORM && ok && inv_2alpha <= 3.402823466e38f) {
+        if constexpr (NONUNIFORM) {
             constexpr int s = (1 << BITS) - 1;
-            for (uint32_t m = kMinGridCells; m <= static_cast<uint32_t>(kMaxGridCells) && cells == 0; m *= 2) {
-                bool distinct = true;
-                uint32_t prev = s >= 2 ? cell_index(s_q.levels[1], alpha, inv_2alpha, m) : 0u;
+            const uint32_t m = static_cast<uint32_t>(kMinGridCells) << lane;     // only lanes with m <= kMaxGridCells count
+            bool distinct = ok && inv_2alpha <= 3.402823466e38f && lane < 16 && m <= static_cast<uint32_t>(kMaxGridCells);
+            uint32_t prev = s >= 2 ? cell_index(s_q.levels[1], alpha, inv_2alpha, m) : 0u;
 #pragma unroll
-                for (int j = 2; j <= s - 1; ++j) {
-                    const uint32_t cur = cell_index(s_q.levels[j], alpha, inv_2alpha, m);
-                    distinct = distinct && cur > prev;
-                    prev = cur;
-                }
-                if (distinct) cells = m;
+            for (int j = 2; j <= s - 1; ++j) {
+                const uint32_t cur = cell_index(s_q.levels[j], alpha, inv_2alpha, m);
+                distinct = distinct && cur > prev;
+                prev = cur;
             }
+            const uint32_t fits = __ballot_sync(0xFFFFFFFFu, distinct);
+            if (fits) cells = static_cast<uint32_t>(kMinGridCells) << (__ffs(static_cast<int>(fits)) - 1);
         }
-        s_q.cells = cells;
-        s_q.cell_scale = __uint_as_float(cells);
+        if (lane == 0) {
+            s_q.alpha = ok ? alpha : 0.0f;
+            s_q.inv_step = inv_step;
+            s_q.inv_step_l = scaled_inv_step(inv_step, 1u << BITS);
+            s_q.top = static_cast<float>((1 << BITS) - 1);
+            s_q.inv_2alpha = inv_2alpha;
+            s_q.cells = cells;
+            s_q.cell_scale = __uint_as_float(cells);
+        }
     }
     __syncthreads();
 }
 
-// Where a job's row and packed words are.  Without segments job wi is worker wi and its whole slice; with
-// segments it is the pair (worker, segment) = (wi / n, wi % n) and a piece of that worker's row.
-struct JobPlace {
-    const char* row; uint32_t* prow; uint64_t d, words_out; uint32_t worker;
+// What a block of the device-parameter kernel keeps in shared memory.  Its place in its range of pieces is there too, and
+// is read back where it is needed, so that the loop over a piece's runs has the registers to itself.
+template <bool NONUNIFORM>
+struct BlockState {
+    float2 grid[NONUNIFORM ? kMaxGridCells + 1 : 1];
+    float2 cell[TQ_MAX_LEVELS];
+    float search[2 * TQ_MAX_LEVELS];
+    WorkerQ q;
+    JobPiece piece;
+    uint64_t cur;
 };
-template <int BITS, bool BF16>
-__device__ __forceinline__ JobPlace place_job(uint32_t wi, const void* grad, uint64_t d, uint64_t grad_stride, uint32_t first_worker,
-                                              uint32_t* packed, uint64_t words_stride, uint64_t words_out, const SegTable& segs) {
+
+// The piece in sh.piece.
+template <int BITS, int SEARCH, bool BF16, class State>
+__device__ __forceinline__ void compress_piece(State& sh, const void* __restrict__ grad, uint64_t grad_stride, const RoundKeys& rk,
+                                               uint32_t first_worker, uint32_t* __restrict__ packed, uint64_t words_stride,
+                                               const TilePlan& plan) {
     constexpr size_t esz = BF16 ? 2 : 4;
-    if (segs.n == 0)
-        return JobPlace{static_cast<const char*>(grad) + static_cast<uint64_t>(wi) * grad_stride * esz,
-                        packed + static_cast<uint64_t>(wi) * words_stride, d, words_out, first_worker + wi};
-    const uint32_t w = wi / segs.n, sg = wi - w * segs.n;
-    const uint64_t len = segs.len[sg];
-    return JobPlace{static_cast<const char*>(grad) + (static_cast<uint64_t>(w) * grad_stride + segs.off[sg]) * esz,
-                    packed + static_cast<uint64_t>(w) * words_stride + segs.woff[sg], len,
-                    (((len * BITS + 31) >> 5) + 3) & ~static_cast<uint64_t>(3), first_worker + w};
+    build_tables<BITS, SEARCH>(sh.q, sh.grid, sh.cell, sh.search);
+    const RunCtx cx{sh.q.alpha, sh.q.inv_step, sh.q.top, sh.q.inv_2alpha, sh.q.cell_scale, uniform_q<BITS>(sh.q),
+                    reinterpret_cast<const char*>(sh.grid), reinterpret_cast<const char*>(sh.cell), sh.search};
+    const char* row = static_cast<const char*>(grad) + (static_cast<uint64_t>(sh.piece.worker) * grad_stride + sh.piece.off) * esz;
+    uint32_t* prow = packed + static_cast<uint64_t>(sh.piece.worker) * words_stride + plan.segs.woff[sh.piece.seg];
+    const uint32_t worker = first_worker + sh.piece.worker;
+    const uint64_t whole = (sh.piece.d - 1) >> 5, stop = sh.piece.tile1 * kThreads;       // runs before the row's last one are whole
+    const uint64_t end = stop < whole ? stop : whole;
+    for (uint64_t run = sh.piece.tile0 * kThreads + threadIdx.x; run < end; run += kThreads)
+        compress_run<BITS, SEARCH, BF16>(row, prow, run, worker, rk, cx);
+    if (sh.piece.last && threadIdx.x < 32) compress_last_run<BITS, is_uniform(SEARCH), BF16>(row, prow, sh.piece.d, worker, rk, sh.q);
 }
 
+// The same for a quantizer that needs one of the rare arithmetics (levels that no grid separates: binary search; alpha too
+// large for the scaled inverse step).  Out of line, so that it costs the common loop no registers: as a second kernel
+// behind the first, which nearly always found nothing to do, it was 2-3 us of every call.
+template <int BITS, int SEARCH, bool BF16, class State>
+__device__ __noinline__ void compress_piece_rare(State& sh, const void* grad, uint64_t grad_stride, const RoundKeys& rk, uint32_t first_worker,
+                                                 uint32_t* packed, uint64_t words_stride, const TilePlan& plan) {
+    compress_piece<BITS, SEARCH, BF16>(sh, grad, grad_stride, rk, first_worker, packed, words_stride, plan);
+}
+
+// The block's pieces of the jobs -- workers, or (worker, segment) pairs, see TilePlan; a tile is one run per thread.
+// Rows of jobs that are marked invalid (alpha = 0) become all code 0.
 template <int BITS, bool NONUNIFORM, bool BF16>
 __global__ void __launch_bounds__(kThreads, TQ_COMPRESS_MIN_BLOCKS)
-compress_kernel_dev(const void* __restrict__ grad, uint64_t d, uint64_t grad_stride,
-                    const tq_params_t* __restrict__ params, const __grid_constant__ RoundKeys rk,
-                    uint32_t first_worker, uint32_t* __restrict__ packed, uint64_t words_stride, uint64_t words_out,
-                    const __grid_constant__ SegTable segs, int table_kernel_ran) {
-    if (table_kernel_ran) {          // rows the decision-table kernel served are done (same rule, evaluated by every thread)
-        uint32_t top, base;
-        if (lut_serves_record(params[blockIdx.y], BITS, &top, &base)) return;
-    }
-    __shared__ __align__(16) float2 s_grid[NONUNIFORM ? kMaxGridCells + 1 : 1];
-    __shared__ __align__(16) float2 s_cell[TQ_MAX_LEVELS];
-    __shared__ float s_search[2 * TQ_MAX_LEVELS];
-    __shared__ WorkerQ s_q;
-    const uint32_t wi = blockIdx.y;
-    const JobPlace job = place_job<BITS, BF16>(wi, grad, d, grad_stride, first_worker, packed, words_stride, words_out, segs);
-    load_worker<BITS, NONUNIFORM>(params, wi, s_q);
-    if (!(s_q.alpha > 0.0f)) {       // invalid parameters: the row is all code 0
-        for (uint64_t w = static_cast<uint64_t>(blockIdx.x) * kThreads + threadIdx.x; w < job.words_out;
-             w += static_cast<uint64_t>(gridDim.x) * kThreads)
-            job.prow[w] = 0u;
-        return;
-    }
-    if constexpr (NONUNIFORM) {
-        if (s_q.cells == 0) return;  // left to compress_kernel_dev_fallback
-    }
-    if constexpr (!NONUNIFORM) {
-        if (s_q.inv_step_l == 0.0f) {    // alpha too large for the scaled inverse step
-            compress_row<BITS, kUniformWide, BF16>(s_q, s_grid, s_cell, s_search, job.row, job.d, rk, job.worker, job.prow, job.words_out);
-            return;
+compress_kernel_dev(const void* __restrict__ grad, uint64_t grad_stride, const tq_params_t* __restrict__ params,
+                    const __grid_constant__ RoundKeys rk, uint32_t first_worker, uint32_t* __restrict__ packed, uint64_t words_stride,
+                    const __grid_constant__ TilePlan plan, int table_kernel_ran) {
+    __shared__ __align__(16) BlockState<NONUNIFORM> sh;
+    if (threadIdx.x == 0) sh.cur = first_tile_of_block(plan, blockIdx.x);
+    while (true) {
+        __syncthreads();                 // the previous piece has been served
+        const uint64_t range_end = first_tile_of_block(plan, blockIdx.x + 1);
+        if (sh.cur >= range_end) return;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            uint64_t cur = sh.cur;
+            sh.piece = next_piece(plan, cur, range_end);
+            sh.cur = cur;
+        }
+        __syncthreads();
+        const tq_params_t& p = params[sh.piece.job];
+        if (table_kernel_ran) {          // rows the decision-table kernel served are done (same rule, evaluated by every thread)
+            uint32_t top, base;
+            if (lut_serves_record(p, BITS, &top, &base)) continue;
+        }
+        load_worker<BITS, NONUNIFORM>(p, sh.q);
+        if (!(sh.q.alpha > 0.0f)) {
+            uint32_t* prow = packed + static_cast<uint64_t>(sh.piece.worker) * words_stride + plan.segs.woff[sh.piece.seg];
+            const uint64_t words_out = (((sh.piece.d * BITS + 31) >> 5) + 3) & ~static_cast<uint64_t>(3);
+            const uint64_t w1 = sh.piece.last ? words_out : sh.piece.tile1 * kThreads * BITS;
+            for (uint64_t w = sh.piece.tile0 * kThreads * BITS + threadIdx.x; w < w1; w += kThreads) prow[w] = 0u;
+        } else if (NONUNIFORM && sh.q.cells == 0) {
+            compress_piece_rare<BITS, kBinary, BF16>(sh, grad, grad_stride, rk, first_worker, packed, words_stride, plan);
+        } else if (!NONUNIFORM && sh.q.inv_step_l == 0.0f) {
+            compress_piece_rare<BITS, kUniformWide, BF16>(sh, grad, grad_stride, rk, first_worker, packed, words_stride, plan);
+        } else {
+            compress_piece<BITS, NONUNIFORM ? kGrid : kUniform, BF16>(sh, grad, grad_stride, rk, first_worker, packed, words_stride, plan);
         }
     }
-    compress_row<BITS, NONUNIFORM ? kGrid : kUniform, BF16>(s_q, s_grid, s_cell, s_search, job.row, job.d, rk, job.worker, job.prow,
-                                                            job.words_out);
-}
-
-template <int BITS, bool BF16>
-__global__ void __launch_bounds__(kThreads, TQ_COMPRESS_MIN_BLOCKS)
-compress_kernel_dev_fallback(const void* __restrict__ grad, uint64_t d, uint64_t grad_stride,
-                             const tq_params_t* __restrict__ params, const __grid_constant__ RoundKeys rk,
-                             uint32_t first_worker, uint32_t* __restrict__ packed, uint64_t words_stride, uint64_t words_out,
-                             const __grid_constant__ SegTable segs, int table_kernel_ran) {
-    if (table_kernel_ran) {
-        uint32_t top, base;
-        if (lut_serves_record(params[blockIdx.y], BITS, &top, &base)) return;
-    }
-    __shared__ __align__(16) float2 s_grid[1];
-    __shared__ __align__(16) float2 s_cell[TQ_MAX_LEVELS];
-    __shared__ float s_search[2 * TQ_MAX_LEVELS];
-    __shared__ WorkerQ s_q;
-    const uint32_t wi = blockIdx.y;
-    const JobPlace job = place_job<BITS, BF16>(wi, grad, d, grad_stride, first_worker, packed, words_stride, words_out, segs);
-    load_worker<BITS, true>(params, wi, s_q);
-    if (!(s_q.alpha > 0.0f) || s_q.cells != 0) return;
-    compress_row<BITS, kBinary, BF16>(s_q, s_grid, s_cell, s_search, job.row, job.d, rk, job.worker, job.prow, job.words_out);
 }
 
 // ---- host side ---------------------------------------------------------------------------------------
@@ -689,7 +671,7 @@ static dim3 compress_grid(uint64_t d, uint32_t n_workers, bool persistent) {
 template <int BITS, int SEARCH, bool BF>
 static cudaError_t launch(const CompressCall& c, const CompressArgs& args, dim3 grid) {
     compress_kernel<BITS, SEARCH, BF><<<grid, kThreads, 0, c.stream>>>(
-        c.grad, c.d, c.grad_stride, args, round_keys(c.seed), c.first_worker, c.packed, c.words_stride, c.words_out);
+        c.grad, c.d, c.grad_stride, args, round_keys(c.seed), c.first_worker, c.packed, c.words_stride);
     return cudaGetLastError();
 }
 
@@ -739,7 +721,7 @@ static cudaError_t launch_tma(const CompressCall& c, const CompressArgs& args, d
     const cudaError_t e = cudaFuncSetAttribute(compress_tma_kernel<BITS, BF>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     compress_tma_kernel<BITS, BF><<<grid, kThreads, smem, c.stream>>>(
-        map, c.grad, c.d, c.grad_stride, args, round_keys(c.seed), c.first_worker, c.packed, c.words_stride, c.words_out);
+        map, c.grad, c.d, c.grad_stride, args, round_keys(c.seed), c.first_worker, c.packed, c.words_stride);
     return cudaGetLastError();
 }
 
@@ -792,52 +774,30 @@ cudaError_t launch_compress(const CompressCall& c) {
     }
 }
 
-static const SegTable kNoSegments{};
-
-template <int BITS, bool NU, bool BF>
-static cudaError_t launch_dev(const CompressCall& c, dim3 grid, int table_kernel_ran) {
-    const RoundKeys rk = round_keys(c.seed);
-    const SegTable& segs = c.segs ? *c.segs : kNoSegments;
-    compress_kernel_dev<BITS, NU, BF><<<grid, kThreads, 0, c.stream>>>(
-        c.grad, c.d, c.grad_stride, c.params_dev, rk, c.first_worker, c.packed, c.words_stride, c.words_out, segs, table_kernel_ran);
-    if constexpr (NU) {
-        if (cudaError_t e = cudaGetLastError()) return e;
-        // a small grid: this pass is empty unless a codebook is too crowded for the lookup grid
-        const dim3 small(grid.x < 16 ? grid.x : 16, grid.y);
-        compress_kernel_dev_fallback<BITS, BF><<<small, kThreads, 0, c.stream>>>(
-            c.grad, c.d, c.grad_stride, c.params_dev, rk, c.first_worker, c.packed, c.words_stride, c.words_out, segs, table_kernel_ran);
-    }
-    return cudaGetLastError();
-}
 template <int BITS>
-static cudaError_t dispatch_dev(const CompressCall& c, dim3 grid, int lut) {
-    if (c.nonuniform) return c.bf16 ? launch_dev<BITS, true, true>(c, grid, lut) : launch_dev<BITS, true, false>(c, grid, lut);
-    return c.bf16 ? launch_dev<BITS, false, true>(c, grid, lut) : launch_dev<BITS, false, false>(c, grid, lut);
+static cudaError_t dispatch_dev(const CompressCall& c, const TilePlan& plan, int table_kernel_ran) {
+    const auto kernel = c.nonuniform ? (c.bf16 ? compress_kernel_dev<BITS, true, true> : compress_kernel_dev<BITS, true, false>)
+                                     : (c.bf16 ? compress_kernel_dev<BITS, false, true> : compress_kernel_dev<BITS, false, false>);
+    kernel<<<plan.blocks, kThreads, 0, c.stream>>>(c.grad, c.grad_stride, c.params_dev, round_keys(c.seed), c.first_worker, c.packed,
+                                                   c.words_stride, plan, table_kernel_ran);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_compress_dev(const CompressCall& c) {
-    // with segments: one grid row per (worker, segment) pair, sized by the longest segment
-    uint64_t d = c.d;
-    uint32_t jobs = c.n_workers;
-    if (c.segs) {
-        d = 0;
-        for (uint32_t sg = 0; sg < c.segs->n; ++sg) d = c.segs->len[sg] > d ? c.segs->len[sg] : d;
-        jobs = c.n_workers * c.segs->n;
-    }
-    // always the persistent grid here: a block first reads its quantizer from device memory and prepares it (two
-    // barriers and a global round trip), which one block per tile would pay 120 000 times on a large row
-    dim3 grid = compress_grid(d, jobs, true);
     // bf16 table codebooks: the decision-table kernel first; it serves the rows its window fits and the element-wise
-    // kernels (a small grid then: they normally find nothing left) take the others
+    // kernel (a small grid then: it normally finds nothing left) takes the others
     bool lut = false;
     if (const cudaError_t e = launch_compress_lut(c, &lut)) return e;
-    if (lut && grid.x > 16) grid.x = 16;
-    if (c.launches) *c.launches = (c.nonuniform ? 2 : 1) + (lut ? 1 : 0);
+    int dev = 0, sms = 148;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    static thread_local TilePlan plan;
+    plan_tiles(&plan, c.segs, c.d, c.n_workers, 32 * kThreads, static_cast<uint64_t>(sms) * (lut ? 1 : TQ_COMPRESS_MIN_BLOCKS));
+    if (c.launches) *c.launches = lut ? 2 : 1;
     switch (c.bits) {
-        case 1: return dispatch_dev<1>(c, grid, lut);
-        case 2: return dispatch_dev<2>(c, grid, lut);
-        case 3: return dispatch_dev<3>(c, grid, lut);
-        default: return dispatch_dev<4>(c, grid, lut);
+        case 1: return dispatch_dev<1>(c, plan, lut);
+        case 2: return dispatch_dev<2>(c, plan, lut);
+        case 3: return dispatch_dev<3>(c, plan, lut);
+        default: return dispatch_dev<4>(c, plan, lut);
     }
 }
 

@@ -4,6 +4,7 @@
 #include <stdint.h>
 
 #include "tq.h"
+#include "tq_launch.h"
 
 namespace tq {
 
@@ -188,6 +189,47 @@ __device__ __forceinline__ void philox_block(uint32_t c0, const PhiloxRun& pr, c
         x3 = lo0;
     }
     out[0] = x0; out[1] = x1; out[2] = x2; out[3] = x3;
+}
+
+// ---- a block's pieces (see TilePlan) ---------------------------------------------------------------
+struct JobPiece {
+    uint32_t worker, seg, job;
+    uint64_t tile0, tile1;         // the piece's tiles, counted from the job's first
+    uint64_t d, off;               // the job's elements, and where they start in the worker's row
+    bool last;                     // the piece holds the job's last tile
+};
+__device__ __forceinline__ uint64_t first_tile_of_block(const TilePlan& plan, uint32_t b) {
+    return b * plan.per_block + b * plan.rest / plan.blocks;           // b * rest < blocks^2 < 2^32
+}
+__device__ __forceinline__ uint32_t block_of_tile(const TilePlan& plan, uint64_t t) {
+    uint32_t b = static_cast<uint32_t>(static_cast<double>(t) * plan.blocks_per_tile);
+    while (first_tile_of_block(plan, b) > t) --b;
+    while (first_tile_of_block(plan, b + 1) <= t) ++b;
+    return b;
+}
+// The piece that starts at tile `cur` of the range [.., end); cur moves on to the next one.
+__device__ __forceinline__ JobPiece next_piece(const TilePlan& plan, uint64_t& cur, uint64_t end) {
+    JobPiece p;
+    p.worker = static_cast<uint32_t>(static_cast<double>(cur) * plan.rows_per_tile);      // below 2^53: at most one off
+    while (p.worker * plan.per_worker > cur) --p.worker;
+    while ((p.worker + 1) * plan.per_worker <= cur) ++p.worker;
+    const uint64_t row0 = p.worker * plan.per_worker, in_row = cur - row0;
+    p.seg = 0;
+    while (p.seg + 1 < plan.segs.n && plan.begin[p.seg + 1] <= in_row) ++p.seg;
+    p.job = p.worker * plan.segs.n + p.seg;
+    const uint64_t job_end = row0 + plan.begin[p.seg + 1], stop = end < job_end ? end : job_end;
+    p.tile0 = in_row - plan.begin[p.seg];
+    p.tile1 = p.tile0 + (stop - cur);
+    p.last = stop == job_end;
+    p.d = plan.segs.len[p.seg]; p.off = plan.segs.off[p.seg];
+    cur = stop;
+    return p;
+}
+// First and last block that have a piece of the job.
+__device__ __forceinline__ void blocks_of_job(const TilePlan& plan, const JobPiece& p, uint32_t& first, uint32_t& last) {
+    const uint64_t row0 = p.worker * plan.per_worker;
+    first = block_of_tile(plan, row0 + plan.begin[p.seg]);
+    last = block_of_tile(plan, row0 + plan.begin[p.seg + 1] - 1);
 }
 
 // ---- warp / block reductions -----------------------------------------------------------------------

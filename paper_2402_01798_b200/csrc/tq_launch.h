@@ -18,6 +18,46 @@ struct SegTable {
     uint64_t woff[TQ_MAX_SEGMENTS];   // first word of the segment's packed bits in the worker's packed row
 };
 
+// All jobs' tiles, numbered worker after worker and segment after segment, cut into one contiguous range per block.
+// A block's share of one job is a "piece"; a range that crosses a job's end consists of several.  Block b and job j
+// have at most one piece, and b + j is different for every piece.
+//
+// Why ranges and not a grid row per job: jobs differ in length (layer groups by a factor of 75 and more) and rarely
+// divide the resident blocks evenly; a range is within one tile of every other.  Measured on
+// 25.6 M x 16 cut into 16 groups of unequal size: statistics 1142 -> 274 us, compress 1076 -> 402 us.
+struct TilePlan {
+    uint64_t per_worker;          // tiles of one worker's row
+    uint64_t per_block;           // block b starts at tile floor(b * total / blocks) = b * per_block + floor(b * rest / blocks)
+    uint32_t rest, blocks;
+    double rows_per_tile, blocks_per_tile;   // 1 / per_worker, blocks / total: estimates of quotients, corrected by the user
+    SegTable segs;                // without segments: one that covers the row
+    uint64_t begin[TQ_MAX_SEGMENTS + 1];   // first tile of each segment within the worker's tiles
+};
+// segs may be null: one segment of d elements per worker.  At least one tile per job, at most `resident` blocks.
+// Equal rows get a whole number of blocks each where that leaves at most 1/24 of the resident blocks out: a block with two
+// pieces pays the end of a piece twice, and all wait for it (11.2 M x 8: statistics 75.7 us with, 73 us without such blocks).
+inline void plan_tiles(TilePlan* plan, const SegTable* segs, uint64_t d, uint32_t n_workers, uint64_t tile_elems, uint64_t resident) {
+    if (segs) plan->segs = *segs;
+    else { plan->segs.n = 1; plan->segs.off[0] = 0; plan->segs.len[0] = d; plan->segs.woff[0] = 0; }
+    uint64_t tiles = 0;
+    for (uint32_t s = 0; s < plan->segs.n; ++s) {
+        plan->begin[s] = tiles;
+        const uint64_t t = (plan->segs.len[s] + tile_elems - 1) / tile_elems;
+        tiles += t ? t : 1;
+    }
+    plan->begin[plan->segs.n] = tiles;
+    plan->per_worker = tiles;
+    const uint64_t total = tiles * n_workers;
+    uint64_t blocks = total < resident ? total : resident;
+    const uint64_t even = blocks / n_workers * n_workers;
+    if (plan->segs.n == 1 && even > 0 && (blocks - even) * 24 <= blocks) blocks = even;
+    plan->blocks = static_cast<uint32_t>(blocks);
+    plan->per_block = total / blocks;
+    plan->rest = static_cast<uint32_t>(total % blocks);
+    plan->rows_per_tile = 1.0 / static_cast<double>(tiles);
+    plan->blocks_per_tile = static_cast<double>(blocks) / static_cast<double>(total);
+}
+
 struct CompressCall {
     const void* grad; bool bf16; uint64_t d, grad_stride; uint32_t n_workers;
     const tq_params_t* params;       // host array, or

@@ -3,10 +3,11 @@
 // sum ln(|g_j| / g_min) (the two ingredients of the maximum-likelihood tail index of Section 5 and of
 // rho, the tail mass of Section 4.1).
 //
-// Shape: grid = (blocks per worker, workers).  A thread walks 16-element chunks with a block-wide
+// Shape: the tiles (4096 elements) of all jobs -- workers, or (worker, segment) pairs -- are cut into one range
+// per resident block (TilePlan).  Within its piece of a job a thread walks 16-element chunks with a block-wide
 // stride, keeps fp32 partial sums inside a chunk and fp64 sums across chunks, then the block reduces
-// with warp shuffles and writes ONE partial record to scratch.  A ticket counter (one atomic per
-// block) tells the last block of a worker to fold that worker's records in index order, so the result
+// with warp shuffles and writes ONE partial record per piece to scratch.  A ticket counter (one atomic per
+// piece) tells the last block of a job to fold that job's records in index order, so the result
 // does not depend on which block finishes last.  No block ever waits for another.
 //
 // With an automatic threshold (g_min = kappa * mean|g|) the tail quantities need the mean first:
@@ -22,17 +23,26 @@
 
 namespace tq {
 
-constexpr int kMaxBlocksPerWorker = 1024;
+constexpr int kRecordsPerJob = 1024;          // scratch records per job: a call has at most blocks + jobs pieces
 constexpr int kChunk = 16;
+constexpr int kTile = kChunk * kThreads;      // elements
 
 struct alignas(64) Partial {
     double sum_abs, sum_sq, sum_log2;
     unsigned long long n_tail, n_bad;
     float max_abs, pad;
 };
-// scratch layout: [n_workers][kMaxBlocksPerWorker] Partial, then [n_workers][2] tickets (uint32)
-__host__ __device__ inline size_t tickets_offset(uint32_t n_workers) {
-    return static_cast<size_t>(n_workers) * kMaxBlocksPerWorker * sizeof(Partial);
+// scratch layout for n jobs: [n * kRecordsPerJob] Partial (piece of block b and job j: record b + j), then [n][2] tickets (uint32)
+__host__ __device__ inline size_t tickets_offset(uint32_t n_jobs) {
+    return static_cast<size_t>(n_jobs) * kRecordsPerJob * sizeof(Partial);
+}
+static void plan_stats(const StatsCall& c, uint32_t n_jobs, int ranges_per_sm, TilePlan* plan) {
+    int dev = 0, sms = 148;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    uint64_t resident = static_cast<uint64_t>(sms) * ranges_per_sm;
+    const uint64_t room = static_cast<uint64_t>(n_jobs) * kRecordsPerJob - n_jobs;
+    if (resident > room) resident = room;
+    plan_tiles(plan, c.segs, c.d, c.n_workers, kTile, resident);
 }
 size_t stats_workspace_bytes(uint32_t n_workers) {
     return tickets_offset(n_workers) + static_cast<size_t>(n_workers) * 2 * sizeof(uint32_t) + 256;
@@ -50,20 +60,29 @@ __device__ __forceinline__ float fma_sat(float a, float b, float c) {
     float r; asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c)); return r;
 }
 
+// Resident blocks per SM.  fp32 rows are bound by HBM and do best with few blocks (25.6 M x 16, moments + tail, 3 / 4 / 5 / 6
+// blocks: 485 / 478 / 503 / 507 us); bf16 rows are bound by instructions and latency and want the warps (124 M x 8, the same:
+// 888 / 754 / 719 / 691 us), and two ranges per resident block, which even out the SMs, where a range stays long enough
+// (668 us; 1 M x 8: 29 instead of 24 us, so short rows keep one).
+constexpr int stats_blocks_per_sm(bool bf16, int pass) { return !bf16 ? 4 : pass == kBoth ? 5 : 6; }
+constexpr uint64_t kTilesForTwoRanges = 64;      // per resident block
+
+struct BlockFold {
+    double d[4][kThreads / 32];
+    unsigned long long u[3][kThreads / 32];
+    float f[kThreads / 32];
+    bool last;
+};
+
+// A block's piece of one job.
 template <bool BF16, int PASS>
-__global__ void __launch_bounds__(kThreads)
-stats_kernel(const void* __restrict__ grad, uint64_t d_row, uint64_t grad_stride, float g_min_in, float kappa,
-             tq_stats_t* __restrict__ stats, Partial* __restrict__ partials, uint32_t* __restrict__ tickets,
-             const __grid_constant__ SegTable segs) {
-    const uint32_t wi = blockIdx.y;          // the job: a worker, or a (worker, segment) pair
+__device__ __forceinline__ void stats_piece(const JobPiece& piece, const TilePlan& plan, const void* __restrict__ grad, uint64_t grad_stride,
+                                            float g_min_in, float kappa, tq_stats_t* __restrict__ stats,
+                                            Partial* __restrict__ partials, uint32_t* __restrict__ tickets, BlockFold& sh) {
     const size_t esz = BF16 ? 2 : 4;
-    uint64_t d = d_row;
-    const char* row = static_cast<const char*>(grad) + static_cast<uint64_t>(wi) * grad_stride * esz;
-    if (segs.n) {
-        const uint32_t worker = wi / segs.n, sg = wi - worker * segs.n;
-        row = static_cast<const char*>(grad) + (static_cast<uint64_t>(worker) * grad_stride + segs.off[sg]) * esz;
-        d = segs.len[sg];
-    }
+    const uint32_t wi = piece.job;
+    const uint64_t d = piece.d;
+    const char* row = static_cast<const char*>(grad) + (static_cast<uint64_t>(piece.worker) * grad_stride + piece.off) * esz;
 
     float g_min = g_min_in;
     if constexpr (PASS == kTail) g_min = stats[wi].g_min;     // finished by the moments pass
@@ -77,9 +96,8 @@ stats_kernel(const void* __restrict__ grad, uint64_t d_row, uint64_t grad_stride
     unsigned long long n_tail = 0, n_bad = 0;
     float max_abs = 0.0f;
 
-    const uint64_t n_chunks = d / kChunk;
-    const uint64_t stride = static_cast<uint64_t>(gridDim.x) * kThreads;
-    for (uint64_t c = static_cast<uint64_t>(blockIdx.x) * kThreads + threadIdx.x; c < n_chunks; c += stride) {
+    const uint64_t n_chunks = d / kChunk, chunk_end = piece.tile1 * kThreads < n_chunks ? piece.tile1 * kThreads : n_chunks;
+    for (uint64_t c = piece.tile0 * kThreads + threadIdx.x; c < chunk_end; c += kThreads) {
         float g[2][8];
         load8<BF16>(row + (c * kChunk) * esz, g[0]);
         load8<BF16>(row + (c * kChunk + 8) * esz, g[1]);
@@ -131,8 +149,8 @@ stats_kernel(const void* __restrict__ grad, uint64_t d_row, uint64_t grad_stride
             }
         }
     }
-    // the d % 16 leftover elements, taken by the first threads of block 0
-    if (blockIdx.x == 0) {
+    // the d % 16 leftover elements, taken by the first threads of the job's last piece
+    if (piece.last) {
         const uint64_t j = n_chunks * kChunk + threadIdx.x;
         if (j < d) {
             const float a = fabsf(load1<BF16>(row, j));
@@ -148,37 +166,35 @@ stats_kernel(const void* __restrict__ grad, uint64_t d_row, uint64_t grad_stride
     }
 
     // block reduction: shuffles inside a warp, shared memory across the 8 warps
-    __shared__ double s_d[3][kThreads / 32];
-    __shared__ unsigned long long s_u[2][kThreads / 32];
-    __shared__ float s_f[kThreads / 32];
-    __shared__ bool s_last;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     sum_abs = warp_sum(sum_abs); sum_sq = warp_sum(sum_sq); sum_log2 = warp_sum(sum_log2);
     n_tail = warp_sum(n_tail); n_bad = warp_sum(n_bad); max_abs = warp_max(max_abs);
     if (lane == 0) {
-        s_d[0][warp] = sum_abs; s_d[1][warp] = sum_sq; s_d[2][warp] = sum_log2;
-        s_u[0][warp] = n_tail; s_u[1][warp] = n_bad; s_f[warp] = max_abs;
+        sh.d[0][warp] = sum_abs; sh.d[1][warp] = sum_sq; sh.d[2][warp] = sum_log2;
+        sh.u[0][warp] = n_tail; sh.u[1][warp] = n_bad; sh.f[warp] = max_abs;
     }
     __syncthreads();
-    Partial* mine = partials + static_cast<size_t>(wi) * kMaxBlocksPerWorker;
+    uint32_t first_block, last_block;
+    blocks_of_job(plan, piece, first_block, last_block);
+    Partial* mine = partials + first_block + wi;                    // the job's records, one per block
     uint32_t* ticket = tickets + wi * 2 + (PASS == kTail ? 1 : 0);
     if (threadIdx.x == 0) {
         Partial p{};
         for (int w = 0; w < kThreads / 32; ++w) {
-            p.sum_abs += s_d[0][w]; p.sum_sq += s_d[1][w]; p.sum_log2 += s_d[2][w];
-            p.n_tail += s_u[0][w]; p.n_bad += s_u[1][w]; p.max_abs = fmaxf(p.max_abs, s_f[w]);
+            p.sum_abs += sh.d[0][w]; p.sum_sq += sh.d[1][w]; p.sum_log2 += sh.d[2][w];
+            p.n_tail += sh.u[0][w]; p.n_bad += sh.u[1][w]; p.max_abs = fmaxf(p.max_abs, sh.f[w]);
         }
-        mine[blockIdx.x] = p;
+        mine[blockIdx.x - first_block] = p;
         __threadfence();                                       // record visible before the ticket
-        s_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+        sh.last = atomicAdd(ticket, 1u) == last_block - first_block;
     }
     __syncthreads();
-    if (!s_last) return;
+    if (!sh.last) return;
 
-    // last block of this worker: fold the records in index order (fixed shape, deterministic)
+    // last block of this job: fold the records in index order (fixed shape, deterministic)
     __threadfence();
     Partial acc{};
-    for (uint32_t b = threadIdx.x; b < gridDim.x; b += kThreads) {
+    for (uint32_t b = threadIdx.x; b <= last_block - first_block; b += kThreads) {
         const volatile Partial* p = mine + b;
         acc.sum_abs += p->sum_abs; acc.sum_sq += p->sum_sq; acc.sum_log2 += p->sum_log2;
         acc.n_tail += p->n_tail; acc.n_bad += p->n_bad; acc.max_abs = fmaxf(acc.max_abs, p->max_abs);
@@ -187,15 +203,15 @@ stats_kernel(const void* __restrict__ grad, uint64_t d_row, uint64_t grad_stride
     acc.n_tail = warp_sum(acc.n_tail); acc.n_bad = warp_sum(acc.n_bad); acc.max_abs = warp_max(acc.max_abs);
     __syncthreads();
     if (lane == 0) {
-        s_d[0][warp] = acc.sum_abs; s_d[1][warp] = acc.sum_sq; s_d[2][warp] = acc.sum_log2;
-        s_u[0][warp] = acc.n_tail; s_u[1][warp] = acc.n_bad; s_f[warp] = acc.max_abs;
+        sh.d[0][warp] = acc.sum_abs; sh.d[1][warp] = acc.sum_sq; sh.d[2][warp] = acc.sum_log2;
+        sh.u[0][warp] = acc.n_tail; sh.u[1][warp] = acc.n_bad; sh.f[warp] = acc.max_abs;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
         Partial t{};
         for (int w = 0; w < kThreads / 32; ++w) {
-            t.sum_abs += s_d[0][w]; t.sum_sq += s_d[1][w]; t.sum_log2 += s_d[2][w];
-            t.n_tail += s_u[0][w]; t.n_bad += s_u[1][w]; t.max_abs = fmaxf(t.max_abs, s_f[w]);
+            t.sum_abs += sh.d[0][w]; t.sum_sq += sh.d[1][w]; t.sum_log2 += sh.d[2][w];
+            t.n_tail += sh.u[0][w]; t.n_bad += sh.u[1][w]; t.max_abs = fmaxf(t.max_abs, sh.f[w]);
         }
         tq_stats_t* st = stats + wi;
         if constexpr (PASS != kTail) {
@@ -216,54 +232,50 @@ stats_kernel(const void* __restrict__ grad, uint64_t d_row, uint64_t grad_stride
             st->n_tail = t.n_tail;
             st->sum_log_tail = (t.sum_log2 - corr) * 0.6931471805599453094;
         }
-        *ticket = 0u;                                          // ready for the next call on this scratch
     }
 }
 
-static const SegTable kNoSegments{};
+template <bool BF16, int PASS>
+__global__ void __launch_bounds__(kThreads, stats_blocks_per_sm(BF16, PASS))
+stats_kernel(const void* __restrict__ grad, uint64_t grad_stride, float g_min_in, float kappa,
+             tq_stats_t* __restrict__ stats, Partial* __restrict__ partials, uint32_t* __restrict__ tickets,
+             const __grid_constant__ TilePlan plan) {
+    __shared__ BlockFold sh;
+    uint64_t cur = first_tile_of_block(plan, blockIdx.x);
+    const uint64_t end = first_tile_of_block(plan, blockIdx.x + 1);
+    while (cur < end) {
+        stats_piece<BF16, PASS>(next_piece(plan, cur, end), plan, grad, grad_stride, g_min_in, kappa, stats, partials, tickets, sh);
+        __syncthreads();                                       // the next piece reuses the shared arrays
+    }
+}
 
 template <bool BF16, int PASS>
-static cudaError_t launch(const StatsCall& c, dim3 grid, Partial* partials, uint32_t* tickets) {
-    stats_kernel<BF16, PASS><<<grid, kThreads, 0, c.stream>>>(c.grad, c.d, c.grad_stride, c.g_min, c.kappa,
-                                                              c.stats, partials, tickets, c.segs ? *c.segs : kNoSegments);
+static cudaError_t launch(const StatsCall& c, const TilePlan& plan, Partial* partials, uint32_t* tickets) {
+    stats_kernel<BF16, PASS><<<plan.blocks, kThreads, 0, c.stream>>>(c.grad, c.grad_stride, c.g_min, c.kappa, c.stats, partials, tickets, plan);
     return cudaGetLastError();
 }
 
-cudaError_t launch_stats(const StatsCall& call, int* launches) {
+cudaError_t launch_stats(const StatsCall& c, int* launches) {
     *launches = 0;
-    // with segments every (worker, segment) pair is a job of its own: same kernels, same scratch layout
-    StatsCall c = call;
     const uint32_t n_jobs = c.segs ? c.n_workers * c.segs->n : c.n_workers;
-    if (c.segs) {
-        c.d = 0;
-        for (uint32_t sg = 0; sg < c.segs->n; ++sg) c.d = c.segs->len[sg] > c.d ? c.segs->len[sg] : c.d;   // sizes the grid
-    }
-    c.n_workers = n_jobs;
     Partial* partials = static_cast<Partial*>(c.workspace);
-    uint32_t* tickets = reinterpret_cast<uint32_t*>(static_cast<char*>(c.workspace) + tickets_offset(c.n_workers));
-    cudaError_t e = cudaMemsetAsync(tickets, 0, static_cast<size_t>(c.n_workers) * 2 * sizeof(uint32_t), c.stream);
+    uint32_t* tickets = reinterpret_cast<uint32_t*>(static_cast<char*>(c.workspace) + tickets_offset(n_jobs));
+    cudaError_t e = cudaMemsetAsync(tickets, 0, static_cast<size_t>(n_jobs) * 2 * sizeof(uint32_t), c.stream);
     if (e != cudaSuccess) return e;
-
-    int dev = 0, sms = 148;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    // 8 resident blocks of 256 threads per SM; spread them over the workers
-    const uint64_t chunks = c.d / kChunk;
-    uint64_t per_worker = static_cast<uint64_t>(sms) * 8 / c.n_workers;       // rounded down: a block beyond the resident set would run as a second wave
-    const uint64_t useful = (chunks + kThreads - 1) / kThreads;
-    if (per_worker > useful) per_worker = useful;
-    if (per_worker > kMaxBlocksPerWorker) per_worker = kMaxBlocksPerWorker;
-    if (per_worker < 1) per_worker = 1;
-    const dim3 grid(static_cast<unsigned>(per_worker), c.n_workers);
+    static thread_local TilePlan plan;
+    const int ranges = stats_blocks_per_sm(c.bf16, c.g_min > 0.0f ? kBoth : kMoments);
+    plan_stats(c, n_jobs, ranges, &plan);
+    if (c.bf16 && plan.per_block >= kTilesForTwoRanges) plan_stats(c, n_jobs, 2 * ranges, &plan);
 
     if (c.g_min > 0.0f) {
-        e = c.bf16 ? launch<true, kBoth>(c, grid, partials, tickets) : launch<false, kBoth>(c, grid, partials, tickets);
+        e = c.bf16 ? launch<true, kBoth>(c, plan, partials, tickets) : launch<false, kBoth>(c, plan, partials, tickets);
         *launches = 1;
         return e;
     }
-    e = c.bf16 ? launch<true, kMoments>(c, grid, partials, tickets) : launch<false, kMoments>(c, grid, partials, tickets);
+    e = c.bf16 ? launch<true, kMoments>(c, plan, partials, tickets) : launch<false, kMoments>(c, plan, partials, tickets);
     if (e != cudaSuccess) return e;
     *launches = 1;
-    e = c.bf16 ? launch<true, kTail>(c, grid, partials, tickets) : launch<false, kTail>(c, grid, partials, tickets);
+    e = c.bf16 ? launch<true, kTail>(c, plan, partials, tickets) : launch<false, kTail>(c, plan, partials, tickets);
     *launches = 2;
     return e;
 }
@@ -297,23 +309,18 @@ __device__ __forceinline__ float pow2_floor(float x) {
 #endif
 
 template <bool BF16, bool FALLBACK>
-__global__ void __launch_bounds__(kThreads, TQ_STATS_HINTED_BLOCKS)
-stats_hinted_kernel(const void* __restrict__ grad, uint64_t d_row, uint64_t grad_stride, float kappa,
-                    tq_gmin_hint_t* __restrict__ hint, tq_stats_t* __restrict__ stats,
-                    PartialH* __restrict__ partials, uint32_t* __restrict__ tickets, const __grid_constant__ SegTable segs) {
+__device__ __forceinline__ void stats_hinted_piece(const JobPiece& piece, const TilePlan& plan, const void* __restrict__ grad,
+                                                   uint64_t grad_stride, float kappa, tq_gmin_hint_t* __restrict__ hint,
+                                                   tq_stats_t* __restrict__ stats, PartialH* __restrict__ partials,
+                                                   uint32_t* __restrict__ tickets, BlockFold& sh) {
     constexpr int K = FALLBACK ? 1 : 2;
-    const uint32_t wi = blockIdx.y;               // the job: a worker, or a (worker, segment) pair
+    const size_t esz = BF16 ? 2 : 4;
+    const uint32_t wi = piece.job;
     if constexpr (FALLBACK) {
         if (hint[wi].hit) return;                 // the one-pass result stands
     }
-    const size_t esz = BF16 ? 2 : 4;
-    uint64_t d = d_row;
-    const char* row = static_cast<const char*>(grad) + static_cast<uint64_t>(wi) * grad_stride * esz;
-    if (segs.n) {
-        const uint32_t worker = wi / segs.n, sg = wi - worker * segs.n;
-        row = static_cast<const char*>(grad) + (static_cast<uint64_t>(worker) * grad_stride + segs.off[sg]) * esz;
-        d = segs.len[sg];
-    }
+    const uint64_t d = piece.d;
+    const char* row = static_cast<const char*>(grad) + (static_cast<uint64_t>(piece.worker) * grad_stride + piece.off) * esz;
 
     // candidate thresholds
     float t[2] = {CUDART_INF_F, CUDART_INF_F};
@@ -400,27 +407,26 @@ stats_hinted_kernel(const void* __restrict__ grad, uint64_t d_row, uint64_t grad
         }
     };
 
-    // A thread's chunks are c0, c0 + stride, ...; the loads of kAhead of them (128 bytes per thread) are
+    // A thread's chunks are c0, c0 + kThreads, ...; the loads of kAhead of them (128 bytes per thread) are
     // issued together, then they are summed in that same order.
     constexpr int kAhead = BF16 ? 4 : 2;
-    const uint64_t n_chunks = d / kChunk;
-    const uint64_t stride = static_cast<uint64_t>(gridDim.x) * kThreads;
-    for (uint64_t c = static_cast<uint64_t>(blockIdx.x) * kThreads + threadIdx.x; c < n_chunks; c += kAhead * stride) {
+    const uint64_t n_chunks = d / kChunk, chunk_end = piece.tile1 * kThreads < n_chunks ? piece.tile1 * kThreads : n_chunks;
+    for (uint64_t c = piece.tile0 * kThreads + threadIdx.x; c < chunk_end; c += kAhead * kThreads) {
         Raw8<BF16> g[kAhead][2];
 #pragma unroll
         for (int u = 0; u < kAhead; ++u) {
-            const uint64_t cu = c + u * stride;
-            if (cu < n_chunks) {
+            const uint64_t cu = c + u * kThreads;
+            if (cu < chunk_end) {
                 load8_raw<BF16>(row + (cu * kChunk) * esz, g[u][0]);
                 load8_raw<BF16>(row + (cu * kChunk + 8) * esz, g[u][1]);
             }
         }
 #pragma unroll
         for (int u = 0; u < kAhead; ++u)
-            if (c + u * stride < n_chunks) take_chunk(g[u]);
+            if (c + u * kThreads < chunk_end) take_chunk(g[u]);
     }
-    // the d % 16 leftover elements, taken by the first threads of block 0
-    if (blockIdx.x == 0) {
+    // the d % 16 leftover elements, taken by the first threads of the job's last piece
+    if (piece.last) {
         const uint64_t j = n_chunks * kChunk + threadIdx.x;
         if (j < d) {
             const float a = fabsf(load1<BF16>(row, j));
@@ -436,10 +442,6 @@ stats_hinted_kernel(const void* __restrict__ grad, uint64_t d_row, uint64_t grad
     }
 
     // block reduction: shuffles inside a warp, shared memory across the 8 warps
-    __shared__ double s_d[4][kThreads / 32];
-    __shared__ unsigned long long s_u[3][kThreads / 32];
-    __shared__ float s_f[kThreads / 32];
-    __shared__ bool s_last;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     auto block_fold = [&](PartialH& p) {       // every thread passes its values; thread 0 gets the block's
         p.sum_abs = warp_sum(p.sum_abs); p.sum_sq = warp_sum(p.sum_sq);
@@ -447,15 +449,15 @@ stats_hinted_kernel(const void* __restrict__ grad, uint64_t d_row, uint64_t grad
         p.n_tail[0] = warp_sum(p.n_tail[0]); p.n_tail[1] = warp_sum(p.n_tail[1]); p.n_bad = warp_sum(p.n_bad);
         p.max_abs = warp_max(p.max_abs);
         if (lane == 0) {
-            s_d[0][warp] = p.sum_abs; s_d[1][warp] = p.sum_sq; s_d[2][warp] = p.sum_log2[0]; s_d[3][warp] = p.sum_log2[1];
-            s_u[0][warp] = p.n_tail[0]; s_u[1][warp] = p.n_tail[1]; s_u[2][warp] = p.n_bad; s_f[warp] = p.max_abs;
+            sh.d[0][warp] = p.sum_abs; sh.d[1][warp] = p.sum_sq; sh.d[2][warp] = p.sum_log2[0]; sh.d[3][warp] = p.sum_log2[1];
+            sh.u[0][warp] = p.n_tail[0]; sh.u[1][warp] = p.n_tail[1]; sh.u[2][warp] = p.n_bad; sh.f[warp] = p.max_abs;
         }
         __syncthreads();
         if (threadIdx.x == 0) {
             PartialH r{};
             for (int w = 0; w < kThreads / 32; ++w) {
-                r.sum_abs += s_d[0][w]; r.sum_sq += s_d[1][w]; r.sum_log2[0] += s_d[2][w]; r.sum_log2[1] += s_d[3][w];
-                r.n_tail[0] += s_u[0][w]; r.n_tail[1] += s_u[1][w]; r.n_bad += s_u[2][w]; r.max_abs = fmaxf(r.max_abs, s_f[w]);
+                r.sum_abs += sh.d[0][w]; r.sum_sq += sh.d[1][w]; r.sum_log2[0] += sh.d[2][w]; r.sum_log2[1] += sh.d[3][w];
+                r.n_tail[0] += sh.u[0][w]; r.n_tail[1] += sh.u[1][w]; r.n_bad += sh.u[2][w]; r.max_abs = fmaxf(r.max_abs, sh.f[w]);
             }
             p = r;
         }
@@ -464,20 +466,22 @@ stats_hinted_kernel(const void* __restrict__ grad, uint64_t d_row, uint64_t grad
     p.sum_abs = sum_abs; p.sum_sq = sum_sq; p.sum_log2[0] = sum_log2[0]; p.sum_log2[1] = sum_log2[1];
     p.n_tail[0] = n_tail[0]; p.n_tail[1] = n_tail[1]; p.n_bad = n_bad; p.max_abs = max_abs;
     block_fold(p);
-    PartialH* mine = partials + static_cast<size_t>(wi) * kMaxBlocksPerWorker;
+    uint32_t first_block, last_block;
+    blocks_of_job(plan, piece, first_block, last_block);
+    PartialH* mine = partials + first_block + wi;                    // the job's records, one per block
     uint32_t* ticket = tickets + wi * 2 + (FALLBACK ? 1 : 0);
     if (threadIdx.x == 0) {
-        mine[blockIdx.x] = p;
+        mine[blockIdx.x - first_block] = p;
         __threadfence();                                       // record visible before the ticket
-        s_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+        sh.last = atomicAdd(ticket, 1u) == last_block - first_block;
     }
     __syncthreads();
-    if (!s_last) return;
+    if (!sh.last) return;
 
-    // last block of this worker: fold the records in index order (fixed shape, deterministic)
+    // last block of this job: fold the records in index order (fixed shape, deterministic)
     __threadfence();
     PartialH acc{};
-    for (uint32_t b = threadIdx.x; b < gridDim.x; b += kThreads) {
+    for (uint32_t b = threadIdx.x; b <= last_block - first_block; b += kThreads) {
         const volatile PartialH* q = mine + b;
         acc.sum_abs += q->sum_abs; acc.sum_sq += q->sum_sq; acc.sum_log2[0] += q->sum_log2[0]; acc.sum_log2[1] += q->sum_log2[1];
         acc.n_tail[0] += q->n_tail[0]; acc.n_tail[1] += q->n_tail[1]; acc.n_bad += q->n_bad; acc.max_abs = fmaxf(acc.max_abs, q->max_abs);
@@ -514,40 +518,39 @@ stats_hinted_kernel(const void* __restrict__ grad, uint64_t d_row, uint64_t grad
             st->n_tail = n;
             st->sum_log_tail = (s2 - static_cast<double>(n) * static_cast<double>(e2)) * 0.6931471805599453094;
         }
-        *ticket = 0u;                                          // ready for the next call on this scratch
     }
 }
 
-cudaError_t launch_stats_hinted(const StatsCall& call, tq_gmin_hint_t* hint, int* launches) {
-    *launches = 0;
-    StatsCall c = call;                          // with segments every (worker, segment) pair is a job of its own
-    if (c.segs) {
-        c.d = 0;
-        for (uint32_t sg = 0; sg < c.segs->n; ++sg) c.d = c.segs->len[sg] > c.d ? c.segs->len[sg] : c.d;   // sizes the grid
-        c.n_workers *= c.segs->n;
+template <bool BF16, bool FALLBACK>
+__global__ void __launch_bounds__(kThreads, TQ_STATS_HINTED_BLOCKS)
+stats_hinted_kernel(const void* __restrict__ grad, uint64_t grad_stride, float kappa,
+                    tq_gmin_hint_t* __restrict__ hint, tq_stats_t* __restrict__ stats,
+                    PartialH* __restrict__ partials, uint32_t* __restrict__ tickets, const __grid_constant__ TilePlan plan) {
+    __shared__ BlockFold sh;
+    uint64_t cur = first_tile_of_block(plan, blockIdx.x);
+    const uint64_t end = first_tile_of_block(plan, blockIdx.x + 1);
+    while (cur < end) {
+        stats_hinted_piece<BF16, FALLBACK>(next_piece(plan, cur, end), plan, grad, grad_stride, kappa, hint, stats, partials, tickets, sh);
+        __syncthreads();                                       // the next piece reuses the shared arrays
     }
-    const SegTable& segs = c.segs ? *c.segs : kNoSegments;
+}
+
+cudaError_t launch_stats_hinted(const StatsCall& c, tq_gmin_hint_t* hint, int* launches) {
+    *launches = 0;
+    const uint32_t n_jobs = c.segs ? c.n_workers * c.segs->n : c.n_workers;
     PartialH* partials = static_cast<PartialH*>(c.workspace);
-    uint32_t* tickets = reinterpret_cast<uint32_t*>(static_cast<char*>(c.workspace) + tickets_offset(c.n_workers));
-    cudaError_t e = cudaMemsetAsync(tickets, 0, static_cast<size_t>(c.n_workers) * 2 * sizeof(uint32_t), c.stream);
+    uint32_t* tickets = reinterpret_cast<uint32_t*>(static_cast<char*>(c.workspace) + tickets_offset(n_jobs));
+    cudaError_t e = cudaMemsetAsync(tickets, 0, static_cast<size_t>(n_jobs) * 2 * sizeof(uint32_t), c.stream);
     if (e != cudaSuccess) return e;
-    int dev = 0, sms = 148;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    // the resident blocks of 256 threads per SM, spread over the workers
-    const uint64_t chunks = c.d / kChunk;
-    uint64_t per_worker = static_cast<uint64_t>(sms) * TQ_STATS_HINTED_BLOCKS / c.n_workers;     // rounded down: no second wave
-    const uint64_t useful = (chunks + kThreads - 1) / kThreads;
-    if (per_worker > useful) per_worker = useful;
-    if (per_worker > kMaxBlocksPerWorker) per_worker = kMaxBlocksPerWorker;
-    if (per_worker < 1) per_worker = 1;
-    const dim3 grid(static_cast<unsigned>(per_worker), c.n_workers);     // the same grid for both kernels: same summation order
-    if (c.bf16) stats_hinted_kernel<true, false><<<grid, kThreads, 0, c.stream>>>(c.grad, c.d, c.grad_stride, c.kappa, hint, c.stats, partials, tickets, segs);
-    else stats_hinted_kernel<false, false><<<grid, kThreads, 0, c.stream>>>(c.grad, c.d, c.grad_stride, c.kappa, hint, c.stats, partials, tickets, segs);
+    static thread_local TilePlan plan;            // the same plan for both kernels: same summation order
+    plan_stats(c, n_jobs, TQ_STATS_HINTED_BLOCKS, &plan);
+    const auto kernel = c.bf16 ? stats_hinted_kernel<true, false> : stats_hinted_kernel<false, false>;
+    const auto tail_kernel = c.bf16 ? stats_hinted_kernel<true, true> : stats_hinted_kernel<false, true>;
+    kernel<<<plan.blocks, kThreads, 0, c.stream>>>(c.grad, c.grad_stride, c.kappa, hint, c.stats, partials, tickets, plan);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     *launches = 1;
-    if (c.bf16) stats_hinted_kernel<true, true><<<grid, kThreads, 0, c.stream>>>(c.grad, c.d, c.grad_stride, c.kappa, hint, c.stats, partials, tickets, segs);
-    else stats_hinted_kernel<false, true><<<grid, kThreads, 0, c.stream>>>(c.grad, c.d, c.grad_stride, c.kappa, hint, c.stats, partials, tickets, segs);
+    tail_kernel<<<plan.blocks, kThreads, 0, c.stream>>>(c.grad, c.grad_stride, c.kappa, hint, c.stats, partials, tickets, plan);
     e = cudaGetLastError();
     if (e == cudaSuccess) *launches = 2;
     return e;
@@ -557,7 +560,7 @@ cudaError_t launch_stats_hinted(const StatsCall& call, tq_gmin_hint_t* hint, int
 // Built-in scratch for callers that cannot allocate: enough for TQ_STATIC_MAX_WORKERS workers.
 // It is part of the library's device image (one copy per GPU that loads the library).
 constexpr size_t kStaticScratchBytes =
-    static_cast<size_t>(TQ_STATIC_MAX_WORKERS) * kMaxBlocksPerWorker * sizeof(Partial) + TQ_STATIC_MAX_WORKERS * 2 * sizeof(uint32_t) + 256;
+    static_cast<size_t>(TQ_STATIC_MAX_WORKERS) * kRecordsPerJob * sizeof(Partial) + TQ_STATIC_MAX_WORKERS * 2 * sizeof(uint32_t) + 256;
 static __device__ __align__(256) unsigned char g_static_scratch[kStaticScratchBytes];
 
 cudaError_t launch_stats_static(const StatsCall& c, int* launches, bool* limit) {

@@ -42,3 +42,56 @@ def test_params_device_record_counts(tq, mode, n):
         assert (got[i].flags, got[i].bits, got[i].mode) == (want.flags, want.bits, want.mode)
         assert math.isclose(got[i].alpha, want.alpha, rel_tol=3e-7)
         assert np.allclose(list(got[i].levels), list(want.levels), rtol=5e-7, atol=0)
+
+
+@pytest.fixture(scope="module")
+def orc():
+    import oracle
+    oracle.lib()
+    return oracle
+
+
+def _oracle_params(orc, p):
+    q = orc.Params()
+    for f in ("bits", "num_levels", "mode", "flags", "alpha", "inv_step", "gamma", "g_min", "rho", "iterations"):
+        setattr(q, f, getattr(p, f))
+    for k in range(16):
+        q.levels[k], q.inv_width[k] = p.levels[k], p.inv_width[k]
+    return q
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("L,mode", [(2, 0), (8, 0), (4, 1), (8, 1), (16, 1)])
+@pytest.mark.parametrize("lengths", [(8192, 8191, 1, 8193, 31, 32, 33), (1, 2, 3), (500_000, 17, 1_300_000, 4097)])
+def test_ranges_that_cross_jobs(tq, orc, dtype, L, mode, lengths):
+    """A block's range of tiles may end anywhere in a job and hold many short ones: every job's statistics (exact counts and
+    maxima; sums of 16-element fp32 partials, 2e-6), packed words and updates (bit-exact) against the oracle."""
+    n, bits, table, at = 3, {2: 1, 4: 2, 8: 3, 16: 4}[L], [], 0
+    for ln in lengths:
+        table.append((at, ln))
+        at += (ln + 15) // 16 * 16
+    gen = torch.Generator(device="cuda").manual_seed(at)
+    g = (torch.randn((n, at), device="cuda", generator=gen) * torch.rand((n, at), device="cuda", generator=gen).pow(-0.4)).to(dtype)
+    S = len(table)
+    stats_dev = tq.tq_stats_segments(g, table)
+    host = g.float().cpu().numpy()
+    for i, r in enumerate(tq.stats_to_host(stats_dev)):
+        off, ln = table[i % S]
+        o = orc.stats(host[i // S, off:off + ln], g_min=r.g_min) if r.g_min > 0 else None
+        assert r.d == ln and (o is None or (r.n_tail, r.max_abs) == (o.n_tail, o.max_abs))
+        assert o is None or math.isclose(r.sum_abs, o.sum_abs, rel_tol=2e-6)
+    params_dev = tq.tq_params_device(stats_dev, n * S, L, mode, 3.0)
+    ps = tq.params_to_host(params_dev)
+    packed = tq.tq_compress_segments(g, table, params_dev, L, mode, seed=99)
+    out = torch.zeros(at, device="cuda")
+    tq.tq_decompress_aggregate_segments(packed, table, params_dev, L, out=out)
+    got, res, w = packed.cpu().numpy().view(np.uint32), out.cpu().numpy(), 0
+    for s, (off, ln) in enumerate(table):
+        words = tq.tq_packed_words(ln, bits)
+        rows = np.ascontiguousarray(got[:, w:w + words])
+        for i in range(n):
+            p = ps[i * S + s]
+            want = np.zeros(words, np.uint32) if p.flags & tq.FLAG_INVALID else orc.compress(host[i, off:off + ln], _oracle_params(orc, p), 99, i)
+            assert np.array_equal(rows[i], want), (s, i)
+        assert np.array_equal(res[off:off + ln], orc.decompress_aggregate(rows, ln, [_oracle_params(orc, ps[i * S + s]) for i in range(n)]))
+        w += words
