@@ -154,6 +154,9 @@ __device__ __forceinline__ void pair_plus_alpha(const Raw8<BF16>& g, int h, floa
 // k = k_lo + [g >= boundary] = max{ j <= s-1 : l_j <= g }.  s_cell[k] = (l_k, 1/|Delta_k|).
 // g is not clipped first: beyond +-alpha the same interval is found as for the clipped value, and
 // p >= 1 (or p < 0, or NaN) saturates to the same decision.
+// What follows an 8-byte lookup is scalar: to use the two halves of two lookups as pairs takes a move per value, which
+// costs an issue slot and often the multiplier pipe, more than pairing saves (25.6 M x 16, 16 levels: 355 -> 349 us, through
+// device parameters 394 -> 350 us; 250 M x 4, 8 levels 958 -> 861 us).
 __device__ __forceinline__ f32x2 code_grid2(float g0, float g1, f32x2 alpha2, float inv_2alpha, f32x2 cell_scale2,
                                             const char* s_grid, const char* s_cell, float rf0, float rf1) {
     const f32x2 g = pair(g0, g1);
@@ -165,15 +168,11 @@ __device__ __forceinline__ f32x2 code_grid2(float g0, float g1, f32x2 alpha2, fl
     unpair(cell8, c0, c1);
     const float2 gc0 = *reinterpret_cast<const float2*>(s_grid + __float_as_uint(c0));
     const float2 gc1 = *reinterpret_cast<const float2*>(s_grid + __float_as_uint(c1));
-    const f32x2 kf = add2(pair(gc0.y, gc1.y), pair(set_ge(g0, gc0.x), set_ge(g1, gc1.x)));
-    float k0, k1;
-    unpair(mul2(kf, both(__uint_as_float(8u))), k0, k1);                     // bits = 8 * k
-    const float2 q0 = *reinterpret_cast<const float2*>(s_cell + __float_as_uint(k0));
-    const float2 q1 = *reinterpret_cast<const float2*>(s_cell + __float_as_uint(k1));
-    const f32x2 p = mul2(sub2(g, pair(q0.x, q1.x)), pair(q0.y, q1.y));
-    float pm0, pm1;
-    unpair(fma2(p, both(65536.0f), both(kMagic)), pm0, pm1);
-    return add2(kf, pair(sub_sat(pm0, rf0), sub_sat(pm1, rf1)));
+    const float k0 = __fadd_rn(gc0.y, set_ge(g0, gc0.x)), k1 = __fadd_rn(gc1.y, set_ge(g1, gc1.x));
+    const float2 q0 = *reinterpret_cast<const float2*>(s_cell + __float_as_uint(__fmul_rn(k0, __uint_as_float(8u))));   // bits = 8 * k
+    const float2 q1 = *reinterpret_cast<const float2*>(s_cell + __float_as_uint(__fmul_rn(k1, __uint_as_float(8u))));
+    const float p0 = __fmul_rn(__fsub_rn(g0, q0.x), q0.y), p1 = __fmul_rn(__fsub_rn(g1, q1.x), q1.y);
+    return pair(__fadd_rn(k0, rounds_up(p0, rf0)), __fadd_rn(k1, rounds_up(p1, rf1)));
 }
 
 // General codebook by branch-free binary search (used when no grid of at most kMaxGridCells cells
