@@ -12,6 +12,12 @@ constexpr int kThreads = 256;
 constexpr float kMagic = 8388608.0f;          // 2^23: adding it leaves an integer in the mantissa
 constexpr uint32_t kMagicBits = 0x4B000000u;  // bit pattern of 2^23
 
+// The kernel before this one on the stream is complete and its writes are visible; the next one may be set up.  Nothing
+// before this may touch global memory.
+__device__ __forceinline__ void pdl_wait() {
+    asm volatile("griddepcontrol.wait;\n\tgriddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // ---- 256-bit global accesses (one full 32-byte sector per lane) ---------------------------------
 __device__ __forceinline__ void ldg256_stream(const void* p, uint32_t (&v)[8]) {
     asm volatile("ld.global.nc.L1::no_allocate.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"

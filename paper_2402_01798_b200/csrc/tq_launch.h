@@ -58,6 +58,29 @@ inline void plan_tiles(TilePlan* plan, const SegTable* segs, uint64_t d, uint32_
     plan->blocks_per_tile = static_cast<double>(blocks) / static_cast<double>(total);
 }
 
+// SMs of the current device.
+inline int sm_count() {
+    int dev = 0, sms = 148;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return sms;
+}
+
+// Every kernel is launched through this: it may be set up (blocks placed, barriers initialised, tables built from kernel
+// parameters) while the kernel before it on the stream is still running, and waits for that one's results at its
+// pdl_wait().  Without it each launch of a round's chain begins about 1 us after the end of the one before it.
+template <class T> struct Same { using type = T; };
+template <class... P>
+inline cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t stream,
+                                 const typename Same<P>::type&... args) {
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid; cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem; cfg.stream = stream; cfg.attrs = &attr; cfg.numAttrs = 1;
+    void* ptrs[] = {const_cast<void*>(static_cast<const void*>(&args))...};
+    return cudaLaunchKernelExC(&cfg, reinterpret_cast<const void*>(kernel), ptrs);
+}
+
 struct CompressCall {
     const void* grad; bool bf16; uint64_t d, grad_stride; uint32_t n_workers;
     const tq_params_t* params;       // host array, or

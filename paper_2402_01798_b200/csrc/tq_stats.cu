@@ -3,16 +3,20 @@
 // sum ln(|g_j| / g_min) (the two ingredients of the maximum-likelihood tail index of Section 5 and of
 // rho, the tail mass of Section 4.1).
 //
-// Shape: the tiles (4096 elements) of all jobs -- workers, or (worker, segment) pairs -- are cut into one range
-// per resident block (TilePlan).  Within its piece of a job a thread walks 16-element chunks with a block-wide
-// stride, keeps fp32 partial sums inside a chunk and fp64 sums across chunks, then the block reduces
-// with warp shuffles and writes ONE partial record per piece to scratch.  A ticket counter (one atomic per
-// piece) tells the last block of a job to fold that job's records in index order, so the result
-// does not depend on which block finishes last.  No block ever waits for another.
+// Arithmetic: a thread takes chunks of 64 bytes (16 fp32 or 32 bf16 elements), keeps fp32 partial sums inside a
+// chunk (at most 16 terms in a row) and fp64 sums across chunks.  A chunk with a NaN or an Inf is redone element by element in
+// fp64.  bf16 pairs are summed, squared and compared as they are (packed and mixed-precision instructions); unpacking
+// them first cost 4 instructions per pair.
 //
-// With an automatic threshold (g_min = kappa * mean|g|) the tail quantities need the mean first:
-// pass 1 (moments) finishes the record's g_min on the device, pass 2 (tail) reads it there; the host
-// is not involved in between.  With a caller-supplied g_min one fused pass does everything.
+// Shapes.  Short rows (stats_small_kernel): a cluster of 8 blocks per job does everything in one launch, with the
+// block sums exchanged through distributed shared memory.  Other rows: the tiles (256 chunks) of all jobs -- workers, or
+// (worker, segment) pairs -- are cut into contiguous ranges, one per block (TilePlan); a block writes one record per
+// piece of a job, and the next launch starts by folding the records of the jobs it needs, in index order, so
+// that the result does not depend on the order in which blocks run and no block waits for another.
+//   automatic threshold, g_min = kappa * mean|g|: pass 1 (moments), pass 2 (tail);
+//   hinted threshold: one pass for two candidate thresholds, then a launch that finishes the record and reads the data
+//   again only for jobs whose hint missed;
+//   caller's threshold: one pass, the last block of a job (a ticket counter) folds the records.
 // HBM traffic per element and pass: 4 bytes (fp32) or 2 bytes (bf16) read.
 #include <math_constants.h>
 
@@ -24,534 +28,752 @@
 namespace tq {
 
 constexpr int kRecordsPerJob = 1024;          // scratch records per job: a call has at most blocks + jobs pieces
-constexpr int kChunk = 16;
-constexpr int kTile = kChunk * kThreads;      // elements
+constexpr int kChunkBytes = 64;
+template <bool BF16> constexpr int kChunk = kChunkBytes / (BF16 ? 2 : 4);      // elements
+constexpr float kMaxFinite = 3.402823466e38f;
 
 struct alignas(64) Partial {
-    double sum_abs, sum_sq, sum_log2;
-    unsigned long long n_tail, n_bad;
+    double sum_abs, sum_sq, sum_log2[2];
+    unsigned long long n_tail[2], n_bad;
     float max_abs, pad;
 };
 // scratch layout for n jobs: [n * kRecordsPerJob] Partial (piece of block b and job j: record b + j), then [n][2] tickets (uint32)
 __host__ __device__ inline size_t tickets_offset(uint32_t n_jobs) {
     return static_cast<size_t>(n_jobs) * kRecordsPerJob * sizeof(Partial);
 }
-static void plan_stats(const StatsCall& c, uint32_t n_jobs, int ranges_per_sm, TilePlan* plan) {
-    int dev = 0, sms = 148;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    uint64_t resident = static_cast<uint64_t>(sms) * ranges_per_sm;
-    const uint64_t room = static_cast<uint64_t>(n_jobs) * kRecordsPerJob - n_jobs;
-    if (resident > room) resident = room;
-    plan_tiles(plan, c.segs, c.d, c.n_workers, kTile, resident);
-}
 size_t stats_workspace_bytes(uint32_t n_workers) {
     return tickets_offset(n_workers) + static_cast<size_t>(n_workers) * 2 * sizeof(uint32_t) + 256;
 }
 
-enum Pass { kMoments = 0, kTail = 1, kBoth = 2 };
+// ---- one chunk -----------------------------------------------------------------------------------------
 
 // Hardware base-2 logarithm (absolute error about 2^-22 for arguments near 1, 2 ulp elsewhere).
-// Subnormal arguments are flushed; only arguments >= 1 (tail elements) are ever used.
 __device__ __forceinline__ float lg2_fast(float x) {
     float r; asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x)); return r;
 }
-
 __device__ __forceinline__ float fma_sat(float a, float b, float c) {
     float r; asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c)); return r;
 }
+// Two bf16 values at a time; the products and sums of the mixed forms are fp32 with one rounding.
+__device__ __forceinline__ uint32_t max_b2(uint32_t a, uint32_t b) { uint32_t r; asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b)); return r; }
+__device__ __forceinline__ void add_halves(uint32_t w, float& lo, float& hi) {          // lo += w.lo, hi += w.hi
+    asm("{\n\t.reg .b16 l, h;\n\tmov.b32 {l, h}, %2;\n\tadd.rn.f32.bf16 %0, l, %0;\n\tadd.rn.f32.bf16 %1, h, %1;\n\t}" : "+f"(lo), "+f"(hi) : "r"(w));
+}
+__device__ __forceinline__ void add_squares(uint32_t w, float& lo, float& hi) {         // lo += w.lo^2, hi += w.hi^2
+    asm("{\n\t.reg .b16 l, h;\n\tmov.b32 {l, h}, %2;\n\tfma.rn.f32.bf16 %0, l, l, %0;\n\tfma.rn.f32.bf16 %1, h, h, %1;\n\t}" : "+f"(lo), "+f"(hi) : "r"(w));
+}
 
-// Resident blocks per SM.  fp32 rows are bound by HBM and do best with few blocks (25.6 M x 16, moments + tail, 3 / 4 / 5 / 6
-// blocks: 485 / 478 / 503 / 507 us); bf16 rows are bound by instructions and latency and want the warps (124 M x 8, the same:
-// 888 / 754 / 719 / 691 us), and two ranges per resident block, which even out the SMs, where a range stays long enough
-// (668 us; 1 M x 8: 29 instead of 24 us, so short rows keep one).
-constexpr int stats_blocks_per_sm(bool bf16, int pass) { return !bf16 ? 4 : pass == kBoth ? 5 : 6; }
-constexpr uint64_t kTilesForTwoRanges = 64;      // per resident block
+using Words = uint32_t[16];                    // a chunk as loaded
+__device__ __forceinline__ void load_chunk(const char* row, uint64_t c, Words& w) {
+    uint32_t v[8];
+    ldg256_stream(row + c * kChunkBytes, v);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) w[i] = v[i];
+    ldg256_stream(row + c * kChunkBytes + 32, v);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) w[8 + i] = v[i];
+}
+// |g| of the chunk (bf16 pairs lose their signs in place; fp32 uses take the absolute value as an operand modifier)
+template <bool BF16>
+__device__ __forceinline__ void drop_signs(Words& w) {
+    if constexpr (BF16) {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) w[i] &= 0x7FFF7FFFu;
+    }
+}
+// fp32 sums of |g| and g^2; their sum is finite exactly when the chunk can be used as it is.
+template <bool BF16>
+__device__ __forceinline__ void moments(const Words& w, float& s_abs, float& s_sq) {
+    if constexpr (BF16) {
+        float a[4] = {0.0f, 0.0f, 0.0f, 0.0f}, q[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+        for (int i = 0; i < 16; i += 2) {
+            add_halves(w[i], a[0], a[1]); add_halves(w[i + 1], a[2], a[3]);
+            add_squares(w[i], q[0], q[1]); add_squares(w[i + 1], q[2], q[3]);
+        }
+        s_abs = (a[0] + a[1]) + (a[2] + a[3]);
+        s_sq = (q[0] + q[1]) + (q[2] + q[3]);
+    } else {
+        s_abs = 0.0f;
+        f32x2 q2 = both(0.0f);
+#pragma unroll
+        for (int i = 0; i < 16; i += 2) {
+            const f32x2 x = pair(__uint_as_float(w[i]), __uint_as_float(w[i + 1]));
+            s_abs += fabsf(__uint_as_float(w[i]));
+            s_abs += fabsf(__uint_as_float(w[i + 1]));
+            q2 = fma2(x, x, q2);
+        }
+        float q0, q1;
+        unpair(q2, q0, q1);
+        s_sq = q0 + q1;
+    }
+}
+// Running maximum of |g|: an fp32 value, or two bf16 values.
+template <bool BF16>
+__device__ __forceinline__ uint32_t chunk_max(const Words& w, uint32_t running) {
+    if constexpr (BF16) {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) running = max_b2(running, w[i]);
+        return running;
+    } else {
+        float m = __uint_as_float(running);
+#pragma unroll
+        for (int i = 0; i < 16; i += 2) m = fmaxf(fmaxf(m, fabsf(__uint_as_float(w[i]))), fabsf(__uint_as_float(w[i + 1])));
+        return __float_as_uint(m);
+    }
+}
+template <bool BF16>
+__device__ __forceinline__ float max_value(uint32_t running) {
+    if constexpr (BF16) return fmaxf(__uint_as_float(running << 16), __uint_as_float(running & 0xFFFF0000u));
+    else return __uint_as_float(running);
+}
 
+// Tail sums for K thresholds that are powers of two, t and 2 t: s_log[k] = sum of log2|g| over |g| > t_k, cnt[k] its number.
+// The integer / compare pipe runs at half rate and would bound this loop (two compares, two selects and two integer
+// adds per threshold), so the tail test m = [|g| > t] is done on the multiply-add pipe, as a saturating fma:
+//   fp32: r = |g| / t is exact (t a power of two), m = sat(r * 2^30 - 2^30): the smallest r above 1 gives 2^7, r <= 1 gives <= 0,
+//         NaN gives 0, Inf gives 1; for 2 t the same r with 2^29;
+//   bf16: the values next above and below t differ from it by 0.011 and 0.006 in log2, a thousand times the error of lg2, so
+//         m = sat((lg - log2 t) * 2^10 - 5.7) is 0 or 1 as well, and r is not needed.
+// Counts are small floats, and the masked sum is s + m * lg, which rounds exactly like adding lg or nothing, so the sums
+// of a threshold do not depend on which of the two it is.  log2 is taken of max(|g|, 2^-126) so that a zero cannot turn
+// 0 * (-inf) into NaN; elements that small are never in a tail (t >= 2^-126).
+struct TailTest {
+    float a, c[2];           // fp32: 1 / t, unused; bf16: unused, the constants of the two saturating operations
+    __device__ __forceinline__ explicit TailTest(float t) {
+        a = __frcp_rn(t);    // exact; 0 for t = Inf (no hint): nothing is in the tail
+        const float e = static_cast<float>(static_cast<int>(__float_as_uint(t) >> 23) - 127);
+        c[0] = -1024.0f * e - 5.7f;
+        c[1] = -1024.0f * e - 1029.7f;
+    }
+};
+template <bool BF16, int K>
+__device__ __forceinline__ void tail_pow2(const Words& w, const TailTest& test, float (&s_log)[K], float (&cnt)[K]) {
+    f32x2 log2s[K], cnts[K];
+#pragma unroll
+    for (int k = 0; k < K; ++k) { log2s[k] = both(0.0f); cnts[k] = both(0.0f); }
+#pragma unroll
+    for (int i = 0; i < 16; i += BF16 ? 1 : 2) {
+        float x0, x1, l0, l1;                                 // what the tail test looks at, log2|g|
+        if constexpr (BF16) {
+            const uint32_t b = max_b2(w[i], 0x00800080u);
+            x0 = l0 = lg2_fast(__uint_as_float(b << 16));
+            x1 = l1 = lg2_fast(__uint_as_float(b & 0xFFFF0000u));
+        } else {
+            unpair(mul2(pair(__uint_as_float(w[i]), __uint_as_float(w[i + 1])), both(test.a)), x0, x1);
+            l0 = lg2_fast(fmaxf(fabsf(__uint_as_float(w[i])), 1.17549435e-38f));
+            l1 = lg2_fast(fmaxf(fabsf(__uint_as_float(w[i + 1])), 1.17549435e-38f));
+        }
+        const f32x2 lg = pair(l0, l1);
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            f32x2 m;
+            if constexpr (BF16) m = pair(fma_sat(x0, 1024.0f, test.c[k]), fma_sat(x1, 1024.0f, test.c[k]));
+            else {
+                const float scale = k ? 536870912.0f : 1073741824.0f;
+                m = pair(fma_sat(fabsf(x0), scale, -1073741824.0f), fma_sat(fabsf(x1), scale, -1073741824.0f));
+            }
+            log2s[k] = fma2(m, lg, log2s[k]);
+            cnts[k] = add2(cnts[k], m);
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        float l0, l1, n0, n1;
+        unpair(log2s[k], l0, l1);
+        unpair(cnts[k], n0, n1);
+        s_log[k] = l0 + l1;
+        cnt[k] = n0 + n1;
+    }
+}
+// Tail sums for any threshold, of log2(|g| * inv) with inv about 1 / g_min.  A NaN is not in the tail; an Inf makes s_log infinite.
+template <bool BF16>
+__device__ __forceinline__ void tail_any(const Words& w, float g_min, float inv, float& s_log, uint32_t& cnt) {
+    float s[2] = {0.0f, 0.0f};
+    cnt = 0;
+    constexpr int n = kChunk<BF16>;
+#pragma unroll
+    for (int i = 0; i < n; ++i) {
+        const uint32_t v = w[BF16 ? i / 2 : i];
+        const float a = BF16 ? __uint_as_float((i & 1) ? (v & 0xFFFF0000u) : (v << 16)) : fabsf(__uint_as_float(v));
+        const bool in_tail = a > g_min;
+        const float lg = lg2_fast(a * inv);
+        s[BF16 ? i & 1 : 0] += in_tail ? lg : 0.0f;          // at most 16 terms in a row
+        cnt += in_tail ? 1u : 0u;
+    }
+    s_log = s[0] + s[1];
+}
+
+// Elements one by one in fp64: chunks with something non-finite, and a row's last d % chunk elements.  Out of line: the double-precision logarithm is long and needed rarely.
+struct Exact {
+    double sum_abs, sum_sq, sum_log2;
+    uint32_t n_tail, n_bad;
+    float max_abs;
+};
+template <bool BF16>
+__device__ __noinline__ Exact exact_sums(const char* row, uint64_t first, uint32_t count, float t, float inv) {
+    Exact r{0.0, 0.0, 0.0, 0u, 0u, 0.0f};
+    for (uint32_t i = 0; i < count; ++i) {
+        const float a = fabsf(load1<BF16>(row, first + i));
+        if (!(a <= kMaxFinite)) { r.n_bad += 1; continue; }
+        r.sum_abs += a;
+        r.sum_sq += static_cast<double>(a) * a;
+        r.max_abs = fmaxf(r.max_abs, a);
+        if (a > t) { r.sum_log2 += log2(static_cast<double>(a) * static_cast<double>(inv)); r.n_tail += 1; }
+    }
+    return r;
+}
+
+// ---- what a thread has gathered, and its reduction over the block ------------------------------------------
+template <bool BF16>
+struct Gathered {
+    double sum_abs = 0.0, sum_sq = 0.0, sum_log2[2] = {0.0, 0.0};
+    float n_tail[2] = {0.0f, 0.0f};            // whole numbers below 2^24: a thread sees at most 2^40 / (2 * 148 * 256) elements
+    unsigned long long n_bad = 0;
+    uint32_t max_bits = 0;
+
+    __device__ __forceinline__ void take_exact(const Exact& e, bool with_moments, int k, bool with_tail) {
+        if (with_moments) {
+            sum_abs += e.sum_abs; sum_sq += e.sum_sq; n_bad += e.n_bad;
+            if constexpr (BF16) max_bits = max_b2(max_bits, __float_as_uint(e.max_abs) >> 16);
+            else max_bits = __float_as_uint(fmaxf(__uint_as_float(max_bits), e.max_abs));
+        }
+        if (with_tail) { sum_log2[k] += e.sum_log2; n_tail[k] += static_cast<float>(e.n_tail); }
+    }
+    __device__ __forceinline__ Partial partial() const {
+        Partial p;
+        p.sum_abs = sum_abs; p.sum_sq = sum_sq; p.sum_log2[0] = sum_log2[0]; p.sum_log2[1] = sum_log2[1];
+        p.n_tail[0] = static_cast<unsigned long long>(n_tail[0]); p.n_tail[1] = static_cast<unsigned long long>(n_tail[1]);
+        p.n_bad = n_bad; p.max_abs = max_value<BF16>(max_bits); p.pad = 0.0f;
+        return p;
+    }
+};
+template <int WARPS>
 struct BlockFold {
-    double d[4][kThreads / 32];
-    unsigned long long u[3][kThreads / 32];
-    float f[kThreads / 32];
+    double d[4][WARPS];
+    unsigned long long u[3][WARPS];
+    float f[WARPS];
+    Partial total;
     bool last;
 };
-
-// A block's piece of one job.
-template <bool BF16, int PASS>
-__device__ __forceinline__ void stats_piece(const JobPiece& piece, const TilePlan& plan, const void* __restrict__ grad, uint64_t grad_stride,
-                                            float g_min_in, float kappa, tq_stats_t* __restrict__ stats,
-                                            Partial* __restrict__ partials, uint32_t* __restrict__ tickets, BlockFold& sh) {
-    const size_t esz = BF16 ? 2 : 4;
-    const uint32_t wi = piece.job;
-    const uint64_t d = piece.d;
-    const char* row = static_cast<const char*>(grad) + (static_cast<uint64_t>(piece.worker) * grad_stride + piece.off) * esz;
-
-    float g_min = g_min_in;
-    if constexpr (PASS == kTail) g_min = stats[wi].g_min;     // finished by the moments pass
-    const bool tail_on = (PASS != kMoments) && (g_min > 0.0f);
-    // Tail elements are scaled by inv_gmin before the logarithm and the exact logarithm of inv_gmin * g_min
-    // is taken out again at the end, so inv_gmin only has to keep |g| * inv_gmin inside the normal range
-    // for |g| > g_min.  1 / g_min overflows for a subnormal g_min; such a threshold is scaled by 2^64 first.
-    const float inv_gmin = tail_on ? __frcp_rn(g_min < 7.8886090522101181e-31f ? g_min * 18446744073709551616.0f : g_min) : 0.0f;
-
-    double sum_abs = 0.0, sum_sq = 0.0, sum_log2 = 0.0;
-    unsigned long long n_tail = 0, n_bad = 0;
-    float max_abs = 0.0f;
-
-    const uint64_t n_chunks = d / kChunk, chunk_end = piece.tile1 * kThreads < n_chunks ? piece.tile1 * kThreads : n_chunks;
-    for (uint64_t c = piece.tile0 * kThreads + threadIdx.x; c < chunk_end; c += kThreads) {
-        float g[2][8];
-        load8<BF16>(row + (c * kChunk) * esz, g[0]);
-        load8<BF16>(row + (c * kChunk + 8) * esz, g[1]);
-        // Fast path: assume every element is finite.  A NaN or Inf (or an overflow of the fp32 partial
-        // sums) shows up as a non-finite partial; the chunk is then redone element by element.
-        float s_abs = 0.0f, s_sq = 0.0f, s_log = 0.0f, c_max = 0.0f;
-        uint32_t c_tail = 0;
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const float a = fabsf(g[h][e]);
-                if constexpr (PASS != kTail) {
-                    s_abs += a;
-                    s_sq = fmaf(a, a, s_sq);
-                    c_max = fmaxf(c_max, a);        // drops NaN, keeps Inf: only used if the chunk is clean
-                }
-                if constexpr (PASS != kMoments) {
-                    const bool in_tail = a > g_min;  // false for NaN, true for Inf (caught below)
-                    const float lg = lg2_fast(a * inv_gmin);
-                    s_log += in_tail ? lg : 0.0f;
-                    c_tail += in_tail ? 1u : 0u;
-                }
-            }
-        bool clean = true;
-        if constexpr (PASS != kTail) clean = (s_abs + s_sq) <= 3.402823466e38f;
-        if constexpr (PASS == kTail) clean = s_log <= 3.402823466e38f;
-        else if constexpr (PASS == kBoth) clean = clean && (s_log <= 3.402823466e38f);
-        if (clean) {
-            if constexpr (PASS != kTail) { sum_abs += s_abs; sum_sq += s_sq; max_abs = fmaxf(max_abs, c_max); }
-            if constexpr (PASS != kMoments) {
-                if (tail_on) { sum_log2 += s_log; n_tail += c_tail; }
-            }
-        } else {
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                const float a = fabsf(g[i >> 3][i & 7]);
-                const bool ok = a <= 3.402823466e38f;          // false for NaN and Inf
-                if constexpr (PASS != kTail) {
-                    if (ok) { sum_abs += a; sum_sq += static_cast<double>(a) * a; max_abs = fmaxf(max_abs, a); }
-                    else n_bad += 1;
-                }
-                if constexpr (PASS != kMoments) {
-                    if (tail_on && ok && a > g_min) {
-                        sum_log2 += log2(static_cast<double>(a) * static_cast<double>(inv_gmin));
-                        n_tail += 1;
-                    }
-                }
-            }
-        }
-    }
-    // the d % 16 leftover elements, taken by the first threads of the job's last piece
-    if (piece.last) {
-        const uint64_t j = n_chunks * kChunk + threadIdx.x;
-        if (j < d) {
-            const float a = fabsf(load1<BF16>(row, j));
-            const bool ok = a <= 3.402823466e38f;
-            const float av = ok ? a : 0.0f;
-            if constexpr (PASS != kTail) {
-                sum_abs += av; sum_sq += static_cast<double>(av) * av; max_abs = fmaxf(max_abs, av); n_bad += ok ? 0 : 1;
-            }
-            if constexpr (PASS != kMoments) {
-                if (tail_on && ok && a > g_min) { sum_log2 += log2(static_cast<double>(a) * static_cast<double>(inv_gmin)); n_tail += 1; }
-            }
-        }
-    }
-
-    // block reduction: shuffles inside a warp, shared memory across the 8 warps
+// Every thread passes its values; thread 0 gets the block's.  MOMENTS / TAILS say which fields are in use (TAILS: how many
+// thresholds).  One block barrier; the shared arrays may be reused after the next one.
+template <int WARPS, bool MOMENTS, int TAILS>
+__device__ __forceinline__ void block_fold(Partial& p, BlockFold<WARPS>& sh) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    sum_abs = warp_sum(sum_abs); sum_sq = warp_sum(sum_sq); sum_log2 = warp_sum(sum_log2);
-    n_tail = warp_sum(n_tail); n_bad = warp_sum(n_bad); max_abs = warp_max(max_abs);
+    if constexpr (MOMENTS) {
+        p.sum_abs = warp_sum(p.sum_abs); p.sum_sq = warp_sum(p.sum_sq); p.n_bad = warp_sum(p.n_bad); p.max_abs = warp_max(p.max_abs);
+    }
+#pragma unroll
+    for (int k = 0; k < TAILS; ++k) { p.sum_log2[k] = warp_sum(p.sum_log2[k]); p.n_tail[k] = warp_sum(p.n_tail[k]); }
     if (lane == 0) {
-        sh.d[0][warp] = sum_abs; sh.d[1][warp] = sum_sq; sh.d[2][warp] = sum_log2;
-        sh.u[0][warp] = n_tail; sh.u[1][warp] = n_bad; sh.f[warp] = max_abs;
-    }
-    __syncthreads();
-    uint32_t first_block, last_block;
-    blocks_of_job(plan, piece, first_block, last_block);
-    Partial* mine = partials + first_block + wi;                    // the job's records, one per block
-    uint32_t* ticket = tickets + wi * 2 + (PASS == kTail ? 1 : 0);
-    if (threadIdx.x == 0) {
-        Partial p{};
-        for (int w = 0; w < kThreads / 32; ++w) {
-            p.sum_abs += sh.d[0][w]; p.sum_sq += sh.d[1][w]; p.sum_log2 += sh.d[2][w];
-            p.n_tail += sh.u[0][w]; p.n_bad += sh.u[1][w]; p.max_abs = fmaxf(p.max_abs, sh.f[w]);
-        }
-        mine[blockIdx.x - first_block] = p;
-        __threadfence();                                       // record visible before the ticket
-        sh.last = atomicAdd(ticket, 1u) == last_block - first_block;
-    }
-    __syncthreads();
-    if (!sh.last) return;
-
-    // last block of this job: fold the records in index order (fixed shape, deterministic)
-    __threadfence();
-    Partial acc{};
-    for (uint32_t b = threadIdx.x; b <= last_block - first_block; b += kThreads) {
-        const volatile Partial* p = mine + b;
-        acc.sum_abs += p->sum_abs; acc.sum_sq += p->sum_sq; acc.sum_log2 += p->sum_log2;
-        acc.n_tail += p->n_tail; acc.n_bad += p->n_bad; acc.max_abs = fmaxf(acc.max_abs, p->max_abs);
-    }
-    acc.sum_abs = warp_sum(acc.sum_abs); acc.sum_sq = warp_sum(acc.sum_sq); acc.sum_log2 = warp_sum(acc.sum_log2);
-    acc.n_tail = warp_sum(acc.n_tail); acc.n_bad = warp_sum(acc.n_bad); acc.max_abs = warp_max(acc.max_abs);
-    __syncthreads();
-    if (lane == 0) {
-        sh.d[0][warp] = acc.sum_abs; sh.d[1][warp] = acc.sum_sq; sh.d[2][warp] = acc.sum_log2;
-        sh.u[0][warp] = acc.n_tail; sh.u[1][warp] = acc.n_bad; sh.f[warp] = acc.max_abs;
+        if constexpr (MOMENTS) { sh.d[0][warp] = p.sum_abs; sh.d[1][warp] = p.sum_sq; sh.u[2][warp] = p.n_bad; sh.f[warp] = p.max_abs; }
+#pragma unroll
+        for (int k = 0; k < TAILS; ++k) { sh.d[2 + k][warp] = p.sum_log2[k]; sh.u[k][warp] = p.n_tail[k]; }
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        Partial t{};
-        for (int w = 0; w < kThreads / 32; ++w) {
-            t.sum_abs += sh.d[0][w]; t.sum_sq += sh.d[1][w]; t.sum_log2 += sh.d[2][w];
-            t.n_tail += sh.u[0][w]; t.n_bad += sh.u[1][w]; t.max_abs = fmaxf(t.max_abs, sh.f[w]);
+        Partial r{};
+#pragma unroll 1
+        for (int w = 0; w < WARPS; ++w) {
+            if constexpr (MOMENTS) { r.sum_abs += sh.d[0][w]; r.sum_sq += sh.d[1][w]; r.n_bad += sh.u[2][w]; r.max_abs = fmaxf(r.max_abs, sh.f[w]); }
+#pragma unroll
+            for (int k = 0; k < TAILS; ++k) { r.sum_log2[k] += sh.d[2 + k][w]; r.n_tail[k] += sh.u[k][w]; }
         }
-        tq_stats_t* st = stats + wi;
-        if constexpr (PASS != kTail) {
-            st->d = d; st->n_nonfinite = t.n_bad; st->sum_abs = t.sum_abs; st->sum_sq = t.sum_sq;
-            st->max_abs = t.max_abs;
-            float gm = g_min_in;
-            if (!(g_min_in > 0.0f))
-                gm = d ? static_cast<float>(static_cast<double>(kappa) * t.sum_abs / static_cast<double>(d)) : 0.0f;
-            st->g_min = gm;
-            st->reserved = 0;
-            if constexpr (PASS == kMoments) { st->n_tail = 0; st->sum_log_tail = 0.0; }
-        }
-        if constexpr (PASS != kMoments) {
-            // elements were scaled by inv_gmin instead of divided by g_min: remove the exact
-            // logarithm of that factor's error, n * log2(inv_gmin * g_min), then convert to ln
-            double corr = 0.0;
-            if (tail_on) corr = static_cast<double>(t.n_tail) * log2(static_cast<double>(inv_gmin) * static_cast<double>(g_min));
-            st->n_tail = t.n_tail;
-            st->sum_log_tail = (t.sum_log2 - corr) * 0.6931471805599453094;
-        }
+        p = r;
     }
 }
-
-template <bool BF16, int PASS>
-__global__ void __launch_bounds__(kThreads, stats_blocks_per_sm(BF16, PASS))
-stats_kernel(const void* __restrict__ grad, uint64_t grad_stride, float g_min_in, float kappa,
-             tq_stats_t* __restrict__ stats, Partial* __restrict__ partials, uint32_t* __restrict__ tickets,
-             const __grid_constant__ TilePlan plan) {
-    __shared__ BlockFold sh;
-    uint64_t cur = first_tile_of_block(plan, blockIdx.x);
-    const uint64_t end = first_tile_of_block(plan, blockIdx.x + 1);
-    while (cur < end) {
-        stats_piece<BF16, PASS>(next_piece(plan, cur, end), plan, grad, grad_stride, g_min_in, kappa, stats, partials, tickets, sh);
-        __syncthreads();                                       // the next piece reuses the shared arrays
-    }
-}
-
-template <bool BF16, int PASS>
-static cudaError_t launch(const StatsCall& c, const TilePlan& plan, Partial* partials, uint32_t* tickets) {
-    stats_kernel<BF16, PASS><<<plan.blocks, kThreads, 0, c.stream>>>(c.grad, c.grad_stride, c.g_min, c.kappa, c.stats, partials, tickets, plan);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_stats(const StatsCall& c, int* launches) {
-    *launches = 0;
-    const uint32_t n_jobs = c.segs ? c.n_workers * c.segs->n : c.n_workers;
-    Partial* partials = static_cast<Partial*>(c.workspace);
-    uint32_t* tickets = reinterpret_cast<uint32_t*>(static_cast<char*>(c.workspace) + tickets_offset(n_jobs));
-    cudaError_t e = cudaMemsetAsync(tickets, 0, static_cast<size_t>(n_jobs) * 2 * sizeof(uint32_t), c.stream);
-    if (e != cudaSuccess) return e;
-    static thread_local TilePlan plan;
-    const int ranges = stats_blocks_per_sm(c.bf16, c.g_min > 0.0f ? kBoth : kMoments);
-    plan_stats(c, n_jobs, ranges, &plan);
-    if (c.bf16 && plan.per_block >= kTilesForTwoRanges) plan_stats(c, n_jobs, 2 * ranges, &plan);
-
-    if (c.g_min > 0.0f) {
-        e = c.bf16 ? launch<true, kBoth>(c, plan, partials, tickets) : launch<false, kBoth>(c, plan, partials, tickets);
-        *launches = 1;
-        return e;
-    }
-    e = c.bf16 ? launch<true, kMoments>(c, plan, partials, tickets) : launch<false, kMoments>(c, plan, partials, tickets);
-    if (e != cudaSuccess) return e;
-    *launches = 1;
-    e = c.bf16 ? launch<true, kTail>(c, plan, partials, tickets) : launch<false, kTail>(c, plan, partials, tickets);
-    *launches = 2;
-    return e;
-}
-
-// ---------------------------------------------------------------------------------------------
-// One pass with a hinted threshold.  The paper leaves the choice of g_min open (Section 4.1 only
-// calls it the lower end of the power-law range); with g_min = kappa * mean|g| rounded DOWN TO A
-// POWER OF TWO the tail sums can be gathered before the mean is known, for a few candidate powers of
-// two at once: a caller-kept hint (the kappa * mean|g| of the previous round) names the two
-// candidates nearest to it, the moments and both candidates' tail sums are accumulated in ONE pass,
-// and the last block keeps the candidate that the finished mean selects.  If neither fits (first
-// round, or the mean moved by more than a factor of about 1.4 to 2), a second kernel redoes the tail
-// pass for the right threshold; it is launched every time and returns at once when not needed, so
-// the host never has to look.  Both kernels sum log2|g| itself (not log2(|g| / g_min)) in the same
-// order and remove n * log2(g_min), an integer multiple, at the end: the record is bit-identical
-// whichever way it was obtained.
-struct alignas(64) PartialH {
-    double sum_abs, sum_sq, sum_log2[2];
-    unsigned long long n_tail[2], n_bad;
-    float max_abs, pad;
-};
-static_assert(sizeof(PartialH) == sizeof(Partial), "the hinted pass shares the scratch layout");
+constexpr int kWarps = kThreads / 32;
 
 // Largest power of two not above x; 0 below the smallest normal number (no tail), Inf for Inf.
 __device__ __forceinline__ float pow2_floor(float x) {
     return x >= 1.17549435e-38f ? __uint_as_float(__float_as_uint(x) & 0xFF800000u) : 0.0f;
 }
+__device__ __forceinline__ float mean_level(float kappa, double sum_abs, uint64_t d) {
+    return d ? static_cast<float>(static_cast<double>(kappa) * sum_abs / static_cast<double>(d)) : 0.0f;
+}
+// Tail elements are scaled by inv before the logarithm and the exact logarithm of inv * g_min is taken out again at
+// the end, so inv only has to keep |g| * inv inside the normal range for |g| > g_min.  1 / g_min overflows for a
+// subnormal g_min; such a threshold is scaled by 2^64 first.
+__device__ __forceinline__ float inverse_of(float g_min) {
+    return g_min > 0.0f ? __frcp_rn(g_min < 7.8886090522101181e-31f ? g_min * 18446744073709551616.0f : g_min) : 0.0f;
+}
+__device__ __forceinline__ void store_moments(tq_stats_t* st, uint64_t d, const Partial& t, float g_min) {
+    st->d = d; st->n_nonfinite = t.n_bad; st->sum_abs = t.sum_abs; st->sum_sq = t.sum_sq; st->max_abs = t.max_abs;
+    st->g_min = g_min; st->reserved = 0;
+}
+// sum_log2 holds the logarithms of |g| * inv
+__device__ __forceinline__ void store_tail(tq_stats_t* st, unsigned long long n, double sum_log2, float g_min, float inv) {
+    const double corr = n ? static_cast<double>(n) * log2(static_cast<double>(inv) * static_cast<double>(g_min)) : 0.0;
+    st->n_tail = n;
+    st->sum_log_tail = (sum_log2 - corr) * 0.6931471805599453094;
+}
+// sum_log2 holds the logarithms of |g|, g_min is a power of two: log2 g_min is an integer
+__device__ __forceinline__ void store_tail_pow2(tq_stats_t* st, unsigned long long n, double sum_log2, float g_min) {
+    const int e2 = static_cast<int>((__float_as_uint(g_min) >> 23) & 0xFFu) - 127;
+    st->n_tail = n;
+    st->sum_log_tail = n ? (sum_log2 - static_cast<double>(n) * static_cast<double>(e2)) * 0.6931471805599453094 : 0.0;
+}
 
-#ifndef TQ_STATS_HINTED_BLOCKS
-#define TQ_STATS_HINTED_BLOCKS 3
-#endif
+// ---- a thread's share of a set of chunks ---------------------------------------------------------------------
+enum Pass { kMoments = 0, kTail = 1, kBoth = 2 };
 
-template <bool BF16, bool FALLBACK>
-__device__ __forceinline__ void stats_hinted_piece(const JobPiece& piece, const TilePlan& plan, const void* __restrict__ grad,
-                                                   uint64_t grad_stride, float kappa, tq_gmin_hint_t* __restrict__ hint,
-                                                   tq_stats_t* __restrict__ stats, PartialH* __restrict__ partials,
-                                                   uint32_t* __restrict__ tickets, BlockFold& sh) {
-    constexpr int K = FALLBACK ? 1 : 2;
-    const size_t esz = BF16 ? 2 : 4;
-    const uint32_t wi = piece.job;
-    if constexpr (FALLBACK) {
-        if (hint[wi].hit) return;                 // the one-pass result stands
+// Threshold g_min (any value; no tail unless positive).
+template <bool BF16, int PASS>
+__device__ __forceinline__ void take_any(const char* row, uint64_t c, Words& w, float g_min, float inv, Gathered<BF16>& g) {
+    drop_signs<BF16>(w);
+    float s_abs = 0.0f, s_sq = 0.0f, s_log = 0.0f;
+    uint32_t cnt = 0;
+    if constexpr (PASS != kTail) moments<BF16>(w, s_abs, s_sq);
+    if constexpr (PASS != kMoments) {
+        if (g_min > 0.0f) tail_any<BF16>(w, g_min, inv, s_log, cnt);
     }
-    const uint64_t d = piece.d;
-    const char* row = static_cast<const char*>(grad) + (static_cast<uint64_t>(piece.worker) * grad_stride + piece.off) * esz;
-
-    // candidate thresholds
-    float t[2] = {CUDART_INF_F, CUDART_INF_F};
-    if constexpr (FALLBACK) {
-        t[0] = stats[wi].g_min;                   // finished by the hinted pass; > 0 here
+    if ((s_abs + s_sq) <= kMaxFinite && fabsf(s_log) <= kMaxFinite) {
+        if constexpr (PASS != kTail) { g.sum_abs += s_abs; g.sum_sq += s_sq; g.max_bits = chunk_max<BF16>(w, g.max_bits); }
+        if constexpr (PASS != kMoments) { g.sum_log2[0] += s_log; g.n_tail[0] += static_cast<float>(cnt); }
     } else {
-        const float level = hint[wi].level;
-        if (level >= 2.3509887e-38f && level <= 3.402823466e38f) {      // from 2^-125: both candidates are normal numbers
-            const uint32_t bits = __float_as_uint(level);
-            const uint32_t e = bits & 0x7F800000u;
-            const uint32_t lo = (bits & 0x00400000u) ? e : e - 0x00800000u;    // mantissa >= 1.5: {2^h, 2^(h+1)}, else {2^(h-1), 2^h}
-            t[0] = __uint_as_float(lo);
-            t[1] = __uint_as_float(lo + 0x00800000u);
-        }
+        g.take_exact(exact_sums<BF16>(row, c * kChunk<BF16>, kChunk<BF16>, PASS != kMoments && g_min > 0.0f ? g_min : CUDART_INF_F, inv),
+                     PASS != kTail, 0, PASS != kMoments);
     }
-
-    double sum_abs = 0.0, sum_sq = 0.0, sum_log2[2] = {0.0, 0.0};
-    unsigned long long n_tail[2] = {0, 0}, n_bad = 0;
-    float max_abs = 0.0f;
-    const f32x2 inv_t2 = both(__frcp_rn(t[0]));     // exact: t is a power of two (0 for t = Inf: nothing is in the tail)
-
-    // One chunk of 16 elements: fp32 partials, then into the fp64 sums (the fast path assumes finite
-    // values; a non-finite partial sends the chunk through the element-wise path).
-    // The integer / compare pipe runs at half rate and would bound this loop (two compares, two
-    // selects and two integer adds per candidate), so the tail test is done on the multiply-add pipe:
-    // with r = |g| / t exact (t a power of two), [|g| > t] = sat(r * 2^30 - 2^30): the smallest r above 1
-    // gives 2^7, r <= 1 gives <= 0, NaN gives 0, Inf gives 1.  The second candidate is 2 t: same r, 2^29.
-    // Counts are kept as small floats inside a chunk, and the masked sum is s + m * lg with m = 0 or 1,
-    // which rounds exactly like adding lg or nothing.  log2 is taken of max(|g|, 2^-126) so that a
-    // zero cannot turn 0 * (-inf) into NaN; elements that small are never in a tail (t >= 2^-126).
-    auto take_chunk = [&](const Raw8<BF16> (&g)[2]) {
-        float s_abs = 0.0f, c_max = 0.0f;
-        f32x2 s_sq2 = both(0.0f), s_log2[2] = {both(0.0f), both(0.0f)}, cnt2[2] = {both(0.0f), both(0.0f)};
+}
+// K thresholds t, 2 t that are powers of two (t = Inf: none), with the moments or without.
+template <bool BF16, int K, bool MOMENTS>
+__device__ __forceinline__ void take_pow2(const char* row, uint64_t c, Words& w, float t, const TailTest& test, Gathered<BF16>& g) {
+    drop_signs<BF16>(w);
+    float s_abs, s_sq, s_log[K], cnt[K];
+    moments<BF16>(w, s_abs, s_sq);               // always: both forms send the same chunks through the exact path
+    tail_pow2<BF16, K>(w, test, s_log, cnt);
+    if ((s_abs + s_sq) <= kMaxFinite) {
+        if constexpr (MOMENTS) { g.sum_abs += s_abs; g.sum_sq += s_sq; g.max_bits = chunk_max<BF16>(w, g.max_bits); }
 #pragma unroll
-        for (int h = 0; h < 2; ++h)
+        for (int k = 0; k < K; ++k) { g.sum_log2[k] += s_log[k]; g.n_tail[k] += cnt[k]; }
+    } else {
 #pragma unroll
-            for (int e = 0; e < 8; e += 2) {
-                const float x0 = elem<BF16>(g[h], e), x1 = elem<BF16>(g[h], e + 1);
-                const float a0 = fabsf(x0), a1 = fabsf(x1);
-                s_abs += a0;
-                s_abs += a1;
-                const f32x2 x = pair(x0, x1);
-                s_sq2 = fma2(x, x, s_sq2);
-                c_max = fmaxf(fmaxf(c_max, a0), a1);
-                const f32x2 lg = pair(lg2_fast(fmaxf(a0, 1.17549435e-38f)), lg2_fast(fmaxf(a1, 1.17549435e-38f)));
-                float r0, r1;
-                unpair(mul2(x, inv_t2), r0, r1);
-#pragma unroll
-                for (int k = 0; k < K; ++k) {
-                    const float scale = k ? 536870912.0f : 1073741824.0f;      // 2^29 for the candidate 2 t, 2^30 for t
-                    const f32x2 m = pair(fma_sat(fabsf(r0), scale, -1073741824.0f), fma_sat(fabsf(r1), scale, -1073741824.0f));
-                    s_log2[k] = fma2(m, lg, s_log2[k]);
-                    cnt2[k] = add2(cnt2[k], m);
-                }
-            }
-        float q0, q1;
-        unpair(s_sq2, q0, q1);
-        const float s_sq = q0 + q1;
-        // same test in both kernels, so that both send the same chunks through the slow path
-        const bool clean = (s_abs + s_sq) <= 3.402823466e38f;
-        if (clean) {
-            if constexpr (!FALLBACK) { sum_abs += s_abs; sum_sq += s_sq; max_abs = fmaxf(max_abs, c_max); }
-#pragma unroll
-            for (int k = 0; k < K; ++k) {
-                float l0, l1, n0, n1;
-                unpair(s_log2[k], l0, l1);
-                unpair(cnt2[k], n0, n1);
-                sum_log2[k] += l0 + l1;
-                n_tail[k] += static_cast<uint32_t>(n0 + n1);
-            }
-        } else {
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                const float a = fabsf(elem<BF16>(g[i >> 3], i & 7));
-                const bool ok = a <= 3.402823466e38f;          // false for NaN and Inf
-                if constexpr (!FALLBACK) {
-                    if (ok) { sum_abs += a; sum_sq += static_cast<double>(a) * a; max_abs = fmaxf(max_abs, a); }
-                    else n_bad += 1;
-                }
-#pragma unroll
-                for (int k = 0; k < K; ++k)
-                    if (ok && a > t[k]) { sum_log2[k] += log2(static_cast<double>(a)); n_tail[k] += 1; }
-            }
-        }
-    };
-
-    // A thread's chunks are c0, c0 + kThreads, ...; the loads of kAhead of them (128 bytes per thread) are
-    // issued together, then they are summed in that same order.
-    constexpr int kAhead = BF16 ? 4 : 2;
-    const uint64_t n_chunks = d / kChunk, chunk_end = piece.tile1 * kThreads < n_chunks ? piece.tile1 * kThreads : n_chunks;
-    for (uint64_t c = piece.tile0 * kThreads + threadIdx.x; c < chunk_end; c += kAhead * kThreads) {
-        Raw8<BF16> g[kAhead][2];
-#pragma unroll
-        for (int u = 0; u < kAhead; ++u) {
-            const uint64_t cu = c + u * kThreads;
-            if (cu < chunk_end) {
-                load8_raw<BF16>(row + (cu * kChunk) * esz, g[u][0]);
-                load8_raw<BF16>(row + (cu * kChunk + 8) * esz, g[u][1]);
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < kAhead; ++u)
-            if (c + u * kThreads < chunk_end) take_chunk(g[u]);
+        for (int k = 0; k < K; ++k)
+            g.take_exact(exact_sums<BF16>(row, c * kChunk<BF16>, kChunk<BF16>, k ? 2.0f * t : t, 1.0f), MOMENTS && k == 0, k, true);
     }
-    // the d % 16 leftover elements, taken by the first threads of the job's last piece
-    if (piece.last) {
-        const uint64_t j = n_chunks * kChunk + threadIdx.x;
-        if (j < d) {
-            const float a = fabsf(load1<BF16>(row, j));
-            const bool ok = a <= 3.402823466e38f;
-            if constexpr (!FALLBACK) {
-                const float av = ok ? a : 0.0f;
-                sum_abs += av; sum_sq += static_cast<double>(av) * av; max_abs = fmaxf(max_abs, av); n_bad += ok ? 0 : 1;
-            }
-#pragma unroll
-            for (int k = 0; k < K; ++k)
-                if (ok && a > t[k]) { sum_log2[k] += log2(static_cast<double>(a)); n_tail[k] += 1; }
-        }
+}
+// A thread's chunks c, c + stride, ... below `end`.  One chunk at a time: with the loads of two issued together the registers
+// cost a resident block, and the larger bursts made HBM slower (25.6 M x 16 fp32, two passes: 510 us instead of 481).
+template <class Take>
+__device__ __forceinline__ void walk(const char* row, uint64_t c, uint64_t end, uint32_t stride, const Take& take) {
+    for (; c < end; c += stride) {
+        Words w;
+        load_chunk(row, c, w);
+        take(c, w);
     }
-
-    // block reduction: shuffles inside a warp, shared memory across the 8 warps
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    auto block_fold = [&](PartialH& p) {       // every thread passes its values; thread 0 gets the block's
-        p.sum_abs = warp_sum(p.sum_abs); p.sum_sq = warp_sum(p.sum_sq);
-        p.sum_log2[0] = warp_sum(p.sum_log2[0]); p.sum_log2[1] = warp_sum(p.sum_log2[1]);
-        p.n_tail[0] = warp_sum(p.n_tail[0]); p.n_tail[1] = warp_sum(p.n_tail[1]); p.n_bad = warp_sum(p.n_bad);
-        p.max_abs = warp_max(p.max_abs);
-        if (lane == 0) {
-            sh.d[0][warp] = p.sum_abs; sh.d[1][warp] = p.sum_sq; sh.d[2][warp] = p.sum_log2[0]; sh.d[3][warp] = p.sum_log2[1];
-            sh.u[0][warp] = p.n_tail[0]; sh.u[1][warp] = p.n_tail[1]; sh.u[2][warp] = p.n_bad; sh.f[warp] = p.max_abs;
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            PartialH r{};
-            for (int w = 0; w < kThreads / 32; ++w) {
-                r.sum_abs += sh.d[0][w]; r.sum_sq += sh.d[1][w]; r.sum_log2[0] += sh.d[2][w]; r.sum_log2[1] += sh.d[3][w];
-                r.n_tail[0] += sh.u[0][w]; r.n_tail[1] += sh.u[1][w]; r.n_bad += sh.u[2][w]; r.max_abs = fmaxf(r.max_abs, sh.f[w]);
-            }
-            p = r;
-        }
-    };
-    PartialH p{};
-    p.sum_abs = sum_abs; p.sum_sq = sum_sq; p.sum_log2[0] = sum_log2[0]; p.sum_log2[1] = sum_log2[1];
-    p.n_tail[0] = n_tail[0]; p.n_tail[1] = n_tail[1]; p.n_bad = n_bad; p.max_abs = max_abs;
-    block_fold(p);
-    uint32_t first_block, last_block;
-    blocks_of_job(plan, piece, first_block, last_block);
-    PartialH* mine = partials + first_block + wi;                    // the job's records, one per block
-    uint32_t* ticket = tickets + wi * 2 + (FALLBACK ? 1 : 0);
+}
+template <bool BF16>
+__device__ __forceinline__ uint64_t chunk_end_of(const JobPiece& piece) {
+    const uint64_t whole = piece.d / kChunk<BF16>, end = piece.tile1 * kThreads;
+    return end < whole ? end : whole;
+}
+// The row's last d % chunk elements, one for each of the first threads.
+template <bool BF16>
+__device__ __forceinline__ bool has_leftover(uint64_t d, uint64_t& j) {
+    j = d / kChunk<BF16> * kChunk<BF16> + threadIdx.x;
+    return j < d;
+}
+template <bool BF16>
+__device__ __forceinline__ const char* row_of(const JobPiece& piece, const void* grad, uint64_t grad_stride) {
+    return static_cast<const char*>(grad) + (static_cast<uint64_t>(piece.worker) * grad_stride + piece.off) * (BF16 ? 2 : 4);
+}
+__device__ __forceinline__ Partial* records_of_job(const TilePlan& plan, const JobPiece& piece, Partial* partials, uint32_t& count) {
+    uint32_t first, last;
+    blocks_of_job(plan, piece, first, last);
+    count = last - first + 1;
+    return partials + first + piece.job;
+}
+__device__ __forceinline__ Partial* record_of_piece(const JobPiece& piece, Partial* partials) { return partials + blockIdx.x + piece.job; }
+// Folds `count` records of an earlier launch (or of blocks whose tickets have been seen).
+template <bool MOMENTS, int TAILS>
+__device__ __forceinline__ void fold_records(const Partial* records, uint32_t count, Partial& p, BlockFold<kWarps>& sh) {
+    p = Partial{};
+    for (uint32_t b = threadIdx.x; b < count; b += kThreads) {
+        const volatile Partial* q = records + b;
+        if constexpr (MOMENTS) { p.sum_abs += q->sum_abs; p.sum_sq += q->sum_sq; p.n_bad += q->n_bad; p.max_abs = fmaxf(p.max_abs, q->max_abs); }
+#pragma unroll
+        for (int k = 0; k < TAILS; ++k) { p.sum_log2[k] += q->sum_log2[k]; p.n_tail[k] += q->n_tail[k]; }
+    }
+    block_fold<kWarps, MOMENTS, TAILS>(p, sh);
+}
+// The sum of |g| over the records, known to every thread.
+__device__ __forceinline__ double fold_sum_abs(const Partial* records, uint32_t count, BlockFold<kWarps>& sh) {
+    double v = 0.0;
+    for (uint32_t b = threadIdx.x; b < count; b += kThreads) v += records[b].sum_abs;
+    v = warp_sum(v);
+    if ((threadIdx.x & 31) == 0) sh.d[0][threadIdx.x >> 5] = v;
+    __syncthreads();
+    double s = 0.0;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) s += sh.d[0][w];
+    __syncthreads();
+    return s;
+}
+// Stores the tail fields of the block's record and says whether all of the job's have been stored (block-uniform).
+__device__ __forceinline__ bool last_of_job(Partial* record, const Partial& p, bool moments, uint32_t* ticket, uint32_t count, BlockFold<kWarps>& sh) {
     if (threadIdx.x == 0) {
-        mine[blockIdx.x - first_block] = p;
+        if (moments) *record = p;
+        else { record->sum_log2[0] = p.sum_log2[0]; record->n_tail[0] = p.n_tail[0]; }
         __threadfence();                                       // record visible before the ticket
-        sh.last = atomicAdd(ticket, 1u) == last_block - first_block;
+        sh.last = atomicAdd(ticket, 1u) == count - 1;
     }
     __syncthreads();
-    if (!sh.last) return;
+    if (sh.last) __threadfence();
+    return sh.last;
+}
 
-    // last block of this job: fold the records in index order (fixed shape, deterministic)
-    __threadfence();
-    PartialH acc{};
-    for (uint32_t b = threadIdx.x; b <= last_block - first_block; b += kThreads) {
-        const volatile PartialH* q = mine + b;
-        acc.sum_abs += q->sum_abs; acc.sum_sq += q->sum_sq; acc.sum_log2[0] += q->sum_log2[0]; acc.sum_log2[1] += q->sum_log2[1];
-        acc.n_tail[0] += q->n_tail[0]; acc.n_tail[1] += q->n_tail[1]; acc.n_bad += q->n_bad; acc.max_abs = fmaxf(acc.max_abs, q->max_abs);
+// ---- any threshold: moments, then tail; or both at once with the caller's ------------------------------------
+
+// Resident blocks per SM, each with one range.  Measured with 3 / 4 / 5 blocks: 25.6 M x 16 fp32, two passes 482 / 477 / 506 us,
+// hinted 258 / 247 / 273 (HBM: 250 us a pass); 124 M x 8 bf16, two passes 668 / 623 / 622 us, hinted 456 / 430 / 470 (555 before; the
+// special-function unit, one log2 per element, is busy 54 % of the time, the multiply-add pipes 57 %, issue 69 %).
+constexpr int kStatsBlocksPerSm = 4;
+
+template <bool BF16, int PASS>
+__device__ __forceinline__ void stats_piece(const JobPiece& piece, const TilePlan& plan, const void* grad, uint64_t grad_stride, float g_min,
+                                            float kappa, tq_stats_t* stats, Partial* partials, uint32_t* tickets, BlockFold<kWarps>& sh) {
+    const char* row = row_of<BF16>(piece, grad, grad_stride);
+    uint32_t count;
+    const Partial* records = records_of_job(plan, piece, partials, count);
+    if constexpr (PASS == kMoments) {
+        if (piece.tile0 == 0 && threadIdx.x == 0) tickets[piece.job] = 0u;          // for the tail pass
     }
-    __syncthreads();
-    block_fold(acc);
-    if (threadIdx.x == 0) {
-        tq_stats_t* st = stats + wi;
-        int pick = -1;                       // candidate whose sums are the record's tail
-        float g_min;
-        if constexpr (FALLBACK) {
-            g_min = t[0];
-            pick = 0;
-        } else {
-            const float level = d ? static_cast<float>(static_cast<double>(kappa) * acc.sum_abs / static_cast<double>(d)) : 0.0f;
-            g_min = pow2_floor(level);
-            st->d = d; st->n_nonfinite = acc.n_bad; st->sum_abs = acc.sum_abs; st->sum_sq = acc.sum_sq;
-            st->max_abs = acc.max_abs; st->g_min = g_min; st->reserved = 0;
-            st->n_tail = 0; st->sum_log_tail = 0.0;
-            uint32_t hit = 1;
-            if (g_min > 0.0f) {
-                if (__float_as_uint(g_min) == __float_as_uint(t[0])) pick = 0;
-                else if (__float_as_uint(g_min) == __float_as_uint(t[1])) pick = 1;
-                else hit = 0;
+    if constexpr (PASS == kTail) {
+        // finish the moments: every piece needs the threshold, the job's first one writes the record
+        if (piece.tile0 == 0) {
+            Partial t;
+            fold_records<true, 0>(records, count, t, sh);
+            if (threadIdx.x == 0) {
+                sh.total = t;
+                store_moments(stats + piece.job, piece.d, t, mean_level(kappa, t.sum_abs, piece.d));
             }
-            hint[wi].level = level;
-            hint[wi].hit = hit;
+            __syncthreads();
+            g_min = mean_level(kappa, sh.total.sum_abs, piece.d);
+        } else {
+            g_min = mean_level(kappa, fold_sum_abs(records, count, sh), piece.d);
         }
-        if (pick >= 0 && g_min <= 3.402823466e38f) {
-            // sum ln(a / g_min) = ln 2 * (sum log2 a - n * log2 g_min), log2 g_min an integer
-            const int e2 = static_cast<int>((__float_as_uint(g_min) >> 23) & 0xFFu) - 127;
-            const unsigned long long n = pick ? acc.n_tail[1] : acc.n_tail[0];
-            const double s2 = pick ? acc.sum_log2[1] : acc.sum_log2[0];
-            st->n_tail = n;
-            st->sum_log_tail = (s2 - static_cast<double>(n) * static_cast<double>(e2)) * 0.6931471805599453094;
+    }
+    const float inv = PASS == kMoments ? 0.0f : inverse_of(g_min);
+    Gathered<BF16> g;
+    walk(row, piece.tile0 * kThreads + threadIdx.x, chunk_end_of<BF16>(piece), kThreads,
+         [&](uint64_t c, Words& w) { take_any<BF16, PASS>(row, c, w, g_min, inv, g); });
+    uint64_t j;
+    if (piece.last && has_leftover<BF16>(piece.d, j))
+        g.take_exact(exact_sums<BF16>(row, j, 1, PASS != kMoments && g_min > 0.0f ? g_min : CUDART_INF_F, inv), PASS != kTail, 0, PASS != kMoments);
+
+    Partial p = g.partial();
+    block_fold<kWarps, PASS != kTail, PASS != kMoments ? 1 : 0>(p, sh);
+    if constexpr (PASS == kMoments) {
+        if (threadIdx.x == 0) *record_of_piece(piece, partials) = p;
+    } else {
+        if (!last_of_job(record_of_piece(piece, partials), p, PASS == kBoth, tickets + piece.job, count, sh)) return;
+        Partial t;
+        fold_records<PASS == kBoth, 1>(records, count, t, sh);
+        if (threadIdx.x == 0) {
+            if (PASS == kBoth) store_moments(stats + piece.job, piece.d, t, g_min);
+            store_tail(stats + piece.job, t.n_tail[0], t.sum_log2[0], g_min, inv);
         }
     }
 }
 
-template <bool BF16, bool FALLBACK>
-__global__ void __launch_bounds__(kThreads, TQ_STATS_HINTED_BLOCKS)
-stats_hinted_kernel(const void* __restrict__ grad, uint64_t grad_stride, float kappa,
-                    tq_gmin_hint_t* __restrict__ hint, tq_stats_t* __restrict__ stats,
-                    PartialH* __restrict__ partials, uint32_t* __restrict__ tickets, const __grid_constant__ TilePlan plan) {
-    __shared__ BlockFold sh;
+template <bool BF16, int PASS>
+__global__ void __launch_bounds__(kThreads, kStatsBlocksPerSm)
+stats_kernel(const void* __restrict__ grad, uint64_t grad_stride, float g_min, float kappa, tq_stats_t* stats, Partial* partials,
+             uint32_t* tickets, const __grid_constant__ TilePlan plan) {
+    __shared__ BlockFold<kWarps> sh;
+    pdl_wait();
     uint64_t cur = first_tile_of_block(plan, blockIdx.x);
     const uint64_t end = first_tile_of_block(plan, blockIdx.x + 1);
     while (cur < end) {
-        stats_hinted_piece<BF16, FALLBACK>(next_piece(plan, cur, end), plan, grad, grad_stride, kappa, hint, stats, partials, tickets, sh);
+        stats_piece<BF16, PASS>(next_piece(plan, cur, end), plan, grad, grad_stride, g_min, kappa, stats, partials, tickets, sh);
         __syncthreads();                                       // the next piece reuses the shared arrays
     }
+}
+
+// ---- hinted threshold -----------------------------------------------------------------------------------------
+// The paper leaves the choice of g_min open (Section 4.1 only calls it the lower end of the power-law range); with g_min =
+// kappa * mean|g| rounded DOWN TO A POWER OF TWO the tail sums can be gathered before the mean is known, for two
+// candidate powers of two at once: a caller-kept hint (the kappa * mean|g| of the previous round) names the two
+// candidates nearest to it, and the launch that folds the records keeps the candidate that the finished mean selects.
+// If neither fits (first round, or the mean moved by more than a factor of about 1.4 to 2), that launch redoes the tail sums for the
+// right threshold, so the host never has to look.  The sums of one threshold are the same, bit for bit, whichever way
+// they were obtained: both sum log2|g| itself and take n * log2(g_min), an integer multiple, out at the end.
+
+// Smaller candidate for a hint; the other one is twice that.  Inf: no hint.
+__device__ __forceinline__ float lower_candidate(float level) {
+    if (!(level >= 2.3509887e-38f && level <= kMaxFinite)) return CUDART_INF_F;      // from 2^-125: both candidates are normal numbers
+    const uint32_t bits = __float_as_uint(level), e = bits & 0x7F800000u;
+    return __uint_as_float((bits & 0x00400000u) ? e : e - 0x00800000u);             // mantissa >= 1.5: {2^h, 2^(h+1)}, else {2^(h-1), 2^h}
+}
+// Which of the candidates t, 2 t is the threshold: 0, 1, -1 neither, 2 there is no tail at all.
+__device__ __forceinline__ int candidate_of(float g_min, float t) {
+    return !(g_min > 0.0f && g_min <= kMaxFinite) ? 2 : g_min == t ? 0 : g_min == 2.0f * t ? 1 : -1;
+}
+
+template <bool BF16>
+__device__ __forceinline__ void hinted_piece(const JobPiece& piece, const void* grad, uint64_t grad_stride,
+                                             const tq_gmin_hint_t* hint, Partial* partials, uint32_t* tickets, BlockFold<kWarps>& sh) {
+    const char* row = row_of<BF16>(piece, grad, grad_stride);
+    const float t = lower_candidate(hint[piece.job].level);
+    const TailTest test(t);
+    Gathered<BF16> g;
+    walk(row, piece.tile0 * kThreads + threadIdx.x, chunk_end_of<BF16>(piece), kThreads,
+         [&](uint64_t c, Words& w) { take_pow2<BF16, 2, true>(row, c, w, t, test, g); });
+    uint64_t j;
+    if (piece.last && has_leftover<BF16>(piece.d, j)) {
+        g.take_exact(exact_sums<BF16>(row, j, 1, t, 1.0f), true, 0, true);
+        g.take_exact(exact_sums<BF16>(row, j, 1, 2.0f * t, 1.0f), false, 1, true);
+    }
+    Partial p = g.partial();
+    block_fold<kWarps, true, 2>(p, sh);
+    if (threadIdx.x == 0) {
+        p.pad = hint[piece.job].level;                           // the finishing launch overwrites the hint
+        *record_of_piece(piece, partials) = p;
+        if (piece.tile0 == 0) tickets[piece.job] = 0u;           // for the finishing launch
+    }
+}
+
+template <bool BF16>
+__device__ __forceinline__ void hinted_finish_piece(const JobPiece& piece, const TilePlan& plan, const void* grad, uint64_t grad_stride,
+                                                    float kappa, tq_gmin_hint_t* hint_out, tq_stats_t* stats,
+                                                    Partial* partials, uint32_t* tickets, BlockFold<kWarps>& sh) {
+    uint32_t count;
+    const Partial* records = records_of_job(plan, piece, partials, count);
+    const float level = mean_level(kappa, fold_sum_abs(records, count, sh), piece.d), g_min = pow2_floor(level);
+    const int pick = candidate_of(g_min, lower_candidate(record_of_piece(piece, partials)->pad));
+    if (piece.tile0 == 0) {
+        Partial r;
+        fold_records<true, 0>(records, count, r, sh);
+        if (threadIdx.x == 0) {
+            store_moments(stats + piece.job, piece.d, r, g_min);
+            hint_out[piece.job].level = level;
+            hint_out[piece.job].hit = pick >= 0 ? 1u : 0u;
+            if (pick == 2) store_tail_pow2(stats + piece.job, 0, 0.0, g_min);
+        }
+        __syncthreads();
+        if (pick == 0 || pick == 1) {
+            fold_records<false, 2>(records, count, r, sh);
+            if (threadIdx.x == 0) store_tail_pow2(stats + piece.job, r.n_tail[pick], r.sum_log2[pick], g_min);
+        }
+    }
+    if (pick >= 0) return;
+
+    const char* row = row_of<BF16>(piece, grad, grad_stride);
+    const TailTest test(g_min);
+    Gathered<BF16> g;
+    walk(row, piece.tile0 * kThreads + threadIdx.x, chunk_end_of<BF16>(piece), kThreads,
+         [&](uint64_t c, Words& w) { take_pow2<BF16, 1, false>(row, c, w, g_min, test, g); });
+    uint64_t j;
+    if (piece.last && has_leftover<BF16>(piece.d, j)) g.take_exact(exact_sums<BF16>(row, j, 1, g_min, 1.0f), false, 0, true);
+    Partial p = g.partial();
+    block_fold<kWarps, false, 1>(p, sh);
+    if (!last_of_job(record_of_piece(piece, partials), p, false, tickets + piece.job, count, sh)) return;
+    fold_records<false, 1>(records, count, p, sh);
+    if (threadIdx.x == 0) store_tail_pow2(stats + piece.job, p.n_tail[0], p.sum_log2[0], g_min);
+}
+
+template <bool BF16>
+__global__ void __launch_bounds__(kThreads, kStatsBlocksPerSm)
+stats_hinted_kernel(const void* __restrict__ grad, uint64_t grad_stride, const tq_gmin_hint_t* hint, Partial* partials, uint32_t* tickets,
+                    const __grid_constant__ TilePlan plan) {
+    __shared__ BlockFold<kWarps> sh;
+    pdl_wait();
+    uint64_t cur = first_tile_of_block(plan, blockIdx.x);
+    const uint64_t end = first_tile_of_block(plan, blockIdx.x + 1);
+    while (cur < end) {
+        hinted_piece<BF16>(next_piece(plan, cur, end), grad, grad_stride, hint, partials, tickets, sh);
+        __syncthreads();                                       // the next piece reuses the shared arrays
+    }
+}
+template <bool BF16>
+__global__ void __launch_bounds__(kThreads, kStatsBlocksPerSm)
+stats_hinted_finish_kernel(const void* __restrict__ grad, uint64_t grad_stride, float kappa, tq_gmin_hint_t* hint, tq_stats_t* stats,
+                           Partial* partials, uint32_t* tickets, const __grid_constant__ TilePlan plan) {
+    __shared__ BlockFold<kWarps> sh;
+    pdl_wait();
+    uint64_t cur = first_tile_of_block(plan, blockIdx.x);
+    const uint64_t end = first_tile_of_block(plan, blockIdx.x + 1);
+    while (cur < end) {
+        hinted_finish_piece<BF16>(next_piece(plan, cur, end), plan, grad, grad_stride, kappa, hint, stats, partials, tickets, sh);
+        __syncthreads();
+    }
+}
+
+// ---- short rows: one cluster per job, one launch -----------------------------------------------------------------
+constexpr int kCluster = 8, kSmallThreads = 512, kSmallWarps = kSmallThreads / 32;
+
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+template <class T>
+__device__ __forceinline__ T of_rank(const T& mine, uint32_t rank) {          // the same shared variable of another block of the cluster
+    static_assert(sizeof(T) == 4 || sizeof(T) == 8, "");
+    uint32_t addr;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(addr) : "r"(smem_addr(&mine)), "r"(rank));
+    if constexpr (sizeof(T) == 8) {
+        unsigned long long v;
+        asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(addr) : "memory");
+        return __builtin_bit_cast(T, v);
+    } else {
+        uint32_t v;
+        asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+        return __builtin_bit_cast(T, v);
+    }
+}
+
+// POW2: g_min = kappa * mean|g| rounded down to a power of two (the hint is kept up, not needed); else the caller's g_min, or
+// kappa * mean|g|.  The first two chunks of a thread stay in registers between the two passes, the others are read again.
+template <bool BF16, bool POW2>
+__global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kSmallThreads)
+stats_small_kernel(const void* __restrict__ grad, uint64_t grad_stride, float g_min, float kappa, tq_gmin_hint_t* hint, tq_stats_t* stats,
+                   const __grid_constant__ SegTable segs) {
+    __shared__ BlockFold<kSmallWarps> sh;
+    __shared__ Partial s_moments, s_tail;
+    pdl_wait();
+    const uint32_t job = blockIdx.x / kCluster, rank = blockIdx.x % kCluster, worker = job / segs.n, seg = job - worker * segs.n;
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint64_t d = segs.len[seg], n_chunks = d / kChunk<BF16>;
+    const char* row = static_cast<const char*>(grad) + (static_cast<uint64_t>(worker) * grad_stride + segs.off[seg]) * (BF16 ? 2 : 4);
+    constexpr uint32_t stride = kCluster * kSmallThreads;
+    const uint64_t c0 = rank * kSmallThreads + threadIdx.x;
+    const bool has0 = c0 < n_chunks, has1 = c0 + stride < n_chunks;
+    Words w0, w1;
+    if (has0) load_chunk(row, c0, w0);
+    if (has1) load_chunk(row, c0 + stride, w1);
+    uint64_t j;
+    const bool leftover = rank == kCluster - 1 && has_leftover<BF16>(d, j);
+
+    Gathered<BF16> g;
+    auto first_pass = [&](uint64_t c, Words& w) { take_any<BF16, kMoments>(row, c, w, 0.0f, 0.0f, g); };
+    if (has0) first_pass(c0, w0);
+    if (has1) first_pass(c0 + stride, w1);
+    walk(row, c0 + 2 * stride, n_chunks, stride, first_pass);
+    if (leftover) g.take_exact(exact_sums<BF16>(row, j, 1, CUDART_INF_F, 0.0f), true, 0, false);
+    Partial p = g.partial();
+    block_fold<kSmallWarps, true, 0>(p, sh);
+    if (threadIdx.x == 0) s_moments = p;
+    cluster_sync();
+
+    auto over_ranks = [&](auto v) {                            // lanes 0..7 hold one block's value each
+        v = lane < kCluster ? v : decltype(v)(0);
+#pragma unroll
+        for (int o = kCluster / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+        return __shfl_sync(0xFFFFFFFFu, v, 0);
+    };
+    const uint32_t from = lane % kCluster;
+    const double sum_abs = over_ranks(of_rank(s_moments.sum_abs, from));      // every warp for itself, in the same order
+    const float level = mean_level(kappa, sum_abs, d);
+    if constexpr (POW2) g_min = pow2_floor(level);
+    else if (!(g_min > 0.0f)) g_min = level;
+    const bool tail_on = g_min > 0.0f && g_min <= kMaxFinite;
+    const float inv = inverse_of(g_min);
+    const TailTest test(g_min);
+
+    g = Gathered<BF16>();
+    if (tail_on) {
+        auto second_pass = [&](uint64_t c, Words& w) {
+            if constexpr (POW2) take_pow2<BF16, 1, false>(row, c, w, g_min, test, g);
+            else take_any<BF16, kTail>(row, c, w, g_min, inv, g);
+        };
+        if (has0) second_pass(c0, w0);
+        if (has1) second_pass(c0 + stride, w1);
+        walk(row, c0 + 2 * stride, n_chunks, stride, second_pass);
+        if (leftover) g.take_exact(exact_sums<BF16>(row, j, 1, g_min, POW2 ? 1.0f : inv), false, 0, true);
+    }
+    p = g.partial();
+    block_fold<kSmallWarps, false, 1>(p, sh);
+    if (threadIdx.x == 0) s_tail = p;
+    cluster_sync();
+    if (rank == 0 && threadIdx.x < 32) {
+        Partial t{};
+        t.sum_abs = sum_abs;
+        t.sum_sq = over_ranks(of_rank(s_moments.sum_sq, from));
+        t.n_bad = over_ranks(of_rank(s_moments.n_bad, from));
+        t.max_abs = warp_max(of_rank(s_moments.max_abs, from));
+        const unsigned long long n = over_ranks(of_rank(s_tail.n_tail[0], from));
+        const double sum_log2 = over_ranks(of_rank(s_tail.sum_log2[0], from));
+        if (lane == 0) {
+            store_moments(stats + job, d, t, g_min);
+            if constexpr (POW2) {
+                store_tail_pow2(stats + job, n, sum_log2, g_min);
+                hint[job].hit = candidate_of(g_min, lower_candidate(hint[job].level)) >= 0 ? 1u : 0u;      // as the long form reports it
+                hint[job].level = level;
+            } else {
+                store_tail(stats + job, n, sum_log2, g_min, inv);
+            }
+        }
+    }
+    cluster_sync();                                            // no block leaves while another reads its shared memory
+}
+
+// ---- launches -----------------------------------------------------------------------------------------------------
+
+// Rows of at most this many bytes, in calls whose clusters are resident at the same time, take the cluster kernel.  Device
+// time against the two launches (hinted / two-pass): 100 k x 1 fp32 6.5 / 6.4 against 8.0 / 8.5 us, 250 k x 8 10.9 / 10.3 against
+// 11.5 / 12.7; beyond, the few SMs of a cluster are too slow (500 k x 1: 13.2 against 9.0 us) or the clusters queue
+// (250 k x 16: 18.7 against 13.9 us).  One launch less on the host (2.5 us) comes on top.
+constexpr uint64_t kSmallRowBytes = 1u << 20;
+constexpr uint32_t kSmallMaxJobs = 8;
+
+static void plan_stats(const StatsCall& c, uint32_t n_jobs, TilePlan* plan) {
+    uint64_t resident = static_cast<uint64_t>(sm_count()) * kStatsBlocksPerSm;
+    const uint64_t room = static_cast<uint64_t>(n_jobs) * kRecordsPerJob - n_jobs;
+    if (resident > room) resident = room;
+    plan_tiles(plan, c.segs, c.d, c.n_workers, kThreads * kChunkBytes / (c.bf16 ? 2 : 4), resident);
+}
+
+// True when the call went to the cluster kernel.
+template <bool POW2>
+static bool launch_small(const StatsCall& c, uint32_t n_jobs, tq_gmin_hint_t* hint, cudaError_t* e) {
+    if (n_jobs > kSmallMaxJobs) return false;
+    SegTable one;
+    if (!c.segs) { one.n = 1; one.off[0] = 0; one.len[0] = c.d; }
+    const SegTable& segs = c.segs ? *c.segs : one;
+    for (uint32_t s = 0; s < segs.n; ++s)
+        if (segs.len[s] * (c.bf16 ? 2 : 4) > kSmallRowBytes) return false;
+    *e = launch_kernel(c.bf16 ? stats_small_kernel<true, POW2> : stats_small_kernel<false, POW2>, dim3(n_jobs * kCluster), kSmallThreads, 0,
+                       c.stream, c.grad, c.grad_stride, c.g_min, c.kappa, hint, c.stats, segs);
+    return true;
+}
+
+cudaError_t launch_stats(const StatsCall& c, int* launches) {
+    *launches = 0;
+    const uint32_t n_jobs = c.segs ? c.n_workers * c.segs->n : c.n_workers;
+    cudaError_t e;
+    if (launch_small<false>(c, n_jobs, nullptr, &e)) { *launches = e == cudaSuccess ? 1 : 0; return e; }
+    Partial* partials = static_cast<Partial*>(c.workspace);
+    uint32_t* tickets = reinterpret_cast<uint32_t*>(static_cast<char*>(c.workspace) + tickets_offset(n_jobs));
+    static thread_local TilePlan plan;
+    plan_stats(c, n_jobs, &plan);
+    auto launch = [&](auto kernel) {
+        e = launch_kernel(kernel, dim3(plan.blocks), kThreads, 0, c.stream, c.grad, c.grad_stride, c.g_min, c.kappa, c.stats, partials, tickets, plan);
+        *launches += e == cudaSuccess ? 1 : 0;
+        return e;
+    };
+    if (c.g_min > 0.0f) {
+        if ((e = cudaMemsetAsync(tickets, 0, static_cast<size_t>(n_jobs) * sizeof(uint32_t), c.stream)) != cudaSuccess) return e;
+        return launch(c.bf16 ? stats_kernel<true, kBoth> : stats_kernel<false, kBoth>);
+    }
+    if (launch(c.bf16 ? stats_kernel<true, kMoments> : stats_kernel<false, kMoments>) != cudaSuccess) return e;
+    return launch(c.bf16 ? stats_kernel<true, kTail> : stats_kernel<false, kTail>);
 }
 
 cudaError_t launch_stats_hinted(const StatsCall& c, tq_gmin_hint_t* hint, int* launches) {
     *launches = 0;
     const uint32_t n_jobs = c.segs ? c.n_workers * c.segs->n : c.n_workers;
-    PartialH* partials = static_cast<PartialH*>(c.workspace);
+    cudaError_t e;
+    if (launch_small<true>(c, n_jobs, hint, &e)) { *launches = e == cudaSuccess ? 1 : 0; return e; }
+    Partial* partials = static_cast<Partial*>(c.workspace);
     uint32_t* tickets = reinterpret_cast<uint32_t*>(static_cast<char*>(c.workspace) + tickets_offset(n_jobs));
-    cudaError_t e = cudaMemsetAsync(tickets, 0, static_cast<size_t>(n_jobs) * 2 * sizeof(uint32_t), c.stream);
-    if (e != cudaSuccess) return e;
-    static thread_local TilePlan plan;            // the same plan for both kernels: same summation order
-    plan_stats(c, n_jobs, TQ_STATS_HINTED_BLOCKS, &plan);
-    const auto kernel = c.bf16 ? stats_hinted_kernel<true, false> : stats_hinted_kernel<false, false>;
-    const auto tail_kernel = c.bf16 ? stats_hinted_kernel<true, true> : stats_hinted_kernel<false, true>;
-    kernel<<<plan.blocks, kThreads, 0, c.stream>>>(c.grad, c.grad_stride, c.kappa, hint, c.stats, partials, tickets, plan);
-    e = cudaGetLastError();
+    static thread_local TilePlan plan;            // the same plan for both launches: same summation order
+    plan_stats(c, n_jobs, &plan);
+    e = launch_kernel(c.bf16 ? stats_hinted_kernel<true> : stats_hinted_kernel<false>, dim3(plan.blocks), kThreads, 0, c.stream, c.grad,
+                      c.grad_stride, static_cast<const tq_gmin_hint_t*>(hint), partials, tickets, plan);
     if (e != cudaSuccess) return e;
     *launches = 1;
-    tail_kernel<<<plan.blocks, kThreads, 0, c.stream>>>(c.grad, c.grad_stride, c.kappa, hint, c.stats, partials, tickets, plan);
-    e = cudaGetLastError();
+    e = launch_kernel(c.bf16 ? stats_hinted_finish_kernel<true> : stats_hinted_finish_kernel<false>, dim3(plan.blocks), kThreads, 0, c.stream,
+                      c.grad, c.grad_stride, c.kappa, hint, c.stats, partials, tickets, plan);
     if (e == cudaSuccess) *launches = 2;
     return e;
 }
