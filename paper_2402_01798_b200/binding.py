@@ -124,9 +124,13 @@ def _check(status: int, where: str) -> None:
         raise TqError(status, where, detail)
 
 
+# torch.cuda.current_stream().cuda_stream without the Stream object (3.3 us of every call's 8)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or (lambda device: torch.cuda.current_stream(device).cuda_stream)
+
+
 def _stream(stream) -> int:
     if stream is None:
-        return torch.cuda.current_stream().cuda_stream
+        return _raw_stream(torch.cuda.current_device())
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 

@@ -400,7 +400,8 @@ compress_kernel(const void* __restrict__ grad, uint64_t d, uint64_t grad_stride,
     const uint32_t worker = first_worker + blockIdx.y;
     const char* row = static_cast<const char*>(grad) + static_cast<uint64_t>(blockIdx.y) * grad_stride * esz;
     uint32_t* prow = packed + static_cast<uint64_t>(blockIdx.y) * words_stride;
-    build_tables<BITS, SEARCH>(q, s_grid, s_cell, s_search);
+    build_tables<BITS, SEARCH>(q, s_grid, s_cell, s_search);          // from kernel parameters: before the wait
+    pdl_wait();
     const RunCtx cx{q.alpha, q.inv_step, q.top, q.inv_2alpha, q.cell_scale, uniform_q<BITS>(q), reinterpret_cast<const char*>(s_grid),
                     reinterpret_cast<const char*>(s_cell), s_search};
     const uint64_t whole = (d - 1) >> 5, stride = static_cast<uint64_t>(gridDim.x) * kThreads;     // runs before the row's last one are whole
@@ -453,9 +454,10 @@ compress_tma_kernel(const __grid_constant__ CUtensorMap tmap, const void* __rest
     if (threadIdx.x == 0) {
         mbar_init(bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        if (tile < n_tiles) issue(tile);
     }
-    build_tables<BITS, kGrid>(q, s_grid, s_cell, nullptr);            // ends with a block barrier
+    build_tables<BITS, kGrid>(q, s_grid, s_cell, nullptr);            // from kernel parameters; ends with a block barrier
+    pdl_wait();
+    if (threadIdx.x == 0 && tile < n_tiles) issue(tile);
 
     constexpr size_t esz = BF16 ? 2 : 4;
     const char* row = static_cast<const char*>(grad) + static_cast<uint64_t>(wi) * grad_stride * esz;
@@ -597,6 +599,7 @@ compress_kernel_dev(const void* __restrict__ grad, uint64_t grad_stride, const t
                     const __grid_constant__ RoundKeys rk, uint32_t first_worker, uint32_t* __restrict__ packed, uint64_t words_stride,
                     const __grid_constant__ TilePlan plan, int table_kernel_ran) {
     __shared__ __align__(16) BlockState<NONUNIFORM> sh;
+    pdl_wait();
     if (threadIdx.x == 0) sh.cur = first_tile_of_block(plan, blockIdx.x);
     while (true) {
         __syncthreads();                 // the previous piece has been served
@@ -658,9 +661,7 @@ static uint32_t choose_cells(const tq_params_t& p, float inv_2alpha) {
 static dim3 compress_grid(uint64_t d, uint32_t n_workers, bool persistent) {
     const uint64_t n_runs = (d + 31) >> 5;
     const uint64_t tiles = (n_runs + kThreads - 1) / kThreads;
-    int dev = 0, sms = 148;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    uint64_t per_worker = static_cast<uint64_t>(sms) * TQ_COMPRESS_MIN_BLOCKS / n_workers;   // rounded down: one wave holds the grid
+    uint64_t per_worker = static_cast<uint64_t>(sm_count()) * TQ_COMPRESS_MIN_BLOCKS / n_workers;   // rounded down: one wave holds the grid
     if (!persistent || per_worker > tiles) per_worker = tiles;
     if (per_worker > 0x7FFFFFFFull) per_worker = 0x7FFFFFFFull;
     if (per_worker < 1) per_worker = 1;
@@ -669,9 +670,8 @@ static dim3 compress_grid(uint64_t d, uint32_t n_workers, bool persistent) {
 
 template <int BITS, int SEARCH, bool BF>
 static cudaError_t launch(const CompressCall& c, const CompressArgs& args, dim3 grid) {
-    compress_kernel<BITS, SEARCH, BF><<<grid, kThreads, 0, c.stream>>>(
-        c.grad, c.d, c.grad_stride, args, round_keys(c.seed), c.first_worker, c.packed, c.words_stride);
-    return cudaGetLastError();
+    return launch_kernel(compress_kernel<BITS, SEARCH, BF>, grid, kThreads, 0, c.stream, c.grad, c.d, c.grad_stride, args, round_keys(c.seed),
+                         c.first_worker, c.packed, c.words_stride);
 }
 
 // ---- tiled copies: the tensor map of the gradient, [N][whole runs][32 elements] ------------------------
@@ -719,9 +719,8 @@ static cudaError_t launch_tma(const CompressCall& c, const CompressArgs& args, d
     const int smem = kThreads * 32 * (BF ? 2 : 4) + 16;
     const cudaError_t e = cudaFuncSetAttribute(compress_tma_kernel<BITS, BF>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    compress_tma_kernel<BITS, BF><<<grid, kThreads, smem, c.stream>>>(
-        map, c.grad, c.d, c.grad_stride, args, round_keys(c.seed), c.first_worker, c.packed, c.words_stride);
-    return cudaGetLastError();
+    return launch_kernel(compress_tma_kernel<BITS, BF>, grid, kThreads, smem, c.stream, map, c.grad, c.d, c.grad_stride, args,
+                         round_keys(c.seed), c.first_worker, c.packed, c.words_stride);
 }
 
 template <int BITS>
@@ -777,9 +776,8 @@ template <int BITS>
 static cudaError_t dispatch_dev(const CompressCall& c, const TilePlan& plan, int table_kernel_ran) {
     const auto kernel = c.nonuniform ? (c.bf16 ? compress_kernel_dev<BITS, true, true> : compress_kernel_dev<BITS, true, false>)
                                      : (c.bf16 ? compress_kernel_dev<BITS, false, true> : compress_kernel_dev<BITS, false, false>);
-    kernel<<<plan.blocks, kThreads, 0, c.stream>>>(c.grad, c.grad_stride, c.params_dev, round_keys(c.seed), c.first_worker, c.packed,
-                                                   c.words_stride, plan, table_kernel_ran);
-    return cudaGetLastError();
+    return launch_kernel(kernel, dim3(plan.blocks), kThreads, 0, c.stream, c.grad, c.grad_stride, c.params_dev, round_keys(c.seed),
+                         c.first_worker, c.packed, c.words_stride, plan, table_kernel_ran);
 }
 
 cudaError_t launch_compress_dev(const CompressCall& c) {
@@ -787,10 +785,8 @@ cudaError_t launch_compress_dev(const CompressCall& c) {
     // kernel (a small grid then: it normally finds nothing left) takes the others
     bool lut = false;
     if (const cudaError_t e = launch_compress_lut(c, &lut)) return e;
-    int dev = 0, sms = 148;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     static thread_local TilePlan plan;
-    plan_tiles(&plan, c.segs, c.d, c.n_workers, 32 * kThreads, static_cast<uint64_t>(sms) * (lut ? 1 : TQ_COMPRESS_MIN_BLOCKS));
+    plan_tiles(&plan, c.segs, c.d, c.n_workers, 32 * kThreads, static_cast<uint64_t>(sm_count()) * (lut ? 1 : TQ_COMPRESS_MIN_BLOCKS));
     if (c.launches) *c.launches = lut ? 2 : 1;
     switch (c.bits) {
         case 1: return dispatch_dev<1>(c, plan, lut);

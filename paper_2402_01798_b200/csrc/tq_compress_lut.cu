@@ -159,7 +159,7 @@ __device__ __forceinline__ void load_piece(const char* row, uint64_t piece, uint
 constexpr int kLutThreads = kThreads;
 
 // A block's share of one row: build the table for quantizer q (n_entries per sign), then quantize.
-template <int BITS>
+template <int BITS, bool WAIT>
 __device__ __forceinline__ void lut_block(const LutWorker& q, uint32_t n_entries, float* s_table, const char* __restrict__ row,
                                           uint32_t* __restrict__ prow, uint64_t d, uint64_t words_out, uint32_t worker,
                                           const RoundKeys& rk) {
@@ -175,6 +175,7 @@ __device__ __forceinline__ void lut_block(const LutWorker& q, uint32_t n_entries
         }
     }
     __syncthreads();
+    if constexpr (WAIT) pdl_wait();          // the table came from kernel parameters
 
     constexpr int E = Piece<BITS>::kElems, PER_ITER = 32 / E;   // 32 elements per thread and iteration: four Philox blocks in flight
     const LutCtx cx{smem_addr(s_table), q.negtop2, q.base2, (n_entries - 1) * 0x00010001u, philox_run(0u, worker, rk)};
@@ -225,7 +226,7 @@ compress_lut_kernel(const void* __restrict__ grad, uint64_t d, uint64_t grad_str
                     uint32_t* __restrict__ packed, uint64_t words_stride, uint64_t words_out) {
     extern __shared__ __align__(16) float s_table[];          // kLutMaxEntries + n_entries: the negative half starts at entry kLutMaxEntries
     const uint32_t wi = blockIdx.y;
-    lut_block<BITS>(args.q[wi], n_entries, s_table, static_cast<const char*>(grad) + static_cast<uint64_t>(wi) * grad_stride * 2,
+    lut_block<BITS, true>(args.q[wi], n_entries, s_table, static_cast<const char*>(grad) + static_cast<uint64_t>(wi) * grad_stride * 2,
                     packed + static_cast<uint64_t>(wi) * words_stride, d, words_out, first_worker + wi, rk);
 }
 
@@ -241,6 +242,7 @@ compress_lut_kernel_dev(const void* __restrict__ grad, uint64_t d, uint64_t grad
     __shared__ LutWorker s_q;
     __shared__ bool s_serves;
     const uint32_t wi = blockIdx.y;
+    pdl_wait();
     if (threadIdx.x < TQ_MAX_LEVELS) {
         s_q.levels[threadIdx.x] = params[wi].levels[threadIdx.x];
         s_q.inv_width[threadIdx.x] = params[wi].inv_width[threadIdx.x];
@@ -254,7 +256,7 @@ compress_lut_kernel_dev(const void* __restrict__ grad, uint64_t d, uint64_t grad
     }
     __syncthreads();
     if (!s_serves) return;
-    lut_block<BITS>(s_q, kLutMaxEntries, s_table, static_cast<const char*>(grad) + static_cast<uint64_t>(wi) * grad_stride * 2,
+    lut_block<BITS, false>(s_q, kLutMaxEntries, s_table, static_cast<const char*>(grad) + static_cast<uint64_t>(wi) * grad_stride * 2,
                     packed + static_cast<uint64_t>(wi) * words_stride, d, words_out, first_worker + wi, rk);
 }
 
@@ -280,18 +282,14 @@ static cudaError_t launch_lut(const CompressCall& c, const LutArgs& args, uint32
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, compress_lut_kernel<BITS>, kLutThreads, smem);
     if (e != cudaSuccess) return e;
     const uint64_t per_worker = lut_blocks_per_worker(c.d, c.n_workers, per_sm, Piece<BITS>::kElems);
-    const RoundKeys rk = round_keys(c.seed);
-    compress_lut_kernel<BITS><<<dim3(static_cast<unsigned>(per_worker), c.n_workers), kLutThreads, smem, c.stream>>>(
-        c.grad, c.d, c.grad_stride, args, rk, n_entries, c.first_worker, c.packed, c.words_stride, c.words_out);
-    return cudaGetLastError();
+    return launch_kernel(compress_lut_kernel<BITS>, dim3(static_cast<unsigned>(per_worker), c.n_workers), kLutThreads, smem, c.stream, c.grad, c.d,
+                         c.grad_stride, args, round_keys(c.seed), n_entries, c.first_worker, c.packed, c.words_stride, c.words_out);
 }
 
 
 static uint64_t lut_blocks_per_worker(uint64_t d, uint32_t n_workers, int per_sm, int pieces_elems) {
-    int dev = 0, sms = 148;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const uint64_t tiles = (d / pieces_elems + kLutThreads - 1) / kLutThreads + 1;
-    uint64_t per_worker = static_cast<uint64_t>(sms) * (per_sm < 1 ? 1 : per_sm) / n_workers;      // rounded down: one wave holds the grid
+    uint64_t per_worker = static_cast<uint64_t>(sm_count()) * (per_sm < 1 ? 1 : per_sm) / n_workers;      // rounded down: one wave holds the grid
     if (per_worker > tiles) per_worker = tiles;
     return per_worker < 1 ? 1 : per_worker;
 }
@@ -305,9 +303,8 @@ static cudaError_t launch_lut_dev(const CompressCall& c) {
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, compress_lut_kernel_dev<BITS>, kLutThreads, smem);
     if (e != cudaSuccess) return e;
     const uint64_t per_worker = lut_blocks_per_worker(c.d, c.n_workers, per_sm, Piece<BITS>::kElems);
-    compress_lut_kernel_dev<BITS><<<dim3(static_cast<unsigned>(per_worker), c.n_workers), kLutThreads, smem, c.stream>>>(
-        c.grad, c.d, c.grad_stride, c.params_dev, round_keys(c.seed), c.first_worker, c.packed, c.words_stride, c.words_out);
-    return cudaGetLastError();
+    return launch_kernel(compress_lut_kernel_dev<BITS>, dim3(static_cast<unsigned>(per_worker), c.n_workers), kLutThreads, smem, c.stream, c.grad,
+                         c.d, c.grad_stride, c.params_dev, round_keys(c.seed), c.first_worker, c.packed, c.words_stride, c.words_out);
 }
 
 // Rows below this many elements keep the element-wise kernels (the table costs more than it saves).

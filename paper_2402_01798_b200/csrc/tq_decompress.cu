@@ -237,7 +237,9 @@ decompress_kernel(const __grid_constant__ RowTable rt, uint64_t words_valid, uin
     // extracts it.  The lookups of one instruction go to one codebook, bank = code + 16 * (worker % 2):
     // they never conflict.
     __shared__ __align__(256) float s_tab[TQ_MAX_WORKERS * kTabStride];
-    fill_tables(s_tab, n, args, dt);
+    if (!dt.params_dev) fill_tables(s_tab, n, args, dt);            // from kernel parameters: before the wait
+    pdl_wait();
+    if (dt.params_dev) fill_tables(s_tab, n, args, dt);
     __syncthreads();
     const char* tab_bytes = reinterpret_cast<const char*>(s_tab);
 
@@ -378,9 +380,12 @@ decompress_bulk_kernel(const __grid_constant__ RowTable rt, uint64_t words_row, 
     if (threadIdx.x == 0) {
         for (int st = 0; st < S; ++st) mbar_init(bar0 + 8 * st, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        for (uint32_t q = 0; q < S && q < n_steps; ++q) issue(q);
     }
-    fill_tables(s_tab, n, args, dt, pstride, poff);
+    if (!dt.params_dev) fill_tables(s_tab, n, args, dt);            // from kernel parameters: before the wait
+    pdl_wait();
+    if (threadIdx.x == 0)
+        for (uint32_t q = 0; q < S && q < n_steps; ++q) issue(q);
+    if (dt.params_dev) fill_tables(s_tab, n, args, dt, pstride, poff);
     __syncthreads();          // barriers initialised and codebooks in place for every thread
     const char* tab_bytes = reinterpret_cast<const char*>(s_tab);
 
@@ -452,9 +457,8 @@ static cudaError_t launch_bulk(const DecompressCall& c, const RowTable& rt, cons
                                                    cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
         if (e != cudaSuccess) return e;
     }
-    decompress_bulk_kernel<BITS, APPLY><<<static_cast<unsigned>(tiles), kDecThreads, smem, c.stream>>>(
-        rt, c.words_valid, c.n_workers, c.d, args, dt, scale, divide, ap, c.out, st);
-    return cudaGetLastError();
+    return launch_kernel(decompress_bulk_kernel<BITS, APPLY>, dim3(static_cast<unsigned>(tiles)), kDecThreads, smem, c.stream, rt, c.words_valid,
+                         c.n_workers, c.d, args, dt, scale, divide, ap, c.out, st);
 }
 
 template <int BITS>
@@ -484,13 +488,8 @@ static cudaError_t launch(const DecompressCall& c, const RowTable& rt, const Dec
     if (blocks >= kBulkMinTiles)
         return c.theta ? launch_bulk<BITS, true>(c, rt, args, dt, scale, divide, ap, blocks)
                        : launch_bulk<BITS, false>(c, rt, args, dt, scale, divide, ap, blocks);
-    if (c.theta)
-        decompress_kernel<BITS, true><<<static_cast<unsigned>(blocks), kDecThreads, 0, c.stream>>>(
-            rt, c.words_valid, c.n_workers, c.d, args, dt, scale, divide, ap, c.out);
-    else
-        decompress_kernel<BITS, false><<<static_cast<unsigned>(blocks), kDecThreads, 0, c.stream>>>(
-            rt, c.words_valid, c.n_workers, c.d, args, dt, scale, divide, ap, c.out);
-    return cudaGetLastError();
+    return launch_kernel(c.theta ? decompress_kernel<BITS, true> : decompress_kernel<BITS, false>, dim3(static_cast<unsigned>(blocks)), kDecThreads,
+                         0, c.stream, rt, c.words_valid, c.n_workers, c.d, args, dt, scale, divide, ap, c.out);
 }
 
 cudaError_t read_wait_expired(unsigned int* count) {

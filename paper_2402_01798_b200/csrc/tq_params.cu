@@ -21,6 +21,7 @@
 #include <cmath>
 
 #include "tq.h"
+#include "tq_device.cuh"
 #include "tq_launch.h"
 
 namespace tq {
@@ -396,9 +397,10 @@ params_kernel(const tq_stats_t* __restrict__ stats, uint32_t n, uint32_t num_lev
               double alpha_user, tq_params_t* __restrict__ out) {
     __shared__ tq_params_t s_p[kParamsWarps];
     const uint32_t warp = threadIdx.x >> 5, i = blockIdx.x * kParamsWarps + warp;
-    if (i >= n) return;
+    if (i >= n) return;              // nothing of this warp reads or writes memory
     const OneWarp lanes;
     tq_params_t* p = &s_p[warp];
+    pdl_wait();
     const tq_stats_t st = stats[i];
     const tq_status s = design(lanes, &st, num_levels, bits, MODE, gamma, rule, alpha_user, p);
     __syncwarp();
@@ -416,10 +418,9 @@ params_kernel(const tq_stats_t* __restrict__ stats, uint32_t n, uint32_t num_lev
 cudaError_t launch_params_device(const tq_stats_t* stats_dev, uint32_t n, uint32_t num_levels, uint32_t bits, uint32_t mode,
                                  double gamma, int rule, double alpha_user, tq_params_t* params_dev, cudaStream_t stream) {
     const uint32_t warps = n < kParamsWarps ? n : kParamsWarps;      // few records: no idle warps to launch
-    const dim3 grid((n + kParamsWarps - 1) / kParamsWarps), block(32 * warps);
+    const dim3 grid((n + kParamsWarps - 1) / kParamsWarps);
     auto* kernel = mode == TQ_UNIFORM ? params_kernel<TQ_UNIFORM> : mode == TQ_NONUNIFORM ? params_kernel<TQ_NONUNIFORM> : params_kernel<TQ_BISCALED>;
-    kernel<<<grid, block, 0, stream>>>(stats_dev, n, num_levels, bits, gamma, rule, alpha_user, params_dev);
-    return cudaGetLastError();
+    return launch_kernel(kernel, grid, 32 * warps, 0, stream, stats_dev, n, num_levels, bits, gamma, rule, alpha_user, params_dev);
 }
 
 bool params_request_ok(uint32_t num_levels, int mode, int rule, uint32_t* bits) { return valid_request(num_levels, mode, rule, bits); }
