@@ -3,9 +3,9 @@
 // fused in one streaming pass.  fp32 adds happen in worker order, so the result does not depend on
 // the launch shape.
 //
-// Work split: a thread owns 32 output elements as units whose codes fill whole 32-bit words (see
-// Unit below), keeps one fp32 accumulator per element in registers and walks the workers four at a
-// time so that many independent loads are in flight before the dependent lookups start.
+// Work split: a thread owns up to 32 output elements as units whose codes fill whole 32-bit words (see
+// Unit below), keeps one fp32 accumulator per element in registers and walks the workers in groups
+// so that many independent loads are in flight before the dependent lookups start.
 // Codebooks live in shared memory, 16 consecutive words per worker, four workers per 256 bytes: any
 // set of codes of one worker maps to distinct banks, so lookups are conflict-free.
 // HBM traffic per output element: N * bits / 8 bytes read, 4 bytes written.
@@ -52,16 +52,12 @@ constexpr int kTabStride = 16;   // floats between consecutive workers' codebook
 
 // A unit is a run of elements decoded from one 32-bit "field": 8 / 16 / 32 elements = one packed word
 // for 4 / 2 / 1 bits; for 3 bits 8 elements = 24 bits that start on a byte boundary and are cut out of
-// two neighbouring words.  A thread owns 32 / kElems units, spaced one block apart, so that every
-// load and every 256-bit store of a warp is contiguous, and keeps 32 accumulators in registers.
+// two neighbouring words.  A thread owns U units, spaced one block apart, so that every
+// load and every 256-bit store of a warp is contiguous, and keeps U * kElems (at most 32) accumulators in registers.
 template <int BITS>
 struct Unit {
     static constexpr int kElems = BITS == 2 ? 16 : (BITS == 1 ? 32 : 8);
-#ifdef TQ_DECOMPRESS_ACC
-    static constexpr int kUnits = TQ_DECOMPRESS_ACC / kElems > 0 ? TQ_DECOMPRESS_ACC / kElems : 1;
-#else
-    static constexpr int kUnits = 32 / kElems;
-#endif
+    static constexpr int kMost = 32 / kElems;      // units of a thread with 32 accumulators
 };
 
 // The field of unit u of one row, all words known to be inside the row.
@@ -139,10 +135,10 @@ constexpr int kDecThreads = 128;
 // Turns the accumulated sums of a thread's units into outputs: the division by N (w_i = 1/N; for N a
 // power of two the product with 2^-k is the same value), then either the store of the aggregate or
 // the fused model update.  Unit k of the thread is unit u0 + k * kDecThreads of the row.
-template <int BITS, bool APPLY>
-__device__ __forceinline__ void finish_units(f32x2 (&acc)[Unit<BITS>::kUnits][Unit<BITS>::kElems / 2], uint64_t u0, uint64_t d,
+template <int BITS, bool APPLY, int U>
+__device__ __forceinline__ void finish_units(f32x2 (&acc)[U][Unit<BITS>::kElems / 2], uint64_t u0, uint64_t d,
                                              float scale, int divide, const ApplyArgs& ap, float* __restrict__ out) {
-    constexpr int E = Unit<BITS>::kElems, U = Unit<BITS>::kUnits;
+    constexpr int E = Unit<BITS>::kElems;
 #pragma unroll
     for (int k = 0; k < U; ++k) {
         float o[E];
@@ -161,11 +157,16 @@ __device__ __forceinline__ void finish_units(f32x2 (&acc)[Unit<BITS>::kUnits][Un
 #pragma unroll
             for (int v = 0; v < E / 8; ++v) {
                 float th[8], mo[8];
+                if (whole) {
+                    ldg256(ap.theta + j0 + 8 * v, th);
+                    if (ap.momentum_buf) ldg256(ap.momentum_buf + j0 + 8 * v, mo);
+                } else {
 #pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                    const uint64_t j = j0 + 8 * v + e;
-                    th[e] = (whole || j < d) ? ap.theta[j] : 0.0f;
-                    mo[e] = (ap.momentum_buf && (whole || j < d)) ? ap.momentum_buf[j] : 0.0f;
+                    for (int e = 0; e < 8; ++e) {
+                        const uint64_t j = j0 + 8 * v + e;
+                        th[e] = j < d ? ap.theta[j] : 0.0f;
+                        mo[e] = (ap.momentum_buf && j < d) ? ap.momentum_buf[j] : 0.0f;
+                    }
                 }
 #pragma unroll
                 for (int e = 0; e < 8; ++e) {
@@ -203,6 +204,9 @@ __device__ __forceinline__ void finish_units(f32x2 (&acc)[Unit<BITS>::kUnits][Un
 // Copies the N codebooks (already multiplied by w_i when weights are given) into shared memory.
 __device__ __forceinline__ void fill_tables(float* s_tab, uint32_t n, const DecompressArgs& args, const DeviceTables& dt,
                                             uint32_t pstride = 1, uint32_t poff = 0) {
+    // lanes read different words, which the constant bank would serve one after the other: read through the generic window
+    uint64_t table = reinterpret_cast<uint64_t>(&args.table[0][0]);
+    asm volatile("" : "+l"(table));
     for (uint32_t t = threadIdx.x; t < n * TQ_MAX_LEVELS; t += kDecThreads) {
         const uint32_t i = t / TQ_MAX_LEVELS, k = t % TQ_MAX_LEVELS;
         float v;
@@ -210,7 +214,7 @@ __device__ __forceinline__ void fill_tables(float* s_tab, uint32_t n, const Deco
             const float l = dt.params_dev[i * pstride + poff].levels[k];
             v = dt.use_weights ? __fmul_rn(dt.weights[i], l) : l;
         } else {
-            v = args.table[i][k];
+            v = reinterpret_cast<const float*>(table)[t];
         }
         s_tab[i * kTabStride + k] = v;
     }
@@ -230,7 +234,7 @@ decompress_kernel(const __grid_constant__ RowTable rt, uint64_t words_valid, uin
                   uint64_t d, const __grid_constant__ DecompressArgs args, const __grid_constant__ DeviceTables dt,
                   float scale, int divide, const __grid_constant__ ApplyArgs ap,
                   float* __restrict__ out) {
-    constexpr int E = Unit<BITS>::kElems, U = Unit<BITS>::kUnits;
+    constexpr int E = Unit<BITS>::kElems, U = 1, G = 16;
 
     // Every group of four codebooks starts on a 256-byte boundary of shared memory, so a table offset
     // (code * 4 < 64) can be merged into the group's base offset by the same byte-permute that
@@ -259,18 +263,31 @@ decompress_kernel(const __grid_constant__ RowTable rt, uint64_t words_valid, uin
 
     uint32_t i = 0;
     if (interior) {
-        for (; i + 4 <= n; i += 4) {          // four workers at a time: 4 * U independent fields in flight
-            uint32_t f[4][U];
+        for (; i + G <= n; i += G) {          // G workers at a time: G * U independent fields in flight
+            uint32_t f[G][U];
 #pragma unroll
-            for (int b = 0; b < 4; ++b)
+            for (int b = 0; b < G; ++b)
 #pragma unroll
                 for (int k = 0; k < U; ++k)
                     f[b][k] = load_field<BITS>(rt.row[i + b], u0 + k * kDecThreads);
 #pragma unroll
-            for (int b = 0; b < 4; ++b)
+            for (int b = 0; b < G; ++b)
 #pragma unroll
                 for (int k = 0; k < U; ++k)
-                    add_unit<BITS>(acc[k], f[b][k], tab_bytes + b * (kTabStride * 4), i * (kTabStride * 4));
+                    add_unit<BITS>(acc[k], f[b][k], tab_bytes + (b & 3) * (kTabStride * 4), (i + (b & ~3)) * (kTabStride * 4));
+        }
+        if constexpr (G > 4) {
+            for (; i + 4 <= n; i += 4) {
+                uint32_t f[4][U];
+#pragma unroll
+                for (int b = 0; b < 4; ++b)
+#pragma unroll
+                    for (int k = 0; k < U; ++k) f[b][k] = load_field<BITS>(rt.row[i + b], u0 + k * kDecThreads);
+#pragma unroll
+                for (int b = 0; b < 4; ++b)
+#pragma unroll
+                    for (int k = 0; k < U; ++k) add_unit<BITS>(acc[k], f[b][k], tab_bytes + b * (kTabStride * 4), i * (kTabStride * 4));
+            }
         }
     }
     for (; i < n; ++i) {                       // remaining workers, or every worker of an edge thread
@@ -284,9 +301,8 @@ decompress_kernel(const __grid_constant__ RowTable rt, uint64_t words_valid, uin
             add_unit<BITS>(acc[k], f[k], tab_bytes + (i & 3u) * (kTabStride * 4), (i & ~3u) * (kTabStride * 4));
     }
 
-    finish_units<BITS, APPLY>(acc, u0, d, scale, divide, ap, out);
+    finish_units<BITS, APPLY, U>(acc, u0, d, scale, divide, ap, out);
 }
-
 
 // ---------------------------------------------------------------------------------------------
 // Bulk-copy variant for large inputs.  One block decodes one tile of kDecThreads * 32 outputs.  The
@@ -307,10 +323,10 @@ constexpr int kGroup = TQ_DECOMPRESS_GROUP;   // workers per stage
 
 __device__ unsigned int g_wait_expired = 0;   // blocks (or threads) whose bounded wait ran out, since load
 
-template <int BITS>
+template <int BITS, int U>
 struct Tile {
     static constexpr int kUnitBytes = BITS == 3 ? 3 : 4;
-    static constexpr int kUnits = kDecThreads * Unit<BITS>::kUnits;     // units per tile (a multiple of 4)
+    static constexpr int kUnits = kDecThreads * U;                           // units per tile (a multiple of 4)
     static constexpr int kSegBytes = kUnits * kUnitBytes;               // one worker's bytes per tile (a multiple of 16)
 };
 
@@ -329,14 +345,14 @@ __device__ __forceinline__ uint32_t stage_field(const uint32_t* seg, uint32_t ul
 #define TQ_DECOMPRESS_BULK_BLOCKS 8
 #endif
 
-template <int BITS, bool APPLY>
+template <int BITS, bool APPLY, int U>
 __global__ void __launch_bounds__(kDecThreads, APPLY ? TQ_DECOMPRESS_BULK_BLOCKS - 2 : TQ_DECOMPRESS_BULK_BLOCKS)
 decompress_bulk_kernel(const __grid_constant__ RowTable rt, uint64_t words_row, uint32_t n,
                        uint64_t d_row, const __grid_constant__ DecompressArgs args, const __grid_constant__ DeviceTables dt,
                        float scale, int divide, const __grid_constant__ ApplyArgs ap_in, float* __restrict__ out_row,
                        const __grid_constant__ SegTiles st) {
-    constexpr int E = Unit<BITS>::kElems, U = Unit<BITS>::kUnits, S = TQ_DECOMPRESS_STAGES;
-    constexpr uint32_t kSeg = Tile<BITS>::kSegBytes;
+    constexpr int E = Unit<BITS>::kElems, S = TQ_DECOMPRESS_STAGES;
+    constexpr uint32_t kSeg = Tile<BITS, U>::kSegBytes;
 
     // [codebooks: n * 64 B][S stages of kGroup segments][16 B that a 3-bit field's second word may touch][S barriers]
     extern __shared__ __align__(1024) unsigned char smem[];
@@ -436,60 +452,71 @@ decompress_bulk_kernel(const __grid_constant__ RowTable rt, uint64_t words_row, 
         return;
     }
 
-    const uint64_t u0 = tile * Tile<BITS>::kUnits + threadIdx.x;
+    const uint64_t u0 = tile * Tile<BITS, U>::kUnits + threadIdx.x;
     if (u0 * E >= d) return;       // nothing of this thread's first unit (hence of any) exists
-    finish_units<BITS, APPLY>(acc, u0, d, scale, divide, ap, out);
+    finish_units<BITS, APPLY, U>(acc, u0, d, scale, divide, ap, out);
 }
-
-// Inputs of at least this many tiles go through the bulk-copy kernel; smaller ones are bound by
-// launch and set-up latency and keep the simpler direct kernel.
-constexpr uint64_t kBulkMinTiles = 8;
 
 static const SegTiles kNoSegTiles{};
 
-template <int BITS, bool APPLY>
+// Below this many tiles of 32 outputs per thread, two per SM, too few warps are in flight for the latency of a walk over the
+// workers: the direct kernel takes one unit per thread (1 M x 64, 3 bits: 27.5 -> 17.3 us; 20 k x 64: 58 -> 7.9 us; 489 tiles, 2 M x
+// 16: 10.8 us in the bulk form, 12.2 in the direct one).
+constexpr uint64_t kTilesForBulk = 296;
+// The fused update has as much to do after the walk as in it; up to this many tiles one unit per thread keeps more blocks
+// in flight (4 M x 4: 18.6 -> 14.3 us, 11.2 M x 8: 39.9 -> 37.3; 25.6 M x 16, 6250 tiles: 97 us against 102; with 64 workers the
+// walk weighs more again, 3 M x 64: 44 us against 56).
+constexpr uint64_t kTilesForLongApply = 4096;
+
+template <int BITS, bool APPLY, int U>
 static cudaError_t launch_bulk(const DecompressCall& c, const RowTable& rt, const DecompressArgs& args, const DeviceTables& dt,
                                float scale, int divide, const ApplyArgs& ap, uint64_t tiles, const SegTiles& st = kNoSegTiles) {
     const size_t smem = static_cast<size_t>(c.n_workers) * (kTabStride * 4) +
-                        static_cast<size_t>(TQ_DECOMPRESS_STAGES) * kGroup * Tile<BITS>::kSegBytes + 16 + 8 * TQ_DECOMPRESS_STAGES;
+                        static_cast<size_t>(TQ_DECOMPRESS_STAGES) * kGroup * Tile<BITS, U>::kSegBytes + 16 + 8 * TQ_DECOMPRESS_STAGES;
     if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(decompress_bulk_kernel<BITS, APPLY>,
+        const cudaError_t e = cudaFuncSetAttribute(decompress_bulk_kernel<BITS, APPLY, U>,
                                                    cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
         if (e != cudaSuccess) return e;
     }
-    return launch_kernel(decompress_bulk_kernel<BITS, APPLY>, dim3(static_cast<unsigned>(tiles)), kDecThreads, smem, c.stream, rt, c.words_valid,
+    return launch_kernel(decompress_bulk_kernel<BITS, APPLY, U>, dim3(static_cast<unsigned>(tiles)), kDecThreads, smem, c.stream, rt, c.words_valid,
                          c.n_workers, c.d, args, dt, scale, divide, ap, c.out, st);
+}
+
+template <int BITS, bool APPLY>
+static cudaError_t launch_apply(const DecompressCall& c, const RowTable& rt, const DecompressArgs& args, const DeviceTables& dt, float scale,
+                                int divide) {
+    constexpr int E = Unit<BITS>::kElems, U = Unit<BITS>::kMost;
+    constexpr uint64_t kPerTile = static_cast<uint64_t>(kDecThreads) * U * E;          // elements
+    const ApplyArgs ap{c.theta, c.momentum_buf, c.lr, c.mu, c.wd};
+    if (c.segs) {      // layer groups: the tiles of every segment in one grid, always through the bulk-copy kernel
+        static thread_local SegTiles st;
+        st.segs = *c.segs;
+        uint64_t total = 0;
+        for (uint32_t sg = 0; sg < c.segs->n; ++sg) {
+            st.tile_begin[sg] = static_cast<uint32_t>(total);
+            total += (c.segs->len[sg] + kPerTile - 1) / kPerTile;
+            if (total > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
+        }
+        st.tile_begin[c.segs->n] = static_cast<uint32_t>(total);
+        return launch_bulk<BITS, APPLY, U>(c, rt, args, dt, scale, divide, ap, total, st);
+    }
+    const uint64_t tiles = (c.d + kPerTile - 1) / kPerTile;
+    if (tiles == 0) return cudaSuccess;
+    if (tiles > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
+    if (tiles < kTilesForBulk) {
+        constexpr uint64_t kPerBlock = static_cast<uint64_t>(kDecThreads) * E;
+        return launch_kernel(decompress_kernel<BITS, APPLY>, dim3(static_cast<unsigned>((c.d + kPerBlock - 1) / kPerBlock)), kDecThreads, 0, c.stream, rt,
+                             c.words_valid, c.n_workers, c.d, args, dt, scale, divide, ap, c.out);
+    }
+    if (APPLY && U > 1 && tiles < kTilesForLongApply && c.n_workers <= 32)
+        return launch_bulk<BITS, APPLY, 1>(c, rt, args, dt, scale, divide, ap, tiles * U);
+    return launch_bulk<BITS, APPLY, U>(c, rt, args, dt, scale, divide, ap, tiles);
 }
 
 template <int BITS>
 static cudaError_t launch(const DecompressCall& c, const RowTable& rt, const DecompressArgs& args, const DeviceTables& dt, float scale,
                           int divide) {
-    if (c.segs) {      // layer groups: the tiles of every segment in one grid, always through the bulk-copy kernel
-        static thread_local SegTiles st;
-        st.segs = *c.segs;
-        const uint64_t per_tile = static_cast<uint64_t>(kDecThreads) * Unit<BITS>::kUnits * Unit<BITS>::kElems;   // elements
-        uint64_t total = 0;
-        for (uint32_t sg = 0; sg < c.segs->n; ++sg) {
-            st.tile_begin[sg] = static_cast<uint32_t>(total);
-            total += (c.segs->len[sg] + per_tile - 1) / per_tile;
-            if (total > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
-        }
-        st.tile_begin[c.segs->n] = static_cast<uint32_t>(total);
-        const ApplyArgs ap{c.theta, c.momentum_buf, c.lr, c.mu, c.wd};
-        return c.theta ? launch_bulk<BITS, true>(c, rt, args, dt, scale, divide, ap, total, st)
-                       : launch_bulk<BITS, false>(c, rt, args, dt, scale, divide, ap, total, st);
-    }
-    const uint64_t n_units = (c.d + Unit<BITS>::kElems - 1) / Unit<BITS>::kElems;
-    const uint64_t per_block = static_cast<uint64_t>(kDecThreads) * Unit<BITS>::kUnits;
-    const uint64_t blocks = (n_units + per_block - 1) / per_block;
-    if (blocks == 0) return cudaSuccess;
-    if (blocks > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
-    const ApplyArgs ap{c.theta, c.momentum_buf, c.lr, c.mu, c.wd};
-    if (blocks >= kBulkMinTiles)
-        return c.theta ? launch_bulk<BITS, true>(c, rt, args, dt, scale, divide, ap, blocks)
-                       : launch_bulk<BITS, false>(c, rt, args, dt, scale, divide, ap, blocks);
-    return launch_kernel(c.theta ? decompress_kernel<BITS, true> : decompress_kernel<BITS, false>, dim3(static_cast<unsigned>(blocks)), kDecThreads,
-                         0, c.stream, rt, c.words_valid, c.n_workers, c.d, args, dt, scale, divide, ap, c.out);
+    return c.theta ? launch_apply<BITS, true>(c, rt, args, dt, scale, divide) : launch_apply<BITS, false>(c, rt, args, dt, scale, divide);
 }
 
 cudaError_t read_wait_expired(unsigned int* count) {

@@ -95,3 +95,31 @@ def test_ranges_that_cross_jobs(tq, orc, dtype, L, mode, lengths):
             assert np.array_equal(rows[i], want), (s, i)
         assert np.array_equal(res[off:off + ln], orc.decompress_aggregate(rows, ln, [_oracle_params(orc, ps[i * S + s]) for i in range(n)]))
         w += words
+
+
+@pytest.mark.parametrize("bits,n", [(1, 3), (2, 17), (3, 64), (4, 5)])
+@pytest.mark.parametrize("d", [1, 1023, 1025, 4097, 295 * 4096 - 5, 295 * 4096 + 5, 300 * 4096 + 1])
+def test_aggregation_forms(tq, orc, bits, n, d):
+    """One unit per thread up to 295 tiles of 4096 outputs, bulk copies beyond; rows one by one, weights, and the fused update
+    (its own split up to 4096 tiles).  Sums are taken in worker order with one rounding per operation: equal to the oracle."""
+    L = 1 << bits
+    r = random.Random(d)
+    ps = [tq.tq_params_from_levels(sorted([-1.0 - i] + [r.uniform(-0.9, 0.9) for _ in range(L - 2)] + [1.0 + i])) for i in range(n)]
+    ops = [_oracle_params(orc, p) for p in ps]
+    words = tq.tq_packed_words(d, bits)
+    gen = torch.Generator(device="cuda").manual_seed(d)
+    packed = torch.randint(-2 ** 31, 2 ** 31 - 1, (n, words), dtype=torch.int32, device="cuda", generator=gen)
+    host = packed.cpu().numpy().view(np.uint32)
+    want = orc.decompress_aggregate(host, d, ops)
+    assert np.array_equal(tq.tq_decompress_aggregate(packed, d, ps).cpu().numpy(), want)
+    weights = [0.01 * (i + 1) for i in range(n)]
+    rows = [packed[i].clone() for i in range(n)]
+    got = tq.tq_decompress_aggregate_rows(rows, d, ps, weights=weights)
+    assert np.array_equal(got.cpu().numpy(), orc.decompress_aggregate(host, d, ops, np.array(weights, np.float32)))
+    theta, mom = torch.randn(d, device="cuda", generator=gen), torch.randn(d, device="cuda", generator=gen)
+    t0, m0, f = theta.cpu().numpy(), mom.cpu().numpy(), np.float32
+    tq.tq_decompress_aggregate_apply(packed, d, ps, theta, mom, lr=0.1, momentum=0.9, weight_decay=1e-3)
+    g = want + f(1e-3) * t0
+    m1 = f(0.9) * m0 + g
+    assert np.array_equal(mom.cpu().numpy(), m1) and np.array_equal(theta.cpu().numpy(), t0 - f(0.1) * m1)
+    assert tq.tq_wait_expired_count() == 0
