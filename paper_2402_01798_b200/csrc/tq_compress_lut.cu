@@ -13,7 +13,7 @@
 // smallest bf16 value >= alpha) every value is truncated to +-alpha; below its base pattern every value is
 // so small that the decision equals that of zero (the host checks this by evaluating the decision at
 // +-base; it is monotone in the value).  The index is clamp(|pattern| - base, 0, n - 1) + n * [negative],
-// n = 2048, 4096 or 8192 entries per sign (16, 32 or 64 binades), computed for the two elements of a
+// n entries per sign, as many whole binades (128 entries) as the quantizer needs, at most 64, computed for the two elements of a
 // 32-bit word at once with 16-bit SIMD integer instructions.  NaN is sent to -alpha before that by a
 // packed bf16 maximum with -top, which returns the operand that is a number, as fmaxf does in the
 // element-wise form.
@@ -240,23 +240,34 @@ compress_lut_kernel_dev(const void* __restrict__ grad, uint64_t d, uint64_t grad
                         uint64_t words_stride, uint64_t words_out) {
     extern __shared__ __align__(16) float s_table[];          // 2 * kLutMaxEntries
     __shared__ LutWorker s_q;
-    __shared__ bool s_serves;
+    __shared__ uint32_t s_fits[2];                            // bit b of the 64: a window of b + 1 binades serves the row
     const uint32_t wi = blockIdx.y;
     pdl_wait();
     if (threadIdx.x < TQ_MAX_LEVELS) {
         s_q.levels[threadIdx.x] = params[wi].levels[threadIdx.x];
         s_q.inv_width[threadIdx.x] = params[wi].inv_width[threadIdx.x];
     }
+    __syncthreads();
+    const tq_params_t& rec = params[wi];
+    uint32_t top = 0, base = 0;
+    if (!lut_usable(rec, BITS)) return;
+    top = top_pattern(rec.alpha);
+    if (threadIdx.x < 64) {
+        const bool fits = lut_window_fits(rec.alpha, s_q.levels, s_q.inv_width, 1u << BITS, top, kLutBinade * (threadIdx.x + 1), &base);
+        const uint32_t bits = __ballot_sync(0xFFFFFFFFu, fits);
+        if ((threadIdx.x & 31u) == 0) s_fits[threadIdx.x >> 5] = bits;
+    }
+    __syncthreads();
+    if (s_fits[1] >> 31 == 0) return;                         // the rule of lut_serves_record: not even the largest window
+    const uint32_t n_entries = kLutBinade * (s_fits[0] ? __ffs(static_cast<int>(s_fits[0])) : 32 + __ffs(static_cast<int>(s_fits[1])));
     if (threadIdx.x == 0) {
-        uint32_t top = 0, base = 0;
-        s_serves = lut_serves_record(params[wi], BITS, &top, &base);
-        s_q.alpha = params[wi].alpha;
+        base = top >= n_entries ? top - (n_entries - 1) : 0u;
+        s_q.alpha = rec.alpha;
         s_q.base2 = ((0u - base) & 0xFFFFu) * 0x00010001u;
         s_q.negtop2 = (top | 0x8000u) * 0x00010001u;
     }
     __syncthreads();
-    if (!s_serves) return;
-    lut_block<BITS, false>(s_q, kLutMaxEntries, s_table, static_cast<const char*>(grad) + static_cast<uint64_t>(wi) * grad_stride * 2,
+    lut_block<BITS, false>(s_q, n_entries, s_table, static_cast<const char*>(grad) + static_cast<uint64_t>(wi) * grad_stride * 2,
                     packed + static_cast<uint64_t>(wi) * words_stride, d, words_out, first_worker + wi, rk);
 }
 
@@ -264,11 +275,14 @@ compress_lut_kernel_dev(const void* __restrict__ grad, uint64_t d, uint64_t grad
 
 // Entries per sign the worker needs, 0 if no window of at most kLutMaxEntries does.
 static uint32_t entries_needed(const tq_params_t& p, uint32_t top) {
-    for (uint32_t n = kLutMinEntries; n <= static_cast<uint32_t>(kLutMaxEntries); n *= 2) {
-        uint32_t base = 0;
-        if (lut_window_fits(p.alpha, p.levels, p.inv_width, p.num_levels, top, n, &base)) return n;
+    // a window that fits stays valid when it is made larger: halve the range of sizes
+    uint32_t lo = 0, hi = kLutMaxEntries / kLutBinade, base = 0;
+    if (!lut_window_fits(p.alpha, p.levels, p.inv_width, p.num_levels, top, kLutMaxEntries, &base)) return 0;
+    while (hi - lo > 1) {
+        const uint32_t mid = (lo + hi) / 2;
+        if (lut_window_fits(p.alpha, p.levels, p.inv_width, p.num_levels, top, mid * kLutBinade, &base)) hi = mid; else lo = mid;
     }
-    return 0;
+    return hi * kLutBinade;
 }
 
 static uint64_t lut_blocks_per_worker(uint64_t d, uint32_t n_workers, int per_sm, int pieces_elems);
@@ -307,12 +321,14 @@ static cudaError_t launch_lut_dev(const CompressCall& c) {
                          c.d, c.grad_stride, c.params_dev, round_keys(c.seed), c.first_worker, c.packed, c.words_stride, c.words_out);
 }
 
-// Rows below this many elements keep the element-wise kernels (the table costs more than it saves).
-constexpr uint64_t kLutMinElements = 1u << 18;
+// Calls with fewer elements (all rows together) keep the element-wise kernels: each of the 444 resident blocks builds a
+// table of some 20 to 40 binades, a few us each (table / element-wise, device parameters: 10 M 19.5 / 15.4 us, 24 M 29.7 / 27.3,
+// 30 M 33.0 / 32.6, 40 M 35.3 / 44.4, 992 M 638 / 843).
+constexpr uint64_t kLutMinElements = 1u << 25;
 
 cudaError_t launch_compress_lut(const CompressCall& c, bool* applied) {
     *applied = false;
-    if (!c.bf16 || !c.nonuniform || c.segs || c.d < kLutMinElements || c.d > (1ull << 35)) return cudaSuccess;
+    if (!c.bf16 || !c.nonuniform || c.segs || c.d * c.n_workers < kLutMinElements || c.d > (1ull << 35)) return cudaSuccess;
     if (c.params_dev) {      // the kernel decides row by row; the caller launches the element-wise kernels for the rest
         *applied = true;
         switch (c.bits) {

@@ -6,8 +6,8 @@
 
 namespace tq {
 
+constexpr int kLutBinade = 128;          // entries per sign and binade
 constexpr int kLutMaxEntries = 8192;     // per sign: 64 binades
-constexpr int kLutMinEntries = 2048;
 
 // X = k * 2^16 + min(T, 2^16) for a gradient value g: the decision of the quantizer equation up to the
 // random draw.  One IEEE operation per step (the build disables contraction on both sides), so host and
@@ -62,8 +62,11 @@ __host__ __device__ inline bool lut_window_fits(float alpha, const float* levels
 
 // Device-resident parameters: a row goes through the table kernel when its record is usable and the largest window
 // serves it; the element-wise kernels evaluate the same rule and leave exactly those rows alone.
+__host__ __device__ inline bool lut_usable(const tq_params_t& p, uint32_t bits) {
+    return p.alpha > 0.0f && p.alpha <= 3.402823466e38f && p.bits == bits && !(p.flags & TQ_FLAG_INVALID);
+}
 __host__ __device__ inline bool lut_serves_record(const tq_params_t& p, uint32_t bits, uint32_t* top, uint32_t* base) {
-    if (!(p.alpha > 0.0f) || !(p.alpha <= 3.402823466e38f) || p.bits != bits || (p.flags & TQ_FLAG_INVALID)) return false;
+    if (!lut_usable(p, bits)) return false;
     *top = top_pattern(p.alpha);
     return lut_window_fits(p.alpha, p.levels, p.inv_width, 1u << bits, *top, kLutMaxEntries, base);
 }
