@@ -90,36 +90,56 @@ __device__ __forceinline__ float rounds_up(float p, float rf) {
 //                                                negatives to 0, which is where the reference sends them
 //   y   = min(y, s/L)                          this is x = s, which the reference codes as s, like every g >= alpha
 //   Xm  = fma(y, L * 2^16, 2^23)               = 2^23 + X, rounded to nearest-even as rint does (2^23 is even)
-//   v   = Xm - (2^23 + r)                      = X - r, exact
-//   cm  = fma.rp(v, 2^-16, 1.5 * 2^23)         = 1.5 * 2^23 + ceil(v / 2^16): the sum stays inside one binade
-// and the caller subtracts the bias.  sum0 / sum1 are g + alpha of the pair.
+//   v   = bits(Xm) - r + 65535                 = 0x4B000000 + (X - r + 65535): the code is byte 2 of v
+// From Xm on the integer pipe does the work: the kernel is bound by the multiplier pipe, which Philox's wide
+// multiplies keep busy for 9 of its 16 cycles per 32 elements, and floating-point operations load that pipe too
+// (30 M x 8 fp32, 16 levels 167 -> 156 us, 4 levels 158 -> 150).  For bf16 storage the widening shares the integer pipe, and the
+// form below it (2- and 4-bit codes) stays the faster one (124 M x 8, 4 / 16 levels 498 / 511 us against 519 / 518).
+// sum0 / sum1 are g + alpha of the pair.
 struct UniformQ {
     float inv_step_l, c_top;      // inv_step / L, s / L
     f32x2 scale2;                 // L * 2^16, twice
-    f32x2 scale2_dn;              // L * 2^16 * 2^-100, twice (codes as denormals, see code_uniform2_dn)
+    f32x2 scale2_dn;              // L * 2^16 * 2^-100, twice (see code_uniform2_dn)
 };
-constexpr float kCodeBias = 12582912.0f;                 // 1.5 * 2^23
-__device__ __forceinline__ f32x2 fma2_ru(f32x2 a, f32x2 b, f32x2 c) {   // round toward +infinity
-    f32x2 r; asm("fma.rp.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v)); return r;
-}
-__device__ __forceinline__ f32x2 mul2_ru(f32x2 a, f32x2 b) {
-    f32x2 r; asm("mul.rp.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v)); return r;
-}
-// min(y, s/L) runs on the integer/compare pipe, which has room here; the multiply-add pipes do not.
-__device__ __forceinline__ f32x2 code_uniform2(float sum0, float sum1, const UniformQ& u, float rf0, float rf1) {
-    const f32x2 y = pair(fminf(mul_sat(sum0, u.inv_step_l), u.c_top), fminf(mul_sat(sum1, u.inv_step_l), u.c_top));
-    const f32x2 v = sub2(fma2(y, u.scale2, both(kMagic)), pair(rf0, rf1));
-    return fma2_ru(v, both(1.52587890625e-5f), both(kCodeBias));
+// min(y, s/L) runs on the integer/compare pipe as well.
+__device__ __forceinline__ void code_uniform2(float sum0, float sum1, const UniformQ& u, uint32_t rnd, uint32_t& v0, uint32_t& v1) {
+    float x0, x1;
+    unpair(fma2(pair(fminf(mul_sat(sum0, u.inv_step_l), u.c_top), fminf(mul_sat(sum1, u.inv_step_l), u.c_top)), u.scale2, both(kMagic)), x0, x1);
+    v0 = __float_as_uint(x0) - (rnd & 0xFFFFu) + 0xFFFFu;
+    v1 = __float_as_uint(x1) - (rnd >> 16) + 0xFFFFu;
 }
 // The same with everything scaled by 2^-100: Xm = fma(y, L * 2^16 * 2^-100, 2^-77) = 2^-77 + X * 2^-100 (rounded
 // at 2^-100 exactly as the unscaled form rounds at 1), the slot arrives as 2^-77 + r * 2^-100, and
 // (X - r) * 2^-100 * 2^-65 rounded up is ceil((X - r) / 2^16) * 2^-149: a denormal whose bit pattern is the code
-// itself, with no bias to take off (or -0 when X < r: pack8_bits' callers drop the sign bit).
+// itself, with no bias to take off (or -0 when X < r: the callers of pack8 drop the sign bit).
 constexpr uint32_t kSlotExpBits = 0x19000000u;            // 2^-77
+__device__ __forceinline__ f32x2 mul2_ru(f32x2 a, f32x2 b) {
+    f32x2 r; asm("mul.rp.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v)); return r;
+}
 __device__ __forceinline__ f32x2 code_uniform2_dn(float sum0, float sum1, const UniformQ& u, float rf0, float rf1) {
     const f32x2 y = pair(fminf(mul_sat(sum0, u.inv_step_l), u.c_top), fminf(mul_sat(sum1, u.inv_step_l), u.c_top));
     const f32x2 v = sub2(fma2(y, u.scale2_dn, both(6.617444900424222e-24f)), pair(rf0, rf1));
     return mul2_ru(v, both(2.710505431213761e-20f));     // 2^-65
+}
+
+// The codes in byte 2 of eight words -> their 8 * BITS packed bits, LSB first.
+template <int BITS>
+__device__ __forceinline__ uint32_t pack_byte2(const uint32_t (&v)[8]) {
+    auto four = [](uint32_t a, uint32_t b, uint32_t c, uint32_t d) {       // byte 2 of each
+        return __byte_perm(__byte_perm(a, b, 0x0062u), __byte_perm(c, d, 0x0062u), 0x5410u);
+    };
+    if constexpr (BITS <= 2) {
+        // c0 .. c3 side by side in the top byte of a product; the other partial products are disjoint bits below it
+        constexpr uint32_t K = (1u << 24) + (1u << (16 + BITS)) + (1u << (8 + 2 * BITS)) + (1u << (3 * BITS));
+        const uint32_t lo = four(v[0], v[1], v[2], v[3]) * K, hi = four(v[4], v[5], v[6], v[7]) * K;
+        if constexpr (BITS == 2) return __byte_perm(lo, hi, 0x0073u);      // 16 bits; the callers merge chunks by byte permutes
+        else return (lo >> 24) | ((hi >> 24) << 4);
+    } else {
+        const uint32_t t = four(v[0], v[2], v[4], v[6]) + (four(v[1], v[3], v[5], v[7]) << BITS);      // two codes per byte
+        if constexpr (BITS == 4) return t;
+        const uint32_t u = (t & 0x003F003Fu) | ((t >> 2) & 0x0FC00FC0u);                                // four codes per half
+        return (u & 0xFFFu) | ((u >> 4) & 0xFFF000u);
+    }
 }
 
 // The same decision without the scaled inverse step (alpha so large that inv_step / L is subnormal):
@@ -201,7 +221,6 @@ __device__ __forceinline__ float code_binary(float g, float alpha, const float* 
 template <int BITS, bool DN>
 __device__ __forceinline__ uint32_t pack8(const f32x2 (&c)[4]) {
     constexpr float B = static_cast<float>(1 << BITS), B2 = B * B;
-    static_assert(!DN || BITS == 2 || BITS == 4, "the callers of the denormal form keep 16 bits of each partial result");
     if constexpr (BITS <= 3) {
         f32x2 a = fma2(c[3], both(B2), c[2]);
         a = fma2(a, both(B2), c[1]);
@@ -253,33 +272,42 @@ __device__ __forceinline__ void quantize_run(const Raw8<BF16> (&g)[4], uint32_t*
     const uint32_t blk_lo = static_cast<uint32_t>(j0 >> 3);
     const PhiloxRun pr = philox_run(static_cast<uint32_t>(j0 >> 35), worker, rk);
     const f32x2 alpha2 = both(cx.alpha), inv_step2 = both(cx.inv_step), cell_scale2 = both(cx.cell_scale);
-    // the scaled uniform path hands pack8 the codes as denormals (2- and 4-bit codes)
-    constexpr bool DN = SEARCH == kUniform && (BITS == 2 || BITS == 4);
+    constexpr bool DN = SEARCH == kUniform && BF16 && (BITS == 2 || BITS == 4);
     uint32_t chunk[4];   // the 8*BITS packed bits of each group
 #pragma unroll
     for (int grp = 0; grp < 4; ++grp) {
         uint32_t rnd[4];
         philox_block(blk_lo + grp, pr, rk, rnd);                      // j0 >> 3 is a multiple of 4: no carry
-        f32x2 code[4];
+        if constexpr (SEARCH == kUniform && !DN) {
+            uint32_t v[8];
 #pragma unroll
-        for (int h = 0; h < 4; ++h) {            // elements 2h, 2h+1 of the group
-            const int e = 2 * h;
-            const float rf0 = slot_as_float<DN>(rnd, e), rf1 = slot_as_float<DN>(rnd, e + 1);
-            if constexpr (is_uniform(SEARCH)) {
+            for (int h = 0; h < 4; ++h) {        // elements 2h, 2h+1 of the group
                 float sum0, sum1;
                 pair_plus_alpha<BF16>(g[grp], h, cx.alpha, sum0, sum1);
-                if constexpr (DN) code[h] = code_uniform2_dn(sum0, sum1, cx.u, rf0, rf1);
-                else if constexpr (SEARCH == kUniform) code[h] = sub2(code_uniform2(sum0, sum1, cx.u, rf0, rf1), both(kCodeBias));
-                else code[h] = code_uniform2_wide(sum0, sum1, inv_step2, cx.top, rf0, rf1);
-            } else {
-                const float g0 = elem<BF16>(g[grp], e), g1 = elem<BF16>(g[grp], e + 1);
-                if constexpr (SEARCH == kGrid)
-                    code[h] = code_grid2(g0, g1, alpha2, cx.inv_2alpha, cell_scale2, cx.s_grid, cx.s_cell, rf0, rf1);
-                else code[h] = pair(code_binary<BITS>(g0, cx.alpha, cx.s_search, reinterpret_cast<const float2*>(cx.s_cell), rf0),
-                                    code_binary<BITS>(g1, cx.alpha, cx.s_search, reinterpret_cast<const float2*>(cx.s_cell), rf1));
+                code_uniform2(sum0, sum1, cx.u, rnd[h], v[2 * h], v[2 * h + 1]);
             }
+            chunk[grp] = pack_byte2<BITS>(v);
+        } else {
+            f32x2 code[4];
+#pragma unroll
+            for (int h = 0; h < 4; ++h) {
+                const int e = 2 * h;
+                const float rf0 = slot_as_float<DN>(rnd, e), rf1 = slot_as_float<DN>(rnd, e + 1);
+                if constexpr (is_uniform(SEARCH)) {
+                    float sum0, sum1;
+                    pair_plus_alpha<BF16>(g[grp], h, cx.alpha, sum0, sum1);
+                    if constexpr (DN) code[h] = code_uniform2_dn(sum0, sum1, cx.u, rf0, rf1);
+                    else code[h] = code_uniform2_wide(sum0, sum1, inv_step2, cx.top, rf0, rf1);
+                } else {
+                    const float g0 = elem<BF16>(g[grp], e), g1 = elem<BF16>(g[grp], e + 1);
+                    if constexpr (SEARCH == kGrid)
+                        code[h] = code_grid2(g0, g1, alpha2, cx.inv_2alpha, cell_scale2, cx.s_grid, cx.s_cell, rf0, rf1);
+                    else code[h] = pair(code_binary<BITS>(g0, cx.alpha, cx.s_search, reinterpret_cast<const float2*>(cx.s_cell), rf0),
+                                        code_binary<BITS>(g1, cx.alpha, cx.s_search, reinterpret_cast<const float2*>(cx.s_cell), rf1));
+                }
+            }
+            chunk[grp] = pack8<BITS, DN>(code);
         }
-        chunk[grp] = pack8<BITS, DN>(code);
     }
 
     // four chunks of 8*BITS bits -> BITS words, LSB first
@@ -577,8 +605,13 @@ __device__ __forceinline__ void compress_piece(State& sh, const void* __restrict
     const uint32_t worker = first_worker + sh.piece.worker;
     const uint64_t whole = (sh.piece.d - 1) >> 5, stop = sh.piece.tile1 * kThreads;       // runs before the row's last one are whole
     const uint64_t end = stop < whole ? stop : whole;
-    for (uint64_t run = sh.piece.tile0 * kThreads + threadIdx.x; run < end; run += kThreads)
-        compress_run<BITS, SEARCH, BF16>(row, prow, run, worker, rk, cx);
+    // from the piece's end to its beginning: what the statistics pass before this one read last is still in L2
+    const uint64_t begin = sh.piece.tile0 * kThreads + threadIdx.x;
+    if (begin < end)
+        for (uint64_t run = begin + (end - 1 - begin) / kThreads * kThreads;; run -= kThreads) {
+            compress_run<BITS, SEARCH, BF16>(row, prow, run, worker, rk, cx);
+            if (run == begin) break;
+        }
     if (sh.piece.last && threadIdx.x < 32) compress_last_run<BITS, is_uniform(SEARCH), BF16>(row, prow, sh.piece.d, worker, rk, sh.q);
 }
 
@@ -655,6 +688,15 @@ static uint32_t choose_cells(const tq_params_t& p, float inv_2alpha) {
     return 0;
 }
 
+// Shares per resident block when each would get `tiles` tiles as one share: the hardware hands the later ones to the blocks
+// that finish first, which evens out SMs and the blocks of an SM, as long as a share repays its set-up.  Device parameters, 1 / 2 /
+// 4 / 8 shares: 25.6 M x 16 (84 tiles) 339 / 327 / 324 / 328 us, 11.2 M x 8 (18 tiles) 70 / 69 / 65 / 68, 1 M x 64 (13) 50 / 48 / 51 / 55,
+// 4 M x 4 (3) 19.8 / 19.7 / 21.4 / 21.4, 124 M x 8 bf16 uniform 541 / 519 / 511 / 513.
+static uint64_t ranges_per_block(uint64_t tiles) {
+    const uint64_t n = tiles / 5;
+    return n < 1 ? 1 : n > 6 ? 6 : n;
+}
+
 // Persistent grid: 4 resident blocks per SM spread over the workers (table modes build their lookup
 // grid once per block); uniform mode has no per-block set-up, so one block per tile lets the hardware
 // scheduler balance the tail.
@@ -662,6 +704,7 @@ static dim3 compress_grid(uint64_t d, uint32_t n_workers, bool persistent) {
     const uint64_t n_runs = (d + 31) >> 5;
     const uint64_t tiles = (n_runs + kThreads - 1) / kThreads;
     uint64_t per_worker = static_cast<uint64_t>(sm_count()) * TQ_COMPRESS_MIN_BLOCKS / n_workers;   // rounded down: one wave holds the grid
+    if (persistent && per_worker > 0) per_worker *= ranges_per_block(tiles / per_worker);
     if (!persistent || per_worker > tiles) per_worker = tiles;
     if (per_worker > 0x7FFFFFFFull) per_worker = 0x7FFFFFFFull;
     if (per_worker < 1) per_worker = 1;
@@ -763,7 +806,9 @@ cudaError_t launch_compress(const CompressCall& c) {
             if (q.cells == 0 || !std::isfinite(q.inv_2alpha)) search = kBinary;
         }
     }
-    const dim3 grid = compress_grid(c.d, c.n_workers, !is_uniform(search));
+    // uniform fp32 rows have no per-block set-up worth sharing: one block per tile (30 M x 8, 16 levels: 156 us, in shares 166);
+    // bf16 ones, bound by instructions, do better in shares (124 M x 8, 4 levels: 543 us by tiles, 506 in shares)
+    const dim3 grid = compress_grid(c.d, c.n_workers, !is_uniform(search) || c.bf16);
     switch (c.bits) {
         case 1: return dispatch<1>(c, args, grid, search);
         case 2: return dispatch<2>(c, args, grid, search);
@@ -786,7 +831,9 @@ cudaError_t launch_compress_dev(const CompressCall& c) {
     bool lut = false;
     if (const cudaError_t e = launch_compress_lut(c, &lut)) return e;
     static thread_local TilePlan plan;
-    plan_tiles(&plan, c.segs, c.d, c.n_workers, 32 * kThreads, static_cast<uint64_t>(sm_count()) * (lut ? 1 : TQ_COMPRESS_MIN_BLOCKS));
+    const uint64_t resident = static_cast<uint64_t>(sm_count()) * TQ_COMPRESS_MIN_BLOCKS;
+    plan_tiles(&plan, c.segs, c.d, c.n_workers, 32 * kThreads, lut ? resident / TQ_COMPRESS_MIN_BLOCKS : resident);
+    if (const uint64_t more = lut ? 1 : ranges_per_block(plan.per_block); more > 1) plan_tiles(&plan, c.segs, c.d, c.n_workers, 32 * kThreads, resident * more);
     if (c.launches) *c.launches = lut ? 2 : 1;
     switch (c.bits) {
         case 1: return dispatch_dev<1>(c, plan, lut);

@@ -721,6 +721,9 @@ static void plan_stats(const StatsCall& c, uint32_t n_jobs, TilePlan* plan) {
     const uint64_t room = static_cast<uint64_t>(n_jobs) * kRecordsPerJob - n_jobs;
     if (resident > room) resident = room;
     plan_tiles(plan, c.segs, c.d, c.n_workers, kThreads * kChunkBytes / (c.bf16 ? 2 : 4), resident);
+    // bf16 rows are bound by instructions: three ranges per resident block even out the SMs (124 M x 8, hinted: 430 -> 407 us;
+    // fp32 rows 249 -> 254 us, short ranges lose more)
+    if (c.bf16 && plan->per_block >= 64 && 3 * resident <= room) plan_tiles(plan, c.segs, c.d, c.n_workers, kThreads * kChunkBytes / 2, 3 * resident);
 }
 
 // True when the call went to the cluster kernel.
