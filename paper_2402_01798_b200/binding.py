@@ -20,6 +20,7 @@ OK, ERR_INVALID_ARG, ERR_DOMAIN, ERR_ALIGNMENT, ERR_BUFFER_TOO_SMALL, ERR_DEGENE
     0, -1, -2, -3, -4, -5, -6
 ERR_STATIC_LIMIT = -7
 STATIC_MAX_WORKERS = 16
+_BITS = {2: 1, 4: 2, 8: 3, 16: 4}          # of a codebook with that many levels
 F32, BF16 = 0, 1
 UNIFORM, NONUNIFORM, BISCALED = 0, 1, 2
 ALPHA_CLOSED, ALPHA_FIXED_POINT, ALPHA_USER, ALPHA_MAXABS = 0, 1, 2, 3
@@ -125,12 +126,13 @@ def _check(status: int, where: str) -> None:
 
 
 # torch.cuda.current_stream().cuda_stream without the Stream object (3.3 us of every call's 8)
+_current_device = getattr(torch._C, "_cuda_getDevice", None) or torch.cuda.current_device
 _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or (lambda device: torch.cuda.current_stream(device).cuda_stream)
 
 
 def _stream(stream) -> int:
     if stream is None:
-        return _raw_stream(torch.cuda.current_device())
+        return _raw_stream(_current_device())
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
@@ -146,12 +148,17 @@ def _grad_layout(grad: torch.Tensor, d: Optional[int]):
     """(n_workers, d, stride) of a [N, stride] or [d] gradient tensor on the GPU."""
     if not grad.is_cuda:
         raise ValueError("gradient must be a CUDA tensor")
-    if grad.dim() == 1:
-        grad = grad.unsqueeze(0)
-    if grad.dim() != 2 or grad.stride(1) != 1:
+    dims = grad.dim()
+    if dims == 1:
+        grad, dims = grad.unsqueeze(0), 2
+    if dims != 2 or grad.stride(1) != 1:
         raise ValueError("gradient must be [N, stride] with unit inner stride")
-    n, width = grad.shape
+    n, width = grad.size(0), grad.size(1)
     return n, (width if d is None else d), (grad.stride(0) if n > 1 else width)
+
+
+def _words_stride(packed: torch.Tensor, n: int) -> int:
+    return packed.stride(0) if n > 1 and packed.dim() == 2 else packed.size(-1)
 
 
 def params_array(params: Sequence[Params]):
@@ -247,13 +254,13 @@ def tq_params_batch(stats_raw, n_workers: int, num_levels: int, mode: int, gamma
     Stats, or a pinned CPU uint8 tensor (used in place).  Returns a ctypes tq_params_t[n] array."""
     out = (Params * n_workers)()
     if isinstance(stats_raw, torch.Tensor):
-        src = C.c_void_p(stats_raw.data_ptr())
+        src = stats_raw.data_ptr()
     elif isinstance(stats_raw, (bytes, bytearray)):
         src = C.cast(C.create_string_buffer(bytes(stats_raw), len(stats_raw)), C.c_void_p)
     else:
         src = C.cast(stats_raw, C.c_void_p)
     _check(lib().tq_params_batch(src, n_workers, num_levels, mode, gamma, alpha_rule, alpha_user,
-                                 C.cast(out, C.c_void_p)), "tq_params_batch")
+                                 out), "tq_params_batch")
     return out
 
 
@@ -272,9 +279,8 @@ def tq_compress(grad: torch.Tensor, params: Sequence[Params], seed: int, first_w
         raise ValueError("one Params per worker")
     if packed is None:
         packed = torch.empty((n, tq_packed_words(d, params[0].bits)), dtype=torch.int32, device=grad.device)
-    words_stride = packed.stride(0) if packed.dim() == 2 and n > 1 else packed.shape[-1]
     _check(lib().tq_compress(grad.data_ptr(), _dtype_code(grad), d, stride, n, _params_array(params),
-                             seed & 0xFFFFFFFFFFFFFFFF, first_worker, packed.data_ptr(), words_stride,
+                             seed & 0xFFFFFFFFFFFFFFFF, first_worker, packed.data_ptr(), _words_stride(packed, n),
                              _stream(stream)), "tq_compress")
     return packed
 
@@ -285,14 +291,13 @@ def tq_decompress_aggregate(packed: torch.Tensor, d: int, params: Sequence[Param
     """Enqueue unpack + dequantize + average of the N packed rows; returns the [d] fp32 update."""
     if not packed.is_cuda or packed.dim() != 2:
         raise ValueError("packed must be a [N, words] CUDA tensor")
-    n = packed.shape[0]
+    n = packed.size(0)
     if len(params) != n:
         raise ValueError("one Params per worker")
     if out is None:
         out = torch.empty(d, dtype=torch.float32, device=packed.device)
     w = None if weights is None else (C.c_float * n)(*[float(x) for x in weights])
-    words_stride = packed.stride(0) if n > 1 else packed.shape[1]
-    _check(lib().tq_decompress_aggregate(packed.data_ptr(), words_stride, n, d, _params_array(params), w,
+    _check(lib().tq_decompress_aggregate(packed.data_ptr(), _words_stride(packed, n), n, d, _params_array(params), w,
                                          out.data_ptr(), _stream(stream)), "tq_decompress_aggregate")
     return out
 
@@ -338,25 +343,22 @@ def tq_compress_device_params(grad: torch.Tensor, params_dev: torch.Tensor, num_
                               first_worker: int = 0, d: Optional[int] = None, packed: Optional[torch.Tensor] = None,
                               stream=None) -> torch.Tensor:
     n, d, stride = _grad_layout(grad, d)
-    bits = {2: 1, 4: 2, 8: 3, 16: 4}[num_levels]
     if packed is None:
-        packed = torch.empty((n, tq_packed_words(d, bits)), dtype=torch.int32, device=grad.device)
-    words_stride = packed.stride(0) if packed.dim() == 2 and n > 1 else packed.shape[-1]
+        packed = torch.empty((n, tq_packed_words(d, _BITS[num_levels])), dtype=torch.int32, device=grad.device)
     _check(lib().tq_compress_device_params(grad.data_ptr(), _dtype_code(grad), d, stride, n, params_dev.data_ptr(),
                                            num_levels, mode, seed & 0xFFFFFFFFFFFFFFFF, first_worker, packed.data_ptr(),
-                                           words_stride, _stream(stream)), "tq_compress_device_params")
+                                           _words_stride(packed, n), _stream(stream)), "tq_compress_device_params")
     return packed
 
 
 def tq_decompress_aggregate_device_params(packed: torch.Tensor, d: int, params_dev: torch.Tensor, num_levels: int,
                                           weights: Optional[Sequence[float]] = None,
                                           out: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
-    n = packed.shape[0]
+    n = packed.size(0)
     if out is None:
         out = torch.empty(d, dtype=torch.float32, device=packed.device)
     w = None if weights is None else (C.c_float * n)(*[float(x) for x in weights])
-    words_stride = packed.stride(0) if n > 1 else packed.shape[1]
-    _check(lib().tq_decompress_aggregate_device_params(packed.data_ptr(), words_stride, n, d, params_dev.data_ptr(),
+    _check(lib().tq_decompress_aggregate_device_params(packed.data_ptr(), _words_stride(packed, n), n, d, params_dev.data_ptr(),
                                                        num_levels, w, out.data_ptr(), _stream(stream)),
            "tq_decompress_aggregate_device_params")
     return out
@@ -410,24 +412,21 @@ def tq_compress_segments(grad: torch.Tensor, segments, params_dev: torch.Tensor,
                          first_worker: int = 0, packed: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     n, _, stride = _grad_layout(grad, None)
     seg = segments if isinstance(segments, C.Array) else segments_array(segments)
-    bits = {2: 1, 4: 2, 8: 3, 16: 4}[num_levels]
     if packed is None:
-        packed = torch.empty((n, tq_segments_packed_words(seg, bits)), dtype=torch.int32, device=grad.device)
-    words_stride = packed.stride(0) if packed.dim() == 2 and n > 1 else packed.shape[-1]
+        packed = torch.empty((n, tq_segments_packed_words(seg, _BITS[num_levels])), dtype=torch.int32, device=grad.device)
     _check(lib().tq_compress_segments(grad.data_ptr(), _dtype_code(grad), stride, n, seg, len(seg), params_dev.data_ptr(),
                                       num_levels, mode, seed & 0xFFFFFFFFFFFFFFFF, first_worker, packed.data_ptr(),
-                                      words_stride, _stream(stream)), "tq_compress_segments")
+                                      _words_stride(packed, n), _stream(stream)), "tq_compress_segments")
     return packed
 
 
 def tq_decompress_aggregate_segments(packed: torch.Tensor, segments, params_dev: torch.Tensor, num_levels: int,
                                      out: torch.Tensor, weights: Optional[Sequence[float]] = None, stream=None) -> torch.Tensor:
     """Aggregates every segment into out[offset : offset + length]; elements of `out` outside the segments are left alone."""
-    n = packed.shape[0]
+    n = packed.size(0)
     seg = segments if isinstance(segments, C.Array) else segments_array(segments)
     w = None if weights is None else (C.c_float * n)(*[float(x) for x in weights])
-    words_stride = packed.stride(0) if n > 1 else packed.shape[1]
-    _check(lib().tq_decompress_aggregate_segments(packed.data_ptr(), words_stride, n, seg, len(seg), params_dev.data_ptr(),
+    _check(lib().tq_decompress_aggregate_segments(packed.data_ptr(), _words_stride(packed, n), n, seg, len(seg), params_dev.data_ptr(),
                                                   num_levels, w, out.data_ptr(), _stream(stream)),
            "tq_decompress_aggregate_segments")
     return out
@@ -437,10 +436,9 @@ def tq_decompress_aggregate_apply(packed: torch.Tensor, d: int, params, theta: t
                                   momentum_buf: Optional[torch.Tensor], lr: float, momentum: float = 0.0,
                                   weight_decay: float = 0.0, weights: Optional[Sequence[float]] = None, stream=None):
     """Aggregate the N packed rows and apply the SGD step in place on ``theta`` (and ``momentum_buf``)."""
-    n = packed.shape[0]
+    n = packed.size(0)
     w = None if weights is None else (C.c_float * n)(*[float(x) for x in weights])
-    words_stride = packed.stride(0) if n > 1 else packed.shape[1]
-    _check(lib().tq_decompress_aggregate_apply(packed.data_ptr(), words_stride, n, d, _params_array(params), w,
+    _check(lib().tq_decompress_aggregate_apply(packed.data_ptr(), _words_stride(packed, n), n, d, _params_array(params), w,
                                                theta.data_ptr(), None if momentum_buf is None else momentum_buf.data_ptr(),
                                                lr, momentum, weight_decay, _stream(stream)), "tq_decompress_aggregate_apply")
     return theta

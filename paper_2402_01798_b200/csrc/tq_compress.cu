@@ -19,8 +19,6 @@
 //     code = ceil((X - r) / 2^16), with the clamps of x done by saturating multiplies and subtracts;
 //   - codes are kept as small floats and packed by exact multiply-adds (sums stay below 2^24);
 //   - table offsets are formed as denormal floats whose bit pattern IS the byte offset.
-#include <cuda.h>
-
 #include <cmath>
 
 #include "tq_device.cuh"
@@ -42,8 +40,11 @@ struct WorkerQ {
     float levels[TQ_MAX_LEVELS];
     float inv_width[TQ_MAX_LEVELS];
 };
+// By-value arguments are copied at every launch: calls of few workers do not pass room for all.
+constexpr uint32_t kFewWorkers = 16;
+template <uint32_t N>
 struct CompressArgs {
-    WorkerQ q[TQ_MAX_WORKERS];
+    WorkerQ q[N];
 };
 
 // kUniformWide: the uniform codebook through the arithmetic that needs no scaled inverse step (used
@@ -415,10 +416,10 @@ __device__ __forceinline__ void build_tables(const WorkerQ& q, float2* s_grid, f
 }
 
 // Quantizers passed by value in the kernel's parameter space (host-side tq_params).
-template <int BITS, int SEARCH, bool BF16>
+template <int BITS, int SEARCH, bool BF16, uint32_t N>
 __global__ void __launch_bounds__(kThreads, TQ_COMPRESS_MIN_BLOCKS)
 compress_kernel(const void* __restrict__ grad, uint64_t d, uint64_t grad_stride,
-                const __grid_constant__ CompressArgs args, const __grid_constant__ RoundKeys rk,
+                const __grid_constant__ CompressArgs<N> args, const __grid_constant__ RoundKeys rk,
                 uint32_t first_worker, uint32_t* __restrict__ packed, uint64_t words_stride) {
     __shared__ __align__(16) float2 s_grid[SEARCH == kGrid ? kMaxGridCells + 1 : 1];
     __shared__ __align__(16) float2 s_cell[TQ_MAX_LEVELS];
@@ -438,107 +439,14 @@ compress_kernel(const void* __restrict__ grad, uint64_t d, uint64_t grad_stride,
     if (blockIdx.x == gridDim.x - 1 && threadIdx.x < 32) compress_last_run<BITS, is_uniform(SEARCH), BF16>(row, prow, d, worker, rk, q);
 }
 
-// ---------------------------------------------------------------------------------------------
-// Table-mode compress with the gradient tiles brought in by the tensor-memory accelerator.
-// A tile is 256 runs of 32 elements (one run per thread).  Thread 0 asks for the block's next tile as
-// ONE tiled copy ({32 elements, 256 runs, 1 worker} of the [N][runs][32] view of the gradient) while
-// the block is still quantizing the current one, so no warp waits on global loads and no registers are
-// held by loads in flight.  The copy lands swizzled (16-byte chunk c of run r at chunk c ^ (r & 7) for
-// 128-byte runs, c ^ ((r >> 1) & 3) for 64-byte runs), which makes a thread's reads of its own run
-// conflict-free.  Runs past the last whole run read as zeros and are not used; the row's last run
-// (possibly partial) goes through the guarded path.  Waits are bounded as in the header.
-__device__ unsigned int g_compress_wait_expired = 0;
-
-__device__ __forceinline__ void lds128(uint32_t addr, uint32_t& a, uint32_t& b, uint32_t& c, uint32_t& d) {
-    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(a), "=r"(b), "=r"(c), "=r"(d) : "r"(addr));
-}
-
-__device__ __forceinline__ void tma_load_tile(uint32_t dst, const CUtensorMap* map, int32_t x, int32_t y, int32_t z, uint32_t bar) {
-    asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
-                 ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(bar) : "memory");
-}
-
-template <int BITS, bool BF16>
-__global__ void __launch_bounds__(kThreads, TQ_COMPRESS_MIN_BLOCKS)
-compress_tma_kernel(const __grid_constant__ CUtensorMap tmap, const void* __restrict__ grad, uint64_t d, uint64_t grad_stride,
-                    const __grid_constant__ CompressArgs args, const __grid_constant__ RoundKeys rk,
-                    uint32_t first_worker, uint32_t* __restrict__ packed, uint64_t words_stride) {
-    constexpr uint32_t kRowBytes = 32 * (BF16 ? 2 : 4), kTileBytes = kThreads * kRowBytes;
-    __shared__ __align__(16) float2 s_grid[kMaxGridCells + 1];
-    __shared__ __align__(16) float2 s_cell[TQ_MAX_LEVELS];
-    extern __shared__ __align__(1024) unsigned char s_tile[];        // kTileBytes, then the barrier
-    const uint32_t wi = blockIdx.y;
-    const WorkerQ& q = args.q[wi];
-    const uint32_t tile0 = smem_addr(s_tile), bar = tile0 + kTileBytes;
-
-    const uint64_t n_runs = (d + 31) >> 5;
-    const uint64_t interior = n_runs - 1;                             // every run before the row's last one is whole
-    const uint32_t n_tiles = static_cast<uint32_t>((interior + kThreads - 1) / kThreads);
-    uint32_t tile = blockIdx.x;
-    auto issue = [&](uint32_t t) {
-        mbar_expect_tx(bar, kTileBytes);
-        tma_load_tile(tile0, &tmap, 0, static_cast<int32_t>(t * kThreads), static_cast<int32_t>(wi), bar);
-    };
-    if (threadIdx.x == 0) {
-        mbar_init(bar, 1);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    build_tables<BITS, kGrid>(q, s_grid, s_cell, nullptr);            // from kernel parameters; ends with a block barrier
-    pdl_wait();
-    if (threadIdx.x == 0 && tile < n_tiles) issue(tile);
-
-    constexpr size_t esz = BF16 ? 2 : 4;
-    const char* row = static_cast<const char*>(grad) + static_cast<uint64_t>(wi) * grad_stride * esz;
-    uint32_t* prow = packed + static_cast<uint64_t>(wi) * words_stride;
-    const RunCtx cx{q.alpha, q.inv_step, q.top, q.inv_2alpha, q.cell_scale, uniform_q<BITS>(q), reinterpret_cast<const char*>(s_grid),
-                    reinterpret_cast<const char*>(s_cell), nullptr};
-    // this thread's run starts at tile0 + tid * kRowBytes; its 16-byte chunk c sits at chunk c ^ sw: the chunk
-    // bits of the run's own address are zero, so the address of chunk c is (run | sw << 4) ^ (c << 4)
-    const uint32_t sw = BF16 ? ((threadIdx.x >> 1) & 3u) : (threadIdx.x & 7u);
-    const uint32_t mine0 = (tile0 + threadIdx.x * kRowBytes) | (sw << 4);
-
-    uint32_t parity = 0;
-    bool expired = false;
-    for (; tile < n_tiles; tile += gridDim.x) {
-        const bool ok = mbar_wait(bar, parity);
-        parity ^= 1u;
-        const uint64_t run = static_cast<uint64_t>(tile) * kThreads + threadIdx.x;
-        Raw8<BF16> g[4];         // read even if the wait ran out: the values are then never used
-#pragma unroll
-        for (int grp = 0; grp < 4; ++grp) {
-            if constexpr (BF16) {
-                lds128(mine0 ^ (static_cast<uint32_t>(grp) << 4), g[grp].v[0], g[grp].v[1], g[grp].v[2], g[grp].v[3]);
-            } else {
-                lds128(mine0 ^ (static_cast<uint32_t>(2 * grp) << 4), g[grp].v[0], g[grp].v[1], g[grp].v[2], g[grp].v[3]);
-                lds128(mine0 ^ (static_cast<uint32_t>(2 * grp + 1) << 4), g[grp].v[4], g[grp].v[5], g[grp].v[6], g[grp].v[7]);
-            }
-        }
-        // every thread has its run in registers: the tile buffer may be refilled.  The same barrier
-        // makes the give-up decision uniform.
-        if (__syncthreads_or(!ok)) { expired = true; break; }
-        if (threadIdx.x == 0 && tile + gridDim.x < n_tiles) issue(tile + gridDim.x);
-        if (run < interior) quantize_run<BITS, kGrid, BF16>(g, prow, run, first_worker + wi, rk, cx);
-    }
-    if (expired) {
-        atomicAdd(&g_compress_wait_expired, 1u);
-        if (threadIdx.x == 0) mbar_wait(bar, parity ^ 1u);            // the copy that did not land in time
-        return;
-    }
-    if (blockIdx.x == gridDim.x - 1 && threadIdx.x < 32) compress_last_run<BITS, false, BF16>(row, prow, d, first_worker + wi, rk, q);
-}
-
-cudaError_t read_compress_wait_expired(unsigned int* count) {
-    return cudaMemcpyFromSymbol(count, g_compress_wait_expired, sizeof(unsigned int));
-}
-
 // The grid cell of a value as a plain integer (device copy of the host's cell_of).
 __device__ __forceinline__ uint32_t cell_index(float g, float alpha, float inv_2alpha, uint32_t cells) {
     return __float_as_uint(grid_cell(g, alpha, inv_2alpha, __uint_as_float(cells)));   // M * 2^-149 has bit pattern M
 }
 
 // Quantizers read from device memory (tq_params_device): no host round trip before the launch.
-// The block turns a job's tq_params_t into the kernel's WorkerQ, including the choice of the lookup grid (the lanes of
-// the first warp try one resolution each).  Ends with a block barrier.
+// The block turns a job's tq_params_t into the kernel's WorkerQ, including the choice of the lookup grid.  Ends with a
+// block barrier.
 template <int BITS, bool NONUNIFORM>
 __device__ __forceinline__ void load_worker(const tq_params_t& p, WorkerQ& s_q) {
     if (threadIdx.x < 32) {
@@ -552,19 +460,15 @@ __device__ __forceinline__ void load_worker(const tq_params_t& p, WorkerQ& s_q) 
         const bool ok = alpha > 0.0f && p.bits == BITS && !(p.flags & TQ_FLAG_INVALID);
         const float inv_2alpha = ok ? __fdiv_rn(1.0f, __fmul_rn(2.0f, alpha)) : 0.0f;
         uint32_t cells = 0;
-        if constexpr (NONUNIFORM) {
+        if constexpr (NONUNIFORM) {      // choose_cells, a lane for each interior level
             constexpr int s = (1 << BITS) - 1;
-            const uint32_t m = static_cast<uint32_t>(kMinGridCells) << lane;     // only lanes with m <= kMaxGridCells count
-            bool distinct = ok && inv_2alpha <= 3.402823466e38f && lane < 16 && m <= static_cast<uint32_t>(kMaxGridCells);
-            uint32_t prev = s >= 2 ? cell_index(s_q.levels[1], alpha, inv_2alpha, m) : 0u;
-#pragma unroll
-            for (int j = 2; j <= s - 1; ++j) {
-                const uint32_t cur = cell_index(s_q.levels[j], alpha, inv_2alpha, m);
-                distinct = distinct && cur > prev;
-                prev = cur;
-            }
-            const uint32_t fits = __ballot_sync(0xFFFFFFFFu, distinct);
-            if (fits) cells = static_cast<uint32_t>(kMinGridCells) << (__ffs(static_cast<int>(fits)) - 1);
+            const bool mine = lane >= 2 && lane <= s - 1;
+            const uint32_t cell = lane < TQ_MAX_LEVELS ? cell_index(s_q.levels[lane], alpha, inv_2alpha, kMaxGridCells) : 0u;
+            const uint32_t prev = __shfl_up_sync(0xFFFFFFFFu, cell, 1);
+            const uint32_t drop = __reduce_min_sync(0xFFFFFFFFu, mine && cell > prev ? 31u - __clz(static_cast<int>(cell ^ prev)) : 31u);
+            const bool distinct = !__any_sync(0xFFFFFFFFu, mine && cell <= prev) && ok && inv_2alpha <= 3.402823466e38f;
+            const uint32_t m = drop >= 31 ? 0u : static_cast<uint32_t>(kMaxGridCells) >> drop;
+            if (distinct) cells = m < static_cast<uint32_t>(kMinGridCells) ? kMinGridCells : m;
         }
         if (lane == 0) {
             s_q.alpha = ok ? alpha : 0.0f;
@@ -668,24 +572,26 @@ compress_kernel_dev(const void* __restrict__ grad, uint64_t grad_stride, const t
 
 // ---- host side ---------------------------------------------------------------------------------------
 
-// The grid cell of a value, exactly as grid_cell() computes it on the device: every step is a single
-// IEEE operation (u * M is exact for M a power of two), so host and device agree bit for bit.
-static uint32_t cell_of(float g, float alpha, float inv_2alpha, uint32_t cells) {
-    float u = (g + alpha) * inv_2alpha;
-    u = !(u > 0.0f) ? 0.0f : (u > 1.0f ? 1.0f : u);
-    return static_cast<uint32_t>(std::floor(u * static_cast<float>(cells)));
-}
-
-// Smallest power-of-two grid (32 .. 2048 cells) that puts the interior levels in distinct cells; 0 if none.
+// Smallest power-of-two grid (32 .. 2048 cells) that puts the interior levels in distinct cells; 0 if none.  The cell of a
+// level is exactly what grid_cell() computes on the device: every step is a single IEEE operation (u * M is exact for M a
+// power of two), and the cell in a grid 2^k times coarser is the cell in the finest one without its last k bits.
 static uint32_t choose_cells(const tq_params_t& p, float inv_2alpha) {
     const int s = static_cast<int>(p.num_levels) - 1;
-    for (uint32_t m = kMinGridCells; m <= static_cast<uint32_t>(kMaxGridCells); m *= 2) {
-        bool distinct = true;
-        for (int j = 2; j <= s - 1 && distinct; ++j)
-            distinct = cell_of(p.levels[j], p.alpha, inv_2alpha, m) > cell_of(p.levels[j - 1], p.alpha, inv_2alpha, m);
-        if (distinct) return m;
+    uint32_t prev = 0;
+    int drop = 31;                       // bits that may go: up to the highest one in which neighbours differ
+    for (int j = 1; j <= s - 1; ++j) {
+        float u = (p.levels[j] + p.alpha) * inv_2alpha;
+        u = !(u > 0.0f) ? 0.0f : (u > 1.0f ? 1.0f : u);
+        const uint32_t cell = static_cast<uint32_t>(u * static_cast<float>(kMaxGridCells));
+        if (j > 1) {
+            if (cell <= prev) return 0;
+            const int top = 31 - __builtin_clz(cell ^ prev);
+            drop = top < drop ? top : drop;
+        }
+        prev = cell;
     }
-    return 0;
+    const uint32_t m = drop >= 31 ? 0u : static_cast<uint32_t>(kMaxGridCells) >> drop;
+    return m < static_cast<uint32_t>(kMinGridCells) ? kMinGridCells : m;
 }
 
 // Shares per resident block when each would get `tiles` tiles as one share: the hardware hands the later ones to the blocks
@@ -711,73 +617,23 @@ static dim3 compress_grid(uint64_t d, uint32_t n_workers, bool persistent) {
     return dim3(static_cast<unsigned>(per_worker), n_workers);
 }
 
-template <int BITS, int SEARCH, bool BF>
-static cudaError_t launch(const CompressCall& c, const CompressArgs& args, dim3 grid) {
-    return launch_kernel(compress_kernel<BITS, SEARCH, BF>, grid, kThreads, 0, c.stream, c.grad, c.d, c.grad_stride, args, round_keys(c.seed),
+template <int BITS, int SEARCH, bool BF, uint32_t N>
+static cudaError_t launch(const CompressCall& c, const CompressArgs<N>& args, dim3 grid) {
+    return launch_kernel(compress_kernel<BITS, SEARCH, BF, N>, grid, kThreads, 0, c.stream, c.grad, c.d, c.grad_stride, args, round_keys(c.seed),
                          c.first_worker, c.packed, c.words_stride);
 }
 
-// ---- tiled copies: the tensor map of the gradient, [N][whole runs][32 elements] ------------------------
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
-                                  const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-static EncodeTiledFn encode_tiled_fn() {
-    static const EncodeTiledFn fn = [] {
-        void* p = nullptr;
-        cudaDriverEntryPointQueryResult how;
-        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &how) != cudaSuccess ||
-            how != cudaDriverEntryPointSuccess)
-            p = nullptr;
-        return reinterpret_cast<EncodeTiledFn>(p);
-    }();
-    return fn;
-}
-
-// Inputs below this many elements per row keep the kernel that loads straight into registers.
-constexpr uint64_t kTmaMinElements = 1u << 16;
-
-// The map copies raw 32- or 16-bit words (no floating-point interpretation), rows past the last whole
-// run read as zeros.  Returns false when the tiled path does not apply (then the direct kernel runs).
-static bool make_tile_map(const CompressCall& c, CUtensorMap* map) {
-    const EncodeTiledFn encode = encode_tiled_fn();
-    const uint64_t whole = c.d / 32;
-    if (!encode || c.d < kTmaMinElements || whole > 0x7FFFFF00ull) return false;
-    const uint64_t esz = c.bf16 ? 2 : 4;
-    const cuuint64_t gdim[3] = {32, whole, c.n_workers};
-    const cuuint64_t row_pitch = c.n_workers > 1 ? c.grad_stride * esz : whole * 32 * esz;
-    const cuuint64_t gstride[2] = {32 * esz, row_pitch};              // bytes between runs, between workers
-    if (row_pitch % 16 != 0 || row_pitch >= (1ull << 40)) return false;
-    const cuuint32_t box[3] = {32, static_cast<cuuint32_t>(kThreads), 1};
-    const cuuint32_t estr[3] = {1, 1, 1};
-    const CUresult r = encode(map, c.bf16 ? CU_TENSOR_MAP_DATA_TYPE_UINT16 : CU_TENSOR_MAP_DATA_TYPE_UINT32, 3,
-                              const_cast<void*>(c.grad), gdim, gstride, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                              c.bf16 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
-                              CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return r == CUDA_SUCCESS;
-}
-
-template <int BITS, bool BF>
-static cudaError_t launch_tma(const CompressCall& c, const CompressArgs& args, dim3 grid, const CUtensorMap& map) {
-    const int smem = kThreads * 32 * (BF ? 2 : 4) + 16;
-    const cudaError_t e = cudaFuncSetAttribute(compress_tma_kernel<BITS, BF>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
-    return launch_kernel(compress_tma_kernel<BITS, BF>, grid, kThreads, smem, c.stream, map, c.grad, c.d, c.grad_stride, args,
-                         round_keys(c.seed), c.first_worker, c.packed, c.words_stride);
-}
-
 template <int BITS>
-static cudaError_t dispatch(const CompressCall& c, const CompressArgs& a, dim3 grid, int search) {
-    // Tiled copies pay for bf16 rows (3 % faster at 124 M x 8: half the bytes per element, so the wait for
-    // global loads weighs more); for fp32 rows the kernel is bound by instruction issue and the extra
-    // shared-memory reads and the barrier per tile cost 2-3 %, so those keep the direct kernel.
-    if (search == kGrid && c.bf16) {
-        alignas(64) CUtensorMap map;
-        if (make_tile_map(c, &map)) return launch_tma<BITS, true>(c, a, grid, map);
+static cudaError_t dispatch(const CompressCall& c, const CompressArgs<TQ_MAX_WORKERS>& a, dim3 grid, int search) {
+    const bool few = c.n_workers <= kFewWorkers;
+    const CompressArgs<kFewWorkers>& f = reinterpret_cast<const CompressArgs<kFewWorkers>&>(a);      // its first entries
+    if (search == kGrid) {
+        if (few) return c.bf16 ? launch<BITS, kGrid, true>(c, f, grid) : launch<BITS, kGrid, false>(c, f, grid);
+        return c.bf16 ? launch<BITS, kGrid, true>(c, a, grid) : launch<BITS, kGrid, false>(c, a, grid);
     }
-    if (search == kGrid) return c.bf16 ? launch<BITS, kGrid, true>(c, a, grid) : launch<BITS, kGrid, false>(c, a, grid);
     if (search == kBinary) return c.bf16 ? launch<BITS, kBinary, true>(c, a, grid) : launch<BITS, kBinary, false>(c, a, grid);
     if (search == kUniformWide) return c.bf16 ? launch<BITS, kUniformWide, true>(c, a, grid) : launch<BITS, kUniformWide, false>(c, a, grid);
+    if (few) return c.bf16 ? launch<BITS, kUniform, true>(c, f, grid) : launch<BITS, kUniform, false>(c, f, grid);
     return c.bf16 ? launch<BITS, kUniform, true>(c, a, grid) : launch<BITS, kUniform, false>(c, a, grid);
 }
 
@@ -789,7 +645,7 @@ cudaError_t launch_compress(const CompressCall& c) {
         const cudaError_t e = launch_compress_lut(c, &applied);
         if (applied || e != cudaSuccess) return e;
     }
-    static thread_local CompressArgs args;   // 9 KB: keep it off the stack
+    static thread_local CompressArgs<TQ_MAX_WORKERS> args;   // 9 KB: keep it off the stack
     int search = c.nonuniform ? kGrid : kUniform;
     for (uint32_t i = 0; i < c.n_workers; ++i) {
         const tq_params_t& p = c.params[i];

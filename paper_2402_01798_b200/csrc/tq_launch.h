@@ -3,6 +3,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "tq.h"
 
 namespace tq {
@@ -60,8 +62,12 @@ inline void plan_tiles(TilePlan* plan, const SegTable* segs, uint64_t d, uint32_
 
 // SMs of the current device.
 inline int sm_count() {
+    static std::atomic<int> known[64];           // per device, 0: not asked yet
     int dev = 0, sms = 148;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (cudaGetDevice(&dev) != cudaSuccess) return sms;
+    if (dev >= 0 && dev < 64 && (sms = known[dev].load(std::memory_order_relaxed)) > 0) return sms;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 148;
+    if (dev >= 0 && dev < 64) known[dev].store(sms, std::memory_order_relaxed);
     return sms;
 }
 
@@ -108,8 +114,7 @@ struct DecompressCall {
     const SegTable* segs = nullptr;          // device parameters only: params_dev[n_workers * segs->n]; d and words_valid are then unused
 };
 cudaError_t launch_decompress(const DecompressCall& c);
-cudaError_t read_wait_expired(unsigned int* count);
-cudaError_t read_compress_wait_expired(unsigned int* count);   // the same for the tiled compress kernel   // give-ups of bounded barrier waits on the current device
+cudaError_t read_wait_expired(unsigned int* count);           // give-ups of bounded barrier waits on the current device
 
 struct StatsCall {
     const void* grad; bool bf16; uint64_t d, grad_stride; uint32_t n_workers;
