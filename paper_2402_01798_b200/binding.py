@@ -1,7 +1,8 @@
-"""ctypes binding of libtq.so: same names and argument order as include/tq.h.
+"""Python binding of libtq.so: same names and argument order as include/tq.h.
 
-Only argument marshalling happens here.  Tensors are torch tensors used as typed device
-buffers; the stream is torch's current CUDA stream unless one is given.
+Only argument marshalling happens here and, for the calls of a round, in the compiled module ``_tq_python``
+(csrc/tq_python.cpp).  Tensors are torch tensors used as typed device buffers; the stream is torch's current
+CUDA stream unless one is given.
 """
 from __future__ import annotations
 
@@ -57,6 +58,7 @@ class TqError(RuntimeError):
 
 
 _lib: Optional[C.CDLL] = None
+_native = None
 
 
 class Segment(C.Structure):
@@ -66,7 +68,7 @@ class Segment(C.Structure):
 
 def lib() -> C.CDLL:
     """Load libtq.so.  There is no fallback: a missing library is an error."""
-    global _lib
+    global _lib, _native
     if _lib is None:
         if not os.path.exists(LIB_PATH):
             raise RuntimeError(
@@ -112,8 +114,32 @@ def lib() -> C.CDLL:
         L.tq_last_cuda_error.restype = C.c_int
         L.tq_kernel_launches.restype = u64
         L.tq_wait_expired_count.argtypes = [C.POINTER(u32)]; L.tq_wait_expired_count.restype = C.c_int
+        _native = _load_native(L)
         _lib = L
     return _lib
+
+
+# the order of the function table in csrc/tq_python.cpp
+_NATIVE = ("tq_stats", "tq_stats_hinted", "tq_stats_static", "tq_params_batch", "tq_params_device", "tq_compress", "tq_compress_device_params",
+           "tq_decompress_aggregate", "tq_decompress_aggregate_rows", "tq_decompress_aggregate_apply",
+           "tq_decompress_aggregate_device_params", "tq_stats_segments", "tq_stats_hinted_segments", "tq_compress_segments",
+           "tq_decompress_aggregate_segments")
+
+
+def _load_native(L: C.CDLL):
+    try:
+        from . import _tq_python
+    except ImportError as e:
+        raise RuntimeError("the compiled marshalling module is missing or does not load: build it with "
+                           "`python -m paper_2402_01798_b200.build`") from e
+    _tq_python.bind([C.cast(getattr(L, name), C.c_void_p).value for name in _NATIVE])
+    return _tq_python
+
+
+def _calls():
+    if _native is None:
+        lib()
+    return _native
 
 
 def _check(status: int, where: str) -> None:
@@ -125,40 +151,9 @@ def _check(status: int, where: str) -> None:
         raise TqError(status, where, detail)
 
 
-# torch.cuda.current_stream().cuda_stream without the Stream object (3.3 us of every call's 8)
-_current_device = getattr(torch._C, "_cuda_getDevice", None) or torch.cuda.current_device
-_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or (lambda device: torch.cuda.current_stream(device).cuda_stream)
-
-
-def _stream(stream) -> int:
-    if stream is None:
-        return _raw_stream(_current_device())
-    return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
-
-
-def _dtype_code(t: torch.Tensor) -> int:
-    if t.dtype == torch.float32:
-        return F32
-    if t.dtype == torch.bfloat16:
-        return BF16
-    raise TypeError("gradient must be float32 or bfloat16")
-
-
-def _grad_layout(grad: torch.Tensor, d: Optional[int]):
-    """(n_workers, d, stride) of a [N, stride] or [d] gradient tensor on the GPU."""
-    if not grad.is_cuda:
-        raise ValueError("gradient must be a CUDA tensor")
-    dims = grad.dim()
-    if dims == 1:
-        grad, dims = grad.unsqueeze(0), 2
-    if dims != 2 or grad.stride(1) != 1:
-        raise ValueError("gradient must be [N, stride] with unit inner stride")
-    n, width = grad.size(0), grad.size(1)
-    return n, (width if d is None else d), (grad.stride(0) if n > 1 else width)
-
-
-def _words_stride(packed: torch.Tensor, n: int) -> int:
-    return packed.stride(0) if n > 1 and packed.dim() == 2 else packed.size(-1)
+def _rows(grad: torch.Tensor) -> int:
+    """Workers of a [N, stride] or [d] gradient tensor."""
+    return grad.size(0) if grad.dim() == 2 else 1
 
 
 def params_array(params: Sequence[Params]):
@@ -182,13 +177,11 @@ def tq_stats_workspace_bytes(n_workers: int) -> int:
 def tq_stats(grad: torch.Tensor, d: Optional[int] = None, g_min: float = 0.0, kappa: float = 1.0,
              stats_dev: Optional[torch.Tensor] = None, workspace: Optional[torch.Tensor] = None, stream=None):
     """Enqueue the statistics reduction; returns the device tensor holding n_workers 64-byte records."""
-    n, d, stride = _grad_layout(grad, d)
     if stats_dev is None:
-        stats_dev = torch.empty(n * 64, dtype=torch.uint8, device=grad.device)
+        stats_dev = torch.empty(_rows(grad) * 64, dtype=torch.uint8, device=grad.device)
     if workspace is None:
-        workspace = torch.empty(tq_stats_workspace_bytes(n), dtype=torch.uint8, device=grad.device)
-    _check(lib().tq_stats(grad.data_ptr(), _dtype_code(grad), d, stride, n, g_min, kappa, stats_dev.data_ptr(),
-                          workspace.data_ptr(), workspace.numel(), _stream(stream)), "tq_stats")
+        workspace = torch.empty(tq_stats_workspace_bytes(_rows(grad)), dtype=torch.uint8, device=grad.device)
+    _check(_calls().stats(grad, d, g_min, kappa, stats_dev, workspace, stream), "tq_stats")
     return stats_dev
 
 
@@ -199,14 +192,11 @@ def tq_stats_hinted(grad: torch.Tensor, hint: torch.Tensor, d: Optional[int] = N
     ``hint`` is a device tensor of n_workers * 8 bytes (tq_gmin_hint_t records) that the caller keeps from
     round to round; zero it before the first one (``new_gmin_hint``).  Returns the records' device tensor.
     """
-    n, d, stride = _grad_layout(grad, d)
     if stats_dev is None:
-        stats_dev = torch.empty(n * 64, dtype=torch.uint8, device=grad.device)
+        stats_dev = torch.empty(_rows(grad) * 64, dtype=torch.uint8, device=grad.device)
     if workspace is None:
-        workspace = torch.empty(tq_stats_workspace_bytes(n), dtype=torch.uint8, device=grad.device)
-    _check(lib().tq_stats_hinted(grad.data_ptr(), _dtype_code(grad), d, stride, n, kappa, hint.data_ptr(),
-                                 stats_dev.data_ptr(), workspace.data_ptr(), workspace.numel(), _stream(stream)),
-           "tq_stats_hinted")
+        workspace = torch.empty(tq_stats_workspace_bytes(_rows(grad)), dtype=torch.uint8, device=grad.device)
+    _check(_calls().stats_hinted(grad, d, kappa, hint, stats_dev, workspace, stream), "tq_stats_hinted")
     return stats_dev
 
 
@@ -228,9 +218,7 @@ def tq_stats_static(grad: torch.Tensor, stats_dev: torch.Tensor, d: Optional[int
     The caller passes the gradient and the output records (``stats_dev``, n_workers * 64 bytes); this
     wrapper allocates nothing either.  At most STATIC_MAX_WORKERS rows; calls that overlap on the GPU race.
     """
-    n, d, stride = _grad_layout(grad, d)
-    _check(lib().tq_stats_static(grad.data_ptr(), _dtype_code(grad), d, stride, n, g_min, kappa,
-                                 stats_dev.data_ptr(), _stream(stream)), "tq_stats_static")
+    _check(_calls().stats_static(grad, d, g_min, kappa, stats_dev, stream), "tq_stats_static")
     return stats_dev
 
 
@@ -253,14 +241,13 @@ def tq_params_batch(stats_raw, n_workers: int, num_levels: int, mode: int, gamma
     """tq_params for n workers at once.  ``stats_raw``: the n 64-byte records as bytes, a ctypes array of
     Stats, or a pinned CPU uint8 tensor (used in place).  Returns a ctypes tq_params_t[n] array."""
     out = (Params * n_workers)()
-    if isinstance(stats_raw, torch.Tensor):
-        src = stats_raw.data_ptr()
-    elif isinstance(stats_raw, (bytes, bytearray)):
-        src = C.cast(C.create_string_buffer(bytes(stats_raw), len(stats_raw)), C.c_void_p)
-    else:
-        src = C.cast(stats_raw, C.c_void_p)
-    _check(lib().tq_params_batch(src, n_workers, num_levels, mode, gamma, alpha_rule, alpha_user,
-                                 out), "tq_params_batch")
+    src, keep = stats_raw, None
+    if isinstance(stats_raw, (bytes, bytearray)):
+        keep = C.create_string_buffer(bytes(stats_raw), len(stats_raw))
+        src = C.addressof(keep)
+    elif not isinstance(stats_raw, torch.Tensor):
+        src = C.cast(stats_raw, C.c_void_p).value
+    _check(_calls().params_batch(src, n_workers, num_levels, mode, gamma, alpha_rule, alpha_user, out), "tq_params_batch")
     return out
 
 
@@ -274,14 +261,10 @@ def tq_params_from_levels(levels: Sequence[float], mode: int = NONUNIFORM) -> Pa
 def tq_compress(grad: torch.Tensor, params: Sequence[Params], seed: int, first_worker: int = 0,
                 d: Optional[int] = None, packed: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """Enqueue truncate + stochastic round + pack for all rows of ``grad``; returns [N, words] int32."""
-    n, d, stride = _grad_layout(grad, d)
-    if len(params) != n:
-        raise ValueError("one Params per worker")
     if packed is None:
-        packed = torch.empty((n, tq_packed_words(d, params[0].bits)), dtype=torch.int32, device=grad.device)
-    _check(lib().tq_compress(grad.data_ptr(), _dtype_code(grad), d, stride, n, _params_array(params),
-                             seed & 0xFFFFFFFFFFFFFFFF, first_worker, packed.data_ptr(), _words_stride(packed, n),
-                             _stream(stream)), "tq_compress")
+        packed = torch.empty((_rows(grad), tq_packed_words(grad.shape[-1] if d is None else d, params[0].bits)), dtype=torch.int32,
+                             device=grad.device)
+    _check(_calls().compress(grad, d, _params_array(params), seed & 0xFFFFFFFFFFFFFFFF, first_worker, packed, stream), "tq_compress")
     return packed
 
 
@@ -289,16 +272,9 @@ def tq_decompress_aggregate(packed: torch.Tensor, d: int, params: Sequence[Param
                             weights: Optional[Sequence[float]] = None, out: Optional[torch.Tensor] = None,
                             stream=None) -> torch.Tensor:
     """Enqueue unpack + dequantize + average of the N packed rows; returns the [d] fp32 update."""
-    if not packed.is_cuda or packed.dim() != 2:
-        raise ValueError("packed must be a [N, words] CUDA tensor")
-    n = packed.size(0)
-    if len(params) != n:
-        raise ValueError("one Params per worker")
     if out is None:
         out = torch.empty(d, dtype=torch.float32, device=packed.device)
-    w = None if weights is None else (C.c_float * n)(*[float(x) for x in weights])
-    _check(lib().tq_decompress_aggregate(packed.data_ptr(), _words_stride(packed, n), n, d, _params_array(params), w,
-                                         out.data_ptr(), _stream(stream)), "tq_decompress_aggregate")
+    _check(_calls().decompress_aggregate(packed, d, _params_array(params), weights, out, stream), "tq_decompress_aggregate")
     return out
 
 
@@ -308,16 +284,10 @@ def tq_decompress_aggregate_rows(rows: Sequence, d: int, params: Sequence[Params
     """tq_decompress_aggregate with one packed row per worker, each given as a 1-D int32 CUDA tensor or as a
     raw device address (an int, e.g. a peer's buffer mapped into this process).  The caller keeps the rows
     alive until the stream has passed the call."""
-    n = len(rows)
-    if len(params) != n:
-        raise ValueError("one Params per worker")
-    ptrs = (C.c_void_p * n)(*[int(r) if isinstance(r, int) else r.data_ptr() for r in rows])
     if out is None:
         dev = next((r.device for r in rows if not isinstance(r, int)), "cuda")
         out = torch.empty(d, dtype=torch.float32, device=dev)
-    w = None if weights is None else (C.c_float * n)(*[float(x) for x in weights])
-    _check(lib().tq_decompress_aggregate_rows(ptrs, n, d, _params_array(params), w, out.data_ptr(), _stream(stream)),
-           "tq_decompress_aggregate_rows")
+    _check(_calls().decompress_aggregate_rows(rows, d, _params_array(params), weights, out, stream), "tq_decompress_aggregate_rows")
     return out
 
 
@@ -327,8 +297,7 @@ def tq_params_device(stats_dev: torch.Tensor, n_workers: int, num_levels: int, m
     """Enqueue the parameter design on the device; returns the device tensor of n_workers 176-byte records."""
     if params_dev is None:
         params_dev = torch.empty(n_workers * C.sizeof(Params), dtype=torch.uint8, device=stats_dev.device)
-    _check(lib().tq_params_device(stats_dev.data_ptr(), n_workers, num_levels, mode, gamma, alpha_rule, alpha_user,
-                                  params_dev.data_ptr(), _stream(stream)), "tq_params_device")
+    _check(_calls().params_device(stats_dev, n_workers, num_levels, mode, gamma, alpha_rule, alpha_user, params_dev, stream), "tq_params_device")
     return params_dev
 
 
@@ -342,25 +311,18 @@ def params_to_host(params_dev: torch.Tensor):
 def tq_compress_device_params(grad: torch.Tensor, params_dev: torch.Tensor, num_levels: int, mode: int, seed: int,
                               first_worker: int = 0, d: Optional[int] = None, packed: Optional[torch.Tensor] = None,
                               stream=None) -> torch.Tensor:
-    n, d, stride = _grad_layout(grad, d)
     if packed is None:
-        packed = torch.empty((n, tq_packed_words(d, _BITS[num_levels])), dtype=torch.int32, device=grad.device)
-    _check(lib().tq_compress_device_params(grad.data_ptr(), _dtype_code(grad), d, stride, n, params_dev.data_ptr(),
-                                           num_levels, mode, seed & 0xFFFFFFFFFFFFFFFF, first_worker, packed.data_ptr(),
-                                           _words_stride(packed, n), _stream(stream)), "tq_compress_device_params")
+        packed = torch.empty((_rows(grad), tq_packed_words(grad.shape[-1] if d is None else d, _BITS[num_levels])), dtype=torch.int32, device=grad.device)
+    _check(_calls().compress_device_params(grad, d, params_dev, num_levels, mode, seed & 0xFFFFFFFFFFFFFFFF, first_worker, packed, stream), "tq_compress_device_params")
     return packed
 
 
 def tq_decompress_aggregate_device_params(packed: torch.Tensor, d: int, params_dev: torch.Tensor, num_levels: int,
                                           weights: Optional[Sequence[float]] = None,
                                           out: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
-    n = packed.size(0)
     if out is None:
         out = torch.empty(d, dtype=torch.float32, device=packed.device)
-    w = None if weights is None else (C.c_float * n)(*[float(x) for x in weights])
-    _check(lib().tq_decompress_aggregate_device_params(packed.data_ptr(), _words_stride(packed, n), n, d, params_dev.data_ptr(),
-                                                       num_levels, w, out.data_ptr(), _stream(stream)),
-           "tq_decompress_aggregate_device_params")
+    _check(_calls().decompress_aggregate_device_params(packed, d, params_dev, num_levels, weights, out, stream), "tq_decompress_aggregate_device_params")
     return out
 
 
@@ -378,16 +340,12 @@ def tq_stats_segments(grad: torch.Tensor, segments, g_min: float = 0.0, kappa: f
                       stats_dev: Optional[torch.Tensor] = None, workspace: Optional[torch.Tensor] = None,
                       stream=None) -> torch.Tensor:
     """One record per (worker, segment), index worker * n_segments + segment; returns the device records."""
-    n, _, stride = _grad_layout(grad, None)
     seg = segments if isinstance(segments, C.Array) else segments_array(segments)
-    jobs = n * len(seg)
     if stats_dev is None:
-        stats_dev = torch.empty(jobs * C.sizeof(Stats), dtype=torch.uint8, device=grad.device)
+        stats_dev = torch.empty(_rows(grad) * len(seg) * C.sizeof(Stats), dtype=torch.uint8, device=grad.device)
     if workspace is None:
-        workspace = torch.empty(tq_stats_workspace_bytes(jobs), dtype=torch.uint8, device=grad.device)
-    _check(lib().tq_stats_segments(grad.data_ptr(), _dtype_code(grad), stride, n, seg, len(seg), g_min, kappa,
-                                   stats_dev.data_ptr(), workspace.data_ptr(), workspace.numel(), _stream(stream)),
-           "tq_stats_segments")
+        workspace = torch.empty(tq_stats_workspace_bytes(_rows(grad) * len(seg)), dtype=torch.uint8, device=grad.device)
+    _check(_calls().stats_segments(grad, seg, g_min, kappa, stats_dev, workspace, stream), "tq_stats_segments")
     return stats_dev
 
 
@@ -395,40 +353,29 @@ def tq_stats_hinted_segments(grad: torch.Tensor, segments, hint: torch.Tensor, k
                              stats_dev: Optional[torch.Tensor] = None, workspace: Optional[torch.Tensor] = None,
                              stream=None) -> torch.Tensor:
     """tq_stats_hinted for every (worker, segment) pair; `hint` = new_gmin_hint(n_workers * n_segments), kept across rounds."""
-    n, _, stride = _grad_layout(grad, None)
     seg = segments if isinstance(segments, C.Array) else segments_array(segments)
-    jobs = n * len(seg)
     if stats_dev is None:
-        stats_dev = torch.empty(jobs * C.sizeof(Stats), dtype=torch.uint8, device=grad.device)
+        stats_dev = torch.empty(_rows(grad) * len(seg) * C.sizeof(Stats), dtype=torch.uint8, device=grad.device)
     if workspace is None:
-        workspace = torch.empty(tq_stats_workspace_bytes(jobs), dtype=torch.uint8, device=grad.device)
-    _check(lib().tq_stats_hinted_segments(grad.data_ptr(), _dtype_code(grad), stride, n, seg, len(seg), kappa, hint.data_ptr(),
-                                          stats_dev.data_ptr(), workspace.data_ptr(), workspace.numel(), _stream(stream)),
-           "tq_stats_hinted_segments")
+        workspace = torch.empty(tq_stats_workspace_bytes(_rows(grad) * len(seg)), dtype=torch.uint8, device=grad.device)
+    _check(_calls().stats_hinted_segments(grad, seg, kappa, hint, stats_dev, workspace, stream), "tq_stats_hinted_segments")
     return stats_dev
 
 
 def tq_compress_segments(grad: torch.Tensor, segments, params_dev: torch.Tensor, num_levels: int, mode: int, seed: int,
                          first_worker: int = 0, packed: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
-    n, _, stride = _grad_layout(grad, None)
     seg = segments if isinstance(segments, C.Array) else segments_array(segments)
     if packed is None:
-        packed = torch.empty((n, tq_segments_packed_words(seg, _BITS[num_levels])), dtype=torch.int32, device=grad.device)
-    _check(lib().tq_compress_segments(grad.data_ptr(), _dtype_code(grad), stride, n, seg, len(seg), params_dev.data_ptr(),
-                                      num_levels, mode, seed & 0xFFFFFFFFFFFFFFFF, first_worker, packed.data_ptr(),
-                                      _words_stride(packed, n), _stream(stream)), "tq_compress_segments")
+        packed = torch.empty((_rows(grad), tq_segments_packed_words(seg, _BITS[num_levels])), dtype=torch.int32, device=grad.device)
+    _check(_calls().compress_segments(grad, seg, params_dev, num_levels, mode, seed & 0xFFFFFFFFFFFFFFFF, first_worker, packed, stream), "tq_compress_segments")
     return packed
 
 
 def tq_decompress_aggregate_segments(packed: torch.Tensor, segments, params_dev: torch.Tensor, num_levels: int,
                                      out: torch.Tensor, weights: Optional[Sequence[float]] = None, stream=None) -> torch.Tensor:
     """Aggregates every segment into out[offset : offset + length]; elements of `out` outside the segments are left alone."""
-    n = packed.size(0)
     seg = segments if isinstance(segments, C.Array) else segments_array(segments)
-    w = None if weights is None else (C.c_float * n)(*[float(x) for x in weights])
-    _check(lib().tq_decompress_aggregate_segments(packed.data_ptr(), _words_stride(packed, n), n, seg, len(seg), params_dev.data_ptr(),
-                                                  num_levels, w, out.data_ptr(), _stream(stream)),
-           "tq_decompress_aggregate_segments")
+    _check(_calls().decompress_aggregate_segments(packed, seg, params_dev, num_levels, weights, out, stream), "tq_decompress_aggregate_segments")
     return out
 
 
@@ -436,11 +383,7 @@ def tq_decompress_aggregate_apply(packed: torch.Tensor, d: int, params, theta: t
                                   momentum_buf: Optional[torch.Tensor], lr: float, momentum: float = 0.0,
                                   weight_decay: float = 0.0, weights: Optional[Sequence[float]] = None, stream=None):
     """Aggregate the N packed rows and apply the SGD step in place on ``theta`` (and ``momentum_buf``)."""
-    n = packed.size(0)
-    w = None if weights is None else (C.c_float * n)(*[float(x) for x in weights])
-    _check(lib().tq_decompress_aggregate_apply(packed.data_ptr(), _words_stride(packed, n), n, d, _params_array(params), w,
-                                               theta.data_ptr(), None if momentum_buf is None else momentum_buf.data_ptr(),
-                                               lr, momentum, weight_decay, _stream(stream)), "tq_decompress_aggregate_apply")
+    _check(_calls().decompress_aggregate_apply(packed, d, _params_array(params), weights, theta, momentum_buf, lr, momentum, weight_decay, stream), "tq_decompress_aggregate_apply")
     return theta
 
 

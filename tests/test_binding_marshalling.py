@@ -1,0 +1,42 @@
+"""What the compiled marshalling module refuses before any library call (no GPU needed)."""
+import pytest
+import torch
+
+
+@pytest.fixture(scope="module")
+def tq():
+    from paper_2402_01798_b200 import binding
+    binding.lib()
+    return binding
+
+
+def test_wrong_arguments_raise(tq):
+    g = torch.zeros(2, 16)
+    ws, st, hint = torch.zeros(8, dtype=torch.uint8), torch.zeros(128, dtype=torch.uint8), torch.zeros(16, dtype=torch.uint8)
+    with pytest.raises(ValueError, match="CUDA tensor"):
+        tq.tq_stats(g, stats_dev=st, workspace=ws)
+    with pytest.raises(ValueError, match="CUDA tensor"):
+        tq.tq_stats_hinted(g, hint, stats_dev=st, workspace=ws)
+    with pytest.raises(TypeError):
+        tq.tq_stats([1.0, 2.0], stats_dev=st, workspace=ws)
+    p = tq.tq_params_from_levels([-1.0, -0.5, 0.5, 1.0])
+    with pytest.raises(ValueError, match=r"\[N, words\] CUDA tensor"):
+        tq.tq_decompress_aggregate(torch.zeros((1, 4), dtype=torch.int32), 16, [p], out=torch.zeros(16))
+    with pytest.raises(ValueError, match="one Params per worker"):
+        tq.tq_decompress_aggregate_rows([16, 32], 16, [p], out=torch.zeros(16))
+    with pytest.raises(TypeError):
+        tq._calls().compress(g)
+
+
+def test_library_status_comes_back(tq):
+    """Addresses and numbers reach the library unchanged: its own argument checks answer."""
+    with pytest.raises(tq.TqError) as e:
+        tq.tq_params_batch(b"\0" * 64, 1, 5, tq.UNIFORM, 3.0)              # five levels
+    assert e.value.status == tq.ERR_INVALID_ARG
+    with pytest.raises(tq.TqError) as e:
+        tq.tq_params_device(torch.zeros(64, dtype=torch.uint8), 1, 4, -1, 3.0, params_dev=torch.zeros(176, dtype=torch.uint8), stream=0)
+    assert e.value.status == tq.ERR_INVALID_ARG
+    p = tq.tq_params_from_levels([-1.0, 1.0])
+    with pytest.raises(tq.TqError) as e:
+        tq.tq_decompress_aggregate_rows([20], 16, [p], out=torch.zeros(16), stream=0)      # a row off its 16-byte boundary
+    assert e.value.status == tq.ERR_ALIGNMENT
