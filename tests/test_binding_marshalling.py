@@ -25,7 +25,7 @@ def test_wrong_arguments_raise(tq):
     with pytest.raises(ValueError, match="one Params per worker"):
         tq.tq_decompress_aggregate_rows([16, 32], 16, [p], out=torch.zeros(16))
     with pytest.raises(TypeError):
-        tq._calls().compress(g)
+        tq._calls().params_device(st)                      # too few arguments
 
 
 def test_library_status_comes_back(tq):
