@@ -534,31 +534,55 @@ __device__ __forceinline__ void hinted_piece(const JobPiece& piece, const void* 
     }
 }
 
-template <bool BF16>
-__device__ __forceinline__ void hinted_finish_piece(const JobPiece& piece, const TilePlan& plan, const void* grad, uint64_t grad_stride,
-                                                    float kappa, tq_gmin_hint_t* hint_out, tq_stats_t* stats,
-                                                    Partial* partials, uint32_t* tickets, BlockFold<kWarps>& sh) {
-    uint32_t count;
-    const Partial* records = records_of_job(plan, piece, partials, count);
-    const float level = mean_level(kappa, fold_sum_abs(records, count, sh), piece.d), g_min = pow2_floor(level);
-    const int pick = candidate_of(g_min, lower_candidate(record_of_piece(piece, partials)->pad));
-    if (piece.tile0 == 0) {
-        Partial r;
-        fold_records<true, 0>(records, count, r, sh);
-        if (threadIdx.x == 0) {
-            store_moments(stats + piece.job, piece.d, r, g_min);
-            hint_out[piece.job].level = level;
-            hint_out[piece.job].hit = pick >= 0 ? 1u : 0u;
-            if (pick == 2) store_tail_pow2(stats + piece.job, 0, 0.0, g_min);
-        }
-        __syncthreads();
-        if (pick == 0 || pick == 1) {
-            fold_records<false, 2>(records, count, r, sh);
-            if (threadIdx.x == 0) store_tail_pow2(stats + piece.job, r.n_tail[pick], r.sum_log2[pick], g_min);
+// What one warp makes of a job's records: the sum of |g|, and with ALL every other field too.  Same order in every warp.
+template <bool ALL>
+__device__ __forceinline__ Partial warp_fold(const Partial* records, uint32_t count) {
+    const uint32_t lane = threadIdx.x & 31u;
+    Partial p{};
+    for (uint32_t b = lane; b < count; b += 32) {
+        const Partial* q = records + b;
+        p.sum_abs += q->sum_abs;
+        if constexpr (ALL) {
+            p.sum_sq += q->sum_sq; p.n_bad += q->n_bad; p.max_abs = fmaxf(p.max_abs, q->max_abs);
+            p.sum_log2[0] += q->sum_log2[0]; p.sum_log2[1] += q->sum_log2[1]; p.n_tail[0] += q->n_tail[0]; p.n_tail[1] += q->n_tail[1];
         }
     }
-    if (pick >= 0) return;
-
+    p.sum_abs = __shfl_sync(0xFFFFFFFFu, warp_sum(p.sum_abs), 0);
+    if constexpr (ALL) {
+        p.sum_sq = warp_sum(p.sum_sq); p.n_bad = warp_sum(p.n_bad); p.max_abs = warp_max(p.max_abs);
+#pragma unroll
+        for (int k = 0; k < 2; ++k) { p.sum_log2[k] = warp_sum(p.sum_log2[k]); p.n_tail[k] = warp_sum(p.n_tail[k]); }
+    }
+    return p;
+}
+// Finishes a piece as far as the first launch allows: by one warp, a block's pieces side by side.  The job's first piece writes the
+// record.  Returns the threshold if the piece's tail has to be read again, else 0.
+__device__ __forceinline__ float hinted_finish_piece(const JobPiece& piece, const TilePlan& plan, float kappa, tq_gmin_hint_t* hint_out,
+                                                     tq_stats_t* stats, Partial* partials) {
+    uint32_t count;
+    const Partial* records = records_of_job(plan, piece, partials, count);
+    const float t = lower_candidate(record_of_piece(piece, partials)->pad);
+    const bool first = piece.tile0 == 0;
+    // a miss lets other blocks overwrite the tail fields of their records, which are then not used here
+    const Partial r = first ? warp_fold<true>(records, count) : warp_fold<false>(records, count);
+    const float level = mean_level(kappa, r.sum_abs, piece.d), g_min = pow2_floor(level);
+    const int pick = candidate_of(g_min, t);
+    if (first && (threadIdx.x & 31u) == 0) {
+        tq_stats_t* st = stats + piece.job;
+        store_moments(st, piece.d, r, g_min);
+        hint_out[piece.job].level = level;
+        hint_out[piece.job].hit = pick >= 0 ? 1u : 0u;
+        if (pick == 2) store_tail_pow2(st, 0, 0.0, g_min);
+        else if (pick >= 0) store_tail_pow2(st, pick ? r.n_tail[1] : r.n_tail[0], pick ? r.sum_log2[1] : r.sum_log2[0], g_min);
+    }
+    return pick >= 0 ? 0.0f : g_min;
+}
+// The tail sums of a piece of a job whose hint missed.
+template <bool BF16>
+__device__ __forceinline__ void hinted_tail_piece(const JobPiece& piece, const TilePlan& plan, const void* grad, uint64_t grad_stride, float g_min,
+                                                  tq_stats_t* stats, Partial* partials, uint32_t* tickets, BlockFold<kWarps>& sh) {
+    uint32_t count;
+    const Partial* records = records_of_job(plan, piece, partials, count);
     const char* row = row_of<BF16>(piece, grad, grad_stride);
     const TailTest test(g_min);
     Gathered<BF16> g;
@@ -591,11 +615,30 @@ __global__ void __launch_bounds__(kThreads, kStatsBlocksPerSm)
 stats_hinted_finish_kernel(const void* __restrict__ grad, uint64_t grad_stride, float kappa, tq_gmin_hint_t* hint, tq_stats_t* stats,
                            Partial* partials, uint32_t* tickets, const __grid_constant__ TilePlan plan) {
     __shared__ BlockFold<kWarps> sh;
+    __shared__ float s_again[kWarps];
     pdl_wait();
     uint64_t cur = first_tile_of_block(plan, blockIdx.x);
     const uint64_t end = first_tile_of_block(plan, blockIdx.x + 1);
-    while (cur < end) {
-        hinted_finish_piece<BF16>(next_piece(plan, cur, end), plan, grad, grad_stride, kappa, hint, stats, partials, tickets, sh);
+    while (cur < end) {                                        // as many pieces at a time as the block has warps
+        const uint64_t batch = cur;
+        const uint32_t warp = threadIdx.x >> 5;
+        uint32_t n = 0;
+        for (; cur < end && n < kWarps; ++n) {
+            const JobPiece piece = next_piece(plan, cur, end);
+            if (n == warp) {
+                const float again = hinted_finish_piece(piece, plan, kappa, hint, stats, partials);
+                if ((threadIdx.x & 31u) == 0) s_again[warp] = again;
+            }
+        }
+        __syncthreads();
+        uint64_t redo = batch;
+        for (uint32_t i = 0; i < n; ++i) {
+            const JobPiece piece = next_piece(plan, redo, end);
+            if (s_again[i] > 0.0f) {
+                hinted_tail_piece<BF16>(piece, plan, grad, grad_stride, s_again[i], stats, partials, tickets, sh);
+                __syncthreads();
+            }
+        }
         __syncthreads();
     }
 }
