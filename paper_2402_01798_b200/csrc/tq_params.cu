@@ -16,7 +16,7 @@
 // x = ln(a / g_min), in which a boxed alpha equation costs one exp and one log; it is solved by Newton
 // steps (4 to 8 evaluations); and everything that exists once per level or per trial point (levels, inverse
 // widths, the split of the two-step quantizer) is spread over the lanes of the warp.  Measured on B200 for
-// one worker, uniform, 4 levels / 8 workers, 16-level two-step quantizer: 5.3 us / 43 us, against
+// one worker, uniform, 4 levels / 8 workers, 16-level two-step quantizer: 5.3 us / 30 us, against
 // 21.1 us / 3590 us with one thread per worker, two pow per evaluation and Aitken steps.
 #include <cmath>
 
@@ -37,6 +37,7 @@ struct OneThread {
     static constexpr int kLanes = 1;
     TQ_HD int lane() const { return 0; }
     TQ_HD uint32_t ballot(bool b) const { return b ? 1u : 0u; }
+    TQ_HD double of(double v, int) const { return v; }          // another lane's value
     TQ_HD void sync() const {}
 };
 struct OneWarp {
@@ -44,10 +45,12 @@ struct OneWarp {
 #ifdef __CUDA_ARCH__
     __device__ int lane() const { return static_cast<int>(threadIdx.x & 31u); }
     __device__ uint32_t ballot(bool b) const { return __ballot_sync(0xFFFFFFFFu, b); }
+    __device__ double of(double v, int lane) const { return __shfl_sync(0xFFFFFFFFu, v, lane); }
     __device__ void sync() const { __syncwarp(); }
 #else
     int lane() const { return 0; }
     uint32_t ballot(bool b) const { return b ? 1u : 0u; }
+    double of(double v, int) const { return v; }
     void sync() const {}
 #endif
 };
@@ -109,14 +112,15 @@ struct SplitGrid {
     double ln_k[kSplitGrid / Lanes::kLanes];
     TQ_HD explicit SplitGrid(const Lanes& lanes, bool wanted) {
         for (int t = 0; wanted && t < kSplitGrid / Lanes::kLanes; ++t)
-            ln_k[t] = log(static_cast<double>(t * Lanes::kLanes + lanes.lane() + 1) / kSplitGrid);
+            ln_k[t] = t * Lanes::kLanes + lanes.lane() + 1 < kSplitGrid ? log(static_cast<double>(t * Lanes::kLanes + lanes.lane() + 1) / kSplitGrid)
+                                                                        : kSplitLnFirst;
     }
 };
-TQ_HD inline int first_bit(uint32_t v, int none) {         // index of the lowest set bit
+TQ_HD inline int first_bit(uint64_t v) {                   // index of the lowest set bit
 #ifdef __CUDA_ARCH__
-    return v ? __ffs(static_cast<int>(v)) - 1 : none;
+    return __ffsll(static_cast<long long>(v)) - 1;
 #else
-    return v ? __builtin_ctz(v) : none;
+    return __builtin_ctzll(v);
 #endif
 }
 
@@ -131,19 +135,19 @@ struct Split {
         return in_body ? m.body * k * a : 1.0 - 2.0 * m.rho * exp((1.0 - m.gamma) * (x + ln_k));
     }
     TQ_HD double inner(double k, bool in_body) const { return inner(k, in_body, in_body ? 0.0 : log(k)); }
-    // Whether Q_B falls with k.  The derivative's sign is that of
+    // Negative where Q_B falls with k.  The derivative's sign is that of
     //     w^(2/3) (1-k)^(1/3) (u' k + 2 u)  -  u^(2/3) k^(1/3) (u' (1-k) + 2 w),      u' = du/dk,
-    // whose terms are non-negative, so their cubes are compared.
-    TQ_HD bool falls(double k, double u, double du) const {
+    // whose terms are non-negative, so their cubes can be compared: the difference of the cubes has the same zeros.
+    TQ_HD double slope(double k, double u, double du) const {
         double w = mass - u;
         if (w < 0.0) w = 0.0;
         const double p = du * k + 2.0 * u, q = du * (1.0 - k) + 2.0 * w;
-        return w * w * (1.0 - k) * (p * p * p) < u * u * k * (q * q * q);
+        return w * w * (1.0 - k) * (p * p * p) - u * u * k * (q * q * q);
     }
-    TQ_HD bool falls_at(double k, double ln_k) const {
+    TQ_HD double slope_at(double k, double ln_k) const {
         const bool in_body = k * a <= 1.0;
         const double u = inner(k, in_body, ln_k);
-        return falls(k, u, in_body ? m.body * a : (m.gamma - 1.0) * (1.0 - u) / k);      // 1 - u = 2 rho (k a)^(1-gamma)
+        return slope(k, u, in_body ? m.body * a : (m.gamma - 1.0) * (1.0 - u) / k);      // 1 - u = 2 rho (k a)^(1-gamma)
     }
     // Q_B(a, k), and d ln Q_B / dx along the minimum: at fixed k where k is a smooth minimum (its own motion does not
     // change Q_B to first order), along k = 1 / a where it is the kink.
@@ -159,64 +163,75 @@ struct Split {
         return t * t * t;
     }
     // Q_B(a, 0) = Q_B(a, 1) = Q_U(a), so the minimum is a point where Q_B turns from falling to rising.  Every
-    // such turn between neighbours of a 128-point grid is closed in on until its bracket is `tol` wide (relative);
-    // the turn with the smallest Q_B wins.  No turn: the minimum is an end.  Where the density jumps (k a = g_min) the
-    // turn may be a kink, which is tested for by itself.  Q_B is flat at a smooth turn, so a bracket of
-    // 2^-34 already fixes it to the last bit: the alpha iteration asks for no more.
+    // such turn between neighbours of a 128-point grid is closed in on; the turn with the smallest Q_B wins.  No turn:
+    // the minimum is an end.  Where the density jumps (k a = g_min) the turn may be a kink, which is tested for by itself.
+    // Q_B is flat at a smooth turn, so an error of 2^-34 there does not show in its last bit: the alpha iteration asks
+    // for no more.
     template <class Lanes>
-    TQ_HD double best(const Lanes& lanes, const SplitGrid<Lanes>& grid, double tol, double* q_best, double* ln_slope) const {
+    TQ_HD double best(const Lanes& lanes, const SplitGrid<Lanes>& grid, bool fine, double* q_best, double* ln_slope) const {
         constexpr int n = Lanes::kLanes;
         *ln_slope = NAN;
         if (x <= 0.0) { *q_best = mass; return 0.5; }            // flat density: Q_B is the same for every k
-        uint32_t down[kSplitGrid / 32] = {};                     // bit j - 1: Q_B falls at k = j / 128 (the end counts as rising)
+        uint64_t down[2] = {0, 0};                               // bit j - 1: Q_B falls at k = j / 128 (the end counts as rising)
 #pragma unroll
         for (int t = 0; t < kSplitGrid / n; ++t) {
-            const int j = t * n + lanes.lane() + 1;
-            const bool falling = j < kSplitGrid && falls_at(static_cast<double>(j) / kSplitGrid, grid.ln_k[t]);
-            down[t * n / 32] |= lanes.ballot(falling) << (t * n % 32);
+            const int j = t * n + lanes.lane() + 1;               // the last place is the grid's first point
+            const bool falling = slope_at(j < kSplitGrid ? static_cast<double>(j) / kSplitGrid : kSplitFirst, grid.ln_k[t]) < 0.0;
+            down[t * n / 64] |= static_cast<uint64_t>(lanes.ballot(falling)) << (t * n % 64);
         }
+        const uint64_t first = down[1] >> 63;
+        down[1] &= ~(1ull << 63);
+        uint64_t turns0 = ~down[0] & ((down[0] << 1) | first), turns1 = ~down[1] & ((down[1] << 1) | (down[0] >> 63));
         double best_k = 0.0, best_q = mass;
-        uint32_t before = falls_at(kSplitFirst, kSplitLnFirst) ? 1u : 0u;
-#pragma unroll
-        for (int v = 0; v < kSplitGrid / 32; ++v) {
-            uint32_t turns = ~down[v] & ((down[v] << 1) | before);
-            before = down[v] >> 31;
-            for (; turns != 0; turns &= turns - 1) {
-                const int j = 32 * v + first_bit(turns, 0) + 1;
-                bool kink = false;
-                const double k = close_in(lanes, j > 1 ? static_cast<double>(j - 1) / kSplitGrid : kSplitFirst,
-                                          static_cast<double>(j) / kSplitGrid, tol, &kink);
-                double slope;
-                const double q = factor(k, kink, &slope);
-                if (q < best_q) { best_q = q; best_k = k; *ln_slope = slope; }
-            }
+#pragma unroll 1
+        while ((turns0 | turns1) != 0) {
+            const int j = (turns0 ? first_bit(turns0) : 64 + first_bit(turns1)) + 1;
+            if (turns0) turns0 &= turns0 - 1; else turns1 &= turns1 - 1;
+            bool kink = false;
+            const double k = close_in(lanes, j > 1 ? static_cast<double>(j - 1) / kSplitGrid : kSplitFirst, static_cast<double>(j) / kSplitGrid, fine, &kink);
+            double slope;
+            const double q = factor(k, kink, &slope);
+            if (q < best_q) { best_q = q; best_k = k; *ln_slope = slope; }
         }
         *q_best = best_q;
         return best_k;
     }
-    // Q_B falls at lo and does not at hi: the lanes' trial points cut the bracket into kLanes + 1 parts each time.
+    // Q_B falls at lo and does not at hi: the lanes' trial points cut the bracket into kLanes + 1 parts each time until it is
+    // 2^-17 wide (relative).  The slope is then a straight line in it, and its zero is off by the square of that width, 2^-34;
+    // `fine` adds a Newton step with the slope of that line, which multiplies the error by 2^-17 once more.
     template <class Lanes>
-    TQ_HD double close_in(const Lanes& lanes, double lo, double hi, double tol, bool* at_kink) const {
+    TQ_HD double close_in(const Lanes& lanes, double lo, double hi, bool fine, bool* at_kink) const {
         constexpr int n = Lanes::kLanes;
         const double kink = 1.0 / a;
         if (kink > lo && kink < hi) {
-            const bool before = falls(kink, m.body, m.body * a), after = falls(kink, m.body, 2.0 * m.rho * (m.gamma - 1.0) * a);
+            const double du_tail = 2.0 * m.rho * (m.gamma - 1.0) * a;
+            const bool before = slope(kink, m.body, m.body * a) < 0.0, after = slope(kink, m.body, du_tail) < 0.0;
             if (before && !after) { *at_kink = true; return kink; }
             if (before) lo = kink; else hi = kink;
         }
-        for (int it = 0; it < 64 && hi - lo > tol * hi; ++it) {
+        double s_lo = NAN, s_hi = NAN;                           // slopes at the ends, where known
+#pragma unroll 1
+        for (int it = 0; it < 64 && (hi - lo > 7.62939453125e-6 * hi || !(s_lo < 0.0) || !(s_hi >= 0.0)); ++it) {
             const double step = (hi - lo) / (n + 1);
-            const double k = lo + step * (lanes.lane() + 1);
-            const int c = first_bit(lanes.ballot(!falls_at(k, log(k))), n);      // trial points before the first one where Q_B rises
-            const double new_lo = lo + step * c, new_hi = c < n ? lo + step * (c + 1) : hi;
+            const double k = lo + step * (lanes.lane() + 1), s = slope_at(k, log(k));
+            const uint32_t rises = lanes.ballot(!(s < 0.0));
+            const int c = rises ? first_bit(rises) : n;            // trial points before the first one where Q_B rises
+            const double new_lo = c > 0 ? lo + step * c : lo, new_hi = c < n ? lo + step * (c + 1) : hi;
+            if (c > 0) s_lo = lanes.of(s, c - 1);
+            if (c < n) s_hi = lanes.of(s, c);
             if (!(new_hi - new_lo < hi - lo)) break;
             lo = new_lo; hi = new_hi;
         }
-        return 0.5 * (lo + hi);
+        if (!(s_lo < 0.0 && s_hi >= 0.0)) return 0.5 * (lo + hi);
+        const double per_slope = (hi - lo) / (s_hi - s_lo);
+        double k = lo - s_lo * per_slope;
+        if (fine) {
+            const double better = k - slope_at(k, log(k)) * per_slope;
+            if (better > lo && better < hi) k = better;
+        }
+        return k;
     }
 };
-constexpr double kSplitCoarse = 5.820766091346741e-11;    // 2^-34
-constexpr double kSplitFine = 4.440892098500626e-16;      // 2^-51
 
 TQ_HD inline float ceil_to_float(double v) {
     float f = static_cast<float>(v);
@@ -271,7 +286,7 @@ TQ_HD inline double solve_alpha(const Lanes& lanes, const SplitGrid<Lanes>& grid
         double slope, f;
         if (mode == TQ_BISCALED) {
             double q, ln_slope;
-            Split(m, x).best(lanes, grid, kSplitCoarse, &q, &ln_slope);
+            Split(m, x).best(lanes, grid, false, &q, &ln_slope);
             f = m.c1 * (m.ln_k - log(q));
             slope = -m.c1 * ln_slope;
         } else {
@@ -352,7 +367,7 @@ TQ_HD inline tq_status design(const Lanes& lanes, const tq_stats_t* st, uint32_t
         // centre reaches k - s/2.  Upper half, then mirrored.
         const Split split(m, log(a / g_min));
         double q, ln_slope;
-        const double k = split.best(lanes, grid, kSplitFine, &q, &ln_slope), beta = k * a;
+        const double k = split.best(lanes, grid, true, &q, &ln_slope), beta = k * a;
         const double u = k > 0.0 ? split.inner(k, k * split.a <= 1.0) : 0.0;
         const double c_in = cbrt(u / (2.0 * beta));
         const double c_out = cbrt((split.mass - u) / (2.0 * (a - beta)));
