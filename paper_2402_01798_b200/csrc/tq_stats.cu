@@ -540,7 +540,7 @@ __device__ __forceinline__ Partial warp_fold(const Partial* records, uint32_t co
     const uint32_t lane = threadIdx.x & 31u;
     Partial p{};
     for (uint32_t b = lane; b < count; b += 32) {
-        const Partial* q = records + b;
+        const volatile Partial* q = records + b;
         p.sum_abs += q->sum_abs;
         if constexpr (ALL) {
             p.sum_sq += q->sum_sq; p.n_bad += q->n_bad; p.max_abs = fmaxf(p.max_abs, q->max_abs);
@@ -593,8 +593,10 @@ __device__ __forceinline__ void hinted_tail_piece(const JobPiece& piece, const T
     Partial p = g.partial();
     block_fold<kWarps, false, 1>(p, sh);
     if (!last_of_job(record_of_piece(piece, partials), p, false, tickets + piece.job, count, sh)) return;
-    fold_records<false, 1>(records, count, p, sh);
-    if (threadIdx.x == 0) store_tail_pow2(stats + piece.job, p.n_tail[0], p.sum_log2[0], g_min);
+    if (threadIdx.x < 32) {                                    // as hinted_finish_piece folds them, or the sums could differ in the last bit
+        const Partial t = warp_fold<true>(records, count);
+        if (threadIdx.x == 0) store_tail_pow2(stats + piece.job, t.n_tail[0], t.sum_log2[0], g_min);
+    }
 }
 
 template <bool BF16>
@@ -645,6 +647,7 @@ stats_hinted_finish_kernel(const void* __restrict__ grad, uint64_t grad_stride, 
 
 // ---- short rows: one cluster per job, one launch -----------------------------------------------------------------
 constexpr int kCluster = 8, kSmallThreads = 512, kSmallWarps = kSmallThreads / 32;
+constexpr int kSmallChunks = 4;              // most per thread
 
 __device__ __forceinline__ void cluster_sync() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -665,9 +668,10 @@ __device__ __forceinline__ T of_rank(const T& mine, uint32_t rank) {          //
     }
 }
 
-// POW2: g_min = kappa * mean|g| rounded down to a power of two (the hint is kept up, not needed); else the caller's g_min, or
-// kappa * mean|g|.  The first two chunks of a thread stay in registers between the two passes, the others are read again.
-template <bool BF16, bool POW2>
+// A thread's CHUNKS chunks stay in registers between the two passes (one kernel for 4 chunks is 0.3 us slower on rows of
+// up to 2, reading the third and fourth again 0.7 us on the others).
+enum Rule { kGiven, kMean, kPow2 };    // g_min: the caller's; kappa * mean|g|; that rounded down to a power of two (the hint is kept up, not needed)
+template <bool BF16, int RULE, int CHUNKS>
 __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kSmallThreads)
 stats_small_kernel(const void* __restrict__ grad, uint64_t grad_stride, float g_min, float kappa, tq_gmin_hint_t* hint, tq_stats_t* stats,
                    const __grid_constant__ SegTable segs) {
@@ -680,22 +684,21 @@ stats_small_kernel(const void* __restrict__ grad, uint64_t grad_stride, float g_
     const char* row = static_cast<const char*>(grad) + (static_cast<uint64_t>(worker) * grad_stride + segs.off[seg]) * (BF16 ? 2 : 4);
     constexpr uint32_t stride = kCluster * kSmallThreads;
     const uint64_t c0 = rank * kSmallThreads + threadIdx.x;
-    const bool has0 = c0 < n_chunks, has1 = c0 + stride < n_chunks;
-    Words w0, w1;
-    if (has0) load_chunk(row, c0, w0);
-    if (has1) load_chunk(row, c0 + stride, w1);
+    Words w[CHUNKS];
+#pragma unroll
+    for (int i = 0; i < CHUNKS; ++i)
+        if (c0 + i * stride < n_chunks) load_chunk(row, c0 + i * stride, w[i]);
     uint64_t j;
     const bool leftover = rank == kCluster - 1 && has_leftover<BF16>(d, j);
 
     Gathered<BF16> g;
-    auto first_pass = [&](uint64_t c, Words& w) { take_any<BF16, kMoments>(row, c, w, 0.0f, 0.0f, g); };
-    if (has0) first_pass(c0, w0);
-    if (has1) first_pass(c0 + stride, w1);
-    walk(row, c0 + 2 * stride, n_chunks, stride, first_pass);
-    if (leftover) g.take_exact(exact_sums<BF16>(row, j, 1, CUDART_INF_F, 0.0f), true, 0, false);
+#pragma unroll
+    for (int i = 0; i < CHUNKS; ++i)
+        if (c0 + i * stride < n_chunks) take_any<BF16, RULE == kGiven ? kBoth : kMoments>(row, c0 + i * stride, w[i], g_min, inverse_of(g_min), g);
+    if (leftover) g.take_exact(exact_sums<BF16>(row, j, 1, RULE == kGiven ? g_min : CUDART_INF_F, inverse_of(g_min)), true, 0, RULE == kGiven);
     Partial p = g.partial();
-    block_fold<kSmallWarps, true, 0>(p, sh);
-    if (threadIdx.x == 0) s_moments = p;
+    block_fold<kSmallWarps, true, RULE == kGiven ? 1 : 0>(p, sh);
+    if (threadIdx.x == 0) { s_moments = p; if constexpr (RULE == kGiven) s_tail = p; }
     cluster_sync();
 
     auto over_ranks = [&](auto v) {                            // lanes 0..7 hold one block's value each
@@ -707,27 +710,29 @@ stats_small_kernel(const void* __restrict__ grad, uint64_t grad_stride, float g_
     const uint32_t from = lane % kCluster;
     const double sum_abs = over_ranks(of_rank(s_moments.sum_abs, from));      // every warp for itself, in the same order
     const float level = mean_level(kappa, sum_abs, d);
-    if constexpr (POW2) g_min = pow2_floor(level);
-    else if (!(g_min > 0.0f)) g_min = level;
+    if constexpr (RULE == kPow2) g_min = pow2_floor(level);
+    if constexpr (RULE == kMean) g_min = level;
     const bool tail_on = g_min > 0.0f && g_min <= kMaxFinite;
     const float inv = inverse_of(g_min);
     const TailTest test(g_min);
 
-    g = Gathered<BF16>();
-    if (tail_on) {
-        auto second_pass = [&](uint64_t c, Words& w) {
-            if constexpr (POW2) take_pow2<BF16, 1, false>(row, c, w, g_min, test, g);
-            else take_any<BF16, kTail>(row, c, w, g_min, inv, g);
-        };
-        if (has0) second_pass(c0, w0);
-        if (has1) second_pass(c0 + stride, w1);
-        walk(row, c0 + 2 * stride, n_chunks, stride, second_pass);
-        if (leftover) g.take_exact(exact_sums<BF16>(row, j, 1, g_min, POW2 ? 1.0f : inv), false, 0, true);
+    if constexpr (RULE != kGiven) {
+        g = Gathered<BF16>();
+        if (tail_on) {
+#pragma unroll
+            for (int i = 0; i < CHUNKS; ++i) {
+                const uint64_t c = c0 + i * stride;
+                if (c >= n_chunks) continue;
+                if constexpr (RULE == kPow2) take_pow2<BF16, 1, false>(row, c, w[i], g_min, test, g);
+                else take_any<BF16, kTail>(row, c, w[i], g_min, inv, g);
+            }
+            if (leftover) g.take_exact(exact_sums<BF16>(row, j, 1, g_min, RULE == kPow2 ? 1.0f : inv), false, 0, true);
+        }
+        p = g.partial();
+        block_fold<kSmallWarps, false, 1>(p, sh);
+        if (threadIdx.x == 0) s_tail = p;
+        cluster_sync();
     }
-    p = g.partial();
-    block_fold<kSmallWarps, false, 1>(p, sh);
-    if (threadIdx.x == 0) s_tail = p;
-    cluster_sync();
     if (rank == 0 && threadIdx.x < 32) {
         Partial t{};
         t.sum_abs = sum_abs;
@@ -738,7 +743,7 @@ stats_small_kernel(const void* __restrict__ grad, uint64_t grad_stride, float g_
         const double sum_log2 = over_ranks(of_rank(s_tail.sum_log2[0], from));
         if (lane == 0) {
             store_moments(stats + job, d, t, g_min);
-            if constexpr (POW2) {
+            if constexpr (RULE == kPow2) {
                 store_tail_pow2(stats + job, n, sum_log2, g_min);
                 hint[job].hit = candidate_of(g_min, lower_candidate(hint[job].level)) >= 0 ? 1u : 0u;      // as the long form reports it
                 hint[job].level = level;
@@ -756,7 +761,7 @@ stats_small_kernel(const void* __restrict__ grad, uint64_t grad_stride, float g_
 // time against the two launches (hinted / two-pass): 100 k x 1 fp32 6.5 / 6.4 against 8.0 / 8.5 us, 250 k x 8 10.9 / 10.3 against
 // 11.5 / 12.7; beyond, the few SMs of a cluster are too slow (500 k x 1: 13.2 against 9.0 us) or the clusters queue
 // (250 k x 16: 18.7 against 13.9 us).  One launch less on the host (2.5 us) comes on top.
-constexpr uint64_t kSmallRowBytes = 1u << 20;
+constexpr uint64_t kSmallRowBytes = static_cast<uint64_t>(kCluster) * kSmallThreads * kSmallChunks * kChunkBytes;      // 1 MiB
 constexpr uint32_t kSmallMaxJobs = 8;
 
 static void plan_stats(const StatsCall& c, uint32_t n_jobs, TilePlan* plan) {
@@ -769,17 +774,23 @@ static void plan_stats(const StatsCall& c, uint32_t n_jobs, TilePlan* plan) {
     if (c.bf16 && plan->per_block >= 64 && 3 * resident <= room) plan_tiles(plan, c.segs, c.d, c.n_workers, kThreads * kChunkBytes / 2, 3 * resident);
 }
 
+template <int RULE, int CHUNKS>
+static cudaError_t launch_clusters(const StatsCall& c, uint32_t n_jobs, tq_gmin_hint_t* hint, const SegTable& segs) {
+    return launch_kernel(c.bf16 ? stats_small_kernel<true, RULE, CHUNKS> : stats_small_kernel<false, RULE, CHUNKS>, dim3(n_jobs * kCluster), kSmallThreads,
+                         0, c.stream, c.grad, c.grad_stride, c.g_min, c.kappa, hint, c.stats, segs);
+}
 // True when the call went to the cluster kernel.
-template <bool POW2>
+template <int RULE>
 static bool launch_small(const StatsCall& c, uint32_t n_jobs, tq_gmin_hint_t* hint, cudaError_t* e) {
     if (n_jobs > kSmallMaxJobs) return false;
     SegTable one;
     if (!c.segs) { one.n = 1; one.off[0] = 0; one.len[0] = c.d; }
     const SegTable& segs = c.segs ? *c.segs : one;
-    for (uint32_t s = 0; s < segs.n; ++s)
-        if (segs.len[s] * (c.bf16 ? 2 : 4) > kSmallRowBytes) return false;
-    *e = launch_kernel(c.bf16 ? stats_small_kernel<true, POW2> : stats_small_kernel<false, POW2>, dim3(n_jobs * kCluster), kSmallThreads, 0,
-                       c.stream, c.grad, c.grad_stride, c.g_min, c.kappa, hint, c.stats, segs);
+    uint64_t most = 0;
+    for (uint32_t s = 0; s < segs.n; ++s) most = segs.len[s] > most ? segs.len[s] : most;
+    most *= c.bf16 ? 2 : 4;
+    if (most > kSmallRowBytes) return false;
+    *e = most <= kSmallRowBytes / 2 ? launch_clusters<RULE, kSmallChunks / 2>(c, n_jobs, hint, segs) : launch_clusters<RULE, kSmallChunks>(c, n_jobs, hint, segs);
     return true;
 }
 
@@ -787,7 +798,10 @@ cudaError_t launch_stats(const StatsCall& c, int* launches) {
     *launches = 0;
     const uint32_t n_jobs = c.segs ? c.n_workers * c.segs->n : c.n_workers;
     cudaError_t e;
-    if (launch_small<false>(c, n_jobs, nullptr, &e)) { *launches = e == cudaSuccess ? 1 : 0; return e; }
+    if (c.g_min > 0.0f ? launch_small<kGiven>(c, n_jobs, nullptr, &e) : launch_small<kMean>(c, n_jobs, nullptr, &e)) {
+        *launches = e == cudaSuccess ? 1 : 0;
+        return e;
+    }
     Partial* partials = static_cast<Partial*>(c.workspace);
     uint32_t* tickets = reinterpret_cast<uint32_t*>(static_cast<char*>(c.workspace) + tickets_offset(n_jobs));
     static thread_local TilePlan plan;
@@ -809,7 +823,7 @@ cudaError_t launch_stats_hinted(const StatsCall& c, tq_gmin_hint_t* hint, int* l
     *launches = 0;
     const uint32_t n_jobs = c.segs ? c.n_workers * c.segs->n : c.n_workers;
     cudaError_t e;
-    if (launch_small<true>(c, n_jobs, hint, &e)) { *launches = e == cudaSuccess ? 1 : 0; return e; }
+    if (launch_small<kPow2>(c, n_jobs, hint, &e)) { *launches = e == cudaSuccess ? 1 : 0; return e; }
     Partial* partials = static_cast<Partial*>(c.workspace);
     uint32_t* tickets = reinterpret_cast<uint32_t*>(static_cast<char*>(c.workspace) + tickets_offset(n_jobs));
     static thread_local TilePlan plan;            // the same plan for both launches: same summation order

@@ -123,3 +123,31 @@ def test_aggregation_forms(tq, orc, bits, n, d):
     m1 = f(0.9) * m0 + g
     assert np.array_equal(mom.cpu().numpy(), m1) and np.array_equal(theta.cpu().numpy(), t0 - f(0.1) * m1)
     assert tq.tq_wait_expired_count() == 0
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("chunks", [0, 1, 4096, 4097, 8192, 8193, 16384, 16385])
+@pytest.mark.parametrize("n", [1, 8, 9])
+def test_statistics_of_short_rows(tq, orc, dtype, chunks, n):
+    """Up to 16384 chunks of 64 bytes and 8 rows one cluster per row does everything; beyond, two launches.  Counts and maxima
+    exact, sums of fp32 partials of at most 16 terms (2e-6), logarithms by the hardware (5e-6), with a few odd values in the row."""
+    d = chunks * (16 if dtype == torch.float32 else 32) + (5 if chunks % 2 else 0)
+    gen = torch.Generator(device="cuda").manual_seed(chunks + n)
+    g = torch.zeros((n, (d + 15) // 16 * 16 + 16), dtype=dtype, device="cuda")
+    g[:, :d] = (torch.randn((n, d), device="cuda", generator=gen) * torch.rand((n, d), device="cuda", generator=gen).add(1e-3).pow(-0.5)).to(dtype)
+    if d > 100:
+        g[0, 17], g[n - 1, d - 1] = float("nan"), float("-inf")
+    host = g.float().cpu().numpy()
+    hint = tq.new_gmin_hint(n)
+    records = {"given": tq.tq_stats(g, d, g_min=0.7), "mean": tq.tq_stats(g, d, kappa=1.5), "pow2": tq.tq_stats_hinted(g, hint, d),
+               "again": tq.tq_stats_hinted(g, hint, d)}
+    assert torch.equal(records["pow2"], records["again"])
+    for name, rec in records.items():
+        for i, r in enumerate(tq.stats_to_host(rec)):
+            x = host[i, :d]
+            o = orc.stats_pow2(x) if name in ("pow2", "again") else orc.stats(x, g_min=0.7 if name == "given" else 0.0, kappa=1.5)
+            assert (r.d, r.n_nonfinite, r.max_abs) == (d, o.n_nonfinite, o.max_abs)
+            assert math.isclose(r.sum_abs, o.sum_abs, rel_tol=2e-6) and math.isclose(r.sum_sq, o.sum_sq, rel_tol=2e-6)
+            assert math.isclose(r.g_min, o.g_min, rel_tol=2e-6)
+            ref = orc.stats(x, g_min=r.g_min) if r.g_min > 0 else o
+            assert r.n_tail == ref.n_tail and math.isclose(r.sum_log_tail, ref.sum_log_tail, rel_tol=5e-6, abs_tol=1e-9)
