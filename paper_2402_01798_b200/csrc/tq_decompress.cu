@@ -463,10 +463,13 @@ static const SegTiles kNoSegTiles{};
 // workers: the direct kernel takes one unit per thread (1 M x 64, 3 bits: 27.5 -> 17.3 us; 20 k x 64: 58 -> 7.9 us; 489 tiles, 2 M x
 // 16: 10.8 us in the bulk form, 12.2 in the direct one).
 constexpr uint64_t kTilesForBulk = 296;
-// The fused update has as much to do after the walk as in it; up to this many tiles one unit per thread keeps more blocks
-// in flight (4 M x 4: 18.6 -> 14.3 us, 11.2 M x 8: 39.9 -> 37.3; 25.6 M x 16, 6250 tiles: 97 us against 102; with 64 workers the
-// walk weighs more again, 3 M x 64: 44 us against 56).
+// The fused update has as much to do after the walk as in it, and fewer registers per thread keep more of its loads in
+// flight: one unit per thread up to this many tiles (4 M x 4: 18.6 -> 14.3 us, 11.2 M x 8: 39.9 -> 37.3; 25.6 M x 16, 6250
+// tiles: 102 us with one unit, 92.9 with two), beyond it two where a tile has four (3 and 4 bits: 25.6 M x 16 96.6 -> 92.9 us,
+// 50 M x 4 142 -> 130, 250 M x 4 684 -> 633).  With 64 workers the walk weighs more again: 3 M x 64 takes 41.5 us with four
+// units, 43.3 with two, 56 with one.
 constexpr uint64_t kTilesForLongApply = 4096;
+constexpr uint32_t kWorkersForShortApply = 32;
 
 template <int BITS, bool APPLY, int U>
 static cudaError_t launch_bulk(const DecompressCall& c, const RowTable& rt, const DecompressArgs& args, const DeviceTables& dt,
@@ -508,8 +511,12 @@ static cudaError_t launch_apply(const DecompressCall& c, const RowTable& rt, con
         return launch_kernel(decompress_kernel<BITS, APPLY>, dim3(static_cast<unsigned>((c.d + kPerBlock - 1) / kPerBlock)), kDecThreads, 0, c.stream, rt,
                              c.words_valid, c.n_workers, c.d, args, dt, scale, divide, ap, c.out);
     }
-    if (APPLY && U > 1 && tiles < kTilesForLongApply && c.n_workers <= 32)
-        return launch_bulk<BITS, APPLY, 1>(c, rt, args, dt, scale, divide, ap, tiles * U);
+    if constexpr (APPLY && U > 1) {
+        if (c.n_workers <= kWorkersForShortApply) {
+            if (tiles < kTilesForLongApply) return launch_bulk<BITS, APPLY, 1>(c, rt, args, dt, scale, divide, ap, tiles * U);
+            if constexpr (U > 2) return launch_bulk<BITS, APPLY, 2>(c, rt, args, dt, scale, divide, ap, tiles * (U / 2));
+        }
+    }
     return launch_bulk<BITS, APPLY, U>(c, rt, args, dt, scale, divide, ap, tiles);
 }
 

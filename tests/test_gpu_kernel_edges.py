@@ -125,6 +125,25 @@ def test_aggregation_forms(tq, orc, bits, n, d):
     assert tq.tq_wait_expired_count() == 0
 
 
+@pytest.mark.parametrize("bits,n,momentum", [(3, 2, 0.9), (4, 1, 0.0), (4, 33, 0.9)])
+@pytest.mark.parametrize("d", [4095 * 4096, 4096 * 4096 - 2047, 4096 * 4096 + 2049])
+def test_fused_update_of_long_rows(tq, bits, n, momentum, d):
+    """From 4096 tiles on two units per thread (one below; four beyond 32 workers).  The aggregate comes from the plain
+    kernel and the update is one rounding per operation: equal."""
+    s = (1 << bits) - 1
+    ps = [tq.tq_params_from_levels([(2 * k - s) * (1.0 + i) / s for k in range(s + 1)]) for i in range(n)]
+    gen = torch.Generator(device="cuda").manual_seed(d)
+    packed = torch.randint(-2 ** 31, 2 ** 31 - 1, (n, tq.tq_packed_words(d, bits)), dtype=torch.int32, device="cuda", generator=gen)
+    g = tq.tq_decompress_aggregate(packed, d, ps)
+    theta = torch.randn(d, device="cuda", generator=gen)
+    mom = torch.randn(d, device="cuda", generator=gen) if momentum else None
+    m1 = momentum * mom + g if momentum else g
+    t1 = theta - 0.1 * m1
+    tq.tq_decompress_aggregate_apply(packed, d, ps, theta, mom, lr=0.1, momentum=momentum)
+    assert torch.equal(theta, t1) and (mom is None or torch.equal(mom, m1))
+    assert tq.tq_wait_expired_count() == 0
+
+
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 @pytest.mark.parametrize("chunks", [0, 1, 4096, 4097, 8192, 8193, 16384, 16385])
 @pytest.mark.parametrize("n", [1, 8, 9])
