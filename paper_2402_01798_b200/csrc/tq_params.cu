@@ -16,8 +16,10 @@
 // x = ln(a / g_min), in which a boxed alpha equation costs one exp and one log; it is solved by Newton
 // steps (4 to 8 evaluations); and everything that exists once per level or per trial point (levels, inverse
 // widths, the split of the two-step quantizer) is spread over the lanes of the warp.  Measured on B200 for
-// one worker, uniform, 4 levels / 8 workers, 16-level two-step quantizer: 5.3 us / 30 us, against
-// 21.1 us / 3590 us with one thread per worker, two pow per evaluation and Aitken steps.
+// one worker, uniform, 4 levels / 8 workers, 16-level two-step quantizer: 5.3 us / 24.5 us, against
+// 21.1 us / 3590 us with one thread per worker, two pow per evaluation and Aitken steps.  The two-step quantizer's
+// trial points are the same for every alpha, so their powers k^-gamma are taken once (29.1 us with an exp
+// and a division per point and alpha; on the host, where one thread does all of them, 22 -> 6.6 us per record).
 #include <cmath>
 
 #include "tq.h"
@@ -73,8 +75,6 @@ struct TailModel {
         ln_body = mode == TQ_NONUNIFORM ? log(body) : 0.0;
         ratio = mode == TQ_NONUNIFORM ? cbrt(2.0 * rho * (gamma - 1.0) / body) : 0.0;
     }
-    // mass inside [-a, a]  (Q_U of Section 4.1)
-    TQ_HD double mass_inside(double x) const { return x <= 0.0 ? body * exp(x) : 1.0 - 2.0 * rho * exp((1.0 - gamma) * x); }
     // Integral of p^(1/3) over [0, a] in units of its value at g_min: a / g_min up to g_min, then
     // 1 + ratio * (e^(b x) - 1) / b  (ratio * x for b = 0).
     TQ_HD double cuberoot_integral(double x) const {
@@ -106,14 +106,17 @@ struct TailModel {
 
 constexpr int kSplitGrid = 128;
 constexpr double kSplitFirst = 9.094947017729282e-13, kSplitLnFirst = -27.72588722239781;   // 2^-40: the grid's first point, in place of 0
-// ln k of the grid points of one lane: j = t * kLanes + lane + 1, k = j / 128
+// k^-gamma at the grid points of one lane, k = j / 128 with j = t * kLanes + lane + 1: the same for every alpha, and for every
+// record of one gamma.
 template <class Lanes>
 struct SplitGrid {
-    double ln_k[kSplitGrid / Lanes::kLanes];
-    TQ_HD explicit SplitGrid(const Lanes& lanes, bool wanted) {
-        for (int t = 0; wanted && t < kSplitGrid / Lanes::kLanes; ++t)
-            ln_k[t] = t * Lanes::kLanes + lanes.lane() + 1 < kSplitGrid ? log(static_cast<double>(t * Lanes::kLanes + lanes.lane() + 1) / kSplitGrid)
-                                                                        : kSplitLnFirst;
+    double gamma = NAN, power[kSplitGrid / Lanes::kLanes];
+    TQ_HD static double ln_k(int j) { return j < kSplitGrid ? log(static_cast<double>(j) / kSplitGrid) : kSplitLnFirst; }
+    TQ_HD void prepare(const Lanes& lanes, double gamma_) {
+        if (gamma == gamma_) return;
+        gamma = gamma_;
+#pragma unroll
+        for (int t = 0; t < kSplitGrid / Lanes::kLanes; ++t) power[t] = exp(-gamma * ln_k(t * Lanes::kLanes + lanes.lane() + 1));
     }
 };
 TQ_HD inline int first_bit(uint64_t v) {                   // index of the lowest set bit
@@ -128,13 +131,15 @@ TQ_HD inline int first_bit(uint64_t v) {                   // index of the lowes
 // Q_B^(1/3) = w^(1/3) (1-k)^(2/3) + u^(1/3) k^(2/3),  u = mass inside k a,  w = mass between k a and a.
 struct Split {
     const TailModel& m;
-    double x, a, mass;          // a in units of g_min, mass inside it
-    TQ_HD Split(const TailModel& m_, double x_) : m(m_), x(x_), a(exp(x_)), mass(m_.mass_inside(x_)) {}
-
-    TQ_HD double inner(double k, bool in_body, double ln_k) const {
-        return in_body ? m.body * k * a : 1.0 - 2.0 * m.rho * exp((1.0 - m.gamma) * (x + ln_k));
+    double x, a;                // a in units of g_min
+    double outside, mass; // 2 rho a^(1-gamma), the mass beyond a; the mass inside
+    TQ_HD Split(const TailModel& m_, double x_) : m(m_), x(x_), a(exp(x_)), outside(2.0 * m_.rho * exp((1.0 - m_.gamma) * x_)) {
+        mass = x <= 0.0 ? m.body * a : 1.0 - outside;
     }
-    TQ_HD double inner(double k, bool in_body) const { return inner(k, in_body, in_body ? 0.0 : log(k)); }
+
+    TQ_HD double inner(double k, bool in_body) const {
+        return in_body ? m.body * k * a : 1.0 - 2.0 * m.rho * exp((1.0 - m.gamma) * (x + log(k)));
+    }
     // Negative where Q_B falls with k.  The derivative's sign is that of
     //     w^(2/3) (1-k)^(1/3) (u' k + 2 u)  -  u^(2/3) k^(1/3) (u' (1-k) + 2 w),      u' = du/dk,
     // whose terms are non-negative, so their cubes can be compared: the difference of the cubes has the same zeros.
@@ -145,9 +150,9 @@ struct Split {
         return w * w * (1.0 - k) * (p * p * p) - u * u * k * (q * q * q);
     }
     TQ_HD double slope_at(double k, double ln_k) const {
-        const bool in_body = k * a <= 1.0;
-        const double u = inner(k, in_body, ln_k);
-        return slope(k, u, in_body ? m.body * a : (m.gamma - 1.0) * (1.0 - u) / k);      // 1 - u = 2 rho (k a)^(1-gamma)
+        if (k * a <= 1.0) return slope(k, m.body * k * a, m.body * a);
+        const double beyond = 2.0 * m.rho * exp((1.0 - m.gamma) * x - m.gamma * ln_k);     // mass beyond k a, over k
+        return slope(k, 1.0 - beyond * k, (m.gamma - 1.0) * beyond);
     }
     // Q_B(a, k), and d ln Q_B / dx along the minimum: at fixed k where k is a smooth minimum (its own motion does not
     // change Q_B to first order), along k = 1 / a where it is the kink.
@@ -173,10 +178,17 @@ struct Split {
         *ln_slope = NAN;
         if (x <= 0.0) { *q_best = mass; return 0.5; }            // flat density: Q_B is the same for every k
         uint64_t down[2] = {0, 0};                               // bit j - 1: Q_B falls at k = j / 128 (the end counts as rising)
+        // (k a)^(1-gamma) as a product of powers, unless one of the two could leave the range of a double
+        const bool powers = m.gamma * fmax(x, -kSplitLnFirst) < 600.0;
 #pragma unroll
         for (int t = 0; t < kSplitGrid / n; ++t) {
             const int j = t * n + lanes.lane() + 1;               // the last place is the grid's first point
-            const bool falling = slope_at(j < kSplitGrid ? static_cast<double>(j) / kSplitGrid : kSplitFirst, grid.ln_k[t]) < 0.0;
+            const double k = j < kSplitGrid ? static_cast<double>(j) / kSplitGrid : kSplitFirst;
+            const bool in_body = k * a <= 1.0;
+            double beyond = outside * grid.power[t];            // mass beyond k a, over k
+            if (!powers) beyond = 2.0 * m.rho * exp((1.0 - m.gamma) * x - m.gamma * grid.ln_k(j));
+            const double u = in_body ? m.body * k * a : 1.0 - beyond * k;
+            const bool falling = slope(k, u, in_body ? m.body * a : (m.gamma - 1.0) * beyond) < 0.0;
             down[t * n / 64] |= static_cast<uint64_t>(lanes.ballot(falling)) << (t * n % 64);
         }
         const uint64_t first = down[1] >> 63;
@@ -212,7 +224,7 @@ struct Split {
         double s_lo = NAN, s_hi = NAN;                           // slopes at the ends, where known
 #pragma unroll 1
         for (int it = 0; it < 64 && (hi - lo > 7.62939453125e-6 * hi || !(s_lo < 0.0) || !(s_hi >= 0.0)); ++it) {
-            const double step = (hi - lo) / (n + 1);
+            const double step = (hi - lo) * (1.0 / (n + 1));
             const double k = lo + step * (lanes.lane() + 1), s = slope_at(k, log(k));
             const uint32_t rises = lanes.ballot(!(s < 0.0));
             const int c = rises ? first_bit(rises) : n;            // trial points before the first one where Q_B rises
@@ -307,7 +319,7 @@ TQ_HD inline double solve_alpha(const Lanes& lanes, const SplitGrid<Lanes>& grid
 // Section 4 as a whole for one worker, by the lanes together.  Arguments are already range-checked; `out` is memory
 // that all lanes see.
 template <class Lanes>
-TQ_HD inline tq_status design(const Lanes& lanes, const tq_stats_t* st, uint32_t num_levels, uint32_t bits, uint32_t mode, double gamma,
+TQ_HD inline tq_status design(const Lanes& lanes, SplitGrid<Lanes>& grid, const tq_stats_t* st, uint32_t num_levels, uint32_t bits, uint32_t mode, double gamma,
                               int rule, double alpha_user, tq_params_t* out) {
     const bool first = lanes.lane() == 0;
     if (first) {
@@ -328,7 +340,7 @@ TQ_HD inline tq_status design(const Lanes& lanes, const tq_stats_t* st, uint32_t
     if (!(rho > 0.0) || !(rho < 0.5)) return TQ_ERR_DOMAIN;
     const double g_min = static_cast<double>(st->g_min);
     const TailModel m(rho, gamma, s, mode);
-    const SplitGrid<Lanes> grid(lanes, mode == TQ_BISCALED);
+    if (mode == TQ_BISCALED) grid.prepare(lanes, gamma);
     int iterations = 0;
 
     double alpha;
@@ -415,9 +427,11 @@ params_kernel(const tq_stats_t* __restrict__ stats, uint32_t n, uint32_t num_lev
     if (i >= n) return;              // nothing of this warp reads or writes memory
     const OneWarp lanes;
     tq_params_t* p = &s_p[warp];
+    SplitGrid<OneWarp> grid;
+    if (MODE == TQ_BISCALED && gamma == gamma) grid.prepare(lanes, gamma);      // while the statistics are still being taken
     pdl_wait();
     const tq_stats_t st = stats[i];
-    const tq_status s = design(lanes, &st, num_levels, bits, MODE, gamma, rule, alpha_user, p);
+    const tq_status s = design(lanes, grid, &st, num_levels, bits, MODE, gamma, rule, alpha_user, p);
     __syncwarp();
     if (s != TQ_OK && lanes.lane() == 0) {
         clear(p);
@@ -459,13 +473,17 @@ extern "C" tq_status tq_params(const tq_stats_t* st, uint32_t num_levels, tq_mod
                                tq_alpha_rule rule, double alpha_user, tq_params_t* out) {
     uint32_t bits = 0;
     if (!st || !out || !tq::valid_request(num_levels, mode, rule, &bits)) return TQ_ERR_INVALID_ARG;
-    return tq::design(tq::OneThread(), st, num_levels, bits, mode, gamma, rule, alpha_user, out);
+    tq::SplitGrid<tq::OneThread> grid;
+    return tq::design(tq::OneThread(), grid, st, num_levels, bits, mode, gamma, rule, alpha_user, out);
 }
 
 extern "C" tq_status tq_params_batch(const tq_stats_t* st, uint32_t n_workers, uint32_t num_levels, tq_mode mode,
                                      double gamma, tq_alpha_rule rule, double alpha_user, tq_params_t* out) {
+    uint32_t bits = 0;
     if (!st || !out || n_workers == 0 || n_workers > TQ_MAX_WORKERS) return TQ_ERR_INVALID_ARG;
+    if (!tq::valid_request(num_levels, mode, rule, &bits)) return TQ_ERR_INVALID_ARG;
+    tq::SplitGrid<tq::OneThread> grid;
     for (uint32_t i = 0; i < n_workers; ++i)
-        if (tq_status s = tq_params(st + i, num_levels, mode, gamma, rule, alpha_user, out + i)) return s;
+        if (tq_status s = tq::design(tq::OneThread(), grid, st + i, num_levels, bits, mode, gamma, rule, alpha_user, out + i)) return s;
     return TQ_OK;
 }
