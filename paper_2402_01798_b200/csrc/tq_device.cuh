@@ -243,20 +243,14 @@ __device__ __forceinline__ void blocks_of_job(const TilePlan& plan, const JobPie
 }
 
 // ---- warp / block reductions -----------------------------------------------------------------------
-__device__ __forceinline__ double warp_sum(double v) {
+// lane 0 gets the sum of the first LANES lanes, all when not stated
+template <int LANES = 32, class T>
+__device__ __forceinline__ T warp_sum(T v) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xFFFFFFFFu, v, o);
+    for (int o = LANES / 2; o > 0; o >>= 1) v += __shfl_down_sync(0xFFFFFFFFu, v, o);
     return v;
 }
-__device__ __forceinline__ unsigned long long warp_sum(unsigned long long v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xFFFFFFFFu, v, o);
-    return v;
-}
-__device__ __forceinline__ float warp_max(float v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_down_sync(0xFFFFFFFFu, v, o));
-    return v;
-}
+// of values that are not negative: their bit patterns are in the same order
+__device__ __forceinline__ float warp_max_abs(float v) { return __uint_as_float(__reduce_max_sync(0xFFFFFFFFu, __float_as_uint(v))); }
 
 }  // namespace tq

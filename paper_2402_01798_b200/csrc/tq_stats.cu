@@ -257,30 +257,42 @@ struct BlockFold {
     bool last;
 };
 // Every thread passes its values; thread 0 gets the block's.  MOMENTS / TAILS say which fields are in use (TAILS: how many
-// thresholds).  One block barrier; the shared arrays may be reused after the next one.
-template <int WARPS, bool MOMENTS, int TAILS>
+// thresholds).  One block barrier; the shared arrays may be reused after the next one.  FEW: a thread's counts are what it
+// has seen itself, below 2^24, so a warp's fit 32 bits (the bf16 hinted kernel does without: its main loop then gets other
+// registers and takes 410 us instead of 404 on 124 M x 8).  The warps' values are added by the lanes of the first: with one thread
+// taking them in turn two passes over 1 M x 8 took 0.4 us more, over 3.5 M bf16 x 1 0.3 us.
+template <int WARPS, bool MOMENTS, int TAILS, bool FEW = true>
 __device__ __forceinline__ void block_fold(Partial& p, BlockFold<WARPS>& sh) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    auto count = [](unsigned long long v) -> unsigned long long {
+        if constexpr (FEW) return __reduce_add_sync(0xFFFFFFFFu, static_cast<unsigned>(v));
+        else return warp_sum(v);
+    };
     if constexpr (MOMENTS) {
-        p.sum_abs = warp_sum(p.sum_abs); p.sum_sq = warp_sum(p.sum_sq); p.n_bad = warp_sum(p.n_bad); p.max_abs = warp_max(p.max_abs);
+        p.sum_abs = warp_sum(p.sum_abs); p.sum_sq = warp_sum(p.sum_sq); p.n_bad = count(p.n_bad); p.max_abs = warp_max_abs(p.max_abs);
     }
 #pragma unroll
-    for (int k = 0; k < TAILS; ++k) { p.sum_log2[k] = warp_sum(p.sum_log2[k]); p.n_tail[k] = warp_sum(p.n_tail[k]); }
+    for (int k = 0; k < TAILS; ++k) { p.sum_log2[k] = warp_sum(p.sum_log2[k]); p.n_tail[k] = count(p.n_tail[k]); }
     if (lane == 0) {
         if constexpr (MOMENTS) { sh.d[0][warp] = p.sum_abs; sh.d[1][warp] = p.sum_sq; sh.u[2][warp] = p.n_bad; sh.f[warp] = p.max_abs; }
 #pragma unroll
         for (int k = 0; k < TAILS; ++k) { sh.d[2 + k][warp] = p.sum_log2[k]; sh.u[k][warp] = p.n_tail[k]; }
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (warp == 0) {                                           // lane w: warp w's values
         Partial r{};
-#pragma unroll 1
-        for (int w = 0; w < WARPS; ++w) {
-            if constexpr (MOMENTS) { r.sum_abs += sh.d[0][w]; r.sum_sq += sh.d[1][w]; r.n_bad += sh.u[2][w]; r.max_abs = fmaxf(r.max_abs, sh.f[w]); }
+        if (lane < WARPS) {
+            if constexpr (MOMENTS) { r.sum_abs = sh.d[0][lane]; r.sum_sq = sh.d[1][lane]; r.n_bad = sh.u[2][lane]; r.max_abs = sh.f[lane]; }
 #pragma unroll
-            for (int k = 0; k < TAILS; ++k) { r.sum_log2[k] += sh.d[2 + k][w]; r.n_tail[k] += sh.u[k][w]; }
+            for (int k = 0; k < TAILS; ++k) { r.sum_log2[k] = sh.d[2 + k][lane]; r.n_tail[k] = sh.u[k][lane]; }
         }
-        p = r;
+        if constexpr (MOMENTS) {
+            r.sum_abs = warp_sum<WARPS>(r.sum_abs); r.sum_sq = warp_sum<WARPS>(r.sum_sq); r.n_bad = warp_sum<WARPS>(r.n_bad);
+            r.max_abs = warp_max_abs(r.max_abs);
+        }
+#pragma unroll
+        for (int k = 0; k < TAILS; ++k) { r.sum_log2[k] = warp_sum<WARPS>(r.sum_log2[k]); r.n_tail[k] = warp_sum<WARPS>(r.n_tail[k]); }
+        if (lane == 0) p = r;
     }
 }
 constexpr int kWarps = kThreads / 32;
@@ -395,7 +407,7 @@ __device__ __forceinline__ void fold_records(const Partial* records, uint32_t co
 #pragma unroll
         for (int k = 0; k < TAILS; ++k) { p.sum_log2[k] += q->sum_log2[k]; p.n_tail[k] += q->n_tail[k]; }
     }
-    block_fold<kWarps, MOMENTS, TAILS>(p, sh);
+    block_fold<kWarps, MOMENTS, TAILS, false>(p, sh);
 }
 // The sum of |g| over the records, known to every thread.
 __device__ __forceinline__ double fold_sum_abs(const Partial* records, uint32_t count, BlockFold<kWarps>& sh) {
@@ -482,12 +494,15 @@ __global__ void __launch_bounds__(kThreads, kStatsBlocksPerSm)
 stats_kernel(const void* __restrict__ grad, uint64_t grad_stride, float g_min, float kappa, tq_stats_t* stats, Partial* partials,
              uint32_t* tickets, const __grid_constant__ TilePlan plan) {
     __shared__ BlockFold<kWarps> sh;
-    pdl_wait();
     uint64_t cur = first_tile_of_block(plan, blockIdx.x);
     const uint64_t end = first_tile_of_block(plan, blockIdx.x + 1);
-    while (cur < end) {
-        stats_piece<BF16, PASS>(next_piece(plan, cur, end), plan, grad, grad_stride, g_min, kappa, stats, partials, tickets, sh);
+    JobPiece piece = next_piece(plan, cur, end);               // no block is empty
+    pdl_wait();
+    while (true) {
+        stats_piece<BF16, PASS>(piece, plan, grad, grad_stride, g_min, kappa, stats, partials, tickets, sh);
+        if (cur >= end) break;
         __syncthreads();                                       // the next piece reuses the shared arrays
+        piece = next_piece(plan, cur, end);
     }
 }
 
@@ -526,7 +541,7 @@ __device__ __forceinline__ void hinted_piece(const JobPiece& piece, const void* 
         g.take_exact(exact_sums<BF16>(row, j, 1, 2.0f * t, 1.0f), false, 1, true);
     }
     Partial p = g.partial();
-    block_fold<kWarps, true, 2>(p, sh);
+    block_fold<kWarps, true, 2, !BF16>(p, sh);
     if (threadIdx.x == 0) {
         p.pad = hint[piece.job].level;                           // the finishing launch overwrites the hint
         *record_of_piece(piece, partials) = p;
@@ -549,7 +564,7 @@ __device__ __forceinline__ Partial warp_fold(const Partial* records, uint32_t co
     }
     p.sum_abs = __shfl_sync(0xFFFFFFFFu, warp_sum(p.sum_abs), 0);
     if constexpr (ALL) {
-        p.sum_sq = warp_sum(p.sum_sq); p.n_bad = warp_sum(p.n_bad); p.max_abs = warp_max(p.max_abs);
+        p.sum_sq = warp_sum(p.sum_sq); p.n_bad = warp_sum(p.n_bad); p.max_abs = warp_max_abs(p.max_abs);
 #pragma unroll
         for (int k = 0; k < 2; ++k) { p.sum_log2[k] = warp_sum(p.sum_log2[k]); p.n_tail[k] = warp_sum(p.n_tail[k]); }
     }
@@ -738,7 +753,7 @@ stats_small_kernel(const void* __restrict__ grad, uint64_t grad_stride, float g_
         t.sum_abs = sum_abs;
         t.sum_sq = over_ranks(of_rank(s_moments.sum_sq, from));
         t.n_bad = over_ranks(of_rank(s_moments.n_bad, from));
-        t.max_abs = warp_max(of_rank(s_moments.max_abs, from));
+        t.max_abs = warp_max_abs(of_rank(s_moments.max_abs, from));
         const unsigned long long n = over_ranks(of_rank(s_tail.n_tail[0], from));
         const double sum_log2 = over_ranks(of_rank(s_tail.sum_log2[0], from));
         if (lane == 0) {
