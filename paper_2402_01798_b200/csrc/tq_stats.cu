@@ -572,10 +572,8 @@ __device__ __forceinline__ Partial warp_fold(const Partial* records, uint32_t co
 }
 // Finishes a piece as far as the first launch allows: by one warp, a block's pieces side by side.  The job's first piece writes the
 // record.  Returns the threshold if the piece's tail has to be read again, else 0.
-__device__ __forceinline__ float hinted_finish_piece(const JobPiece& piece, const TilePlan& plan, float kappa, tq_gmin_hint_t* hint_out,
-                                                     tq_stats_t* stats, Partial* partials) {
-    uint32_t count;
-    const Partial* records = records_of_job(plan, piece, partials, count);
+__device__ __forceinline__ float hinted_finish_piece(const JobPiece& piece, float kappa, tq_gmin_hint_t* hint_out,
+                                                     tq_stats_t* stats, Partial* partials, const Partial* records, uint32_t count) {
     const float t = lower_candidate(record_of_piece(piece, partials)->pad);
     const bool first = piece.tile0 == 0;
     // a miss lets other blocks overwrite the tail fields of their records, which are then not used here
@@ -633,19 +631,25 @@ stats_hinted_finish_kernel(const void* __restrict__ grad, uint64_t grad_stride, 
                            Partial* partials, uint32_t* tickets, const __grid_constant__ TilePlan plan) {
     __shared__ BlockFold<kWarps> sh;
     __shared__ float s_again[kWarps];
-    pdl_wait();
-    uint64_t cur = first_tile_of_block(plan, blockIdx.x);
+    const uint32_t warp = threadIdx.x >> 5;
+    uint64_t cur = first_tile_of_block(plan, blockIdx.x), batch;
     const uint64_t end = first_tile_of_block(plan, blockIdx.x + 1);
-    while (cur < end) {                                        // as many pieces at a time as the block has warps
-        const uint64_t batch = cur;
-        const uint32_t warp = threadIdx.x >> 5;
-        uint32_t n = 0;
-        for (; cur < end && n < kWarps; ++n) {
+    JobPiece mine;
+    const Partial* records = nullptr;
+    uint32_t n, count = 0;
+    auto next_batch = [&] {                                    // as many pieces at a time as the block has warps
+        batch = cur;
+        for (n = 0; cur < end && n < kWarps; ++n) {
             const JobPiece piece = next_piece(plan, cur, end);
-            if (n == warp) {
-                const float again = hinted_finish_piece(piece, plan, kappa, hint, stats, partials);
-                if ((threadIdx.x & 31u) == 0) s_again[warp] = again;
-            }
+            if (n == warp) { mine = piece; records = records_of_job(plan, mine, partials, count); }
+        }
+    };
+    next_batch();                                              // which are known before the records are there
+    pdl_wait();
+    while (true) {
+        if (warp < n) {
+            const float again = hinted_finish_piece(mine, kappa, hint, stats, partials, records, count);
+            if ((threadIdx.x & 31u) == 0) s_again[warp] = again;
         }
         __syncthreads();
         uint64_t redo = batch;
@@ -656,7 +660,9 @@ stats_hinted_finish_kernel(const void* __restrict__ grad, uint64_t grad_stride, 
                 __syncthreads();
             }
         }
+        if (cur >= end) break;
         __syncthreads();
+        next_batch();
     }
 }
 
