@@ -1,25 +1,29 @@
 // Client side of Algorithm 1: truncate (Section 3.1, truncation equation), stochastically round onto
 // the codebook (Section 3.1, quantizer equation) and pack b-bit codes, fused in one pass.
 //
-// Work split: persistent blocks walk tiles of 8192 elements of one worker; in a tile a thread owns a
-// run of 32 consecutive elements = four groups of 8.  A group is the unit of randomness: one
-// Philox4x32-10 call (counter = group index, worker) yields 128 bits = eight 16-bit slots, one per
-// element.  A run packs into exactly `bits` 32-bit words, so no thread ever shares a word with
-// another and no shuffles or atomics are needed.
+// Work split: a thread owns a run of 32 consecutive elements = four groups of 8, a tile is one run for each of a block's 256
+// threads.  A group is the unit of randomness: one Philox4x32-10 call (counter = group index, worker) yields 128
+// bits = eight 16-bit slots, one per element.  A run packs into exactly `bits` 32-bit words, so no thread ever shares a
+// word with another and no shuffles or atomics are needed.
+//   Quantizers in kernel parameters (compress_kernel): a grid row per worker, the lookup tables built before the data is
+//   waited for; blocks of table codebooks and of bf16 rows take several tiles.
+//   Quantizers in device memory (compress_kernel_dev): the tiles of all jobs cut into contiguous ranges (TilePlan).
 // HBM traffic per element: 4 (fp32) or 2 (bf16) bytes read, bits/8 bytes written.
 //
-// The kernel is bound by instruction issue, and within that by the half-rate integer/compare pipe,
-// so the per-element arithmetic is arranged to run on the fp32 multiply-add pipe wherever the
-// result is provably the same:
+// What bounds it: fp32 rows come close to HBM (25.6 M x 16, 16 levels: 327 us, 282 at the rate of a plain copy; 4 levels
+// 30 M x 8: 150 us, 156), bf16 rows the multiplier pipe, which Philox's wide multiplies occupy for 9 cycles per 32
+// elements.  So the per-element arithmetic runs on the multiply-add pipes or on the integer / compare pipe,
+// whichever has room, where the result is provably the same:
 //   - floor / int conversion: add 2^23 rounding down, the integer appears in the mantissa;
 //   - threshold T = rint(p * 2^16): one fused multiply-add with 2^23;
 //   - the random slot r as the float 2^23 + r: one byte-permute; [r < T] = sat((2^23 + T) - (2^23 + r)),
 //     a saturating subtract of two exactly representable integers;
 //   - uniform codebook: interval and threshold together as the one integer X = rint(x * 2^16) = k * 2^16 + T,
-//     code = ceil((X - r) / 2^16), with the clamps of x done by saturating multiplies and subtracts;
-//   - codes are kept as small floats and packed by exact multiply-adds (sums stay below 2^24);
+//     code = ceil((X - r) / 2^16), with the clamps of x done by saturating multiplies and a minimum;
+//   - codes are packed by exact multiply-adds, or by products and byte-permutes of integers;
 //   - table offsets are formed as denormal floats whose bit pattern IS the byte offset.
 #include <cmath>
+#include <cstring>
 
 #include "tq_device.cuh"
 #include "tq_launch.h"
@@ -36,7 +40,8 @@ struct WorkerQ {
     float inv_step_l;             // inv_step / L when that quotient is exact and normal, else 0 (uniform mode)
     float inv_2alpha;             // maps [-alpha, alpha] to [0, 1] for the lookup grid
     float cell_scale;             // grid cells M as the denormal M * 2^-149
-    uint32_t cells;               // M
+    uint32_t cells;               // M, 0: no linear grid separates the levels
+    uint32_t log_base, log_cells; // logarithmic grid: 8 * first cell, cells per sign (0: it does not separate them either)
     float levels[TQ_MAX_LEVELS];
     float inv_width[TQ_MAX_LEVELS];
 };
@@ -49,7 +54,7 @@ struct CompressArgs {
 
 // kUniformWide: the uniform codebook through the arithmetic that needs no scaled inverse step (used
 // only when inv_step / L would be subnormal, i.e. alpha beyond about 2^121).
-enum Search { kUniform = 0, kGrid = 1, kBinary = 2, kUniformWide = 3 };
+enum Search { kUniform = 0, kGrid = 1, kBinary = 2, kUniformWide = 3, kLogGrid = 4 };
 __host__ __device__ constexpr bool is_uniform(int search) { return search == kUniform || search == kUniformWide; }
 
 cudaError_t launch_compress_dev(const CompressCall& c);
@@ -178,6 +183,13 @@ __device__ __forceinline__ void pair_plus_alpha(const Raw8<BF16>& g, int h, floa
 // What follows an 8-byte lookup is scalar: to use the two halves of two lookups as pairs takes a move per value, which
 // costs an issue slot and often the multiplier pipe, more than pairing saves (25.6 M x 16, 16 levels: 355 -> 349 us, through
 // device parameters 394 -> 350 us; 250 M x 4, 8 levels 958 -> 861 us).
+__device__ __forceinline__ f32x2 code_cells2(float g0, float g1, float2 gc0, float2 gc1, const char* s_cell, float rf0, float rf1) {
+    const float k0 = __fadd_rn(gc0.y, set_ge(g0, gc0.x)), k1 = __fadd_rn(gc1.y, set_ge(g1, gc1.x));
+    const float2 q0 = *reinterpret_cast<const float2*>(s_cell + __float_as_uint(__fmul_rn(k0, __uint_as_float(8u))));   // bits = 8 * k
+    const float2 q1 = *reinterpret_cast<const float2*>(s_cell + __float_as_uint(__fmul_rn(k1, __uint_as_float(8u))));
+    const float p0 = __fmul_rn(__fsub_rn(g0, q0.x), q0.y), p1 = __fmul_rn(__fsub_rn(g1, q1.x), q1.y);
+    return pair(__fadd_rn(k0, rounds_up(p0, rf0)), __fadd_rn(k1, rounds_up(p1, rf1)));
+}
 __device__ __forceinline__ f32x2 code_grid2(float g0, float g1, f32x2 alpha2, float inv_2alpha, f32x2 cell_scale2,
                                             const char* s_grid, const char* s_cell, float rf0, float rf1) {
     const f32x2 g = pair(g0, g1);
@@ -189,11 +201,30 @@ __device__ __forceinline__ f32x2 code_grid2(float g0, float g1, f32x2 alpha2, fl
     unpair(cell8, c0, c1);
     const float2 gc0 = *reinterpret_cast<const float2*>(s_grid + __float_as_uint(c0));
     const float2 gc1 = *reinterpret_cast<const float2*>(s_grid + __float_as_uint(c1));
-    const float k0 = __fadd_rn(gc0.y, set_ge(g0, gc0.x)), k1 = __fadd_rn(gc1.y, set_ge(g1, gc1.x));
-    const float2 q0 = *reinterpret_cast<const float2*>(s_cell + __float_as_uint(__fmul_rn(k0, __uint_as_float(8u))));   // bits = 8 * k
-    const float2 q1 = *reinterpret_cast<const float2*>(s_cell + __float_as_uint(__fmul_rn(k1, __uint_as_float(8u))));
-    const float p0 = __fmul_rn(__fsub_rn(g0, q0.x), q0.y), p1 = __fmul_rn(__fsub_rn(g1, q1.x), q1.y);
-    return pair(__fadd_rn(k0, rounds_up(p0, rf0)), __fadd_rn(k1, rounds_up(p1, rf1)));
+    return code_cells2(g0, g1, gc0, gc1, s_cell, rf0, rf1);
+}
+
+// The same through a logarithmic grid, whose cells are the exponent and the four highest mantissa bits of |g|, 16 per binade,
+// mirrored for negative values.  Levels 1/16 apart, relatively, are in different cells, however small they are against alpha:
+// this serves the codebooks of heavy tails (exponent 2.5, 16 levels, alpha at 10^4 g_min), whose inner levels are closer
+// than 1/2048 of the range.  Its index arithmetic takes 4.5 operations of the integer / compare pipe per element where the
+// linear grid's floor takes as many of the multiply-add pipes, which have more room, so the linear grid goes first.
+// 25.6 M x 16, 16 levels, exponent 2.5: 575 us by binary search, 366 this way (device parameters 579, 404); where both grids
+// serve, exponent 3: 327 us linear, 379 logarithmic; 250 M x 4, 8 levels 782 and 874.
+// The high half of a float, without its three lowest bits, is 8 times its cell: the byte offset of an 8-byte entry.  Two values
+// at a time in the halves of a word.  t = max(g, -alpha): a NaN takes the lowest cell and code 0.
+__device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {          // with sign replication, unlike __byte_perm
+    uint32_t r; asm("prmt.b32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(sel)); return r;
+}
+__host__ __device__ inline uint32_t log_cell8(uint32_t bits) { return (bits >> 16) & 0x7FF8u; }
+__device__ __forceinline__ f32x2 code_log2(float g0, float g1, float alpha, uint32_t nbase2, uint32_t top2, const char* s_middle,
+                                           const char* s_cell, float rf0, float rf1) {
+    const float t0 = fmaxf(g0, -alpha), t1 = fmaxf(g1, -alpha);
+    const uint32_t y = __byte_perm(__float_as_uint(t0), __float_as_uint(t1), 0x7632u);
+    const uint32_t z = __viaddmin_s16x2_relu(y & 0x7FF87FF8u, nbase2, top2) ^ (prmt(y, y, 0xBB99u) & 0xFFF8FFF8u);
+    const float2 gc0 = *reinterpret_cast<const float2*>(s_middle + static_cast<int>(prmt(z, z, 0x9910u)));
+    const float2 gc1 = *reinterpret_cast<const float2*>(s_middle + static_cast<int>(prmt(z, z, 0xBB32u)));
+    return code_cells2(t0, t1, gc0, gc1, s_cell, rf0, rf1);
 }
 
 // General codebook by branch-free binary search (used when no grid of at most kMaxGridCells cells
@@ -240,8 +271,25 @@ __device__ __forceinline__ uint32_t pack8(const f32x2 (&c)[4]) {
     }
 }
 
+// The cell of a level, counted from the middle (negative below it), and whether the grid's cells separate the levels: each cell
+// holds at most one, and there are at most kMaxGridCells.  A level 0 is left to the search: -0 is below its cell.
+__host__ __device__ inline uint32_t float_bits(float x) {
+#ifdef __CUDA_ARCH__
+    return __float_as_uint(x);
+#else
+    uint32_t b;
+    memcpy(&b, &x, 4);
+    return b;
+#endif
+}
+__host__ __device__ inline uint32_t log_cell(float level, uint32_t base8) {
+    const uint32_t b = float_bits(level), z = (log_cell8(b) - base8) >> 3;
+    return b >> 31 ? ~z : z;
+}
+
 struct RunCtx {
     float alpha, inv_step, top, inv_2alpha, cell_scale;
+    uint32_t log_nbase2, log_top2;             // logarithmic grid; s_grid is then its middle
     UniformQ u;
     const char* s_grid; const char* s_cell; const float* s_search;
 };
@@ -250,6 +298,13 @@ template <int BITS>
 __device__ __forceinline__ UniformQ uniform_q(const WorkerQ& q) {
     constexpr float L = static_cast<float>(1 << BITS);
     return UniformQ{q.inv_step_l, (L - 1.0f) / L, both(L * 65536.0f), both(L * 65536.0f * 7.888609052210118e-31f)};
+}
+
+template <int BITS, int SEARCH>
+__device__ __forceinline__ RunCtx run_ctx(const WorkerQ& q, const float2* s_grid, const float2* s_cell, const float* s_search) {
+    const uint32_t n = SEARCH == kLogGrid ? q.log_cells : 0u;
+    return RunCtx{q.alpha, q.inv_step, q.top, q.inv_2alpha, q.cell_scale, ((0u - q.log_base) & 0xFFFFu) * 0x00010001u, 8u * (n - 1) * 0x00010001u,
+                  uniform_q<BITS>(q), reinterpret_cast<const char*>(s_grid + n), reinterpret_cast<const char*>(s_cell), s_search};
 }
 
 // inv_step / L for the scaled uniform path: exact when the quotient is a normal number (L is a power of
@@ -303,6 +358,8 @@ __device__ __forceinline__ void quantize_run(const Raw8<BF16> (&g)[4], uint32_t*
                     const float g0 = elem<BF16>(g[grp], e), g1 = elem<BF16>(g[grp], e + 1);
                     if constexpr (SEARCH == kGrid)
                         code[h] = code_grid2(g0, g1, alpha2, cx.inv_2alpha, cell_scale2, cx.s_grid, cx.s_cell, rf0, rf1);
+                    else if constexpr (SEARCH == kLogGrid)
+                        code[h] = code_log2(g0, g1, cx.alpha, cx.log_nbase2, cx.log_top2, cx.s_grid, cx.s_cell, rf0, rf1);
                     else code[h] = pair(code_binary<BITS>(g0, cx.alpha, cx.s_search, reinterpret_cast<const float2*>(cx.s_cell), rf0),
                                         code_binary<BITS>(g1, cx.alpha, cx.s_search, reinterpret_cast<const float2*>(cx.s_cell), rf1));
                 }
@@ -385,7 +442,7 @@ __device__ __forceinline__ void compress_last_run(const char* row, uint32_t* pro
 #endif
 
 // Per-block set-up of the shared tables for quantizer q (ends with a block barrier unless the codebook is uniform).
-// s_grid must hold kMaxGridCells + 1 entries when SEARCH == kGrid.
+// s_grid must hold kMaxGridCells + 1 entries when SEARCH is a grid.
 template <int BITS, int SEARCH>
 __device__ __forceinline__ void build_tables(const WorkerQ& q, float2* s_grid, float2* s_cell, float* s_search) {
     constexpr int L = 1 << BITS;
@@ -396,13 +453,15 @@ __device__ __forceinline__ void build_tables(const WorkerQ& q, float2* s_grid, f
         if (threadIdx.x < 2 * TQ_MAX_LEVELS)
             s_search[threadIdx.x] = (threadIdx.x >= 1 && threadIdx.x <= L - 2) ? q.levels[threadIdx.x] : __int_as_float(0x7F800000);
     }
-    if constexpr (SEARCH == kGrid) {
-        // cells of the interior levels l_1 .. l_{s-1} (distinct by the choice of M)
+    if constexpr (SEARCH == kGrid || SEARCH == kLogGrid) {
+        // cells of the interior levels l_1 .. l_{s-1} (distinct, or the grid would not have been chosen)
         uint32_t lc[L];
 #pragma unroll
         for (int j = 1; j <= L - 2; ++j)
-            lc[j] = __float_as_uint(grid_cell(q.levels[j], q.alpha, q.inv_2alpha, q.cell_scale));
-        for (uint32_t c = threadIdx.x; c <= q.cells; c += kThreads) {
+            lc[j] = SEARCH == kGrid ? __float_as_uint(grid_cell(q.levels[j], q.alpha, q.inv_2alpha, q.cell_scale))
+                                    : log_cell(q.levels[j], q.log_base) + q.log_cells;
+        const uint32_t last = SEARCH == kGrid ? q.cells : 2 * q.log_cells - 1;
+        for (uint32_t c = threadIdx.x; c <= last; c += kThreads) {
             float below = 0.0f, boundary = __int_as_float(0x7FC00000);   // NaN: no value compares >= it
 #pragma unroll
             for (int j = 1; j <= L - 2; ++j) {
@@ -421,7 +480,7 @@ __global__ void __launch_bounds__(kThreads, TQ_COMPRESS_MIN_BLOCKS)
 compress_kernel(const void* __restrict__ grad, uint64_t d, uint64_t grad_stride,
                 const __grid_constant__ CompressArgs<N> args, const __grid_constant__ RoundKeys rk,
                 uint32_t first_worker, uint32_t* __restrict__ packed, uint64_t words_stride) {
-    __shared__ __align__(16) float2 s_grid[SEARCH == kGrid ? kMaxGridCells + 1 : 1];
+    __shared__ __align__(16) float2 s_grid[SEARCH == kGrid || SEARCH == kLogGrid ? kMaxGridCells + 1 : 1];
     __shared__ __align__(16) float2 s_cell[TQ_MAX_LEVELS];
     __shared__ float s_search[2 * TQ_MAX_LEVELS];
     constexpr size_t esz = BF16 ? 2 : 4;
@@ -431,8 +490,7 @@ compress_kernel(const void* __restrict__ grad, uint64_t d, uint64_t grad_stride,
     uint32_t* prow = packed + static_cast<uint64_t>(blockIdx.y) * words_stride;
     build_tables<BITS, SEARCH>(q, s_grid, s_cell, s_search);          // from kernel parameters: before the wait
     pdl_wait();
-    const RunCtx cx{q.alpha, q.inv_step, q.top, q.inv_2alpha, q.cell_scale, uniform_q<BITS>(q), reinterpret_cast<const char*>(s_grid),
-                    reinterpret_cast<const char*>(s_cell), s_search};
+    const RunCtx cx = run_ctx<BITS, SEARCH>(q, s_grid, s_cell, s_search);
     const uint64_t whole = (d - 1) >> 5, stride = static_cast<uint64_t>(gridDim.x) * kThreads;     // runs before the row's last one are whole
     for (uint64_t run = static_cast<uint64_t>(blockIdx.x) * kThreads + threadIdx.x; run < whole; run += stride)
         compress_run<BITS, SEARCH, BF16>(row, prow, run, worker, rk, cx);
@@ -459,7 +517,7 @@ __device__ __forceinline__ void load_worker(const tq_params_t& p, WorkerQ& s_q) 
         const float alpha = p.alpha, inv_step = p.inv_step;
         const bool ok = alpha > 0.0f && p.bits == BITS && !(p.flags & TQ_FLAG_INVALID);
         const float inv_2alpha = ok ? __fdiv_rn(1.0f, __fmul_rn(2.0f, alpha)) : 0.0f;
-        uint32_t cells = 0;
+        uint32_t cells = 0, log_base = 0, log_cells = 0;
         if constexpr (NONUNIFORM) {      // choose_cells, a lane for each interior level
             constexpr int s = (1 << BITS) - 1;
             const bool mine = lane >= 2 && lane <= s - 1;
@@ -469,6 +527,16 @@ __device__ __forceinline__ void load_worker(const tq_params_t& p, WorkerQ& s_q) 
             const bool distinct = !__any_sync(0xFFFFFFFFu, mine && cell <= prev) && ok && inv_2alpha <= 3.402823466e38f;
             const uint32_t m = drop >= 31 ? 0u : static_cast<uint32_t>(kMaxGridCells) >> drop;
             if (distinct) cells = m < static_cast<uint32_t>(kMinGridCells) ? kMinGridCells : m;
+            else if (ok) {               // choose_log_grid
+                const bool interior = lane >= 1 && lane <= s - 1;
+                const float level = lane < TQ_MAX_LEVELS ? s_q.levels[lane] : 0.0f;
+                const uint32_t c8 = log_cell8(__float_as_uint(level));
+                log_base = __reduce_min_sync(0xFFFFFFFFu, interior ? c8 : 0x7FF8u);
+                const uint32_t n = ((__reduce_max_sync(0xFFFFFFFFu, interior ? c8 : 0u) - log_base) >> 3) + 1;
+                const int lc = static_cast<int>(log_cell(level, log_base)), below = __shfl_up_sync(0xFFFFFFFFu, lc, 1);
+                const bool bad = (interior && level == 0.0f) || (mine && lc <= below) || n > kMaxGridCells / 2;
+                if (!__any_sync(0xFFFFFFFFu, bad)) log_cells = n;
+            }
         }
         if (lane == 0) {
             s_q.alpha = ok ? alpha : 0.0f;
@@ -476,7 +544,7 @@ __device__ __forceinline__ void load_worker(const tq_params_t& p, WorkerQ& s_q) 
             s_q.inv_step_l = scaled_inv_step(inv_step, 1u << BITS);
             s_q.top = static_cast<float>((1 << BITS) - 1);
             s_q.inv_2alpha = inv_2alpha;
-            s_q.cells = cells;
+            s_q.cells = cells; s_q.log_base = log_base; s_q.log_cells = log_cells;
             s_q.cell_scale = __uint_as_float(cells);
         }
     }
@@ -502,8 +570,7 @@ __device__ __forceinline__ void compress_piece(State& sh, const void* __restrict
                                                const TilePlan& plan) {
     constexpr size_t esz = BF16 ? 2 : 4;
     build_tables<BITS, SEARCH>(sh.q, sh.grid, sh.cell, sh.search);
-    const RunCtx cx{sh.q.alpha, sh.q.inv_step, sh.q.top, sh.q.inv_2alpha, sh.q.cell_scale, uniform_q<BITS>(sh.q),
-                    reinterpret_cast<const char*>(sh.grid), reinterpret_cast<const char*>(sh.cell), sh.search};
+    const RunCtx cx = run_ctx<BITS, SEARCH>(sh.q, sh.grid, sh.cell, sh.search);
     const char* row = static_cast<const char*>(grad) + (static_cast<uint64_t>(sh.piece.worker) * grad_stride + sh.piece.off) * esz;
     uint32_t* prow = packed + static_cast<uint64_t>(sh.piece.worker) * words_stride + plan.segs.woff[sh.piece.seg];
     const uint32_t worker = first_worker + sh.piece.worker;
@@ -560,6 +627,8 @@ compress_kernel_dev(const void* __restrict__ grad, uint64_t grad_stride, const t
             const uint64_t words_out = (((sh.piece.d * BITS + 31) >> 5) + 3) & ~static_cast<uint64_t>(3);
             const uint64_t w1 = sh.piece.last ? words_out : sh.piece.tile1 * kThreads * BITS;
             for (uint64_t w = sh.piece.tile0 * kThreads * BITS + threadIdx.x; w < w1; w += kThreads) prow[w] = 0u;
+        } else if (NONUNIFORM && sh.q.cells == 0 && sh.q.log_cells != 0) {
+            compress_piece_rare<BITS, kLogGrid, BF16>(sh, grad, grad_stride, rk, first_worker, packed, words_stride, plan);
         } else if (NONUNIFORM && sh.q.cells == 0) {
             compress_piece_rare<BITS, kBinary, BF16>(sh, grad, grad_stride, rk, first_worker, packed, words_stride, plan);
         } else if (!NONUNIFORM && sh.q.inv_step_l == 0.0f) {
@@ -592,6 +661,23 @@ static uint32_t choose_cells(const tq_params_t& p, float inv_2alpha) {
     }
     const uint32_t m = drop >= 31 ? 0u : static_cast<uint32_t>(kMaxGridCells) >> drop;
     return m < static_cast<uint32_t>(kMinGridCells) ? kMinGridCells : m;
+}
+
+// The logarithmic grid of a codebook: 8 * its first cell, and its cells per sign, 0 if it does not separate the levels.
+static uint32_t choose_log_grid(const tq_params_t& p, uint32_t* base8) {
+    const int s = static_cast<int>(p.num_levels) - 1;
+    uint32_t lo = 0x7FF8u, hi = 0;
+    for (int j = 1; j <= s - 1; ++j) {
+        const uint32_t c8 = log_cell8(float_bits(p.levels[j]));
+        lo = c8 < lo ? c8 : lo;
+        hi = c8 > hi ? c8 : hi;
+        if (p.levels[j] == 0.0f) return 0;
+    }
+    *base8 = lo;
+    for (int j = 2; j <= s - 1; ++j)
+        if (static_cast<int>(log_cell(p.levels[j], lo)) <= static_cast<int>(log_cell(p.levels[j - 1], lo))) return 0;
+    const uint32_t n = s > 1 ? ((hi - lo) >> 3) + 1 : 0;
+    return n > kMaxGridCells / 2 ? 0 : n;
 }
 
 // Shares per resident block when each would get `tiles` tiles as one share: the hardware hands the later ones to the blocks
@@ -631,6 +717,7 @@ static cudaError_t dispatch(const CompressCall& c, const CompressArgs<TQ_MAX_WOR
         if (few) return c.bf16 ? launch<BITS, kGrid, true>(c, f, grid) : launch<BITS, kGrid, false>(c, f, grid);
         return c.bf16 ? launch<BITS, kGrid, true>(c, a, grid) : launch<BITS, kGrid, false>(c, a, grid);
     }
+    if (search == kLogGrid) return c.bf16 ? launch<BITS, kLogGrid, true>(c, a, grid) : launch<BITS, kLogGrid, false>(c, a, grid);
     if (search == kBinary) return c.bf16 ? launch<BITS, kBinary, true>(c, a, grid) : launch<BITS, kBinary, false>(c, a, grid);
     if (search == kUniformWide) return c.bf16 ? launch<BITS, kUniformWide, true>(c, a, grid) : launch<BITS, kUniformWide, false>(c, a, grid);
     if (few) return c.bf16 ? launch<BITS, kUniform, true>(c, f, grid) : launch<BITS, kUniform, false>(c, f, grid);
@@ -654,14 +741,17 @@ cudaError_t launch_compress(const CompressCall& c) {
         q.inv_2alpha = 1.0f / (2.0f * p.alpha);
         q.inv_step_l = scaled_inv_step(p.inv_step, p.num_levels);
         if (!c.nonuniform && q.inv_step_l == 0.0f) search = kUniformWide;
-        q.cells = 0; q.cell_scale = 0.0f;
+        q.cells = q.log_base = q.log_cells = 0; q.cell_scale = 0.0f;
         for (int k = 0; k < TQ_MAX_LEVELS; ++k) { q.levels[k] = p.levels[k]; q.inv_width[k] = p.inv_width[k]; }
         if (c.nonuniform) {
             q.cells = choose_cells(p, q.inv_2alpha);
             q.cell_scale = std::ldexp(static_cast<float>(q.cells), -149);
-            if (q.cells == 0 || !std::isfinite(q.inv_2alpha)) search = kBinary;
+            if (q.cells == 0 || !std::isfinite(q.inv_2alpha)) search = kLogGrid;
         }
     }
+    if (search == kLogGrid)                                  // one form for the launch
+        for (uint32_t i = 0; i < c.n_workers; ++i)
+            if ((args.q[i].log_cells = choose_log_grid(c.params[i], &args.q[i].log_base)) == 0) search = kBinary;
     // uniform fp32 rows have no per-block set-up worth sharing: one block per tile (30 M x 8, 16 levels: 156 us, in shares 166);
     // bf16 ones, bound by instructions, do better in shares (124 M x 8, 4 levels: 543 us by tiles, 506 in shares)
     const dim3 grid = compress_grid(c.d, c.n_workers, !is_uniform(search) || c.bf16);

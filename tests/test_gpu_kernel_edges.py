@@ -170,3 +170,32 @@ def test_statistics_of_short_rows(tq, orc, dtype, chunks, n):
             assert math.isclose(r.g_min, o.g_min, rel_tol=2e-6)
             ref = orc.stats(x, g_min=r.g_min) if r.g_min > 0 else o
             assert r.n_tail == ref.n_tail and math.isclose(r.sum_log_tail, ref.sum_log_tail, rel_tol=5e-6, abs_tol=1e-9)
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("L,alpha,inner", [(16, 1.0, 2.0 ** -20), (16, 3e-3, 3e-3 * 2.0 ** -63), (8, 5e30, 1e25), (8, 1e-30, 1e-37), (16, 0.37, 0.37 * 1.07 ** -6)])
+def test_codebooks_of_the_logarithmic_grid(tq, orc, dtype, L, alpha, inner):
+    """Levels in geometric steps from `inner` to alpha, of both signs and on one side only: too close together for 2048 equal cells
+    (but for the last, whose neighbours are 1.07 apart), up to 64 binades deep, large and small.  Values at every level and one
+    ulp beside it, at the edges of cells, NaN, infinities, zeros.  Codes equal the oracle's, parameters on the host and on the device."""
+    f = np.float32
+    mags = np.geomspace(inner, alpha, L // 2).astype(f)
+    books = [np.concatenate([-mags[::-1], mags]), np.concatenate([[-f(alpha)], np.geomspace(inner, alpha, L - 1).astype(f)])]
+    d = 20_003
+    for lv in books:
+        lv[-1] = -lv[0]
+        p = tq.tq_params_from_levels([float(x) for x in lv])
+        r = np.random.default_rng(L)
+        at = np.concatenate([lv, np.nextafter(lv, f(np.inf)), np.nextafter(lv, f(-np.inf)), mags.view(np.uint32).__and__(0xFFF80000).view(f),
+                             np.array([0.0, -0.0, np.nan, -np.nan, np.inf, -np.inf, 1e-45, -1e-45, 3e38, -3e38], f)]).astype(f)
+        x = (np.exp2(r.uniform(np.log2(float(inner)) - 3, np.log2(alpha) + 2, d)) * r.choice([-1.0, 1.0], d)).astype(f)
+        x[: 8 * at.size] = np.tile(at, 8)
+        g = torch.zeros(2, (d + 31) // 32 * 32, dtype=dtype, device="cuda")
+        g[:, :d] = torch.from_numpy(x).to(dtype).cuda()
+        host = g[:, :d].float().cpu().numpy()
+        got = tq.tq_compress(g, [p, p], seed=11, first_worker=3, d=d).cpu().numpy().view(np.uint32)
+        raw = torch.frombuffer(bytearray(bytes(p) * 2), dtype=torch.uint8).cuda()
+        dev = tq.tq_compress_device_params(g, raw, L, tq.NONUNIFORM, seed=11, first_worker=3, d=d).cpu().numpy().view(np.uint32)
+        for i in range(2):
+            want = orc.compress(host[i], _oracle_params(orc, p), 11, 3 + i)
+            assert np.array_equal(got[i], want) and np.array_equal(dev[i], want)
