@@ -201,13 +201,14 @@ __device__ __forceinline__ void finish_units(f32x2 (&acc)[U][Unit<BITS>::kElems 
     }
 }
 
-// Copies the N codebooks (already multiplied by w_i when weights are given) into shared memory.
+// Copies the N codebooks (already multiplied by w_i when weights are given) into shared memory; the block's first `idle` threads do not
+// take part.
 __device__ __forceinline__ void fill_tables(float* s_tab, uint32_t n, const DecompressArgs& args, const DeviceTables& dt,
-                                            uint32_t pstride = 1, uint32_t poff = 0) {
+                                            uint32_t pstride = 1, uint32_t poff = 0, uint32_t idle = 0) {
     // lanes read different words, which the constant bank would serve one after the other: read through the generic window
     uint64_t table = reinterpret_cast<uint64_t>(&args.table[0][0]);
     asm volatile("" : "+l"(table));
-    for (uint32_t t = threadIdx.x; t < n * TQ_MAX_LEVELS; t += kDecThreads) {
+    for (uint32_t t = threadIdx.x - idle; t < n * TQ_MAX_LEVELS; t += kDecThreads - idle) {
         const uint32_t i = t / TQ_MAX_LEVELS, k = t % TQ_MAX_LEVELS;
         float v;
         if (dt.params_dev) {     // same rounded product w_i * l as the host forms for the by-value table
@@ -393,15 +394,22 @@ decompress_bulk_kernel(const __grid_constant__ RowTable rt, uint64_t words_row, 
             bulk_load(stage0 + (st * kGroup + b) * kSeg, reinterpret_cast<const char*>(rt.row[i0 + b]) + tile_off, seg_bytes, bar);
     };
 
-    if (threadIdx.x == 0) {
-        for (int st = 0; st < S; ++st) mbar_init(bar0 + 8 * st, 1);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    // The first warp sends the first copies off as soon as the rows may be read; the others fill in the codebooks meanwhile, before
+    // they wait where these are kernel parameters.  (Codebooks first, by all, then the copies: 250 M x 4, 3 bits 280 us instead of
+    // 274, 50 M x 4 61.9 instead of 59.7, 124 M x 8, 2 bits 162.4 instead of 159.5.)
+    if (threadIdx.x < 32) {
+        if (threadIdx.x == 0) {
+            for (int st = 0; st < S; ++st) mbar_init(bar0 + 8 * st, 1);
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        }
+        pdl_wait();
+        if (threadIdx.x == 0)
+            for (uint32_t q = 0; q < S && q < n_steps; ++q) issue(q);
+    } else {
+        if (!dt.params_dev) fill_tables(s_tab, n, args, dt, 1, 0, 32);
+        pdl_wait();
+        if (dt.params_dev) fill_tables(s_tab, n, args, dt, pstride, poff, 32);
     }
-    if (!dt.params_dev) fill_tables(s_tab, n, args, dt);            // from kernel parameters: before the wait
-    pdl_wait();
-    if (threadIdx.x == 0)
-        for (uint32_t q = 0; q < S && q < n_steps; ++q) issue(q);
-    if (dt.params_dev) fill_tables(s_tab, n, args, dt, pstride, poff);
     __syncthreads();          // barriers initialised and codebooks in place for every thread
     const char* tab_bytes = reinterpret_cast<const char*>(s_tab);
 
