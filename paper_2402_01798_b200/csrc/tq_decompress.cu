@@ -489,7 +489,9 @@ static cudaError_t launch_bulk(const DecompressCall& c, const RowTable& rt, cons
                                                    cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
         if (e != cudaSuccess) return e;
     }
-    return launch_kernel(decompress_bulk_kernel<BITS, APPLY, U>, dim3(static_cast<unsigned>(tiles)), kDecThreads, smem, c.stream, rt, c.words_valid,
+    // fewer blocks than fit at a time: see launch_kernel (rounds, early / late: 3 M x 64 336 / 325 us, 2 M x 16 72.4 / 68.1, 2 M x 8 56.2 / 53.9)
+    const Start start = tiles < static_cast<uint64_t>(sm_count()) * TQ_DECOMPRESS_BULK_BLOCKS ? Start::kLate : Start::kEarly;
+    return launch_kernel(start, decompress_bulk_kernel<BITS, APPLY, U>, dim3(static_cast<unsigned>(tiles)), kDecThreads, smem, c.stream, rt, c.words_valid,
                          c.n_workers, c.d, args, dt, scale, divide, ap, c.out, st);
 }
 
@@ -516,7 +518,14 @@ static cudaError_t launch_apply(const DecompressCall& c, const RowTable& rt, con
     if (tiles > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
     if (tiles < kTilesForBulk) {
         constexpr uint64_t kPerBlock = static_cast<uint64_t>(kDecThreads) * E;
-        return launch_kernel(decompress_kernel<BITS, APPLY>, dim3(static_cast<unsigned>((c.d + kPerBlock - 1) / kPerBlock)), kDecThreads, 0, c.stream, rt,
+        const uint64_t blocks = (c.d + kPerBlock - 1) / kPerBlock;
+        // At most half of what fits at a time, with a long walk over the workers: see launch_kernel.  Rounds, early / late start:
+        // 250 k x 64 63.1 / 49.6 us, 50 k x 64 37.9 / 24.9, 250 k x 16 29.6 / 26.6; behind short compressions there is room
+        // everywhere, and only codebooks in device memory, which an early start cannot read, leave it no advantage: 20 k x 64 29.6 /
+        // 22.8, with the codebooks in kernel parameters 16.1 / 17.9; 50 k x 16 20.0 / 20.1 and 13.0 / 13.7; 1 M x 16 (977 blocks) 55.0 / 55.3.
+        const bool late = c.n_workers >= 16 && blocks <= static_cast<uint64_t>(sm_count()) * (TQ_DECOMPRESS_MIN_BLOCKS / 2) &&
+                          (c.n_workers * c.d >= (1u << 21) || (c.params_dev && c.n_workers >= 32));
+        return launch_kernel(late ? Start::kLate : Start::kEarly, decompress_kernel<BITS, APPLY>, dim3(static_cast<unsigned>(blocks)), kDecThreads, 0, c.stream, rt,
                              c.words_valid, c.n_workers, c.d, args, dt, scale, divide, ap, c.out);
     }
     if constexpr (APPLY && U > 1) {
