@@ -795,6 +795,12 @@ static void plan_stats(const StatsCall& c, uint32_t n_jobs, TilePlan* plan) {
     if (c.bf16 && plan->per_block >= 64 && 3 * resident <= room) plan_tiles(plan, c.segs, c.d, c.n_workers, kThreads * kChunkBytes / 2, 3 * resident);
 }
 
+// Equal rows in a whole number of blocks each may leave some places empty: see launch_kernel.  Rounds of 3 M x 64, 576 blocks of 81
+// tiles, early / late: hinted 336 / 315 us, two passes 461 / 416; of 1 M x 64, 27 tiles, two passes 152.8 / 153.4.
+static Start start_of(const TilePlan& plan) {
+    return plan.blocks < static_cast<uint32_t>(sm_count()) * kStatsBlocksPerSm && plan.per_block >= 48 ? Start::kLate : Start::kEarly;
+}
+
 template <int RULE, int CHUNKS>
 static cudaError_t launch_clusters(const StatsCall& c, uint32_t n_jobs, tq_gmin_hint_t* hint, const SegTable& segs) {
     return launch_kernel(c.bf16 ? stats_small_kernel<true, RULE, CHUNKS> : stats_small_kernel<false, RULE, CHUNKS>, dim3(n_jobs * kCluster), kSmallThreads,
@@ -827,17 +833,17 @@ cudaError_t launch_stats(const StatsCall& c, int* launches) {
     uint32_t* tickets = reinterpret_cast<uint32_t*>(static_cast<char*>(c.workspace) + tickets_offset(n_jobs));
     static thread_local TilePlan plan;
     plan_stats(c, n_jobs, &plan);
-    auto launch = [&](auto kernel) {
-        e = launch_kernel(kernel, dim3(plan.blocks), kThreads, 0, c.stream, c.grad, c.grad_stride, c.g_min, c.kappa, c.stats, partials, tickets, plan);
+    auto launch = [&](auto kernel, Start start) {
+        e = launch_kernel(start, kernel, dim3(plan.blocks), kThreads, 0, c.stream, c.grad, c.grad_stride, c.g_min, c.kappa, c.stats, partials, tickets, plan);
         *launches += e == cudaSuccess ? 1 : 0;
         return e;
     };
     if (c.g_min > 0.0f) {
         if ((e = cudaMemsetAsync(tickets, 0, static_cast<size_t>(n_jobs) * sizeof(uint32_t), c.stream)) != cudaSuccess) return e;
-        return launch(c.bf16 ? stats_kernel<true, kBoth> : stats_kernel<false, kBoth>);
+        return launch(c.bf16 ? stats_kernel<true, kBoth> : stats_kernel<false, kBoth>, start_of(plan));
     }
-    if (launch(c.bf16 ? stats_kernel<true, kMoments> : stats_kernel<false, kMoments>) != cudaSuccess) return e;
-    return launch(c.bf16 ? stats_kernel<true, kTail> : stats_kernel<false, kTail>);
+    if (launch(c.bf16 ? stats_kernel<true, kMoments> : stats_kernel<false, kMoments>, start_of(plan)) != cudaSuccess) return e;
+    return launch(c.bf16 ? stats_kernel<true, kTail> : stats_kernel<false, kTail>, Start::kEarly);
 }
 
 cudaError_t launch_stats_hinted(const StatsCall& c, tq_gmin_hint_t* hint, int* launches) {
@@ -849,9 +855,7 @@ cudaError_t launch_stats_hinted(const StatsCall& c, tq_gmin_hint_t* hint, int* l
     uint32_t* tickets = reinterpret_cast<uint32_t*>(static_cast<char*>(c.workspace) + tickets_offset(n_jobs));
     static thread_local TilePlan plan;            // the same plan for both launches: same summation order
     plan_stats(c, n_jobs, &plan);
-    // rows that are not cut into whole blocks leave some places empty: see launch_kernel (rounds of 3 M x 64, 576 blocks: early 336, late 315 us)
-    const Start start = plan.blocks < static_cast<uint32_t>(sm_count()) * kStatsBlocksPerSm ? Start::kLate : Start::kEarly;
-    e = launch_kernel(start, c.bf16 ? stats_hinted_kernel<true> : stats_hinted_kernel<false>, dim3(plan.blocks), kThreads, 0, c.stream, c.grad,
+    e = launch_kernel(start_of(plan), c.bf16 ? stats_hinted_kernel<true> : stats_hinted_kernel<false>, dim3(plan.blocks), kThreads, 0, c.stream, c.grad,
                       c.grad_stride, static_cast<const tq_gmin_hint_t*>(hint), partials, tickets, plan);
     if (e != cudaSuccess) return e;
     *launches = 1;
