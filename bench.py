@@ -358,7 +358,7 @@ def measure_round(args, tq, w, g, stride, dev, local_rank, world, steps, warmup,
     value = whole_job_gbs(world, in_bytes, ms_per_step)
 
     # per-kernel durations inside the timed region (CUDA events on the launching stream)
-    t_stats = stats_t([e[0].elapsed_time(e[1]) for e in evs])       # two launches
+    t_stats = stats_t([e[0].elapsed_time(e[1]) for e in evs])
     t_params = stats_t([e[1].elapsed_time(e[2]) for e in evs])      # device kernel, or copy + sync + host design
     t_comp = stats_t([e[2].elapsed_time(e[3]) for e in evs])
     t_dec = stats_t([e[3].elapsed_time(e[4]) for e in evs])

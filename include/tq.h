@@ -138,9 +138,10 @@ typedef struct {
  * power-of-two threshold can be tried before the mean is known: the pass gathers the tail count and
  * sum ln|g| for the two powers of two nearest to hint->level (the previous round's kappa * mean|g|),
  * and when the finished mean selects one of them the record is complete after reading the data once.
- * When it selects neither (first round; mean moved by more than a factor of about 1.4 to 2) a second
- * kernel, which is always enqueued and otherwise returns at once, redoes the tail sums for the right
- * threshold: the record is the same, bit for bit, either way, and the host never has to look.
+ * When it selects neither (first round; mean moved by more than a factor of about 1.4 to 2) the
+ * launch that finishes the record redoes the tail sums for the right threshold (short rows are kept on
+ * the chip until the threshold is known, and need no second reading): the record is the same, bit for
+ * bit, either way, and the host never has to look.
  *   hint_dev     [n_workers] tq_gmin_hint_t, device memory, 8-byte aligned, in/out (updated by every call).
  *   kappa        > 0.
  *   other arguments, the record's fields, workspace rules and errors as for tq_stats; stats_dev[i].g_min
@@ -362,7 +363,7 @@ uint64_t tq_kernel_launches(void); /* kernels launched by this library in this p
  * copies and waits for them on shared-memory barriers; every such wait gives up after a fixed number
  * of polls.  While barriers remain in the tile's loop the whole block takes the decision (it stores nothing for
  * the tile and counts itself once); in the last three steps of a tile there is no barrier left, and a thread whose
- * wait runs out there drops its own 32 outputs and counts itself, so a tile can then be partly stored.
+ * wait runs out there drops its own outputs and counts itself, so a tile can then be partly stored.
  * *count_host receives the number of such give-ups on the current device since the library was loaded
  * (0 in a healthy run: a non-zero value means the outputs of the affected launch are incomplete).
  * Synchronises the device.  Returns TQ_ERR_INVALID_ARG for a null pointer, TQ_ERR_CUDA if the read fails.
