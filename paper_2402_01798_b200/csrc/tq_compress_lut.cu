@@ -153,10 +153,10 @@ __device__ __forceinline__ void load_piece(const char* row, uint64_t piece, uint
                      : "l"(row + piece * (2 * E) + 32 * i));
 }
 
-#ifndef TQ_LUT_MIN_BLOCKS
-#define TQ_LUT_MIN_BLOCKS 3
-#endif
-constexpr int kLutThreads = kThreads;
+// One block per SM.  80 registers a thread allow 24 warps, as one block of 768 threads, two of 384 or three of 256: with one there is
+// one table to build (124 M x 8 in equal shares, 16 levels, host / device parameters: 604 / 613 us, 603 / 613, 622 / 624; 15 M x 4: 42.6 / 47.0, 44.2 /
+// 49.1, 45.5 / 51.1).  28 warps spill at 72 registers: 639 / 684.
+constexpr int kLutThreads = 768;
 
 // A block's share of one row: build the table for quantizer q (n_entries per sign), then quantize.
 template <int BITS, bool WAIT>
@@ -220,7 +220,7 @@ __device__ __forceinline__ void lut_block(const LutWorker& q, uint32_t n_entries
 
 // Quantizers passed by value (host-side tq_params); the host has chosen the window.
 template <int BITS>
-__global__ void __launch_bounds__(kLutThreads, TQ_LUT_MIN_BLOCKS)
+__global__ void __launch_bounds__(kLutThreads, 1)
 compress_lut_kernel(const void* __restrict__ grad, uint64_t d, uint64_t grad_stride, const __grid_constant__ LutArgs args,
                     const __grid_constant__ RoundKeys rk, uint32_t n_entries, uint32_t first_worker,
                     uint32_t* __restrict__ packed, uint64_t words_stride, uint64_t words_out) {
@@ -234,7 +234,7 @@ compress_lut_kernel(const void* __restrict__ grad, uint64_t d, uint64_t grad_str
 // table form serves its row, with the largest window; rows it does not serve are left to the element-wise
 // device-parameter kernels, which are launched after this one and skip the rows served here.
 template <int BITS>
-__global__ void __launch_bounds__(kLutThreads, TQ_LUT_MIN_BLOCKS)
+__global__ void __launch_bounds__(kLutThreads, 1)
 compress_lut_kernel_dev(const void* __restrict__ grad, uint64_t d, uint64_t grad_stride, const tq_params_t* __restrict__ params,
                         const __grid_constant__ RoundKeys rk, uint32_t first_worker, uint32_t* __restrict__ packed,
                         uint64_t words_stride, uint64_t words_out) {
@@ -285,60 +285,61 @@ static uint32_t entries_needed(const tq_params_t& p, uint32_t top) {
     return hi * kLutBinade;
 }
 
-static uint64_t lut_blocks_per_worker(uint64_t d, uint32_t n_workers, int per_sm, int pieces_elems);
-
 template <int BITS>
-static cudaError_t launch_lut(const CompressCall& c, const LutArgs& args, uint32_t n_entries) {
+static cudaError_t launch_lut(const CompressCall& c, const LutArgs& args, uint32_t n_entries, uint32_t per_worker) {
     const int smem = static_cast<int>((kLutMaxEntries + n_entries) * sizeof(float));
     cudaError_t e = cudaFuncSetAttribute(compress_lut_kernel<BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, compress_lut_kernel<BITS>, kLutThreads, smem);
-    if (e != cudaSuccess) return e;
-    const uint64_t per_worker = lut_blocks_per_worker(c.d, c.n_workers, per_sm, Piece<BITS>::kElems);
-    return launch_kernel(compress_lut_kernel<BITS>, dim3(static_cast<unsigned>(per_worker), c.n_workers), kLutThreads, smem, c.stream, c.grad, c.d,
+    return launch_kernel(compress_lut_kernel<BITS>, dim3(per_worker, c.n_workers), kLutThreads, smem, c.stream, c.grad, c.d,
                          c.grad_stride, args, round_keys(c.seed), n_entries, c.first_worker, c.packed, c.words_stride, c.words_out);
 }
 
 
-static uint64_t lut_blocks_per_worker(uint64_t d, uint32_t n_workers, int per_sm, int pieces_elems) {
-    const uint64_t tiles = (d / pieces_elems + kLutThreads - 1) / kLutThreads + 1;
-    uint64_t per_worker = static_cast<uint64_t>(sm_count()) * (per_sm < 1 ? 1 : per_sm) / n_workers;      // rounded down: one wave holds the grid
-    // two shares per resident block even out the SMs where a share repays its table (124 M x 8: 637 -> 619 us; 5 M x 8, 90 000
-    // elements a block: 31.6 -> 33.9 us)
-    if (per_worker > 0 && d / per_worker >= (1u << 19)) per_worker *= 2;
-    if (per_worker > tiles) per_worker = tiles;
-    return per_worker < 1 ? 1 : per_worker;
+// Blocks per row, and what the longest chain of blocks costs with them, in elements that a block quantizes in that time: a table costs
+// as much as 40000 (3.5 us), the waves follow one another, and SMs differ by 3 % of a share, which more and shorter shares
+// even out (124 M x 8, 36 / 55 / 74 blocks a row: 604 / 608 / 611 us); rows that do not divide the SMs waste less in several (37 blocks
+// a row, 296 in all, two for each SM: 591 us).
+static uint64_t lut_plan(uint64_t d, uint32_t n_workers, uint32_t* per_worker) {
+    const uint64_t sms = static_cast<uint64_t>(sm_count());
+    uint64_t best = ~0ull;
+    for (uint64_t shares = 1; shares <= 8; ++shares) {
+        uint64_t p = sms * shares / n_workers;
+        if (p == 0) p = 1;
+        const uint64_t waves = (p * n_workers + sms - 1) / sms, share = d / p + 1, cost = waves * (40000 + share) + share / 32;
+        if (cost < best) { best = cost; *per_worker = static_cast<uint32_t>(p); }
+    }
+    return best;
 }
 
 template <int BITS>
-static cudaError_t launch_lut_dev(const CompressCall& c) {
+static cudaError_t launch_lut_dev(const CompressCall& c, uint32_t per_worker) {
     const int smem = static_cast<int>(2 * kLutMaxEntries * sizeof(float));
     cudaError_t e = cudaFuncSetAttribute(compress_lut_kernel_dev<BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, compress_lut_kernel_dev<BITS>, kLutThreads, smem);
-    if (e != cudaSuccess) return e;
-    const uint64_t per_worker = lut_blocks_per_worker(c.d, c.n_workers, per_sm, Piece<BITS>::kElems);
-    return launch_kernel(compress_lut_kernel_dev<BITS>, dim3(static_cast<unsigned>(per_worker), c.n_workers), kLutThreads, smem, c.stream, c.grad,
+    return launch_kernel(compress_lut_kernel_dev<BITS>, dim3(per_worker, c.n_workers), kLutThreads, smem, c.stream, c.grad,
                          c.d, c.grad_stride, c.params_dev, round_keys(c.seed), c.first_worker, c.packed, c.words_stride, c.words_out);
 }
 
-// Calls with fewer elements (all rows together) keep the element-wise kernels: each of the 444 resident blocks builds a
-// table of some 20 to 40 binades, a few us each (table / element-wise, device parameters: 10 M 19.5 / 15.4 us, 24 M 29.7 / 27.3,
-// 30 M 33.0 / 32.6, 40 M 35.3 / 44.4, 992 M 638 / 843).
-constexpr uint64_t kLutMinElements = 1u << 25;
+// The element-wise kernels take 1.65 times as long per element (and no table; 1.43 times where the call with device parameters needs a second launch
+// for the rows that the table does not serve).  Table / element-wise, host and device parameters: 8 M 13.0 / 12.6 and 16.2 / 14.2
+// us, 10 M 12.7 / 13.6 and 16.2 / 15.3, 2 M x 8 17.0 / 21.0 and 20.9 / 22.4, 300 k x 64 (128 blocks for 148 SMs) 20.4 / 22.9 and 25.4 /
+// 24.6, 30 M 24.9 / 31.2 and 28.3 / 33.4, 124 M x 8 591 / 843 and 599 / 843.
+static bool lut_pays(const CompressCall& c, uint32_t* per_worker) {
+    const uint64_t cost = lut_plan(c.d, c.n_workers, per_worker), others = c.d * c.n_workers / static_cast<uint64_t>(sm_count());
+    return cost * 100 < others * (c.params_dev ? 143 : 165);
+}
 
 cudaError_t launch_compress_lut(const CompressCall& c, bool* applied) {
     *applied = false;
-    if (!c.bf16 || !c.nonuniform || c.segs || c.d * c.n_workers < kLutMinElements || c.d > (1ull << 35)) return cudaSuccess;
+    uint32_t per_worker = 0;
+    if (!c.bf16 || !c.nonuniform || c.segs || c.d > (1ull << 35) || !lut_pays(c, &per_worker)) return cudaSuccess;
     if (c.params_dev) {      // the kernel decides row by row; the caller launches the element-wise kernels for the rest
         *applied = true;
         switch (c.bits) {
-            case 1: return launch_lut_dev<1>(c);
-            case 2: return launch_lut_dev<2>(c);
-            case 3: return launch_lut_dev<3>(c);
-            default: return launch_lut_dev<4>(c);
+            case 1: return launch_lut_dev<1>(c, per_worker);
+            case 2: return launch_lut_dev<2>(c, per_worker);
+            case 3: return launch_lut_dev<3>(c, per_worker);
+            default: return launch_lut_dev<4>(c, per_worker);
         }
     }
     static thread_local LutArgs args;
@@ -363,10 +364,10 @@ cudaError_t launch_compress_lut(const CompressCall& c, bool* applied) {
     }
     *applied = true;
     switch (c.bits) {
-        case 1: return launch_lut<1>(c, args, n_entries);
-        case 2: return launch_lut<2>(c, args, n_entries);
-        case 3: return launch_lut<3>(c, args, n_entries);
-        default: return launch_lut<4>(c, args, n_entries);
+        case 1: return launch_lut<1>(c, args, n_entries, per_worker);
+        case 2: return launch_lut<2>(c, args, n_entries, per_worker);
+        case 3: return launch_lut<3>(c, args, n_entries, per_worker);
+        default: return launch_lut<4>(c, args, n_entries, per_worker);
     }
 }
 

@@ -199,3 +199,21 @@ def test_codebooks_of_the_logarithmic_grid(tq, orc, dtype, L, alpha, inner):
         for i in range(2):
             want = orc.compress(host[i], _oracle_params(orc, p), 11, 3 + i)
             assert np.array_equal(got[i], want) and np.array_equal(dev[i], want)
+
+
+@pytest.mark.parametrize("bits,d,n", [(4, 8_200_003, 1), (4, 9_500_001, 1), (3, 2_000_003, 8), (2, 300_001, 40), (4, 200_000, 64), (1, 17_000_033, 1), (4, 20_000_016, 2)])
+def test_decision_table_dispatch(tq, orc, bits, d, n):
+    """bf16 rows on both sides of the line from which the decision table serves a call (earlier with host parameters than with
+    device ones), few and many rows per SM, ragged ends.  The same codes whichever kernel ran: the oracle's on the last row."""
+    L = 1 << bits
+    mags = np.geomspace(1e-5, 3e-3, L // 2).astype(np.float32) if L > 2 else np.array([3e-3], np.float32)
+    p = tq.tq_params_from_levels([float(x) for x in np.concatenate([-mags[::-1], mags])])
+    gen = torch.Generator(device="cuda").manual_seed(d)
+    g = torch.zeros(n, (d + 31) // 32 * 32, dtype=torch.bfloat16, device="cuda")
+    for i in range(n):
+        g[i, :d] = (torch.randn(d, device="cuda", generator=gen) * torch.exp(torch.randn(d, device="cuda", generator=gen)) * 2e-4).to(torch.bfloat16)
+    g[:, 5], g[:, d - 1] = float("nan"), float("-inf")
+    got = tq.tq_compress(g, [p] * n, seed=3, d=d)
+    raw = torch.frombuffer(bytearray(bytes(p) * n), dtype=torch.uint8).cuda()
+    assert torch.equal(got, tq.tq_compress_device_params(g, raw, L, tq.NONUNIFORM, seed=3, d=d))
+    assert np.array_equal(got[n - 1].cpu().numpy().view(np.uint32), orc.compress(g[n - 1, :d].float().cpu().numpy(), _oracle_params(orc, p), 3, n - 1))
