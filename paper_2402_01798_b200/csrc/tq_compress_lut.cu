@@ -158,11 +158,12 @@ __device__ __forceinline__ void load_piece(const char* row, uint64_t piece, uint
 // 49.1, 45.5 / 51.1).  28 warps spill at 72 registers: 639 / 684.
 constexpr int kLutThreads = 768;
 
-// A block's share of one row: build the table for quantizer q (n_entries per sign), then quantize.
+// A block's share of one row: build the table for quantizer q (n_entries per sign), then quantize the pieces begin + thread, + stride,
+// ... below `end`, and with LAST the row's last one, possibly partial.
 template <int BITS, bool WAIT>
 __device__ __forceinline__ void lut_block(const LutWorker& q, uint32_t n_entries, float* s_table, const char* __restrict__ row,
                                           uint32_t* __restrict__ prow, uint64_t d, uint64_t words_out, uint32_t worker,
-                                          const RoundKeys& rk) {
+                                          const RoundKeys& rk, uint64_t begin, uint64_t stride, uint64_t end, bool last) {
     // the table: the decision for every bit pattern of the window, both signs
     {
         const uint32_t base = (0u - q.base2) & 0xFFFFu;
@@ -179,11 +180,10 @@ __device__ __forceinline__ void lut_block(const LutWorker& q, uint32_t n_entries
 
     constexpr int E = Piece<BITS>::kElems, PER_ITER = 32 / E;   // 32 elements per thread and iteration: four Philox blocks in flight
     const LutCtx cx{smem_addr(s_table), q.negtop2, q.base2, (n_entries - 1) * 0x00010001u, philox_run(0u, worker, rk)};
-    const uint64_t interior = (d - 1) / E;                     // whole pieces before the row's last one
-    const uint64_t stride = static_cast<uint64_t>(gridDim.x) * kLutThreads;
+    const uint64_t row_interior = (d - 1) / E, interior = end < row_interior ? end : row_interior;      // whole pieces before the row's last one
 
     // two sets of registers take turns: the next iteration's loads are in flight while this one is quantized
-    uint64_t piece = static_cast<uint64_t>(blockIdx.x) * kLutThreads + threadIdx.x;
+    uint64_t piece = begin + threadIdx.x;
     uint32_t a[PER_ITER][E / 2], b[PER_ITER][E / 2];
     auto fetch = [&](uint32_t (&buf)[PER_ITER][E / 2], uint64_t first) {
 #pragma unroll
@@ -205,16 +205,16 @@ __device__ __forceinline__ void lut_block(const LutWorker& q, uint32_t n_entries
         fetch(a, piece);
         quantize(b, next);
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {                 // the row's last piece, possibly partial
+    if (last && threadIdx.x == 0) {
         const unsigned short* e = reinterpret_cast<const unsigned short*>(row);
         uint32_t t[E / 2];
 #pragma unroll
         for (int i = 0; i < E / 2; ++i) {
-            const uint64_t j = interior * E + 2 * i;
+            const uint64_t j = row_interior * E + 2 * i;
             const uint32_t lo = j < d ? __ldg(e + j) : 0u, hi = j + 1 < d ? __ldg(e + j + 1) : 0u;
             t[i] = lo | (hi << 16);
         }
-        lut_piece<BITS, true>(t, prow, interior, d, words_out, rk, cx);
+        lut_piece<BITS, true>(t, prow, row_interior, d, words_out, rk, cx);
     }
 }
 
@@ -227,48 +227,84 @@ compress_lut_kernel(const void* __restrict__ grad, uint64_t d, uint64_t grad_str
     extern __shared__ __align__(16) float s_table[];          // kLutMaxEntries + n_entries: the negative half starts at entry kLutMaxEntries
     const uint32_t wi = blockIdx.y;
     lut_block<BITS, true>(args.q[wi], n_entries, s_table, static_cast<const char*>(grad) + static_cast<uint64_t>(wi) * grad_stride * 2,
-                    packed + static_cast<uint64_t>(wi) * words_stride, d, words_out, first_worker + wi, rk);
+                    packed + static_cast<uint64_t>(wi) * words_stride, d, words_out, first_worker + wi, rk,
+                    static_cast<uint64_t>(blockIdx.x) * kLutThreads, static_cast<uint64_t>(gridDim.x) * kLutThreads, ~0ull, blockIdx.x == 0);
 }
 
 // Quantizers read from device memory (tq_params_device).  Every block decides by lut_serves_record whether the
 // table form serves its row, with the largest window; rows it does not serve are left to the element-wise
 // device-parameter kernels, which are launched after this one and skip the rows served here.
+struct LutState {
+    LutWorker q;
+    uint32_t fits[2];                                         // bit b of the 64: a window of b + 1 binades serves the row
+};
+// The record's quantizer into s.q; returns the entries per sign, 0 if the table does not serve it.  Block-uniform; ends with a barrier.
+template <int BITS>
+__device__ __forceinline__ uint32_t lut_record(const tq_params_t& rec, LutState& s) {
+    if (threadIdx.x < TQ_MAX_LEVELS) {
+        s.q.levels[threadIdx.x] = rec.levels[threadIdx.x];
+        s.q.inv_width[threadIdx.x] = rec.inv_width[threadIdx.x];
+    }
+    __syncthreads();
+    if (!lut_usable(rec, BITS)) return 0;
+    const uint32_t top = top_pattern(rec.alpha);
+    uint32_t base = 0;
+    if (threadIdx.x < 64) {
+        const bool fits = lut_window_fits(rec.alpha, s.q.levels, s.q.inv_width, 1u << BITS, top, kLutBinade * (threadIdx.x + 1), &base);
+        const uint32_t bits = __ballot_sync(0xFFFFFFFFu, fits);
+        if ((threadIdx.x & 31u) == 0) s.fits[threadIdx.x >> 5] = bits;
+    }
+    __syncthreads();
+    if (s.fits[1] >> 31 == 0) return 0;                       // the rule of lut_serves_record: not even the largest window
+    const uint32_t n_entries = kLutBinade * (s.fits[0] ? __ffs(static_cast<int>(s.fits[0])) : 32 + __ffs(static_cast<int>(s.fits[1])));
+    if (threadIdx.x == 0) {
+        base = top >= n_entries ? top - (n_entries - 1) : 0u;
+        s.q.alpha = rec.alpha;
+        s.q.base2 = ((0u - base) & 0xFFFFu) * 0x00010001u;
+        s.q.negtop2 = (top | 0x8000u) * 0x00010001u;
+    }
+    __syncthreads();
+    return n_entries;
+}
+
 template <int BITS>
 __global__ void __launch_bounds__(kLutThreads, 1)
 compress_lut_kernel_dev(const void* __restrict__ grad, uint64_t d, uint64_t grad_stride, const tq_params_t* __restrict__ params,
                         const __grid_constant__ RoundKeys rk, uint32_t first_worker, uint32_t* __restrict__ packed,
                         uint64_t words_stride, uint64_t words_out) {
     extern __shared__ __align__(16) float s_table[];          // 2 * kLutMaxEntries
-    __shared__ LutWorker s_q;
-    __shared__ uint32_t s_fits[2];                            // bit b of the 64: a window of b + 1 binades serves the row
+    __shared__ LutState s;
     const uint32_t wi = blockIdx.y;
     pdl_wait();
-    if (threadIdx.x < TQ_MAX_LEVELS) {
-        s_q.levels[threadIdx.x] = params[wi].levels[threadIdx.x];
-        s_q.inv_width[threadIdx.x] = params[wi].inv_width[threadIdx.x];
+    const uint32_t n_entries = lut_record<BITS>(params[wi], s);
+    if (n_entries == 0) return;
+    lut_block<BITS, false>(s.q, n_entries, s_table, static_cast<const char*>(grad) + static_cast<uint64_t>(wi) * grad_stride * 2,
+                    packed + static_cast<uint64_t>(wi) * words_stride, d, words_out, first_worker + wi, rk,
+                    static_cast<uint64_t>(blockIdx.x) * kLutThreads, static_cast<uint64_t>(gridDim.x) * kLutThreads, ~0ull, blockIdx.x == 0);
+}
+
+// Layer groups: a block's range of the jobs' tiles (kLutThreads pieces each), a table for every piece of a job.
+template <int BITS>
+__global__ void __launch_bounds__(kLutThreads, 1)
+compress_lut_kernel_segs(const void* __restrict__ grad, uint64_t grad_stride, const tq_params_t* __restrict__ params,
+                         const __grid_constant__ RoundKeys rk, uint32_t first_worker, uint32_t* __restrict__ packed, uint64_t words_stride,
+                         const __grid_constant__ TilePlan plan) {
+    extern __shared__ __align__(16) float s_table[];          // 2 * kLutMaxEntries
+    __shared__ LutState s;
+    uint64_t cur = first_tile_of_block(plan, blockIdx.x);
+    const uint64_t range_end = first_tile_of_block(plan, blockIdx.x + 1);
+    pdl_wait();
+    while (cur < range_end) {
+        const JobPiece job = next_piece(plan, cur, range_end);
+        const uint32_t n_entries = lut_record<BITS>(params[job.job], s);
+        if (n_entries != 0)
+            lut_block<BITS, false>(s.q, n_entries, s_table,
+                                   static_cast<const char*>(grad) + (static_cast<uint64_t>(job.worker) * grad_stride + job.off) * 2,
+                                   packed + static_cast<uint64_t>(job.worker) * words_stride + plan.segs.woff[job.seg], job.d,
+                                   (((job.d * BITS + 31) >> 5) + 3) & ~static_cast<uint64_t>(3), first_worker + job.worker, rk,
+                                   job.tile0 * kLutThreads, kLutThreads, job.tile1 * kLutThreads, job.last);
+        __syncthreads();                                       // the next piece reuses the table
     }
-    __syncthreads();
-    const tq_params_t& rec = params[wi];
-    uint32_t top = 0, base = 0;
-    if (!lut_usable(rec, BITS)) return;
-    top = top_pattern(rec.alpha);
-    if (threadIdx.x < 64) {
-        const bool fits = lut_window_fits(rec.alpha, s_q.levels, s_q.inv_width, 1u << BITS, top, kLutBinade * (threadIdx.x + 1), &base);
-        const uint32_t bits = __ballot_sync(0xFFFFFFFFu, fits);
-        if ((threadIdx.x & 31u) == 0) s_fits[threadIdx.x >> 5] = bits;
-    }
-    __syncthreads();
-    if (s_fits[1] >> 31 == 0) return;                         // the rule of lut_serves_record: not even the largest window
-    const uint32_t n_entries = kLutBinade * (s_fits[0] ? __ffs(static_cast<int>(s_fits[0])) : 32 + __ffs(static_cast<int>(s_fits[1])));
-    if (threadIdx.x == 0) {
-        base = top >= n_entries ? top - (n_entries - 1) : 0u;
-        s_q.alpha = rec.alpha;
-        s_q.base2 = ((0u - base) & 0xFFFFu) * 0x00010001u;
-        s_q.negtop2 = (top | 0x8000u) * 0x00010001u;
-    }
-    __syncthreads();
-    lut_block<BITS, false>(s_q, n_entries, s_table, static_cast<const char*>(grad) + static_cast<uint64_t>(wi) * grad_stride * 2,
-                    packed + static_cast<uint64_t>(wi) * words_stride, d, words_out, first_worker + wi, rk);
 }
 
 // ---- host --------------------------------------------------------------------------------------------
@@ -320,6 +356,17 @@ static cudaError_t launch_lut_dev(const CompressCall& c, uint32_t per_worker) {
                          c.d, c.grad_stride, c.params_dev, round_keys(c.seed), c.first_worker, c.packed, c.words_stride, c.words_out);
 }
 
+template <int BITS>
+static cudaError_t launch_lut_segs(const CompressCall& c, uint32_t blocks) {
+    static thread_local TilePlan plan;
+    plan_tiles(&plan, c.segs, c.d, c.n_workers, static_cast<uint64_t>(kLutThreads) * Piece<BITS>::kElems, blocks);
+    const int smem = static_cast<int>(2 * kLutMaxEntries * sizeof(float));
+    const cudaError_t e = cudaFuncSetAttribute(compress_lut_kernel_segs<BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    return launch_kernel(compress_lut_kernel_segs<BITS>, dim3(plan.blocks), kLutThreads, smem, c.stream, c.grad, c.grad_stride, c.params_dev,
+                         round_keys(c.seed), c.first_worker, c.packed, c.words_stride, plan);
+}
+
 // The element-wise kernels take 1.65 times as long per element (and no table; 1.43 times where the call with device parameters needs a second launch
 // for the rows that the table does not serve).  Table / element-wise, host and device parameters: 8 M 13.0 / 12.6 and 16.2 / 14.2
 // us, 10 M 12.7 / 13.6 and 16.2 / 15.3, 2 M x 8 17.0 / 21.0 and 20.9 / 22.4, 300 k x 64 (128 blocks for 148 SMs) 20.4 / 22.9 and 25.4 /
@@ -332,7 +379,27 @@ static bool lut_pays(const CompressCall& c, uint32_t* per_worker) {
 cudaError_t launch_compress_lut(const CompressCall& c, bool* applied) {
     *applied = false;
     uint32_t per_worker = 0;
-    if (!c.bf16 || !c.nonuniform || c.segs || c.d > (1ull << 35) || !lut_pays(c, &per_worker)) return cudaSuccess;
+    if (!c.bf16 || !c.nonuniform) return cudaSuccess;
+    if (c.segs) {
+        uint64_t total = 0;
+        for (uint32_t s = 0; s < c.segs->n; ++s) {
+            if (c.segs->len[s] > (1ull << 35)) return cudaSuccess;
+            total += c.segs->len[s] * c.n_workers;
+        }
+        // two ranges per SM; a table for every piece, of which there are at most blocks + jobs; the element-wise kernel as above
+        // (25.6 M x 16, 16 levels, 16 groups of lengths up to 75 apart: 358 us element-wise, 305 with tables, 302 / 312 in one / three
+        // ranges per SM; 25.6 M x 8, 8 levels 183 / 179 / 184)
+        const uint32_t blocks = static_cast<uint32_t>(sm_count()) * 2;
+        if ((blocks + static_cast<uint64_t>(c.n_workers) * c.segs->n) * 40000 * 100 >= total * 43) return cudaSuccess;
+        *applied = true;
+        switch (c.bits) {
+            case 1: return launch_lut_segs<1>(c, blocks);
+            case 2: return launch_lut_segs<2>(c, blocks);
+            case 3: return launch_lut_segs<3>(c, blocks);
+            default: return launch_lut_segs<4>(c, blocks);
+        }
+    }
+    if (c.d > (1ull << 35) || !lut_pays(c, &per_worker)) return cudaSuccess;
     if (c.params_dev) {      // the kernel decides row by row; the caller launches the element-wise kernels for the rest
         *applied = true;
         switch (c.bits) {

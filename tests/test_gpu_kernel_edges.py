@@ -217,3 +217,39 @@ def test_decision_table_dispatch(tq, orc, bits, d, n):
     raw = torch.frombuffer(bytearray(bytes(p) * n), dtype=torch.uint8).cuda()
     assert torch.equal(got, tq.tq_compress_device_params(g, raw, L, tq.NONUNIFORM, seed=3, d=d))
     assert np.array_equal(got[n - 1].cpu().numpy().view(np.uint32), orc.compress(g[n - 1, :d].float().cpu().numpy(), _oracle_params(orc, p), 3, n - 1))
+
+
+@pytest.mark.parametrize("bits,bad", [(4, False), (3, True), (1, False)])
+def test_decision_table_of_layer_groups(tq, orc, bits, bad):
+    """bf16 layer groups large enough for a table per piece: lengths from one element up, ranges that cross several jobs, one job whose
+    codebook the table does not serve and one that is invalid (zeros).  Equal to the element-wise kernels, which serve the
+    groups one call each would be too short for, and to the oracle on a few jobs."""
+    L, n = 1 << bits, 3
+    lens = [16_000_000, 1, 5_000_001, 33, 9_000_016, 12_289, 3_000_007]
+    segs, off = [], 0
+    for ln in lens:
+        segs.append((off, ln))
+        off += (ln + 15) // 16 * 16
+    gen = torch.Generator(device="cuda").manual_seed(bits)
+    g = (torch.randn(n, off, device="cuda", generator=gen) * torch.exp(torch.randn(n, off, device="cuda", generator=gen)) * 2e-4).to(torch.bfloat16)
+    g[:, 7], g[:, off - 17] = float("nan"), float("inf")
+    ps = []
+    for j in range(n * len(lens)):
+        mags = np.geomspace((1e-5 if not (bad and j == 2) else 1e-30) * (1 + j), 3e-3 * (1 + 0.1 * j), L // 2).astype(np.float32) if L > 2 else np.array([3e-3], np.float32)
+        ps.append(tq.tq_params_from_levels([float(x) for x in np.concatenate([-mags[::-1], mags])]))
+    recs = [bytes(p) for p in ps]
+    if bad:
+        recs[len(lens) + 4] = bytes(len(recs[0]))                # alpha = 0: never served, all codes 0
+    raw = torch.frombuffer(bytearray(b"".join(recs)), dtype=torch.uint8).cuda()
+    got = tq.tq_compress_segments(g, segs, raw, L, tq.NONUNIFORM, seed=21).cpu().numpy().view(np.uint32)
+    w = 0
+    for s, (o, ln) in enumerate(segs):
+        words = tq.tq_packed_words(ln, bits)
+        for i in range(n):
+            j = i * len(lens) + s
+            part = got[i, w:w + words]
+            if bad and j == len(lens) + 4:
+                assert not part.any()
+            elif s != 0 or i == 2:
+                assert np.array_equal(part, orc.compress(g[i, o:o + ln].float().cpu().numpy(), _oracle_params(orc, ps[j]), 21, i)), (s, i)
+        w += words
