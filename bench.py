@@ -39,7 +39,7 @@ if ROOT not in sys.path:
 METRIC = "compress & decompress-aggregate GB/s of fp32 gradient, % of B200 HBM peak"
 FALLBACK_HBM_GBS = 6650.0
 # dram__bytes_read.sum + dram__bytes_write.sum per launch from the ncu capture summarised in
-# profiles/compress_kernel_resnet50-25.6M.md (valid for the kernel as it stands; None elsewhere)
+# profiles/compress_kernel_resnet50-25.6M.md (the kernel's loads and stores have not changed since; None elsewhere)
 NCU_DRAM_BYTES = {("resnet50-25.6M", "tq_compress"): 1_837_323_352}
 
 
