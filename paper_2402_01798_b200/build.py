@@ -13,7 +13,7 @@ LIB = os.path.join(PKG, "libtq.so")
 NATIVE = os.path.join(PKG, "_tq_python" + sysconfig.get_config_var("EXT_SUFFIX"))
 NATIVE_SOURCE = os.path.join(CSRC, "tq_python.cpp")
 SOURCES = ["tq_api.cu", "tq_stats.cu", "tq_compress.cu", "tq_compress_lut.cu", "tq_decompress.cu", "tq_params.cu"]
-HEADERS = ["tq_device.cuh", "tq_launch.h", "tq_lut.cuh"]
+HEADERS = ["tq_aggregation_plan.h", "tq_device.cuh", "tq_launch.h", "tq_lut.cuh"]
 
 NVCC_FLAGS = [
     "-std=c++17", "-O3", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo",

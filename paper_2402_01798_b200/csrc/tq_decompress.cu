@@ -9,6 +9,7 @@
 // Codebooks live in shared memory, 16 consecutive words per worker, four workers per 256 bytes: any
 // set of codes of one worker maps to distinct banks, so lookups are conflict-free.
 // HBM traffic per output element: N * bits / 8 bytes read, 4 bytes written.
+#include "tq_aggregation_plan.h"
 #include "tq_device.cuh"
 #include "tq_launch.h"
 
@@ -50,14 +51,10 @@ __device__ __forceinline__ uint32_t ldg32_stream(const uint32_t* p) {
 
 constexpr int kTabStride = 16;   // floats between consecutive workers' codebooks in shared memory: four codebooks per 256 bytes
 
-// A unit is a run of elements decoded from one 32-bit "field": 8 / 16 / 32 elements = one packed word
-// for 4 / 2 / 1 bits; for 3 bits 8 elements = 24 bits that start on a byte boundary and are cut out of
-// two neighbouring words.  A thread owns U units, spaced one block apart, so that every
-// load and every 256-bit store of a warp is contiguous, and keeps U * kElems (at most 32) accumulators in registers.
 template <int BITS>
 struct Unit {
-    static constexpr int kElems = BITS == 2 ? 16 : (BITS == 1 ? 32 : 8);
-    static constexpr int kMost = 32 / kElems;      // units of a thread with 32 accumulators
+    static constexpr int kElems = unit_elems(BITS);
+    static constexpr int kMost = most_units(BITS);
 };
 
 // The field of unit u of one row, all words known to be inside the row.
@@ -129,8 +126,6 @@ __device__ __forceinline__ void add_unit(f32x2* acc, uint32_t f, const char* tab
         }
     }
 }
-
-constexpr int kDecThreads = 128;
 
 // Turns the accumulated sums of a thread's units into outputs: the division by N (w_i = 1/N; for N a
 // power of two the product with 2^-k is the same value), then either the store of the aggregate or
@@ -324,13 +319,6 @@ constexpr int kGroup = TQ_DECOMPRESS_GROUP;   // workers per stage
 
 __device__ unsigned int g_wait_expired = 0;   // blocks (or threads) whose bounded wait ran out, since load
 
-template <int BITS, int U>
-struct Tile {
-    static constexpr int kUnitBytes = BITS == 3 ? 3 : 4;
-    static constexpr int kUnits = kDecThreads * U;                           // units per tile (a multiple of 4)
-    static constexpr int kSegBytes = kUnits * kUnitBytes;               // one worker's bytes per tile (a multiple of 16)
-};
-
 // The field of local unit ul of a tile segment in shared memory (same cut as load_field; the tile's
 // first unit is a multiple of 4, so the byte phase of a 3-bit unit is that of its local index).
 template <int BITS>
@@ -353,7 +341,7 @@ decompress_bulk_kernel(const __grid_constant__ RowTable rt, uint64_t words_row, 
                        float scale, int divide, const __grid_constant__ ApplyArgs ap_in, float* __restrict__ out_row,
                        const __grid_constant__ SegTiles st) {
     constexpr int E = Unit<BITS>::kElems, S = TQ_DECOMPRESS_STAGES;
-    constexpr uint32_t kSeg = Tile<BITS, U>::kSegBytes;
+    constexpr uint32_t kSeg = tile_bytes(BITS, U);
 
     // [codebooks: n * 64 B][S stages of kGroup segments][16 B that a 3-bit field's second word may touch][S barriers]
     extern __shared__ __align__(1024) unsigned char smem[];
@@ -381,7 +369,7 @@ decompress_bulk_kernel(const __grid_constant__ RowTable rt, uint64_t words_row, 
     }
     const uint64_t tile_off = tile * kSeg + row_shift * 4;                   // byte offset of the tile in every row
     const uint64_t row_bytes = (words_valid + row_shift) * 4;
-    const uint32_t seg_bytes = static_cast<uint32_t>(row_bytes - tile_off < kSeg ? row_bytes - tile_off : kSeg);
+    const uint32_t seg_bytes = tile_bytes_in_row(row_bytes, tile_off, kSeg);  // every block has a tile inside its row
     const uint32_t n_steps = (n + kGroup - 1) / kGroup;
 
     // step q = workers q*kGroup .. ; its bytes go to stage q % S
@@ -460,30 +448,18 @@ decompress_bulk_kernel(const __grid_constant__ RowTable rt, uint64_t words_row, 
         return;
     }
 
-    const uint64_t u0 = tile * Tile<BITS, U>::kUnits + threadIdx.x;
+    const uint64_t u0 = tile * (kDecThreads * U) + threadIdx.x;
     if (u0 * E >= d) return;       // nothing of this thread's first unit (hence of any) exists
     finish_units<BITS, APPLY, U>(acc, u0, d, scale, divide, ap, out);
 }
 
 static const SegTiles kNoSegTiles{};
 
-// Below this many tiles of 32 outputs per thread, two per SM, too few warps are in flight for the latency of a walk over the
-// workers: the direct kernel takes one unit per thread (1 M x 64, 3 bits: 27.5 -> 17.3 us; 20 k x 64: 58 -> 7.9 us; 489 tiles, 2 M x
-// 16: 10.8 us in the bulk form, 12.2 in the direct one).
-constexpr uint64_t kTilesForBulk = 296;
-// The fused update has as much to do after the walk as in it, and fewer registers per thread keep more of its loads in
-// flight: one unit per thread up to this many tiles (4 M x 4: 18.6 -> 14.3 us, 11.2 M x 8: 39.9 -> 37.3; 25.6 M x 16, 6250
-// tiles: 102 us with one unit, 92.9 with two), beyond it two where a tile has four (3 and 4 bits: 25.6 M x 16 96.6 -> 92.9 us,
-// 50 M x 4 142 -> 130, 250 M x 4 684 -> 633).  With 64 workers the walk weighs more again: 3 M x 64 takes 41.5 us with four
-// units, 43.3 with two, 56 with one.
-constexpr uint64_t kTilesForLongApply = 4096;
-constexpr uint32_t kWorkersForShortApply = 32;
-
 template <int BITS, bool APPLY, int U>
 static cudaError_t launch_bulk(const DecompressCall& c, const RowTable& rt, const DecompressArgs& args, const DeviceTables& dt,
                                float scale, int divide, const ApplyArgs& ap, uint64_t tiles, const SegTiles& st = kNoSegTiles) {
     const size_t smem = static_cast<size_t>(c.n_workers) * (kTabStride * 4) +
-                        static_cast<size_t>(TQ_DECOMPRESS_STAGES) * kGroup * Tile<BITS, U>::kSegBytes + 16 + 8 * TQ_DECOMPRESS_STAGES;
+                        static_cast<size_t>(TQ_DECOMPRESS_STAGES) * kGroup * tile_bytes(BITS, U) + 16 + 8 * TQ_DECOMPRESS_STAGES;
     if (smem > 48 * 1024) {
         const cudaError_t e = cudaFuncSetAttribute(decompress_bulk_kernel<BITS, APPLY, U>,
                                                    cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
@@ -498,8 +474,7 @@ static cudaError_t launch_bulk(const DecompressCall& c, const RowTable& rt, cons
 template <int BITS, bool APPLY>
 static cudaError_t launch_apply(const DecompressCall& c, const RowTable& rt, const DecompressArgs& args, const DeviceTables& dt, float scale,
                                 int divide) {
-    constexpr int E = Unit<BITS>::kElems, U = Unit<BITS>::kMost;
-    constexpr uint64_t kPerTile = static_cast<uint64_t>(kDecThreads) * U * E;          // elements
+    constexpr int U = Unit<BITS>::kMost;
     const ApplyArgs ap{c.theta, c.momentum_buf, c.lr, c.mu, c.wd};
     if (c.segs) {      // layer groups: the tiles of every segment in one grid, always through the bulk-copy kernel
         static thread_local SegTiles st;
@@ -507,34 +482,32 @@ static cudaError_t launch_apply(const DecompressCall& c, const RowTable& rt, con
         uint64_t total = 0;
         for (uint32_t sg = 0; sg < c.segs->n; ++sg) {
             st.tile_begin[sg] = static_cast<uint32_t>(total);
-            total += (c.segs->len[sg] + kPerTile - 1) / kPerTile;
+            total += tiles_of(BITS, U, c.segs->len[sg]);
             if (total > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
         }
         st.tile_begin[c.segs->n] = static_cast<uint32_t>(total);
         return launch_bulk<BITS, APPLY, U>(c, rt, args, dt, scale, divide, ap, total, st);
     }
-    const uint64_t tiles = (c.d + kPerTile - 1) / kPerTile;
-    if (tiles == 0) return cudaSuccess;
-    if (tiles > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
-    if (tiles < kTilesForBulk) {
-        constexpr uint64_t kPerBlock = static_cast<uint64_t>(kDecThreads) * E;
-        const uint64_t blocks = (c.d + kPerBlock - 1) / kPerBlock;
+    const AggregationPlan plan = plan_aggregation(BITS, c.d, c.n_workers, APPLY);
+    if (plan.blocks == 0) return cudaSuccess;
+    if (plan.blocks > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
+    if (!plan.bulk) {
         // At most half of what fits at a time, with a long walk over the workers: see launch_kernel.  Rounds, early / late start:
         // 250 k x 64 63.1 / 49.6 us, 50 k x 64 37.9 / 24.9, 250 k x 16 29.6 / 26.6; behind short compressions there is room
         // everywhere, and only codebooks in device memory, which an early start cannot read, leave it no advantage: 20 k x 64 29.6 /
         // 22.8, with the codebooks in kernel parameters 16.1 / 17.9; 50 k x 16 20.0 / 20.1 and 13.0 / 13.7; 1 M x 16 (977 blocks) 55.0 / 55.3.
-        const bool late = c.n_workers >= 16 && blocks <= static_cast<uint64_t>(sm_count()) * (TQ_DECOMPRESS_MIN_BLOCKS / 2) &&
+        const bool late = c.n_workers >= 16 && plan.blocks <= static_cast<uint64_t>(sm_count()) * (TQ_DECOMPRESS_MIN_BLOCKS / 2) &&
                           (c.n_workers * c.d >= (1u << 21) || (c.params_dev && c.n_workers >= 32));
-        return launch_kernel(late ? Start::kLate : Start::kEarly, decompress_kernel<BITS, APPLY>, dim3(static_cast<unsigned>(blocks)), kDecThreads, 0, c.stream, rt,
+        return launch_kernel(late ? Start::kLate : Start::kEarly, decompress_kernel<BITS, APPLY>, dim3(static_cast<unsigned>(plan.blocks)), kDecThreads, 0, c.stream, rt,
                              c.words_valid, c.n_workers, c.d, args, dt, scale, divide, ap, c.out);
     }
     if constexpr (APPLY && U > 1) {
-        if (c.n_workers <= kWorkersForShortApply) {
-            if (tiles < kTilesForLongApply) return launch_bulk<BITS, APPLY, 1>(c, rt, args, dt, scale, divide, ap, tiles * U);
-            if constexpr (U > 2) return launch_bulk<BITS, APPLY, 2>(c, rt, args, dt, scale, divide, ap, tiles * (U / 2));
-        }
+        if (plan.units == 1) return launch_bulk<BITS, APPLY, 1>(c, rt, args, dt, scale, divide, ap, plan.blocks);
     }
-    return launch_bulk<BITS, APPLY, U>(c, rt, args, dt, scale, divide, ap, tiles);
+    if constexpr (APPLY && U > 2) {
+        if (plan.units == 2) return launch_bulk<BITS, APPLY, 2>(c, rt, args, dt, scale, divide, ap, plan.blocks);
+    }
+    return launch_bulk<BITS, APPLY, U>(c, rt, args, dt, scale, divide, ap, plan.blocks);
 }
 
 template <int BITS>
