@@ -151,9 +151,8 @@ struct Packed {
     size_t stride;
     uint32_t n;
 };
-Packed packed_rows(Args& a) {
-    const at::Tensor& t = a.tensor();
-    if (!t.is_cuda() || t.dim() != 2) fail(PyExc_ValueError, "packed must be a [N, words] CUDA tensor");
+Packed packed_rows(const at::Tensor& t) {       // in any memory the GPU reads (pinned host memory too); a row may have several dimensions
+    if (t.dim() < 1) fail(PyExc_ValueError, "packed must have a row per worker");
     return Packed{static_cast<uint32_t*>(t.data_ptr()), static_cast<size_t>(t.size(0) > 1 ? t.stride(0) : t.size(1)), static_cast<uint32_t>(t.size(0))};
 }
 Packed packed_out(Args& a, uint32_t n) {        // as many rows as the gradient has; one row may be given as a vector
@@ -246,7 +245,9 @@ tq_status compress_device_params(Args& a) {     // grad, d, params, num_levels, 
                                     first, p.data, p.stride, a.stream());
 }
 tq_status decompress_aggregate(Args& a) {       // packed, d, params, weights, out, stream
-    const Packed p = packed_rows(a);
+    const at::Tensor& t = a.tensor();
+    if (!t.is_cuda() || t.dim() != 2) fail(PyExc_ValueError, "packed must be a [N, words] CUDA tensor");
+    const Packed p = packed_rows(t);
     const uint64_t d = a.u64();
     const tq_params_t* params = host_params(a, p.n);
     const float* w = a.weights(p.n);
@@ -272,7 +273,7 @@ tq_status decompress_aggregate_rows(Args& a) {  // rows (tensors or addresses), 
     return F.decompress_aggregate_rows(rows, static_cast<uint32_t>(n), d, params, w, static_cast<float*>(out), a.stream());
 }
 tq_status decompress_aggregate_apply(Args& a) { // packed, d, params, weights, theta, momentum, lr, mu, weight_decay, stream
-    const Packed p = packed_rows(a);
+    const Packed p = packed_rows(a.tensor());
     const uint64_t d = a.u64();
     const tq_params_t* params = host_params(a, p.n);
     const float* w = a.weights(p.n);
@@ -283,7 +284,7 @@ tq_status decompress_aggregate_apply(Args& a) { // packed, d, params, weights, t
                                         a.stream());
 }
 tq_status decompress_aggregate_device_params(Args& a) {      // packed, d, params, num_levels, weights, out, stream
-    const Packed p = packed_rows(a);
+    const Packed p = packed_rows(a.tensor());
     const uint64_t d = a.u64();
     void* params = a.address();
     const uint32_t levels = a.u32();
@@ -325,7 +326,7 @@ tq_status compress_segments(Args& a) {          // grad, segments, params, num_l
                                first, p.data, p.stride, a.stream());
 }
 tq_status decompress_aggregate_segments(Args& a) {           // packed, segments, params, num_levels, weights, out, stream
-    const Packed p = packed_rows(a);
+    const Packed p = packed_rows(a.tensor());
     uint32_t n_seg;
     const tq_segment_t* seg = segments(a, &n_seg);
     void* params = a.address();

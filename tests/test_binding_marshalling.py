@@ -40,3 +40,19 @@ def test_library_status_comes_back(tq):
     with pytest.raises(tq.TqError) as e:
         tq.tq_decompress_aggregate_rows([20], 16, [p], out=torch.zeros(16), stream=0)      # a row off its 16-byte boundary
     assert e.value.status == tq.ERR_ALIGNMENT
+
+
+def test_packed_rows_outside_the_gpu_and_with_more_dimensions(tq):
+    """The fused update and the device-parameter calls read packed rows wherever the GPU can, pinned host memory included, and a
+    row may be folded ([N, 2, 4]): such a block reaches the library, whose own checks answer."""
+    buf = torch.zeros(20, dtype=torch.int32)
+    rows = buf[(-buf.data_ptr() // 4) % 4 + 1:][:16]                                           # four bytes off a 16-byte boundary
+    out, params = torch.zeros(16), torch.zeros(2 * 176, dtype=torch.uint8)
+    p = tq.tq_params_from_levels([-1.0, -0.5, 0.5, 1.0])
+    for packed in (rows.view(2, 8), rows.view(2, 2, 4)):
+        for call in (lambda: tq.tq_decompress_aggregate_device_params(packed, 16, params, 4, out=out, stream=0),
+                     lambda: tq.tq_decompress_aggregate_segments(packed, [(0, 16)], params, 4, out=out, stream=0),
+                     lambda: tq.tq_decompress_aggregate_apply(packed, 16, [p, p], out, None, lr=0.1, stream=0)):
+            with pytest.raises(tq.TqError) as e:
+                call()
+            assert e.value.status == tq.ERR_ALIGNMENT
