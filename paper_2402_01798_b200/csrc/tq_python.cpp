@@ -94,18 +94,22 @@ public:
         if (PyErr_Occurred()) throw Failed();
         return s;
     }
-    // None, or n numbers
+    // None, or up to n numbers, the rest zeros.  Only the first TQ_MAX_WORKERS are kept: the library refuses more rows before
+    // it reads a weight.
     const float* weights(uint32_t n) {
         PyObject* o = next();
         if (o == Py_None) return nullptr;
         PyObject* seq = PySequence_Fast(o, "weights must be a sequence of numbers");
         if (!seq) throw Failed();
         const Py_ssize_t have = PySequence_Fast_GET_SIZE(seq);
-        for (Py_ssize_t i = 0; i < have && i < n; ++i) weights_[i] = static_cast<float>(PyFloat_AsDouble(PySequence_Fast_GET_ITEM(seq, i)));
+        for (Py_ssize_t i = 0; i < have && !PyErr_Occurred(); ++i) {
+            const float w = static_cast<float>(PyFloat_AsDouble(PySequence_Fast_GET_ITEM(seq, i)));
+            if (i < TQ_MAX_WORKERS) weights_[i] = w;
+        }
         Py_DECREF(seq);
         if (PyErr_Occurred()) throw Failed();
         if (have > n) fail(PyExc_IndexError, "invalid index");
-        for (Py_ssize_t i = have; i < n; ++i) weights_[i] = 0.0f;
+        for (Py_ssize_t i = have; i < TQ_MAX_WORKERS; ++i) weights_[i] = 0.0f;
         return weights_;
     }
 

@@ -56,3 +56,36 @@ def test_packed_rows_outside_the_gpu_and_with_more_dimensions(tq):
             with pytest.raises(tq.TqError) as e:
                 call()
             assert e.value.status == tq.ERR_ALIGNMENT
+
+
+@pytest.mark.parametrize("rows", [64, 65, 1000])
+def test_weights_of_more_rows_than_the_library_takes(tq, rows):
+    """One weight per row, a list too short (zeros follow) and one too long.  More than 64 rows are the library's to refuse, without a
+    weight written beyond the 64 that the binding keeps; with 64 the misaligned rows are what it refuses."""
+    packed = torch.zeros(4 * rows + 8, dtype=torch.int32)
+    packed = packed[(-packed.data_ptr() // 4) % 4 + 1:][:4 * rows].view(rows, 4)
+    out, params = torch.zeros(16), torch.zeros(176 * rows, dtype=torch.uint8)
+    p = tq.tq_params_from_levels([-1.0, -0.5, 0.5, 1.0])
+    for weights in ([0.5] * rows, [], (0.5,) * (rows - 1), torch.ones(rows)):
+        for call in (lambda: tq.tq_decompress_aggregate_device_params(packed, 16, params, 4, weights=weights, out=out, stream=0),
+                     lambda: tq.tq_decompress_aggregate_segments(packed, [(0, 16)], params, 4, weights=weights, out=out, stream=0),
+                     lambda: tq.tq_decompress_aggregate_apply(packed, 16, [p] * rows, out, None, lr=0.1, weights=weights, stream=0),
+                     lambda: tq.tq_decompress_aggregate_rows([8] * rows, 16, [p] * rows, weights=weights, out=out, stream=0)):
+            with pytest.raises(tq.TqError) as e:
+                call()
+            assert e.value.status == (tq.ERR_ALIGNMENT if rows == 64 else tq.ERR_INVALID_ARG)
+    for call in (lambda w: tq.tq_decompress_aggregate_device_params(packed, 16, params, 4, weights=w, out=out, stream=0),
+                 lambda w: tq.tq_decompress_aggregate_apply(packed, 16, [p] * rows, out, None, lr=0.1, weights=w, stream=0)):
+        with pytest.raises(IndexError):
+            call([0.5] * (rows + 1))
+        with pytest.raises(TypeError):
+            call([0.5, None])
+
+
+@pytest.mark.gpu
+def test_weights_of_more_rows_than_the_library_takes_in_a_block(tq):
+    """As above for the call that asks for a CUDA block."""
+    p = tq.tq_params_from_levels([-1.0, 1.0])
+    with pytest.raises(tq.TqError) as e:
+        tq.tq_decompress_aggregate(torch.zeros((65, 4), dtype=torch.int32, device="cuda"), 16, [p] * 65, weights=[0.1] * 65)
+    assert e.value.status == tq.ERR_INVALID_ARG
