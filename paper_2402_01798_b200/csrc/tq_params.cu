@@ -282,12 +282,15 @@ TQ_HD inline void clear(tq_params_t* p) {
 
 // The boxed alpha equation x = F(x), from x0 = ln(alpha' / g_min) until a plain step changes alpha by <= 1e-12
 // relative.  The plain iteration converges linearly (70 steps for gamma = 3, s = 15).  F' comes with F, so a step goes to
-// the root of the tangent of F(x) - x wherever F' < 0.999 (Newton).  For the quantizers of Sections 4.1 and 4.2, F' grows
-// with x on x > 0, and every iterate is >= x0 because Q <= 1; so if F'(x0) >= -0.9 the plain iteration is a
-// contraction, or runs monotonically into the same first fixed point that the tangents of the convex F - x cannot
-// pass.  Elsewhere (the plain iteration may then end in a 2-cycle, which is its result) steps stay plain where F' < 0,
-// as they do for the two-step quantizer; F has a kink at x = 0, which no tangent step crosses.  Either way the result is
-// accepted only through the plain-step test.  Stops when alpha has passed max|g| (no fixed point below it).
+// the root of the tangent of F(x) - x where that cannot change the outcome; x = F(x) is tested on the way in any case.  For the
+// quantizers of Sections 4.1 and 4.2 and x > 0, every iterate is >= x0 because Q <= 1, and wherever F' < 1 it grows with x and
+// stays below 1, so F - x is convex and falls: one fixed point, which no tangent from its left passes.
+//   x0 > 0 and -0.9 <= F'(x0): no 2-cycle (F' > -1), so the plain iteration reaches that point too.  Its largest iterate is F(x0)
+//   or the fixed point; it is stopped by max|g| exactly when one of the two is beyond, and either shows as a plain step beyond.
+//   Elsewhere steps stay plain (the plain iteration may end in a 2-cycle, which is its result) but where F rises from x on
+//   (F' >= 0, F(x) >= x): it then runs up to the point that the tangents approach from the same side.
+// The two-step quantizer takes tangents wherever F' >= 0.  F has a kink at x = 0, which no tangent step crosses.  Stops when a plain
+// step has passed max|g|.
 template <class Lanes>
 TQ_HD inline double solve_alpha(const Lanes& lanes, const SplitGrid<Lanes>& grid, const TailModel& m, uint32_t mode, double x_cap,
                                 int* iterations) {
@@ -307,7 +310,8 @@ TQ_HD inline double solve_alpha(const Lanes& lanes, const SplitGrid<Lanes>& grid
         if (it == 0 && !(slope >= least)) least = 0.0;
         ++it;
         const double d = f - x, root = f + d * slope / (1.0 - slope);      // = x + d / (1 - slope)
-        const bool take = slope >= least && slope < 0.999 && x > 0.0 && root > 0.0 && finite_d(root) && !(root > x_cap);
+        const bool same = mode == TQ_BISCALED || least < 0.0 || d >= 0.0;
+        const bool take = same && slope >= least && slope < 0.999 && x > 0.0 && root > 0.0 && finite_d(root) && !(f > x_cap) && !(root > x_cap);
         x = f;
         if (fabs(d) <= 1e-12) break;
         if (take) x = root;

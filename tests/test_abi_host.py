@@ -6,6 +6,7 @@ No kernel is launched here; argument errors are detected before any CUDA call is
 import ctypes as C
 import math
 import os
+import random
 import re
 
 import numpy as np
@@ -137,6 +138,23 @@ def test_tq_params_agrees_with_oracle(tq, orc, L, mode, gamma, rule):
         assert np.all(np.diff(lv) > 0) and lv[0] == -a.alpha and lv[-1] == a.alpha
         for k in range(L - 1):                                  # inverse widths are rounded UP
             assert a.inv_width[k] >= 1.0 / float(np.float32(lv[k + 1] - lv[k]))
+
+
+@pytest.mark.parametrize("mode,records", [(0, 4000), (1, 4000), (2, 120)])
+def test_alpha_is_stopped_by_the_largest_gradient_as_the_plain_iteration_is(tq, orc, mode, records):
+    """Flat tails with max|g| within a factor of 3 of g_min: the plain iteration overshoots its fixed point, and where one of its
+    steps passes max|g|, alpha is max|g|, flagged.  The exponents are no whole numbers: for gamma = 3 and two levels every
+    orbit of the uniform equation is a 2-cycle and its end touches g_min to rounding, which leaves that flag open."""
+    r, capped = random.Random(mode), 0
+    for _ in range(records):
+        d = 10 ** r.randint(3, 9)
+        n_tail, g_min = int(2 * d * r.uniform(0.2, 0.49)), math.exp(r.uniform(-12, -2))
+        kw = dict(d=d, n_tail=n_tail, sum_log_tail=n_tail / r.uniform(1.01, 4.0), g_min=g_min, max_abs=g_min * r.uniform(1.0, 3.0))
+        L, gamma = r.choice([2, 4, 8, 16]), r.choice([math.nan, 2.0 + math.exp(r.uniform(-5.0, 2.5))])
+        a, b = tq.tq_params(_stats(tq.Stats, **kw), L, mode, gamma), orc.params(_stats(orc.Stats, **kw), L, mode, gamma)
+        assert a.flags == b.flags and math.isclose(a.alpha, b.alpha, rel_tol=3e-7), (L, gamma, kw)
+        capped += bool(a.flags & tq.FLAG_ALPHA_CAPPED)
+    assert records // 20 < capped < records
 
 
 def test_tq_params_errors(tq):
