@@ -409,18 +409,18 @@ __device__ __forceinline__ void fold_records(const Partial* records, uint32_t co
     }
     block_fold<kWarps, MOMENTS, TAILS, false>(p, sh);
 }
-// The sum of |g| over the records, known to every thread.
+// The sum of |g| over the records, known to every thread; added as fold_records adds it, because a threshold that follows from the
+// one has to equal that from the other.
 __device__ __forceinline__ double fold_sum_abs(const Partial* records, uint32_t count, BlockFold<kWarps>& sh) {
+    const int lane = threadIdx.x & 31;
     double v = 0.0;
     for (uint32_t b = threadIdx.x; b < count; b += kThreads) v += records[b].sum_abs;
     v = warp_sum(v);
-    if ((threadIdx.x & 31) == 0) sh.d[0][threadIdx.x >> 5] = v;
+    if (lane == 0) sh.d[0][threadIdx.x >> 5] = v;
     __syncthreads();
-    double s = 0.0;
-#pragma unroll
-    for (int w = 0; w < kWarps; ++w) s += sh.d[0][w];
+    v = __shfl_sync(0xFFFFFFFFu, warp_sum<kWarps>(lane < kWarps ? sh.d[0][lane] : 0.0), 0);
     __syncthreads();
-    return s;
+    return v;
 }
 // Stores the tail fields of the block's record and says whether all of the job's have been stored (block-uniform).
 __device__ __forceinline__ bool last_of_job(Partial* record, const Partial& p, bool moments, uint32_t* ticket, uint32_t count, BlockFold<kWarps>& sh) {

@@ -253,3 +253,42 @@ def test_decision_table_of_layer_groups(tq, orc, bits, bad):
             elif s != 0 or i == 2:
                 assert np.array_equal(part, orc.compress(g[i, o:o + ln].float().cpu().numpy(), _oracle_params(orc, ps[j]), 21, i)), (s, i)
         w += words
+
+
+def test_two_pass_threshold_is_one_number(tq):
+    """The tail pass derives g_min = mean|g| in every block from the 512 block sums of the row.  Here the mean lies on the tie between
+    two fp32 numbers, and the order in which the warps' sums are added decides to which side it falls; 1 + 2^-23 stands in every
+    block, above the one threshold and not above the other.  Each block's sum is exact in fp64, so the sum over the blocks is the
+    tree's, bit for bit, and the tail holds all of those elements or none."""
+    T, P = 512, 1.0 + 2.0 ** -23
+
+    def fold(rec, tree):                                       # as one block of 256 threads adds the records
+        v = (rec[:256] + rec[256:]).reshape(8, 32)
+        for o in (16, 8, 4, 2, 1):
+            v = v[:, :o] + v[:, o:2 * o]
+        w = v[:, 0]
+        if tree:
+            for o in (4, 2, 1):
+                w = w[:o] + w[o:2 * o]
+            return float(w[0])
+        s = 0.0
+        for x in w:
+            s += float(x)
+        return s
+
+    r = np.random.default_rng(1)
+    large = np.full(T, 47.0 + 2.0 ** -12)
+    large[:16] -= 2.0 ** -18                                   # the blocks' sums without `small` add up to the tie, T * 4096 * (1 + 2^-24)
+    while True:
+        small = np.where(r.random(T) < 0.03, r.integers(1, 17, T), 0) * 2.0 ** -38
+        rec = 253 * 16 + P + large + small
+        tree, turn = fold(rec, True), fold(rec, False)
+        if np.float32(tree / (T * 4096)) != np.float32(turn / (T * 4096)):
+            break
+    x = np.ones((T, 256, 16), np.float32)                      # a block's tile: 256 chunks of 16
+    x[:, :3] = 0.0
+    x[:, 0, 0], x[:, 1, 0], x[:, 2, 0] = P, small, large
+    g = torch.from_numpy(x.reshape(-1)).cuda()
+    for st in (tq.stats_to_host(tq.tq_stats(g))[0], tq.stats_to_host(tq.tq_stats_segments(g, [(0, g.numel())]))[0]):
+        assert st.sum_abs == tree and st.g_min == float(np.float32(tree / (T * 4096)))
+        assert st.n_tail == T + (T if st.g_min == 1.0 else 0)
