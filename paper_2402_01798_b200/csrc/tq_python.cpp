@@ -40,6 +40,17 @@ struct Failed {};                              // a Python exception is set
     throw Failed();
 }
 
+// Calls the library with the interpreter lock released, as ctypes does: a launch may wait for room in a full queue, behind a host
+// callback that needs the lock.  Arguments are ready before; what they point to is held by the caller's arguments or by Args.
+template <class... P, class... A>
+tq_status call(tq_status (*f)(P...), const A&... args) {
+    struct Unlocked {
+        PyThreadState* state = PyEval_SaveThread();
+        ~Unlocked() { PyEval_RestoreThread(state); }
+    } unlocked;
+    return f(args...);
+}
+
 // One call's positional arguments, taken in order.
 class Args {
 public:
@@ -188,7 +199,7 @@ tq_status stats(Args& a) {                      // grad, d, g_min, kappa, stats,
     const float g_min = a.f32(), kappa = a.f32();
     void* st = a.address();
     const Scratch ws = scratch(a);
-    return F.stats(g.data, g.dtype, d, g.stride, g.n, g_min, kappa, static_cast<tq_stats_t*>(st), ws.data, ws.bytes, a.stream());
+    return call(F.stats, g.data, g.dtype, d, g.stride, g.n, g_min, kappa, static_cast<tq_stats_t*>(st), ws.data, ws.bytes, a.stream());
 }
 tq_status stats_hinted(Args& a) {               // grad, d, kappa, hint, stats, workspace, stream
     const Grad g = gradient(a);
@@ -197,7 +208,7 @@ tq_status stats_hinted(Args& a) {               // grad, d, kappa, hint, stats, 
     void* hint = a.address();
     void* st = a.address();
     const Scratch ws = scratch(a);
-    return F.stats_hinted(g.data, g.dtype, d, g.stride, g.n, kappa, static_cast<tq_gmin_hint_t*>(hint), static_cast<tq_stats_t*>(st), ws.data,
+    return call(F.stats_hinted, g.data, g.dtype, d, g.stride, g.n, kappa, static_cast<tq_gmin_hint_t*>(hint), static_cast<tq_stats_t*>(st), ws.data,
                           ws.bytes, a.stream());
 }
 tq_status stats_static(Args& a) {               // grad, d, g_min, kappa, stats, stream
@@ -205,7 +216,7 @@ tq_status stats_static(Args& a) {               // grad, d, g_min, kappa, stats,
     const uint64_t d = elements(a, g);
     const float g_min = a.f32(), kappa = a.f32();
     void* st = a.address();
-    return F.stats_static(g.data, g.dtype, d, g.stride, g.n, g_min, kappa, static_cast<tq_stats_t*>(st), a.stream());
+    return call(F.stats_static, g.data, g.dtype, d, g.stride, g.n, g_min, kappa, static_cast<tq_stats_t*>(st), a.stream());
 }
 tq_status params_batch(Args& a) {               // address of the records, n, num_levels, mode, gamma, rule, alpha_user, out
     PyObject* src = a.next();
@@ -215,7 +226,7 @@ tq_status params_batch(Args& a) {               // address of the records, n, nu
     const double gamma = a.f64();
     const uint32_t rule = a.u32();
     const double alpha = a.f64();
-    return F.params_batch(static_cast<const tq_stats_t*>(records), n, levels, static_cast<tq_mode>(mode), gamma, static_cast<tq_alpha_rule>(rule),
+    return call(F.params_batch, static_cast<const tq_stats_t*>(records), n, levels, static_cast<tq_mode>(mode), gamma, static_cast<tq_alpha_rule>(rule),
                           alpha, static_cast<tq_params_t*>(a.buffer()));
 }
 tq_status params_device(Args& a) {              // stats, n, num_levels, mode, gamma, rule, alpha_user, params, stream
@@ -225,7 +236,7 @@ tq_status params_device(Args& a) {              // stats, n, num_levels, mode, g
     const uint32_t rule = a.u32();
     const double alpha = a.f64();
     void* out = a.address();
-    return F.params_device(static_cast<tq_stats_t*>(st), n, levels, static_cast<tq_mode>(mode), gamma, static_cast<tq_alpha_rule>(rule), alpha,
+    return call(F.params_device, static_cast<tq_stats_t*>(st), n, levels, static_cast<tq_mode>(mode), gamma, static_cast<tq_alpha_rule>(rule), alpha,
                            static_cast<tq_params_t*>(out), a.stream());
 }
 tq_status compress(Args& a) {                   // grad, d, params, seed, first_worker, packed, stream
@@ -235,7 +246,7 @@ tq_status compress(Args& a) {                   // grad, d, params, seed, first_
     const uint64_t seed = a.u64();
     const uint32_t first = a.u32();
     const Packed p = packed_out(a, g.n);
-    return F.compress(g.data, g.dtype, d, g.stride, g.n, params, seed, first, p.data, p.stride, a.stream());
+    return call(F.compress, g.data, g.dtype, d, g.stride, g.n, params, seed, first, p.data, p.stride, a.stream());
 }
 tq_status compress_device_params(Args& a) {     // grad, d, params, num_levels, mode, seed, first_worker, packed, stream
     const Grad g = gradient(a);
@@ -245,7 +256,7 @@ tq_status compress_device_params(Args& a) {     // grad, d, params, num_levels, 
     const uint64_t seed = a.u64();
     const uint32_t first = a.u32();
     const Packed p = packed_out(a, g.n);
-    return F.compress_device_params(g.data, g.dtype, d, g.stride, g.n, static_cast<tq_params_t*>(params), levels, static_cast<tq_mode>(mode), seed,
+    return call(F.compress_device_params, g.data, g.dtype, d, g.stride, g.n, static_cast<tq_params_t*>(params), levels, static_cast<tq_mode>(mode), seed,
                                     first, p.data, p.stride, a.stream());
 }
 tq_status decompress_aggregate(Args& a) {       // packed, d, params, weights, out, stream
@@ -256,7 +267,7 @@ tq_status decompress_aggregate(Args& a) {       // packed, d, params, weights, o
     const tq_params_t* params = host_params(a, p.n);
     const float* w = a.weights(p.n);
     void* out = a.address();
-    return F.decompress_aggregate(p.data, p.stride, p.n, d, params, w, static_cast<float*>(out), a.stream());
+    return call(F.decompress_aggregate, p.data, p.stride, p.n, d, params, w, static_cast<float*>(out), a.stream());
 }
 tq_status decompress_aggregate_rows(Args& a) {  // rows (tensors or addresses), d, params, weights, out, stream
     PyObject* seq = PySequence_Fast(a.next(), "rows must be a sequence");
@@ -274,7 +285,7 @@ tq_status decompress_aggregate_rows(Args& a) {  // rows (tensors or addresses), 
     if (n > TQ_MAX_WORKERS) return TQ_ERR_INVALID_ARG;
     const float* w = a.weights(static_cast<uint32_t>(n));
     void* out = a.address();
-    return F.decompress_aggregate_rows(rows, static_cast<uint32_t>(n), d, params, w, static_cast<float*>(out), a.stream());
+    return call(F.decompress_aggregate_rows, rows, static_cast<uint32_t>(n), d, params, w, static_cast<float*>(out), a.stream());
 }
 tq_status decompress_aggregate_apply(Args& a) { // packed, d, params, weights, theta, momentum, lr, mu, weight_decay, stream
     const Packed p = packed_rows(a.tensor());
@@ -284,7 +295,7 @@ tq_status decompress_aggregate_apply(Args& a) { // packed, d, params, weights, t
     void* theta = a.address();
     void* momentum = a.address();
     const float lr = a.f32(), mu = a.f32(), wd = a.f32();
-    return F.decompress_aggregate_apply(p.data, p.stride, p.n, d, params, w, static_cast<float*>(theta), static_cast<float*>(momentum), lr, mu, wd,
+    return call(F.decompress_aggregate_apply, p.data, p.stride, p.n, d, params, w, static_cast<float*>(theta), static_cast<float*>(momentum), lr, mu, wd,
                                         a.stream());
 }
 tq_status decompress_aggregate_device_params(Args& a) {      // packed, d, params, num_levels, weights, out, stream
@@ -294,7 +305,7 @@ tq_status decompress_aggregate_device_params(Args& a) {      // packed, d, param
     const uint32_t levels = a.u32();
     const float* w = a.weights(p.n);
     void* out = a.address();
-    return F.decompress_aggregate_device_params(p.data, p.stride, p.n, d, static_cast<tq_params_t*>(params), levels, w, static_cast<float*>(out),
+    return call(F.decompress_aggregate_device_params, p.data, p.stride, p.n, d, static_cast<tq_params_t*>(params), levels, w, static_cast<float*>(out),
                                                 a.stream());
 }
 tq_status stats_segments(Args& a) {             // grad, segments, g_min, kappa, stats, workspace, stream
@@ -304,7 +315,7 @@ tq_status stats_segments(Args& a) {             // grad, segments, g_min, kappa,
     const float g_min = a.f32(), kappa = a.f32();
     void* st = a.address();
     const Scratch ws = scratch(a);
-    return F.stats_segments(g.data, g.dtype, g.stride, g.n, seg, n_seg, g_min, kappa, static_cast<tq_stats_t*>(st), ws.data, ws.bytes, a.stream());
+    return call(F.stats_segments, g.data, g.dtype, g.stride, g.n, seg, n_seg, g_min, kappa, static_cast<tq_stats_t*>(st), ws.data, ws.bytes, a.stream());
 }
 tq_status stats_hinted_segments(Args& a) {      // grad, segments, kappa, hint, stats, workspace, stream
     const Grad g = gradient(a);
@@ -314,7 +325,7 @@ tq_status stats_hinted_segments(Args& a) {      // grad, segments, kappa, hint, 
     void* hint = a.address();
     void* st = a.address();
     const Scratch ws = scratch(a);
-    return F.stats_hinted_segments(g.data, g.dtype, g.stride, g.n, seg, n_seg, kappa, static_cast<tq_gmin_hint_t*>(hint), static_cast<tq_stats_t*>(st),
+    return call(F.stats_hinted_segments, g.data, g.dtype, g.stride, g.n, seg, n_seg, kappa, static_cast<tq_gmin_hint_t*>(hint), static_cast<tq_stats_t*>(st),
                                    ws.data, ws.bytes, a.stream());
 }
 tq_status compress_segments(Args& a) {          // grad, segments, params, num_levels, mode, seed, first_worker, packed, stream
@@ -326,7 +337,7 @@ tq_status compress_segments(Args& a) {          // grad, segments, params, num_l
     const uint64_t seed = a.u64();
     const uint32_t first = a.u32();
     const Packed p = packed_out(a, g.n);
-    return F.compress_segments(g.data, g.dtype, g.stride, g.n, seg, n_seg, static_cast<tq_params_t*>(params), levels, static_cast<tq_mode>(mode), seed,
+    return call(F.compress_segments, g.data, g.dtype, g.stride, g.n, seg, n_seg, static_cast<tq_params_t*>(params), levels, static_cast<tq_mode>(mode), seed,
                                first, p.data, p.stride, a.stream());
 }
 tq_status decompress_aggregate_segments(Args& a) {           // packed, segments, params, num_levels, weights, out, stream
@@ -337,7 +348,7 @@ tq_status decompress_aggregate_segments(Args& a) {           // packed, segments
     const uint32_t levels = a.u32();
     const float* w = a.weights(p.n);
     void* out = a.address();
-    return F.decompress_aggregate_segments(p.data, p.stride, p.n, seg, n_seg, static_cast<tq_params_t*>(params), levels, w, static_cast<float*>(out),
+    return call(F.decompress_aggregate_segments, p.data, p.stride, p.n, seg, n_seg, static_cast<tq_params_t*>(params), levels, w, static_cast<float*>(out),
                                            a.stream());
 }
 

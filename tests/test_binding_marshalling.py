@@ -1,4 +1,8 @@
 """What the compiled marshalling module refuses before any library call (no GPU needed)."""
+import ctypes
+import subprocess
+import threading
+
 import pytest
 import torch
 
@@ -89,3 +93,35 @@ def test_weights_of_more_rows_than_the_library_takes_in_a_block(tq):
     with pytest.raises(tq.TqError) as e:
         tq.tq_decompress_aggregate(torch.zeros((65, 4), dtype=torch.int32, device="cuda"), 16, [p] * 65, weights=[0.1] * 65)
     assert e.value.status == tq.ERR_INVALID_ARG
+
+
+def test_other_threads_run_while_the_library_works(tq, tmp_path):
+    """A call may last: a launch waits for room in a full queue, the parameter design of 64 records takes its time.  With a library
+    function that sleeps 0.2 s in place of each of the library's, another thread goes on meanwhile."""
+    (tmp_path / "slow.c").write_text("#include <unistd.h>\nint slow(void) { usleep(200000); return 0; }\n")
+    subprocess.run(["gcc", "-shared", "-fPIC", "-o", str(tmp_path / "slow.so"), str(tmp_path / "slow.c")], check=True)
+    slow = ctypes.CDLL(str(tmp_path / "slow.so"))
+    native, at = tq._calls(), lambda f: ctypes.cast(f, ctypes.c_void_p).value
+    buf, p = torch.zeros(1024, dtype=torch.int32), tq.params_array([tq.tq_params_from_levels([-1.0, 1.0])])
+    packed, seg = buf.view(1, 1024), tq.segments_array([(0, 16)])
+    calls = {"params_batch": (buf, 1, 16, 1, 3.0, 1, 0.0, p), "params_device": (buf, 1, 16, 1, 3.0, 1, 0.0, buf, 0),
+             "decompress_aggregate_rows": ([buf], 16, p, None, buf, 0), "decompress_aggregate_apply": (packed, 16, p, [1.0], buf, None, 0.1, 0.9, 0.0, 0),
+             "decompress_aggregate_device_params": (packed, 16, buf, 2, None, buf, 0), "decompress_aggregate_segments": (packed, seg, buf, 2, None, buf, 0)}
+    ticks, stop = [0], threading.Event()
+
+    def count():
+        while not stop.wait(0.002):
+            ticks[0] += 1
+
+    other = threading.Thread(target=count)
+    other.start()
+    native.bind([at(slow.slow)] * len(tq._NATIVE))
+    try:
+        for name, args in calls.items():
+            before = ticks[0]
+            assert getattr(native, name)(*args) == tq.OK
+            assert ticks[0] - before >= 10, name
+    finally:
+        native.bind([at(getattr(tq.lib(), name)) for name in tq._NATIVE])
+        stop.set()
+        other.join()
