@@ -94,11 +94,11 @@ public:
         return v;
     }
     float f32() { return static_cast<float>(f64()); }
-    // None: torch's current stream; else a stream object or a raw handle
+    // None: torch's current stream; else a stream object, or a raw handle: anything that int() takes (other libraries' handles do)
     void* stream() {
         PyObject* o = next();
         if (o == Py_None) return c10::cuda::getCurrentCUDAStream().stream();
-        PyObject* handle = PyObject_HasAttrString(o, "cuda_stream") ? PyObject_GetAttrString(o, "cuda_stream") : (Py_INCREF(o), o);
+        PyObject* handle = PyObject_HasAttrString(o, "cuda_stream") ? PyObject_GetAttrString(o, "cuda_stream") : PyNumber_Long(o);
         if (!handle) throw Failed();
         void* s = PyLong_AsVoidPtr(handle);
         Py_DECREF(handle);

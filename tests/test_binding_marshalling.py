@@ -3,6 +3,7 @@ import ctypes
 import subprocess
 import threading
 
+import numpy as np
 import pytest
 import torch
 
@@ -125,3 +126,18 @@ def test_other_threads_run_while_the_library_works(tq, tmp_path):
         native.bind([at(getattr(tq.lib(), name)) for name in tq._NATIVE])
         stop.set()
         other.join()
+
+
+def test_stream_handles(tq):
+    """A raw handle may be anything that int() takes: numpy integers, the handle objects of other libraries."""
+    class Handle:
+        def __int__(self):
+            return 0
+
+    p, out = tq.tq_params_from_levels([-1.0, 1.0]), torch.zeros(16)
+    for stream in (0, np.int64(0), np.uint64(0), Handle()):
+        with pytest.raises(tq.TqError) as e:
+            tq.tq_decompress_aggregate_rows([20], 16, [p], out=out, stream=stream)
+        assert e.value.status == tq.ERR_ALIGNMENT
+    with pytest.raises(TypeError):
+        tq.tq_decompress_aggregate_rows([20], 16, [p], out=out, stream=object())
