@@ -51,6 +51,20 @@ tq_status call(tq_status (*f)(P...), const A&... args) {
     return f(args...);
 }
 
+// Device address of a tensor, or of anything else with a data_ptr() (a storage, say).
+void* address_of(PyObject* o) {
+    if (THPVariable_Check(o)) return THPVariable_Unpack(o).data_ptr();
+    PyObject* v = PyObject_CallMethod(o, "data_ptr", nullptr);
+    if (!v) {
+        if (PyErr_ExceptionMatches(PyExc_AttributeError)) fail(PyExc_TypeError, "a tensor is needed");
+        throw Failed();
+    }
+    void* p = PyLong_AsVoidPtr(v);
+    Py_DECREF(v);
+    if (PyErr_Occurred()) throw Failed();
+    return p;
+}
+
 // One call's positional arguments, taken in order.
 class Args {
 public:
@@ -68,12 +82,9 @@ public:
         if (!THPVariable_Check(o)) fail(PyExc_TypeError, "a tensor is needed");
         return THPVariable_Unpack(o);
     }
-    // device address of a tensor, or nullptr for None
-    void* address() {
+    void* address() {                          // nullptr for None
         PyObject* o = next();
-        if (o == Py_None) return nullptr;
-        if (!THPVariable_Check(o)) fail(PyExc_TypeError, "a tensor is needed");
-        return THPVariable_Unpack(o).data_ptr();
+        return o == Py_None ? nullptr : address_of(o);
     }
     // a ctypes array (or anything else with a buffer): its address and size
     void* buffer(Py_ssize_t* bytes = nullptr) {
@@ -274,12 +285,17 @@ tq_status decompress_aggregate_rows(Args& a) {  // rows (tensors or addresses), 
     if (!seq) throw Failed();
     const uint32_t* rows[TQ_MAX_WORKERS];
     const Py_ssize_t n = PySequence_Fast_GET_SIZE(seq);
-    for (Py_ssize_t i = 0; i < n && i < TQ_MAX_WORKERS; ++i) {
-        PyObject* r = PySequence_Fast_GET_ITEM(seq, i);
-        rows[i] = static_cast<const uint32_t*>(THPVariable_Check(r) ? THPVariable_Unpack(r).data_ptr() : PyLong_AsVoidPtr(r));
+    try {
+        for (Py_ssize_t i = 0; i < n && i < TQ_MAX_WORKERS; ++i) {
+            PyObject* r = PySequence_Fast_GET_ITEM(seq, i);
+            rows[i] = static_cast<const uint32_t*>(PyLong_Check(r) ? PyLong_AsVoidPtr(r) : address_of(r));
+            if (PyErr_Occurred()) throw Failed();
+        }
+    } catch (...) {
+        Py_DECREF(seq);
+        throw;
     }
     Py_DECREF(seq);
-    if (PyErr_Occurred()) throw Failed();
     const uint64_t d = a.u64();
     const tq_params_t* params = host_params(a, static_cast<uint32_t>(n));
     if (n > TQ_MAX_WORKERS) return TQ_ERR_INVALID_ARG;

@@ -141,3 +141,21 @@ def test_stream_handles(tq):
         assert e.value.status == tq.ERR_ALIGNMENT
     with pytest.raises(TypeError):
         tq.tq_decompress_aggregate_rows([20], 16, [p], out=out, stream=object())
+
+
+def test_objects_with_an_address(tq):
+    """Buffers that are not typed by a tensor: whatever has a data_ptr(), a storage for one."""
+    class Buffer:
+        def __init__(self, at):
+            self.data_ptr = lambda: at
+
+    p, t = tq.tq_params_from_levels([-1.0, 1.0]), torch.zeros(64)
+    for call in (lambda: tq.tq_decompress_aggregate_rows([Buffer(20)], 16, [p], out=t, stream=0),
+                 lambda: tq.tq_decompress_aggregate_rows([16], 16, [p], out=Buffer(16), stream=0),
+                 lambda: tq.tq_params_device(Buffer(4), 1, 4, 0, 3.0, params_dev=t.untyped_storage(), stream=0)):
+        with pytest.raises(tq.TqError) as e:
+            call()
+        assert e.value.status == tq.ERR_ALIGNMENT
+    for bad in (object(), "text", 1.5):
+        with pytest.raises(TypeError):
+            tq.tq_decompress_aggregate_rows([bad], 16, [p], out=t, stream=0)
