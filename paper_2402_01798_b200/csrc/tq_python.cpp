@@ -116,7 +116,7 @@ public:
         if (PyErr_Occurred()) throw Failed();
         return s;
     }
-    // None, or up to n numbers, the rest zeros.  Only the first TQ_MAX_WORKERS are kept: the library refuses more rows before
+    // None, or up to n values that float() takes, the rest zeros.  Only the first TQ_MAX_WORKERS are kept: the library refuses more rows before
     // it reads a weight.
     const float* weights(uint32_t n) {
         PyObject* o = next();
@@ -124,9 +124,11 @@ public:
         PyObject* seq = PySequence_Fast(o, "weights must be a sequence of numbers");
         if (!seq) throw Failed();
         const Py_ssize_t have = PySequence_Fast_GET_SIZE(seq);
-        for (Py_ssize_t i = 0; i < have && !PyErr_Occurred(); ++i) {
-            const float w = static_cast<float>(PyFloat_AsDouble(PySequence_Fast_GET_ITEM(seq, i)));
-            if (i < TQ_MAX_WORKERS) weights_[i] = w;
+        for (Py_ssize_t i = 0; i < have; ++i) {
+            PyObject* w = PyNumber_Float(PySequence_Fast_GET_ITEM(seq, i));
+            if (!w) break;
+            if (i < TQ_MAX_WORKERS) weights_[i] = static_cast<float>(PyFloat_AS_DOUBLE(w));
+            Py_DECREF(w);
         }
         Py_DECREF(seq);
         if (PyErr_Occurred()) throw Failed();
@@ -186,10 +188,11 @@ Packed packed_out(Args& a, uint32_t n) {        // as many rows as the gradient 
     const bool rows = t.dim() == 2 && n > 1;
     return Packed{static_cast<uint32_t*>(t.data_ptr()), static_cast<size_t>(rows ? t.stride(0) : t.size(t.dim() - 1)), n};
 }
-const tq_params_t* host_params(Args& a, uint32_t n) {
+const tq_params_t* host_params(Args& a, uint32_t n, bool or_more = false) {
     Py_ssize_t bytes = 0;
     void* p = a.buffer(&bytes);
-    if (bytes != static_cast<Py_ssize_t>(n * sizeof(tq_params_t))) fail(PyExc_ValueError, "one Params per worker");
+    const Py_ssize_t need = static_cast<Py_ssize_t>(n * sizeof(tq_params_t));
+    if (or_more ? bytes < need : bytes != need) fail(PyExc_ValueError, "one Params per worker");
     return static_cast<const tq_params_t*>(p);
 }
 const tq_segment_t* segments(Args& a, uint32_t* n) {
@@ -306,7 +309,7 @@ tq_status decompress_aggregate_rows(Args& a) {  // rows (tensors or addresses), 
 tq_status decompress_aggregate_apply(Args& a) { // packed, d, params, weights, theta, momentum, lr, mu, weight_decay, stream
     const Packed p = packed_rows(a.tensor());
     const uint64_t d = a.u64();
-    const tq_params_t* params = host_params(a, p.n);
+    const tq_params_t* params = host_params(a, p.n, true);
     const float* w = a.weights(p.n);
     void* theta = a.address();
     void* momentum = a.address();

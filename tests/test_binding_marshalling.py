@@ -159,3 +159,18 @@ def test_objects_with_an_address(tq):
     for bad in (object(), "text", 1.5):
         with pytest.raises(TypeError):
             tq.tq_decompress_aggregate_rows([bad], 16, [p], out=t, stream=0)
+
+
+def test_records_and_weights_of_the_fused_update(tq):
+    """The fused update takes the records of a larger job for its first rows, but not too few; weights are what float() takes."""
+    p, t = tq.tq_params_from_levels([-1.0, 1.0]), torch.zeros(64)
+    packed = torch.zeros(9, dtype=torch.int32)
+    packed = packed[(-packed.data_ptr() // 4) % 4 + 1:][:4].view(1, 4)                        # misaligned: the library's check answers
+    for params, weights in (([p], None), ([p, p, p], None), ((tq.Params * 2)(p, p), [np.float32(1)]), ([p], ["0.5"]), ([p], torch.ones(1)), ([p], (w for w in [1]))):
+        with pytest.raises(tq.TqError) as e:
+            tq.tq_decompress_aggregate_apply(packed, 16, params, t, None, lr=0.1, weights=weights, stream=0)
+        assert e.value.status == tq.ERR_ALIGNMENT
+    with pytest.raises(ValueError, match="one Params per worker"):
+        tq.tq_decompress_aggregate_apply(packed, 16, [], t, None, lr=0.1, stream=0)
+    with pytest.raises(ValueError):
+        tq.tq_decompress_aggregate_apply(packed, 16, [p], t, None, lr=0.1, weights=["half"], stream=0)
