@@ -68,7 +68,7 @@ class Segment(C.Structure):
 
 def lib() -> C.CDLL:
     """Load libtq.so.  There is no fallback: a missing library is an error."""
-    global _lib, _native
+    global _lib
     if _lib is None:
         if not os.path.exists(LIB_PATH):
             raise RuntimeError(
@@ -114,7 +114,6 @@ def lib() -> C.CDLL:
         L.tq_last_cuda_error.restype = C.c_int
         L.tq_kernel_launches.restype = u64
         L.tq_wait_expired_count.argtypes = [C.POINTER(u32)]; L.tq_wait_expired_count.restype = C.c_int
-        _native = _load_native(L)
         _lib = L
     return _lib
 
@@ -127,6 +126,11 @@ _NATIVE = ("tq_stats", "tq_stats_hinted", "tq_stats_static", "tq_params_batch", 
 
 
 def _load_native(L: C.CDLL):
+    from . import build
+    built_for = build.native_torch()
+    if built_for not in (None, str(torch.__version__)):
+        raise RuntimeError(f"the compiled marshalling module was built against torch {built_for}, this is {torch.__version__}: "
+                           "build it again with `python -m paper_2402_01798_b200.build`")
     try:
         from . import _tq_python
     except ImportError as e:
@@ -137,8 +141,10 @@ def _load_native(L: C.CDLL):
 
 
 def _calls():
+    """The compiled module, loaded by the first call that needs it: the host-side calls do without."""
+    global _native
     if _native is None:
-        lib()
+        _native = _load_native(lib())
     return _native
 
 

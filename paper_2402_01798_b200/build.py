@@ -12,6 +12,7 @@ CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libtq.so")
 NATIVE = os.path.join(PKG, "_tq_python" + sysconfig.get_config_var("EXT_SUFFIX"))
 NATIVE_SOURCE = os.path.join(CSRC, "tq_python.cpp")
+NATIVE_TORCH = os.path.join(PKG, "_tq_python.torch")       # the torch version that the module was built against: its C++ interface changes
 SOURCES = ["tq_api.cu", "tq_stats.cu", "tq_compress.cu", "tq_compress_lut.cu", "tq_decompress.cu", "tq_params.cu"]
 HEADERS = ["tq_aggregation_plan.h", "tq_device.cuh", "tq_launch.h", "tq_lut.cuh"]
 
@@ -38,11 +39,19 @@ def _run(cmd, verbose: bool, what: str) -> None:
         raise RuntimeError(f"building {what} failed")
 
 
+def native_torch():
+    """The torch version that the marshalling module was built against, None if that was not written down."""
+    if not os.path.exists(NATIVE_TORCH):
+        return None
+    with open(NATIVE_TORCH) as f:
+        return f.read().strip()
+
+
 def build_native(force: bool = False, verbose: bool = False) -> str:
     """The marshalling module: C++ against torch's and Python's headers."""
-    if not force and not _stale(NATIVE, [NATIVE_SOURCE]):
-        return NATIVE
     import torch
+    if not force and native_torch() == torch.__version__ and not _stale(NATIVE, [NATIVE_SOURCE]):
+        return NATIVE
     base = os.path.dirname(torch.__file__)
     inc = [os.path.join(base, "include"), os.path.join(base, "include", "torch", "csrc", "api", "include"),
            sysconfig.get_paths()["include"], os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include"), os.path.join(ROOT, "include")]
@@ -52,6 +61,8 @@ def build_native(force: bool = False, verbose: bool = False) -> str:
           *[f"-I{p}" for p in inc], NATIVE_SOURCE, "-o", tmp, f"-L{libs}", f"-Wl,-rpath,{libs}", "-ltorch_python", "-ltorch_cpu", "-lc10_cuda", "-lc10"],
          verbose, os.path.basename(NATIVE))
     os.replace(tmp, NATIVE)
+    with open(NATIVE_TORCH, "w") as f:
+        f.write(torch.__version__)
     return NATIVE
 
 

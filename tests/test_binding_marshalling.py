@@ -1,6 +1,7 @@
 """What the compiled marshalling module refuses before any library call (no GPU needed)."""
 import ctypes
 import subprocess
+import sys
 import threading
 
 import numpy as np
@@ -174,3 +175,33 @@ def test_records_and_weights_of_the_fused_update(tq):
         tq.tq_decompress_aggregate_apply(packed, 16, [], t, None, lr=0.1, stream=0)
     with pytest.raises(ValueError):
         tq.tq_decompress_aggregate_apply(packed, 16, [p], t, None, lr=0.1, weights=["half"], stream=0)
+
+
+def test_host_calls_do_without_the_compiled_module(tq, monkeypatch):
+    """The parameter design and the sizes go through ctypes; only a call of a round asks for the module, and says what to do."""
+    monkeypatch.setattr(tq, "_native", None)
+    monkeypatch.setattr(tq, "_lib", None)
+    monkeypatch.delattr("paper_2402_01798_b200._tq_python")
+    monkeypatch.setitem(sys.modules, "paper_2402_01798_b200._tq_python", None)                # an import fails
+    assert tq.tq_params_from_levels([-1.0, 1.0]).bits == 1 and tq.tq_packed_words(100, 3) == 12
+    with pytest.raises(RuntimeError, match="paper_2402_01798_b200.build"):
+        tq.tq_params_batch(b"\0" * 64, 1, 4, tq.UNIFORM, 3.0)
+
+
+def test_module_of_another_torch(tq, monkeypatch, tmp_path):
+    """torch's C++ interface changes between versions: a module of another one is refused, and built again by the next build."""
+    from paper_2402_01798_b200 import build
+    monkeypatch.setattr(tq, "_native", None)
+    monkeypatch.setattr(build, "NATIVE_TORCH", str(tmp_path / "version"))
+    ran = []
+    monkeypatch.setattr(build, "_run", lambda cmd, verbose, what: (ran.append(what), open(cmd[cmd.index("-o") + 1], "w").close()))
+    monkeypatch.setattr(build.os, "replace", lambda a, b: build.os.unlink(a))
+    (tmp_path / "version").write_text("1.0.0")
+    with pytest.raises(RuntimeError, match="torch 1.0.0"):
+        tq.tq_params_batch(b"\0" * 64, 1, 4, tq.UNIFORM, 3.0)
+    build.build_native()
+    assert len(ran) == 1 and build.native_torch() == torch.__version__
+    build.build_native()
+    assert len(ran) == 1
+    with pytest.raises(tq.TqError):
+        tq.tq_params_batch(b"\0" * 64, 1, 4, tq.UNIFORM, 3.0)
