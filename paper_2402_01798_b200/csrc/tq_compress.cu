@@ -599,7 +599,7 @@ __device__ __noinline__ void compress_piece_rare(State& sh, const void* grad, ui
 // Rows of jobs that are marked invalid (alpha = 0) become all code 0.
 template <int BITS, bool NONUNIFORM, bool BF16>
 __global__ void __launch_bounds__(kThreads, TQ_COMPRESS_MIN_BLOCKS)
-compress_kernel_dev(const void* __restrict__ grad, uint64_t grad_stride, const tq_params_t* __restrict__ params,
+compress_kernel_dev(const void* __restrict__ grad, uint64_t grad_stride, const tq_params_t* params,
                     const __grid_constant__ RoundKeys rk, uint32_t first_worker, uint32_t* __restrict__ packed, uint64_t words_stride,
                     const __grid_constant__ TilePlan plan, int table_kernel_ran) {
     __shared__ __align__(16) BlockState<NONUNIFORM> sh;

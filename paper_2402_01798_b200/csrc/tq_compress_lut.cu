@@ -211,7 +211,7 @@ __device__ __forceinline__ void lut_block(const LutWorker& q, uint32_t n_entries
 #pragma unroll
         for (int i = 0; i < E / 2; ++i) {
             const uint64_t j = row_interior * E + 2 * i;
-            const uint32_t lo = j < d ? __ldg(e + j) : 0u, hi = j + 1 < d ? __ldg(e + j + 1) : 0u;
+            const uint32_t lo = j < d ? ldg16(e + j) : 0u, hi = j + 1 < d ? ldg16(e + j + 1) : 0u;
             t[i] = lo | (hi << 16);
         }
         lut_piece<BITS, true>(t, prow, row_interior, d, words_out, rk, cx);
@@ -269,7 +269,7 @@ __device__ __forceinline__ uint32_t lut_record(const tq_params_t& rec, LutState&
 
 template <int BITS>
 __global__ void __launch_bounds__(kLutThreads, 1)
-compress_lut_kernel_dev(const void* __restrict__ grad, uint64_t d, uint64_t grad_stride, const tq_params_t* __restrict__ params,
+compress_lut_kernel_dev(const void* __restrict__ grad, uint64_t d, uint64_t grad_stride, const tq_params_t* params,
                         const __grid_constant__ RoundKeys rk, uint32_t first_worker, uint32_t* __restrict__ packed,
                         uint64_t words_stride, uint64_t words_out) {
     extern __shared__ __align__(16) float s_table[];          // 2 * kLutMaxEntries
@@ -286,7 +286,7 @@ compress_lut_kernel_dev(const void* __restrict__ grad, uint64_t d, uint64_t grad
 // Layer groups: a block's range of the jobs' tiles (kLutThreads pieces each), a table for every piece of a job.
 template <int BITS>
 __global__ void __launch_bounds__(kLutThreads, 1)
-compress_lut_kernel_segs(const void* __restrict__ grad, uint64_t grad_stride, const tq_params_t* __restrict__ params,
+compress_lut_kernel_segs(const void* __restrict__ grad, uint64_t grad_stride, const tq_params_t* params,
                          const __grid_constant__ RoundKeys rk, uint32_t first_worker, uint32_t* __restrict__ packed, uint64_t words_stride,
                          const __grid_constant__ TilePlan plan) {
     extern __shared__ __align__(16) float s_table[];          // 2 * kLutMaxEntries

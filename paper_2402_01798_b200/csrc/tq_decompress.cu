@@ -64,7 +64,7 @@ __device__ __forceinline__ uint32_t load_field(const uint32_t* row, uint64_t u) 
     else {
         const uint64_t wi = (3 * u) >> 2;                      // 24 u bits = 3 u bytes into the row
         const uint32_t sh = (static_cast<uint32_t>(u) * 24u) & 31u;
-        const uint32_t lo = __ldg(row + wi), hi = __ldg(row + wi + 1);   // cached: neighbours share words
+        const uint32_t lo = ldg32(row + wi), hi = ldg32(row + wi + 1);   // cached: neighbours share words
         return __funnelshift_r(lo, hi, sh);
     }
 }
@@ -75,8 +75,8 @@ __device__ __forceinline__ uint32_t load_field_guarded(const uint32_t* row, uint
     else {
         const uint64_t wi = (3 * u) >> 2;
         const uint32_t sh = (static_cast<uint32_t>(u) * 24u) & 31u;
-        const uint32_t lo = wi < words_valid ? __ldg(row + wi) : 0u;
-        const uint32_t hi = wi + 1 < words_valid ? __ldg(row + wi + 1) : 0u;
+        const uint32_t lo = wi < words_valid ? ldg32(row + wi) : 0u;
+        const uint32_t hi = wi + 1 < words_valid ? ldg32(row + wi + 1) : 0u;
         return __funnelshift_r(lo, hi, sh);
     }
 }

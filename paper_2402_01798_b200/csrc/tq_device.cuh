@@ -13,7 +13,9 @@ constexpr float kMagic = 8388608.0f;          // 2^23: adding it leaves an integ
 constexpr uint32_t kMagicBits = 0x4B000000u;  // bit pattern of 2^23
 
 // The kernel before this one on the stream is complete and its writes are visible; the next one may be set up.  Nothing
-// before this may touch global memory.
+// before this may touch global memory, and nothing may let the compiler move a load up to there: what other kernels write is read
+// through volatile asm, or through pointers that make no promise (const together with __restrict__, like __ldg, says that the
+// data does not change while the kernel runs, and an early start begins while it still does).
 __device__ __forceinline__ void pdl_wait() {
     asm volatile("griddepcontrol.wait;\n\tgriddepcontrol.launch_dependents;" ::: "memory");
 }
@@ -80,11 +82,18 @@ __device__ __forceinline__ void set_elem(Raw8<BF16>& r, int e, float x) {   // f
                                : ((r.v[e >> 1] & 0xFFFF0000u) | (__float_as_uint(x) >> 16));
 }
 
+// Single words, any alignment of the run they belong to.
+__device__ __forceinline__ uint32_t ldg32(const void* p) {
+    uint32_t v; asm volatile("ld.global.nc.b32 %0, [%1];" : "=r"(v) : "l"(p)); return v;
+}
+__device__ __forceinline__ uint32_t ldg16(const void* p) {
+    unsigned short v; asm volatile("ld.global.nc.b16 %0, [%1];" : "=h"(v) : "l"(p)); return v;
+}
 // One element, any alignment (ragged tails).
 template <bool BF16>
 __device__ __forceinline__ float load1(const void* base, uint64_t j) {
-    if constexpr (!BF16) return __ldg(reinterpret_cast<const float*>(base) + j);
-    else return __uint_as_float(static_cast<uint32_t>(__ldg(reinterpret_cast<const unsigned short*>(base) + j)) << 16);
+    if constexpr (!BF16) return __uint_as_float(ldg32(static_cast<const float*>(base) + j));
+    else return __uint_as_float(ldg16(static_cast<const unsigned short*>(base) + j) << 16);
 }
 
 // ---- asynchronous copies into shared memory, counted on an mbarrier ----------------------------------

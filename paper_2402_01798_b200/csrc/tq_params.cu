@@ -424,8 +424,8 @@ static bool valid_request(uint32_t num_levels, int mode, int rule, uint32_t* bit
 constexpr int kParamsWarps = 4;
 template <uint32_t MODE>
 __global__ void __launch_bounds__(32 * kParamsWarps)
-params_kernel(const tq_stats_t* __restrict__ stats, uint32_t n, uint32_t num_levels, uint32_t bits, double gamma, int rule,
-              double alpha_user, tq_params_t* __restrict__ out) {
+params_kernel(const tq_stats_t* stats, uint32_t n, uint32_t num_levels, uint32_t bits, double gamma, int rule,
+              double alpha_user, tq_params_t* out) {
     __shared__ tq_params_t s_p[kParamsWarps];
     const uint32_t warp = threadIdx.x >> 5, i = blockIdx.x * kParamsWarps + warp;
     if (i >= n) return;              // nothing of this warp reads or writes memory
