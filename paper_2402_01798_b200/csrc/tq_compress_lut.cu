@@ -324,7 +324,8 @@ static uint32_t entries_needed(const tq_params_t& p, uint32_t top) {
 template <int BITS>
 static cudaError_t launch_lut(const CompressCall& c, const LutArgs& args, uint32_t n_entries, uint32_t per_worker) {
     const int smem = static_cast<int>((kLutMaxEntries + n_entries) * sizeof(float));
-    cudaError_t e = cudaFuncSetAttribute(compress_lut_kernel<BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    // always the same limit: another thread may set it between this call's and the launch
+    const cudaError_t e = cudaFuncSetAttribute(compress_lut_kernel<BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * kLutMaxEntries * static_cast<int>(sizeof(float)));
     if (e != cudaSuccess) return e;
     return launch_kernel(compress_lut_kernel<BITS>, dim3(per_worker, c.n_workers), kLutThreads, smem, c.stream, c.grad, c.d,
                          c.grad_stride, args, round_keys(c.seed), n_entries, c.first_worker, c.packed, c.words_stride, c.words_out);

@@ -1,6 +1,7 @@
 """Sizes at which the kernels' work splits change: edges of tiles, remainders, the ends of a dispatch range."""
 import math
 import random
+import threading
 
 import numpy as np
 import pytest
@@ -292,3 +293,33 @@ def test_two_pass_threshold_is_one_number(tq):
     for st in (tq.stats_to_host(tq.tq_stats(g))[0], tq.stats_to_host(tq.tq_stats_segments(g, [(0, g.numel())]))[0]):
         assert st.sum_abs == tree and st.g_min == float(np.float32(tree / (T * 4096)))
         assert st.n_tail == T + (T if st.g_min == 1.0 else 0)
+
+
+def test_decision_tables_of_two_threads(tq):
+    """Two threads compress bf16 rows whose quantizers need tables of different sizes, each on its own stream: every call is accepted
+    and gives what it gives alone."""
+    d = 17_000_000
+    g = (torch.randn(1, d, device="cuda", generator=torch.Generator(device="cuda").manual_seed(1)) * 1e-3).to(torch.bfloat16)
+    books = []
+    for inner in (1e-3, 1e-12):                                  # two binades of entries, thirty-odd
+        mags = np.geomspace(inner, 3e-3, 8).astype(np.float32)
+        books.append([tq.tq_params_from_levels([float(x) for x in np.concatenate([-mags[::-1], mags])])])
+    want = [tq.tq_compress(g, p, seed=5, d=d) for p in books]
+    torch.cuda.synchronize()
+    failed = []
+
+    def work(k):
+        try:
+            stream, out = torch.cuda.Stream(), torch.empty_like(want[k])
+            with torch.cuda.stream(stream):
+                for _ in range(2000):
+                    tq.tq_compress(g, books[k], seed=5, d=d, packed=out)
+                stream.synchronize()
+                assert torch.equal(out, want[k])
+        except BaseException as e:
+            failed.append(e)
+
+    threads = [threading.Thread(target=work, args=(k,)) for k in (0, 1)]
+    [t.start() for t in threads]
+    [t.join() for t in threads]
+    assert not failed, failed
