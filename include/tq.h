@@ -169,8 +169,7 @@ tq_status tq_stats_hinted(const void* grad_dev, tq_dtype dtype, uint64_t d, uint
  * The call allocates nothing and frees nothing.  The first call on each device looks up the array's
  * device address (once per device, with that device current); make that first call outside any
  * stream capture.  All calls on a device share the one array and it keeps the previous call's
- * contents: the library clears the ticket counters itself at the start of every call, nothing else
- * needs to start at zero.  Two calls whose kernels overlap on the same GPU (different streams, or
+ * contents; nothing in it needs to start at zero.  Two calls whose kernels overlap on the same GPU (different streams, or
  * different host threads) race on the array and give wrong statistics: serialise them.
  * The looked-up address is remembered per device ordinal for the life of the process.  It does not
  * survive cudaDeviceReset, nor a second CUDA context on the same ordinal: a process that resets a device
