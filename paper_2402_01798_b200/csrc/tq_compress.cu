@@ -513,9 +513,9 @@ __device__ __forceinline__ void load_worker(const tq_params_t& p, WorkerQ& s_q) 
             s_q.levels[lane] = p.levels[lane];
             s_q.inv_width[lane] = p.inv_width[lane];
         }
-        __syncwarp();
         const float alpha = p.alpha, inv_step = p.inv_step;
         const bool ok = alpha > 0.0f && p.bits == BITS && !(p.flags & TQ_FLAG_INVALID);
+        __syncwarp();
         const float inv_2alpha = ok ? __fdiv_rn(1.0f, __fmul_rn(2.0f, alpha)) : 0.0f;
         uint32_t cells = 0, log_base = 0, log_cells = 0;
         if constexpr (NONUNIFORM) {      // choose_cells, a lane for each interior level

@@ -245,12 +245,14 @@ __device__ __forceinline__ uint32_t lut_record(const tq_params_t& rec, LutState&
         s.q.levels[threadIdx.x] = rec.levels[threadIdx.x];
         s.q.inv_width[threadIdx.x] = rec.inv_width[threadIdx.x];
     }
+    const float alpha = rec.alpha;                            // read beside the levels: after a barrier it would be one more trip to memory
+    const bool usable = lut_usable(rec, BITS);
     __syncthreads();
-    if (!lut_usable(rec, BITS)) return 0;
-    const uint32_t top = top_pattern(rec.alpha);
+    if (!usable) return 0;
+    const uint32_t top = top_pattern(alpha);
     uint32_t base = 0;
     if (threadIdx.x < 64) {
-        const bool fits = lut_window_fits(rec.alpha, s.q.levels, s.q.inv_width, 1u << BITS, top, kLutBinade * (threadIdx.x + 1), &base);
+        const bool fits = lut_window_fits(alpha, s.q.levels, s.q.inv_width, 1u << BITS, top, kLutBinade * (threadIdx.x + 1), &base);
         const uint32_t bits = __ballot_sync(0xFFFFFFFFu, fits);
         if ((threadIdx.x & 31u) == 0) s.fits[threadIdx.x >> 5] = bits;
     }
@@ -259,7 +261,7 @@ __device__ __forceinline__ uint32_t lut_record(const tq_params_t& rec, LutState&
     const uint32_t n_entries = kLutBinade * (s.fits[0] ? __ffs(static_cast<int>(s.fits[0])) : 32 + __ffs(static_cast<int>(s.fits[1])));
     if (threadIdx.x == 0) {
         base = top >= n_entries ? top - (n_entries - 1) : 0u;
-        s.q.alpha = rec.alpha;
+        s.q.alpha = alpha;
         s.q.base2 = ((0u - base) & 0xFFFFu) * 0x00010001u;
         s.q.negtop2 = (top | 0x8000u) * 0x00010001u;
     }

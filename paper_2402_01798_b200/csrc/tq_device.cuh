@@ -233,7 +233,8 @@ __device__ __forceinline__ JobPiece next_piece(const TilePlan& plan, uint64_t& c
     while (p.worker * plan.per_worker > cur) --p.worker;
     while ((p.worker + 1) * plan.per_worker <= cur) ++p.worker;
     const uint64_t row0 = p.worker * plan.per_worker, in_row = cur - row0;
-    p.seg = 0;
+    p.seg = 0;                     // eight at a time first: one after the other, 40 groups cost more than a microsecond a piece
+    while (p.seg + 8 < plan.segs.n && plan.begin[p.seg + 8] <= in_row) p.seg += 8;
     while (p.seg + 1 < plan.segs.n && plan.begin[p.seg + 1] <= in_row) ++p.seg;
     p.job = p.worker * plan.segs.n + p.seg;
     const uint64_t job_end = row0 + plan.begin[p.seg + 1], stop = end < job_end ? end : job_end;

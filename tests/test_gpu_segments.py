@@ -193,3 +193,26 @@ def test_segment_argument_checks(tq):
     with pytest.raises(tq.TqError) as e:
         tq.tq_stats_segments(gb, [(8, 64)])              # 16 bytes into a bf16 row
     assert e.value.status == tq.ERR_ALIGNMENT
+
+
+@pytest.mark.parametrize("S", [1, 2, 8, 9, 16, 17, 63, 64])
+def test_every_number_of_groups(tq, orc, S):
+    """A block finds the group of a tile eight groups at a time, then one: numbers of groups around multiples of eight up to the most, groups of one tile and of
+    several, three workers.  Counts and maxima exact and sums to fp32 partials in every group's record, for every threshold rule.
+    A tail of a few elements just above g_min has a sum of logarithms near 0; the hinted form adds log2|g|, below 16 here, so an element
+    adds up to 16 * (2 ulp of the hardware's logarithm + 16 roundings of a partial sum) * 2^-24 * ln 2 = 1.3e-5."""
+    n, table, at = 3, [], 0
+    for s in range(S):
+        ln = [4096, 17, 9000, 4097][s % 4] * (300 if S < 3 else 1)
+        table.append((at, ln))
+        at += (ln + 15) // 16 * 16
+    g = make_rows(n, at, torch.float32, seed=S)
+    hint = tq.new_gmin_hint(n * S)
+    host = g.cpu().numpy()
+    for rec in (tq.tq_stats_segments(g, table, g_min=2e-3), tq.tq_stats_segments(g, table), tq.tq_stats_hinted_segments(g, table, hint),
+                tq.tq_stats_hinted_segments(g, table, hint)):
+        for j, r in enumerate(tq.stats_to_host(rec)):
+            off, ln = table[j % S]
+            o = orc.stats(host[j // S, off:off + ln], g_min=r.g_min)
+            assert (r.d, r.max_abs, r.n_tail) == (ln, o.max_abs, o.n_tail), (j, S)
+            assert math.isclose(r.sum_abs, o.sum_abs, rel_tol=TOL_SUM) and math.isclose(r.sum_log_tail, o.sum_log_tail, rel_tol=TOL_LOG, abs_tol=1.3e-5 * r.n_tail)
