@@ -10,7 +10,7 @@
 //
 // Shapes.  Short rows (stats_small_kernel): a cluster of 8 blocks per job does everything in one launch, with the
 // block sums exchanged through distributed shared memory.  Other rows: the tiles (256 chunks) of all jobs -- workers, or
-// (worker, segment) pairs -- are cut into contiguous ranges, one per block (TilePlan); a block writes one record per
+// (worker, segment) pairs -- are cut into contiguous ranges, one per block (StatsPlan); a block writes one record per
 // piece of a job, and the next launch starts by folding the records of the jobs it needs, in index order, so
 // that the result does not depend on the order in which blocks run and no block waits for another.
 //   automatic threshold, g_min = kappa * mean|g|: pass 1 (moments), pass 2 (tail);
@@ -386,13 +386,39 @@ __device__ __forceinline__ bool has_leftover(uint64_t d, uint64_t& j) {
     j = d / kChunk<BF16> * kChunk<BF16> + threadIdx.x;
     return j < d;
 }
+// ---- how the work is cut ------------------------------------------------------------------------------------
+// Ranges (TilePlan), or blocks that keep to one job each: see plan_stats.
+struct StatsPlan : TilePlan {
+    uint32_t per_row;                              // blocks per worker where every block has one piece; 0: ranges
+    uint32_t block_begin[TQ_MAX_SEGMENTS + 1];     // then: first block of each segment within the worker's blocks
+};
+__device__ __forceinline__ void range_of_block(const StatsPlan& plan, uint32_t b, uint64_t& cur, uint64_t& end) {
+    if (plan.per_row == 0) {
+        cur = first_tile_of_block(plan, b);
+        end = first_tile_of_block(plan, b + 1);
+        return;
+    }
+    const uint32_t worker = b / plan.per_row, in_row = b - worker * plan.per_row;
+    uint32_t seg = 0;
+    while (seg + 8 < plan.segs.n && plan.block_begin[seg + 8] <= in_row) seg += 8;
+    while (seg + 1 < plan.segs.n && plan.block_begin[seg + 1] <= in_row) ++seg;
+    const uint32_t parts = plan.block_begin[seg + 1] - plan.block_begin[seg], part = in_row - plan.block_begin[seg];
+    const uint64_t first = worker * plan.per_worker + plan.begin[seg], tiles = plan.begin[seg + 1] - plan.begin[seg];
+    cur = first + tiles * part / parts;
+    end = first + tiles * (part + 1) / parts;
+}
+
 template <bool BF16>
 __device__ __forceinline__ const char* row_of(const JobPiece& piece, const void* grad, uint64_t grad_stride) {
     return static_cast<const char*>(grad) + (static_cast<uint64_t>(piece.worker) * grad_stride + piece.off) * (BF16 ? 2 : 4);
 }
-__device__ __forceinline__ Partial* records_of_job(const TilePlan& plan, const JobPiece& piece, Partial* partials, uint32_t& count) {
+__device__ __forceinline__ Partial* records_of_job(const StatsPlan& plan, const JobPiece& piece, Partial* partials, uint32_t& count) {
     uint32_t first, last;
-    blocks_of_job(plan, piece, first, last);
+    if (plan.per_row == 0) blocks_of_job(plan, piece, first, last);
+    else {
+        first = piece.worker * plan.per_row + plan.block_begin[piece.seg];
+        last = piece.worker * plan.per_row + plan.block_begin[piece.seg + 1] - 1;
+    }
     count = last - first + 1;
     return partials + first + piece.job;
 }
@@ -444,7 +470,7 @@ __device__ __forceinline__ bool last_of_job(Partial* record, const Partial& p, u
 constexpr int kStatsBlocksPerSm = 4;
 
 template <bool BF16, int PASS>
-__device__ __forceinline__ void stats_piece(const JobPiece& piece, const TilePlan& plan, const void* grad, uint64_t grad_stride, float g_min,
+__device__ __forceinline__ void stats_piece(const JobPiece& piece, const StatsPlan& plan, const void* grad, uint64_t grad_stride, float g_min,
                                             float kappa, tq_stats_t* stats, Partial* partials, uint32_t* tickets, BlockFold<kWarps>& sh) {
     const char* row = row_of<BF16>(piece, grad, grad_stride);
     uint32_t count;
@@ -490,10 +516,10 @@ __device__ __forceinline__ void stats_piece(const JobPiece& piece, const TilePla
 template <bool BF16, int PASS>
 __global__ void __launch_bounds__(kThreads, kStatsBlocksPerSm)
 stats_kernel(const void* __restrict__ grad, uint64_t grad_stride, float g_min, float kappa, tq_stats_t* stats, Partial* partials,
-             uint32_t* tickets, const __grid_constant__ TilePlan plan) {
+             uint32_t* tickets, const __grid_constant__ StatsPlan plan) {
     __shared__ BlockFold<kWarps> sh;
-    uint64_t cur = first_tile_of_block(plan, blockIdx.x);
-    const uint64_t end = first_tile_of_block(plan, blockIdx.x + 1);
+    uint64_t cur, end;
+    range_of_block(plan, blockIdx.x, cur, end);
     JobPiece piece = next_piece(plan, cur, end);               // no block is empty
     pdl_wait();
     while (true) {
@@ -508,7 +534,7 @@ stats_kernel(const void* __restrict__ grad, uint64_t grad_stride, float g_min, f
 // each piece of a block waited for the one before it, and the first for a memset (8 rows of 1 M in 16 groups 20.5 us, now 10.9; 25.6 M x 16
 // 242, now 239).
 __global__ void __launch_bounds__(kThreads)
-stats_given_finish_kernel(float g_min, tq_stats_t* stats, Partial* partials, const __grid_constant__ TilePlan plan) {
+stats_given_finish_kernel(float g_min, tq_stats_t* stats, Partial* partials, const __grid_constant__ StatsPlan plan) {
     __shared__ BlockFold<kWarps> sh;
     const uint32_t worker = blockIdx.x / plan.segs.n, seg = blockIdx.x - worker * plan.segs.n;
     uint64_t cur = worker * plan.per_worker + plan.begin[seg];
@@ -610,7 +636,7 @@ __device__ __forceinline__ float hinted_finish_piece(const JobPiece& piece, floa
 }
 // The tail sums of a piece of a job whose hint missed.
 template <bool BF16>
-__device__ __forceinline__ void hinted_tail_piece(const JobPiece& piece, const TilePlan& plan, const void* grad, uint64_t grad_stride, float g_min,
+__device__ __forceinline__ void hinted_tail_piece(const JobPiece& piece, const StatsPlan& plan, const void* grad, uint64_t grad_stride, float g_min,
                                                   tq_stats_t* stats, Partial* partials, uint32_t* tickets, BlockFold<kWarps>& sh) {
     uint32_t count;
     const Partial* records = records_of_job(plan, piece, partials, count);
@@ -633,11 +659,11 @@ __device__ __forceinline__ void hinted_tail_piece(const JobPiece& piece, const T
 template <bool BF16>
 __global__ void __launch_bounds__(kThreads, kStatsBlocksPerSm)
 stats_hinted_kernel(const void* __restrict__ grad, uint64_t grad_stride, const tq_gmin_hint_t* hint, Partial* partials, uint32_t* tickets,
-                    const __grid_constant__ TilePlan plan) {
+                    const __grid_constant__ StatsPlan plan) {
     __shared__ BlockFold<kWarps> sh;
     pdl_wait();
-    uint64_t cur = first_tile_of_block(plan, blockIdx.x);
-    const uint64_t end = first_tile_of_block(plan, blockIdx.x + 1);
+    uint64_t cur, end;
+    range_of_block(plan, blockIdx.x, cur, end);
     while (cur < end) {
         hinted_piece<BF16>(next_piece(plan, cur, end), grad, grad_stride, hint, partials, tickets, sh);
         __syncthreads();                                       // the next piece reuses the shared arrays
@@ -646,12 +672,12 @@ stats_hinted_kernel(const void* __restrict__ grad, uint64_t grad_stride, const t
 template <bool BF16>
 __global__ void __launch_bounds__(kThreads, kStatsBlocksPerSm)
 stats_hinted_finish_kernel(const void* __restrict__ grad, uint64_t grad_stride, float kappa, tq_gmin_hint_t* hint, tq_stats_t* stats,
-                           Partial* partials, uint32_t* tickets, const __grid_constant__ TilePlan plan) {
+                           Partial* partials, uint32_t* tickets, const __grid_constant__ StatsPlan plan) {
     __shared__ BlockFold<kWarps> sh;
     __shared__ float s_again[kWarps];
     const uint32_t warp = threadIdx.x >> 5;
-    uint64_t cur = first_tile_of_block(plan, blockIdx.x), batch;
-    const uint64_t end = first_tile_of_block(plan, blockIdx.x + 1);
+    uint64_t cur, end, batch;
+    range_of_block(plan, blockIdx.x, cur, end);
     JobPiece mine;
     const Partial* records = nullptr;
     uint32_t n, count = 0;
@@ -803,11 +829,33 @@ stats_small_kernel(const void* __restrict__ grad, uint64_t grad_stride, float g_
 constexpr uint64_t kSmallRowBytes = static_cast<uint64_t>(kCluster) * kSmallThreads * kSmallChunks * kChunkBytes;      // 1 MiB
 constexpr uint32_t kSmallMaxJobs = 8;
 
-static void plan_stats(const StatsCall& c, uint32_t n_jobs, TilePlan* plan) {
+// Where layer groups are short, the pieces of a range stand in a chain: in the tail pass each folds its job's records and ends with a
+// ticket.  Calls without a hint whose resident blocks would get up to 8 tiles give each block a piece of one job instead, of
+// about 1.25 times an even share (fewer blocks than places where jobs allow it, so that one wave holds them).  Ranges / one job each,
+// us: two passes over 32 rows of 500 k in 30 groups 56.1 / 30.1, 64 x 200 k in 40 60.2 / 45.7, 8 x 1 M in 40 30.1 / 18.4; threshold given
+// 23.1 / 20.4, 30.9 / 27.4, 12.5 / 10.3.  From 14 tiles on ranges are faster (11 x 3 M fp32 in 16, threshold given: 27.4 / 31.9), as they are
+// behind a hint, whose records a block folds side by side (64 x 200 k in 40: 32.2 / 36.0).
+constexpr uint64_t kTilesForRanges = 8;
+
+static void plan_stats(const StatsCall& c, uint32_t n_jobs, bool hinted, StatsPlan* plan) {
     uint64_t resident = static_cast<uint64_t>(sm_count()) * kStatsBlocksPerSm;
     const uint64_t room = static_cast<uint64_t>(n_jobs) * kRecordsPerJob - n_jobs;
     if (resident > room) resident = room;
     plan_tiles(plan, c.segs, c.d, c.n_workers, kThreads * kChunkBytes / (c.bf16 ? 2 : 4), resident);
+    plan->per_row = 0;
+    const uint64_t total = plan->per_worker * c.n_workers;
+    if (!hinted && plan->segs.n > 1 && total > resident && total <= kTilesForRanges * resident) {
+        const uint64_t target = total * 5 / (resident * 4);      // at least 1
+        uint32_t blocks = 0;
+        for (uint32_t s = 0; s < plan->segs.n; ++s) {
+            plan->block_begin[s] = blocks;
+            const uint64_t parts = (plan->begin[s + 1] - plan->begin[s] + target / 2) / target;
+            blocks += parts > 0 ? static_cast<uint32_t>(parts) : 1u;
+        }
+        plan->block_begin[plan->segs.n] = plan->per_row = blocks;
+        plan->blocks = blocks * c.n_workers;
+        return;
+    }
     // bf16 rows are bound by instructions: three ranges per resident block even out the SMs (124 M x 8, hinted: 430 -> 407 us;
     // fp32 rows 249 -> 254 us, short ranges lose more)
     if (c.bf16 && plan->per_block >= 64 && 3 * resident <= room) plan_tiles(plan, c.segs, c.d, c.n_workers, kThreads * kChunkBytes / 2, 3 * resident);
@@ -815,7 +863,7 @@ static void plan_stats(const StatsCall& c, uint32_t n_jobs, TilePlan* plan) {
 
 // Equal rows in a whole number of blocks each may leave some places empty: see launch_kernel.  Rounds of 3 M x 64, 576 blocks of 81
 // tiles, early / late: hinted 336 / 315 us, two passes 461 / 416; of 1 M x 64, 27 tiles, two passes 152.8 / 153.4.
-static Start start_of(const TilePlan& plan) {
+static Start start_of(const StatsPlan& plan) {
     return plan.blocks < static_cast<uint32_t>(sm_count()) * kStatsBlocksPerSm && plan.per_block >= 48 ? Start::kLate : Start::kEarly;
 }
 
@@ -849,8 +897,8 @@ cudaError_t launch_stats(const StatsCall& c, int* launches) {
     }
     Partial* partials = static_cast<Partial*>(c.workspace);
     uint32_t* tickets = reinterpret_cast<uint32_t*>(static_cast<char*>(c.workspace) + tickets_offset(n_jobs));
-    static thread_local TilePlan plan;
-    plan_stats(c, n_jobs, &plan);
+    static thread_local StatsPlan plan;
+    plan_stats(c, n_jobs, false, &plan);
     auto launch = [&](auto kernel, Start start) {
         e = launch_kernel(start, kernel, dim3(plan.blocks), kThreads, 0, c.stream, c.grad, c.grad_stride, c.g_min, c.kappa, c.stats, partials, tickets, plan);
         *launches += e == cudaSuccess ? 1 : 0;
@@ -873,8 +921,8 @@ cudaError_t launch_stats_hinted(const StatsCall& c, tq_gmin_hint_t* hint, int* l
     if (launch_small<kPow2>(c, n_jobs, hint, &e)) { *launches = e == cudaSuccess ? 1 : 0; return e; }
     Partial* partials = static_cast<Partial*>(c.workspace);
     uint32_t* tickets = reinterpret_cast<uint32_t*>(static_cast<char*>(c.workspace) + tickets_offset(n_jobs));
-    static thread_local TilePlan plan;            // the same plan for both launches: same summation order
-    plan_stats(c, n_jobs, &plan);
+    static thread_local StatsPlan plan;            // the same plan for both launches: same summation order
+    plan_stats(c, n_jobs, true, &plan);
     e = launch_kernel(start_of(plan), c.bf16 ? stats_hinted_kernel<true> : stats_hinted_kernel<false>, dim3(plan.blocks), kThreads, 0, c.stream, c.grad,
                       c.grad_stride, static_cast<const tq_gmin_hint_t*>(hint), partials, tickets, plan);
     if (e != cudaSuccess) return e;

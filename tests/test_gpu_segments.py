@@ -216,3 +216,29 @@ def test_every_number_of_groups(tq, orc, S):
             o = orc.stats(host[j // S, off:off + ln], g_min=r.g_min)
             assert (r.d, r.max_abs, r.n_tail) == (ln, o.max_abs, o.n_tail), (j, S)
             assert math.isclose(r.sum_abs, o.sum_abs, rel_tol=TOL_SUM) and math.isclose(r.sum_log_tail, o.sum_log_tail, rel_tol=TOL_LOG, abs_tol=1.3e-5 * r.n_tail)
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("n,S,share", [(1, 40, (1, 1)), (1, 64, (8, 0)), (1, 2, (8, 1)), (16, 37, (5, 3)), (64, 64, (7, 9))])
+def test_blocks_that_keep_to_one_group(tq, orc, dtype, n, S, share):
+    """Statistics without a hint of more tiles than resident blocks and up to eight for each: a block takes a piece of one group.  Totals
+    at both ends of that range, groups of one tile beside groups of hundreds, one element to spare or to lack in a tile.  Counts and
+    maxima exact, sums to fp32 partials, and one threshold in all pieces of a group (the tail's count is that of the record's)."""
+    tile, resident = (4096 if dtype == torch.float32 else 8192), 4 * torch.cuda.get_device_properties(0).multi_processor_count
+    tiles = (share[0] * resident + share[1]) // n              # per worker; the last group takes what the others leave
+    lens = [tile * (1 + (7 * s) % (2 * tiles // S - 1) if tiles >= 3 * S else 1) - (s % 3) for s in range(S - 1)]
+    lens.append(tile * max(1, tiles - sum((x + 2) // tile for x in lens)) - 5)
+    table, at = [], 0
+    for ln in lens:
+        table.append((at, ln))
+        at += (ln + 15) // 16 * 16
+    g = make_rows(n, at, dtype, seed=n + S)
+    for rec in (tq.tq_stats_segments(g, table), tq.tq_stats_segments(g, table, g_min=2e-3)):
+        for j, r in enumerate(tq.stats_to_host(rec)):
+            if n * S > 100 and j % 7 and j < n * S - S:
+                continue
+            off, ln = table[j % S]
+            o = orc.stats(host_f32(orc, g[j // S, off:off + ln]), g_min=r.g_min)
+            assert (r.d, r.max_abs, r.n_tail) == (ln, o.max_abs, o.n_tail), (j, S)
+            assert math.isclose(r.sum_abs, o.sum_abs, rel_tol=TOL_SUM) and math.isclose(r.sum_sq, o.sum_sq, rel_tol=2 * TOL_SUM)
+            assert math.isclose(r.sum_log_tail, o.sum_log_tail, rel_tol=TOL_LOG, abs_tol=1.3e-5 * r.n_tail)
