@@ -301,7 +301,7 @@ decompress_kernel(const __grid_constant__ RowTable rt, uint64_t words_valid, uin
 }
 
 // ---------------------------------------------------------------------------------------------
-// Bulk-copy variant for large inputs.  One block decodes one tile of kDecThreads * 32 outputs.  The
+// Bulk-copy variant for large inputs.  One block decodes one tile of kDecThreads * U * Unit<BITS>::kElems outputs.  The
 // packed bytes of the tile, kGroup workers at a time, are brought into a ring of shared-memory stages
 // by asynchronous bulk copies (one per worker row, completion counted on an mbarrier), so the next
 // workers' bytes are in flight while the current ones are looked up, and no registers are tied up by
@@ -440,7 +440,7 @@ decompress_bulk_kernel(const __grid_constant__ RowTable rt, uint64_t words_row, 
     }
     // A block barrier here would make the give-up of the last steps uniform as well; it was measured to cost 2-5 %
     // of the kernel (0.163 -> 0.167 ms and 0.161 -> 0.169 ms on 124 M x 8 with 4- and 2-bit codes), so a thread whose
-    // wait runs out in one of the last S steps drops its own 32 outputs and counts itself.
+    // wait runs out in one of the last S steps drops its own U * Unit<BITS>::kElems outputs and counts itself.
     if (expired) {
         atomicAdd(&g_wait_expired, 1u);
         if (threadIdx.x == 0)      // the copies issued and not yet seen to land: steps q .. q + S - 1

@@ -36,30 +36,9 @@ __device__ __forceinline__ void stg256(void* p, const float (&v)[8]) {
                  : "memory");
 }
 
-// Eight consecutive gradient elements as fp32.  `p` is 32-byte aligned for fp32 and 16-byte aligned
-// for bf16.  bf16 -> fp32 is exact: the stored 16 bits become the high half of the fp32 pattern.
-template <bool BF16>
-__device__ __forceinline__ void load8(const void* p, float (&g)[8]) {
-    if constexpr (!BF16) {
-        uint32_t v[8];
-        ldg256_stream(p, v);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) g[i] = __uint_as_float(v[i]);
-    } else {
-        uint4 v;
-        asm volatile("ld.global.nc.L1::no_allocate.v4.b32 {%0,%1,%2,%3}, [%4];"
-                     : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
-        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            g[2 * i] = __uint_as_float(w[i] << 16);
-            g[2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u);
-        }
-    }
-}
-
 // Eight consecutive gradient elements kept as loaded (fp32: 8 words; bf16: 4 words of two), decoded
-// on use.  Keeping bf16 packed halves the registers a loaded group occupies.
+// on use.  Keeping bf16 packed halves the registers a loaded group occupies.  The address is 32-byte aligned for fp32 and 16-byte
+// aligned for bf16.  bf16 -> fp32 is exact: the stored 16 bits become the high half of the fp32 pattern.
 template <bool BF16>
 struct Raw8 {
     uint32_t v[BF16 ? 4 : 8];
@@ -74,12 +53,6 @@ template <bool BF16>
 __device__ __forceinline__ float elem(const Raw8<BF16>& r, int e) {
     if constexpr (!BF16) return __uint_as_float(r.v[e]);
     else return __uint_as_float((e & 1) ? (r.v[e >> 1] & 0xFFFF0000u) : (r.v[e >> 1] << 16));
-}
-template <bool BF16>
-__device__ __forceinline__ void set_elem(Raw8<BF16>& r, int e, float x) {   // fp32 bits, or an exact bf16 value
-    if constexpr (!BF16) r.v[e] = __float_as_uint(x);
-    else r.v[e >> 1] = (e & 1) ? ((r.v[e >> 1] & 0x0000FFFFu) | (__float_as_uint(x) & 0xFFFF0000u))
-                               : ((r.v[e >> 1] & 0xFFFF0000u) | (__float_as_uint(x) >> 16));
 }
 
 // Single words, any alignment of the run they belong to.
