@@ -38,9 +38,9 @@ if ROOT not in sys.path:
 
 METRIC = "compress & decompress-aggregate GB/s of fp32 gradient, % of B200 HBM peak"
 FALLBACK_HBM_GBS = 6650.0
-# dram__bytes_read.sum + dram__bytes_write.sum per launch from the ncu capture summarised in
-# profiles/compress_kernel_resnet50-25.6M.md (the kernel's loads and stores have not changed since; None elsewhere)
-NCU_DRAM_BYTES = {("resnet50-25.6M", "tq_compress"): 1_837_323_352}
+# dram__bytes_read.sum + dram__bytes_write.sum over the algorithmic bytes, from the ncu capture of the same kernel at 6.4 M x 16 in
+# profiles/ (454.3 MB of 460.8; the last few MB written are still in L2 when it ends); None for workloads that take another kernel
+NCU_DRAM_PER_ALGORITHMIC_BYTE = {("resnet50-25.6M", "tq_compress"): 454_296_832 / 460_800_000}
 
 
 def hbm_peak():
@@ -500,10 +500,11 @@ def measure_round(args, tq, w, g, stride, dev, local_rank, world, steps, warmup,
     except Exception as e:                                   # capture is an extra: report why it did not work
         result["cuda_graph"] = {"error": repr(e)[:300]}
 
-    dom = "tq_compress"      # the single kernel with the largest share of the round (see profiles/launch_list_*)
+    dom = "tq_compress"      # the single kernel with the largest share of the round
+    per_byte = NCU_DRAM_PER_ALGORITHMIC_BYTE.get((w.name, dom))
     result["roofline"] = {"kernel": dom, "bound": "hbm", "achieved": kernels[dom]["gbs"], "peak": peak, "peak_source": peak_kind,
                           "unit": "GB/s", "frac": kernels[dom]["gbs"] / peak, "algorithmic_bytes": alg[dom][0],
-                          "traffic": NCU_DRAM_BYTES.get((w.name, dom))}
+                          "traffic": None if per_byte is None else round(per_byte * alg[dom][0])}
 
     # end to end through the public API with HOST buffers: H2D of every worker's gradient, the round,
     # D2H of the aggregated update, all inside the timed region

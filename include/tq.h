@@ -116,7 +116,8 @@ size_t tq_stats_workspace_bytes(uint32_t n_workers);
  *   workspace_dev, ws_bytes   device scratch of at least tq_stats_workspace_bytes(n_workers), 256-byte
  *                aligned; contents need not be initialised and are not meaningful afterwards.  Calls
  *                sharing one workspace must not overlap on the device.
- * Sums are accumulated in fp32 over runs of 16 elements and in fp64 beyond; counts and max are exact.
+ * Sums are accumulated in fp32 inside chunks of 64 bytes (16 fp32 or 32 bf16 elements, at most 16 terms in a row) and in fp64
+ * beyond, in an order that depends on the call's sizes alone; counts and max are exact.
  * d = 0 is allowed (all-zero records).  Errors: INVALID_ARG, ALIGNMENT, BUFFER_TOO_SMALL, CUDA.
  */
 tq_status tq_stats(const void* grad_dev, tq_dtype dtype, uint64_t d, uint64_t grad_stride,
@@ -313,7 +314,8 @@ tq_status tq_decompress_aggregate_device_params(const uint32_t* packed_dev, size
  * its own alpha and codebook, and its own packed stream.  A group is a segment [offset, offset + length)
  * of every worker's row, the same for all workers.  These calls do for all (worker, segment) pairs at once
  * what one tq_stats / tq_params_device / tq_compress_device_params / tq_decompress_aggregate_device_params
- * call per group does on the sub-range, with the same results bit for bit:
+ * call per group does on the sub-range, with the same results bit for bit but for the sums of the statistics, which are added in
+ * another order (a threshold from them may differ in its last fp32 bit):
  *   - records are indexed [worker * n_segments + segment];
  *   - element j of a segment is element j of that group's gradient: the random bits of Section 3.1's
  *     rounding come from (seed, first_worker + worker, j) with j counted from the segment's start;
