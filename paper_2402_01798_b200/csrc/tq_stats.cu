@@ -392,12 +392,12 @@ struct StatsPlan : TilePlan {
     uint32_t per_row;                              // blocks per worker where every block has one piece; 0: ranges
     uint32_t block_begin[TQ_MAX_SEGMENTS + 1];     // then: first block of each segment within the worker's blocks
 };
+__device__ __forceinline__ void range_of_block(const TilePlan& plan, uint32_t b, uint64_t& cur, uint64_t& end) {
+    cur = first_tile_of_block(plan, b);
+    end = first_tile_of_block(plan, b + 1);
+}
 __device__ __forceinline__ void range_of_block(const StatsPlan& plan, uint32_t b, uint64_t& cur, uint64_t& end) {
-    if (plan.per_row == 0) {
-        cur = first_tile_of_block(plan, b);
-        end = first_tile_of_block(plan, b + 1);
-        return;
-    }
+    if (plan.per_row == 0) return range_of_block(static_cast<const TilePlan&>(plan), b, cur, end);
     const uint32_t worker = b / plan.per_row, in_row = b - worker * plan.per_row;
     uint32_t seg = 0;
     while (seg + 8 < plan.segs.n && plan.block_begin[seg + 8] <= in_row) seg += 8;
@@ -412,15 +412,16 @@ template <bool BF16>
 __device__ __forceinline__ const char* row_of(const JobPiece& piece, const void* grad, uint64_t grad_stride) {
     return static_cast<const char*>(grad) + (static_cast<uint64_t>(piece.worker) * grad_stride + piece.off) * (BF16 ? 2 : 4);
 }
-__device__ __forceinline__ Partial* records_of_job(const StatsPlan& plan, const JobPiece& piece, Partial* partials, uint32_t& count) {
+__device__ __forceinline__ Partial* records_of_job(const TilePlan& plan, const JobPiece& piece, Partial* partials, uint32_t& count) {
     uint32_t first, last;
-    if (plan.per_row == 0) blocks_of_job(plan, piece, first, last);
-    else {
-        first = piece.worker * plan.per_row + plan.block_begin[piece.seg];
-        last = piece.worker * plan.per_row + plan.block_begin[piece.seg + 1] - 1;
-    }
+    blocks_of_job(plan, piece, first, last);
     count = last - first + 1;
     return partials + first + piece.job;
+}
+__device__ __forceinline__ Partial* records_of_job(const StatsPlan& plan, const JobPiece& piece, Partial* partials, uint32_t& count) {
+    if (plan.per_row == 0) return records_of_job(static_cast<const TilePlan&>(plan), piece, partials, count);
+    count = plan.block_begin[piece.seg + 1] - plan.block_begin[piece.seg];
+    return partials + piece.worker * plan.per_row + plan.block_begin[piece.seg] + piece.job;
 }
 __device__ __forceinline__ Partial* record_of_piece(const JobPiece& piece, Partial* partials) { return partials + blockIdx.x + piece.job; }
 // Folds `count` records of an earlier launch (or of blocks whose tickets have been seen).
@@ -636,7 +637,7 @@ __device__ __forceinline__ float hinted_finish_piece(const JobPiece& piece, floa
 }
 // The tail sums of a piece of a job whose hint missed.
 template <bool BF16>
-__device__ __forceinline__ void hinted_tail_piece(const JobPiece& piece, const StatsPlan& plan, const void* grad, uint64_t grad_stride, float g_min,
+__device__ __forceinline__ void hinted_tail_piece(const JobPiece& piece, const TilePlan& plan, const void* grad, uint64_t grad_stride, float g_min,
                                                   tq_stats_t* stats, Partial* partials, uint32_t* tickets, BlockFold<kWarps>& sh) {
     uint32_t count;
     const Partial* records = records_of_job(plan, piece, partials, count);
@@ -659,7 +660,7 @@ __device__ __forceinline__ void hinted_tail_piece(const JobPiece& piece, const S
 template <bool BF16>
 __global__ void __launch_bounds__(kThreads, kStatsBlocksPerSm)
 stats_hinted_kernel(const void* __restrict__ grad, uint64_t grad_stride, const tq_gmin_hint_t* hint, Partial* partials, uint32_t* tickets,
-                    const __grid_constant__ StatsPlan plan) {
+                    const __grid_constant__ TilePlan plan) {
     __shared__ BlockFold<kWarps> sh;
     pdl_wait();
     uint64_t cur, end;
@@ -672,7 +673,7 @@ stats_hinted_kernel(const void* __restrict__ grad, uint64_t grad_stride, const t
 template <bool BF16>
 __global__ void __launch_bounds__(kThreads, kStatsBlocksPerSm)
 stats_hinted_finish_kernel(const void* __restrict__ grad, uint64_t grad_stride, float kappa, tq_gmin_hint_t* hint, tq_stats_t* stats,
-                           Partial* partials, uint32_t* tickets, const __grid_constant__ StatsPlan plan) {
+                           Partial* partials, uint32_t* tickets, const __grid_constant__ TilePlan plan) {
     __shared__ BlockFold<kWarps> sh;
     __shared__ float s_again[kWarps];
     const uint32_t warp = threadIdx.x >> 5;
@@ -834,36 +835,40 @@ constexpr uint32_t kSmallMaxJobs = 8;
 // about 1.25 times an even share (fewer blocks than places where jobs allow it, so that one wave holds them).  Ranges / one job each,
 // us: two passes over 32 rows of 500 k in 30 groups 56.1 / 30.1, 64 x 200 k in 40 60.2 / 45.7, 8 x 1 M in 40 30.1 / 18.4; threshold given
 // 23.1 / 20.4, 30.9 / 27.4, 12.5 / 10.3.  From 14 tiles on ranges are faster (11 x 3 M fp32 in 16, threshold given: 27.4 / 31.9), as they are
-// behind a hint, whose records a block folds side by side (64 x 200 k in 40: 32.2 / 36.0).
+// behind a hint, whose records a block folds side by side (64 x 200 k in 40: 32.2 / 36.0); its kernels do not
+// know the other form, which moved the registers of the bf16 main loop (38 M x 11: 579 -> 587 us a round).
 constexpr uint64_t kTilesForRanges = 8;
 
-static void plan_stats(const StatsCall& c, uint32_t n_jobs, bool hinted, StatsPlan* plan) {
-    uint64_t resident = static_cast<uint64_t>(sm_count()) * kStatsBlocksPerSm;
-    const uint64_t room = static_cast<uint64_t>(n_jobs) * kRecordsPerJob - n_jobs;
-    if (resident > room) resident = room;
+static uint64_t resident_blocks(uint32_t n_jobs) {
+    const uint64_t resident = static_cast<uint64_t>(sm_count()) * kStatsBlocksPerSm, room = static_cast<uint64_t>(n_jobs) * kRecordsPerJob - n_jobs;
+    return resident < room ? resident : room;
+}
+static void plan_ranges(const StatsCall& c, uint32_t n_jobs, TilePlan* plan) {
+    const uint64_t resident = resident_blocks(n_jobs), room = static_cast<uint64_t>(n_jobs) * kRecordsPerJob - n_jobs;
     plan_tiles(plan, c.segs, c.d, c.n_workers, kThreads * kChunkBytes / (c.bf16 ? 2 : 4), resident);
-    plan->per_row = 0;
-    const uint64_t total = plan->per_worker * c.n_workers;
-    if (!hinted && plan->segs.n > 1 && total > resident && total <= kTilesForRanges * resident) {
-        const uint64_t target = total * 5 / (resident * 4);      // at least 1
-        uint32_t blocks = 0;
-        for (uint32_t s = 0; s < plan->segs.n; ++s) {
-            plan->block_begin[s] = blocks;
-            const uint64_t parts = (plan->begin[s + 1] - plan->begin[s] + target / 2) / target;
-            blocks += parts > 0 ? static_cast<uint32_t>(parts) : 1u;
-        }
-        plan->block_begin[plan->segs.n] = plan->per_row = blocks;
-        plan->blocks = blocks * c.n_workers;
-        return;
-    }
     // bf16 rows are bound by instructions: three ranges per resident block even out the SMs (124 M x 8, hinted: 430 -> 407 us;
     // fp32 rows 249 -> 254 us, short ranges lose more)
     if (c.bf16 && plan->per_block >= 64 && 3 * resident <= room) plan_tiles(plan, c.segs, c.d, c.n_workers, kThreads * kChunkBytes / 2, 3 * resident);
 }
+static void plan_stats(const StatsCall& c, uint32_t n_jobs, StatsPlan* plan) {
+    plan_ranges(c, n_jobs, plan);
+    plan->per_row = 0;
+    const uint64_t total = plan->per_worker * c.n_workers, resident = resident_blocks(n_jobs);
+    if (plan->segs.n == 1 || total <= resident || total > kTilesForRanges * resident) return;
+    const uint64_t target = total * 5 / (resident * 4);          // at least 1
+    uint32_t blocks = 0;
+    for (uint32_t s = 0; s < plan->segs.n; ++s) {
+        plan->block_begin[s] = blocks;
+        const uint64_t parts = (plan->begin[s + 1] - plan->begin[s] + target / 2) / target;
+        blocks += parts > 0 ? static_cast<uint32_t>(parts) : 1u;
+    }
+    plan->block_begin[plan->segs.n] = plan->per_row = blocks;
+    plan->blocks = blocks * c.n_workers;
+}
 
 // Equal rows in a whole number of blocks each may leave some places empty: see launch_kernel.  Rounds of 3 M x 64, 576 blocks of 81
 // tiles, early / late: hinted 336 / 315 us, two passes 461 / 416; of 1 M x 64, 27 tiles, two passes 152.8 / 153.4.
-static Start start_of(const StatsPlan& plan) {
+static Start start_of(const TilePlan& plan) {
     return plan.blocks < static_cast<uint32_t>(sm_count()) * kStatsBlocksPerSm && plan.per_block >= 48 ? Start::kLate : Start::kEarly;
 }
 
@@ -898,7 +903,7 @@ cudaError_t launch_stats(const StatsCall& c, int* launches) {
     Partial* partials = static_cast<Partial*>(c.workspace);
     uint32_t* tickets = reinterpret_cast<uint32_t*>(static_cast<char*>(c.workspace) + tickets_offset(n_jobs));
     static thread_local StatsPlan plan;
-    plan_stats(c, n_jobs, false, &plan);
+    plan_stats(c, n_jobs, &plan);
     auto launch = [&](auto kernel, Start start) {
         e = launch_kernel(start, kernel, dim3(plan.blocks), kThreads, 0, c.stream, c.grad, c.grad_stride, c.g_min, c.kappa, c.stats, partials, tickets, plan);
         *launches += e == cudaSuccess ? 1 : 0;
@@ -921,8 +926,8 @@ cudaError_t launch_stats_hinted(const StatsCall& c, tq_gmin_hint_t* hint, int* l
     if (launch_small<kPow2>(c, n_jobs, hint, &e)) { *launches = e == cudaSuccess ? 1 : 0; return e; }
     Partial* partials = static_cast<Partial*>(c.workspace);
     uint32_t* tickets = reinterpret_cast<uint32_t*>(static_cast<char*>(c.workspace) + tickets_offset(n_jobs));
-    static thread_local StatsPlan plan;            // the same plan for both launches: same summation order
-    plan_stats(c, n_jobs, true, &plan);
+    static thread_local TilePlan plan;            // the same plan for both launches: same summation order
+    plan_ranges(c, n_jobs, &plan);
     e = launch_kernel(start_of(plan), c.bf16 ? stats_hinted_kernel<true> : stats_hinted_kernel<false>, dim3(plan.blocks), kThreads, 0, c.stream, c.grad,
                       c.grad_stride, static_cast<const tq_gmin_hint_t*>(hint), partials, tickets, plan);
     if (e != cudaSuccess) return e;
