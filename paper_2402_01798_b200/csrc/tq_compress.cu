@@ -128,26 +128,6 @@ __device__ __forceinline__ f32x2 code_uniform2_dn(float sum0, float sum1, const 
     return mul2_ru(v, both(2.710505431213761e-20f));     // 2^-65
 }
 
-// The codes in byte 2 of eight words -> their 8 * BITS packed bits, LSB first.
-template <int BITS>
-__device__ __forceinline__ uint32_t pack_byte2(const uint32_t (&v)[8]) {
-    auto four = [](uint32_t a, uint32_t b, uint32_t c, uint32_t d) {       // byte 2 of each
-        return __byte_perm(__byte_perm(a, b, 0x0062u), __byte_perm(c, d, 0x0062u), 0x5410u);
-    };
-    if constexpr (BITS <= 2) {
-        // c0 .. c3 side by side in the top byte of a product; the other partial products are disjoint bits below it
-        constexpr uint32_t K = (1u << 24) + (1u << (16 + BITS)) + (1u << (8 + 2 * BITS)) + (1u << (3 * BITS));
-        const uint32_t lo = four(v[0], v[1], v[2], v[3]) * K, hi = four(v[4], v[5], v[6], v[7]) * K;
-        if constexpr (BITS == 2) return __byte_perm(lo, hi, 0x0073u);      // 16 bits; the callers merge chunks by byte permutes
-        else return (lo >> 24) | ((hi >> 24) << 4);
-    } else {
-        const uint32_t t = four(v[0], v[2], v[4], v[6]) + (four(v[1], v[3], v[5], v[7]) << BITS);      // two codes per byte
-        if constexpr (BITS == 4) return t;
-        const uint32_t u = (t & 0x003F003Fu) | ((t >> 2) & 0x0FC00FC0u);                                // four codes per half
-        return (u & 0xFFFu) | ((u >> 4) & 0xFFF000u);
-    }
-}
-
 // The same decision without the scaled inverse step (alpha so large that inv_step / L is subnormal):
 // x = clip((g + alpha) * inv_step, 0, s), k' = floor x, p' = x - k'; at x = s this yields k' = s, p' = 0,
 // i.e. the same code s as k = s-1, p >= 1.  NaN becomes 0 (fmaxf drops it).  Returns the plain code.
@@ -618,8 +598,7 @@ compress_kernel_dev(const void* __restrict__ grad, uint64_t grad_stride, const t
         __syncthreads();
         const tq_params_t& p = params[sh.piece.job];
         if (table_kernel_ran) {          // rows the decision-table kernel served are done (same rule, evaluated by every thread)
-            uint32_t top, base;
-            if (lut_serves_record(p, BITS, &top, &base)) continue;
+            if (lut_serves_record(p, BITS)) continue;
         }
         load_worker<BITS, NONUNIFORM>(p, sh.q);
         if (!(sh.q.alpha > 0.0f)) {

@@ -9,21 +9,22 @@
 // element then costs one table read, and code = k + [r < T] = floor((X + 65535 - r) / 2^16) for the
 // element's 16 random bits r.
 //
-// Table index.  Only a window of magnitudes needs entries.  Above the window's top pattern P_top (the
-// smallest bf16 value >= alpha) every value is truncated to +-alpha; below its base pattern every value is
-// so small that the decision equals that of zero (the host checks this by evaluating the decision at
-// +-base; it is monotone in the value).  The index is clamp(|pattern| - base, 0, n - 1) + n * [negative],
-// n entries per sign, as many whole binades (128 entries) as the quantizer needs, at most 64, computed for the two elements of a
-// 32-bit word at once with 16-bit SIMD integer instructions.  NaN is sent to -alpha before that by a
-// packed bf16 maximum with -top, which returns the operand that is a number, as fmaxf does in the
-// element-wise form.
+// The table is indexed by the pattern itself: positive values from entry 0, negative ones from entry 2^15, each up to P_top,
+// the smallest bf16 value >= alpha; nothing is stored between P_top and 2^15.  A packed maximum with -P_top and a packed
+// minimum with P_top bring every value into the table, both halves of a word in one operation each; the maximum
+// returns the operand that is a number, so a NaN becomes -alpha as in the element-wise form.  Values so small that the
+// decision equals that of zero (the host or the block checks this by evaluating the decision at +-base; it is monotone in
+// the value) are filled in, not evaluated.
 //
-// Arithmetic on the floating-point pipe, without conversions: a table entry is the float with bit
-// pattern 0x19000000 + (X + 65535) = 2^-77 + (X + 65535) * 2^-100, the random slot is made into
-// 2^-77 + r * 2^-100 by one byte permute; their difference is exact, and a multiplication by 2^-65
-// rounded down yields floor(.../2^16) * 2^-149, a denormal whose bit pattern IS the code.  Packing
-// multiplies and adds such denormals (exact: fixed-point arithmetic below 2^24 * 2^-149), so the packed
-// bits appear as a bit pattern too.
+// What bounds it: table reads.  32 random words take 3.6 wavefronts of the shared-memory pipe, with the loads 4.3 per 32 elements, 17.2 of
+// the 18.5 cycles that the SM's four schedulers take for 32 elements each (a copy's bandwidth would leave 13).  The
+// multiplier pipe is busy for 14.9 of them, the integer / compare pipe for 10.2, and the wide multiplies of Philox hold the
+// latter up further, so the index and the comparison with r are given to neither more than needed: the two-way dot product of 16-bit
+// halves (one operation of the multiplier pipe, 2 cycles) makes the address, table + 4 * pattern, from either half of a word, and
+// X + 65535 - r from either half of a word of random bits.  The code is then byte 2 of the difference, and codes are packed by
+// byte permutes.  124 M x 8, 16 levels, against an index of clamped binades with the sign moved beside it and r made into a
+// float by a byte permute (14.3 instructions per element, now 12.2; integer pipe 14.8 cycles): 601 -> 515 us through device
+// parameters, 591 -> 497 with the host's; 4 levels 600 -> 504.
 #include <cmath>
 
 #include "tq_device.cuh"
@@ -32,12 +33,9 @@
 
 namespace tq {
 
-constexpr uint32_t kSlotExpBits = 0x19000000u;   // 2^-77: exponent field 50, ulp 2^-100
-
 struct LutWorker {
     float alpha;
-    uint32_t base2;       // -(base pattern) in both 16-bit halves
-    uint32_t negtop2;     // the bf16 value -top in both halves
+    uint32_t top, base;   // the largest pattern, the smallest one that is evaluated
     float levels[TQ_MAX_LEVELS];
     float inv_width[TQ_MAX_LEVELS];
 };
@@ -50,34 +48,18 @@ struct LutArgs {
 __device__ __forceinline__ uint32_t max_bf16x2(uint32_t a, uint32_t b) {
     uint32_t r; asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b)); return r;
 }
-// Four pairs of codes held as denormals (bit pattern = code) -> their 8 * BITS packed bits, LSB first,
-// as a bit pattern.  Every intermediate is an integer below 2^24 in units of 2^-149: exact.
-template <int BITS>
-__device__ __forceinline__ uint32_t pack8_bits(const f32x2 (&c)[4]) {
-    constexpr float B = static_cast<float>(1 << BITS), B2 = B * B;
-    if constexpr (BITS <= 3) {
-        f32x2 a = fma2(c[3], both(B2), c[2]);
-        a = fma2(a, both(B2), c[1]);
-        a = fma2(a, both(B2), c[0]);
-        float ev, od;
-        unpair(a, ev, od);
-        return __float_as_uint(__fmaf_rn(od, B, ev));
-    } else {
-        float e0, o0, e1, o1;
-        unpair(fma2(c[1], both(B2), c[0]), e0, o0);
-        unpair(fma2(c[3], both(B2), c[2]), e1, o1);
-        return __byte_perm(__float_as_uint(__fmaf_rn(o0, B, e0)), __float_as_uint(__fmaf_rn(o1, B, e1)), 0x5410u);
-    }
+__device__ __forceinline__ uint32_t min_bf16x2(uint32_t a, uint32_t b) {
+    uint32_t r; asm("min.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b)); return r;
 }
 
 struct LutCtx {
-    uint32_t table;          // shared-memory address of the entries: positive values from byte 0, negative values from byte 32768
-    uint32_t negtop2, nbase2, cap2;
+    uint32_t table;          // shared-memory address of entry 0
+    uint32_t negtop2, top2;  // the bf16 values -P_top and P_top in both halves
     PhiloxRun pr;
 };
 
-__device__ __forceinline__ float lds_f32(uint32_t addr) {
-    float v; asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr)); return v;
+__device__ __forceinline__ uint32_t lds_u32(uint32_t addr) {
+    uint32_t v; asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr)); return v;
 }
 
 // Elements a thread quantizes as one piece: consecutive, loaded with 256-bit loads (lane after lane, so a
@@ -91,31 +73,22 @@ __device__ __forceinline__ void lut_piece(const uint32_t (&g)[Piece<BITS>::kElem
     constexpr int E = Piece<BITS>::kElems, GROUPS = E / 8, WORDS = E * BITS / 32;
     const uint64_t j0 = piece * E;
     const uint32_t blk_lo = static_cast<uint32_t>(j0 >> 3);   // rows of more than 2^35 elements do not come here
-    const f32x2 down = both(2.710505431213761e-20f);          // 2^-65
     uint32_t chunk[GROUPS];
 #pragma unroll
     for (int grp = 0; grp < GROUPS; ++grp) {
-        uint32_t rnd[4];
+        uint32_t rnd[4], v[8];
         philox_block(blk_lo + grp, cx.pr, rk, rnd);           // j0 >> 3 is a multiple of GROUPS: no carry
-        f32x2 code[4];
 #pragma unroll
         for (int h = 0; h < 4; ++h) {                          // elements 2h, 2h+1 of the group
-            const uint32_t w = max_bf16x2(g[4 * grp + h], cx.negtop2);
-            // byte offsets of the two entries: 4 * clamp(|pattern| - base, 0, n - 1), negative values 32 KB further on
-            const uint32_t off = __viaddmin_s16x2_relu(w & 0x7FFF7FFFu, cx.nbase2, cx.cap2) * 4u + (w & 0x80008000u);
-            const float y0 = lds_f32(cx.table + (off & 0xFFFFu)), y1 = lds_f32(cx.table + (off >> 16));
-            const float r0 = __uint_as_float(__byte_perm(rnd[h], kSlotExpBits, 0x7610u));
-            const float r1 = __uint_as_float(__byte_perm(rnd[h], kSlotExpBits, 0x7632u));
-            code[h] = mul2_rd(sub2(pair(y0, y1), pair(r0, r1)), down);
+            const uint32_t w = min_bf16x2(max_bf16x2(g[4 * grp + h], cx.negtop2), cx.top2);
+            v[2 * h] = dot_halves_signed(rnd[h], 0x00FFu, lds_u32(dot_halves(w, 0x0004u, cx.table)));           // X + 65535 - r
+            v[2 * h + 1] = dot_halves_signed(rnd[h], 0xFF00u, lds_u32(dot_halves(w, 0x0400u, cx.table)));
             if constexpr (TAIL) {                              // padding bits are zero
-                float c0, c1;
-                unpair(code[h], c0, c1);
-                if (j0 + 8 * grp + 2 * h >= d) c0 = 0.0f;
-                if (j0 + 8 * grp + 2 * h + 1 >= d) c1 = 0.0f;
-                code[h] = pair(c0, c1);
+                if (j0 + 8 * grp + 2 * h >= d) v[2 * h] = 0u;
+                if (j0 + 8 * grp + 2 * h + 1 >= d) v[2 * h + 1] = 0u;
             }
         }
-        chunk[grp] = pack8_bits<BITS>(code);
+        chunk[grp] = pack_byte2<BITS>(v);
     }
 
     uint32_t w[WORDS];
@@ -153,38 +126,43 @@ __device__ __forceinline__ void load_piece(const char* row, uint64_t piece, uint
                      : "l"(row + piece * (2 * E) + 32 * i));
 }
 
-// One block per SM.  80 registers a thread allow 24 warps, as one block of 768 threads, two of 384 or three of 256: with one there is
-// one table to build (124 M x 8 in equal shares, 16 levels, host / device parameters: 604 / 613 us, 603 / 613, 622 / 624; 15 M x 4: 42.6 / 47.0, 44.2 /
-// 49.1, 45.5 / 51.1).  28 warps spill at 72 registers: 639 / 684.
-constexpr int kLutThreads = 768;
+// One block per SM, with the table that all its warps share.  Codes of 2 and 4 bits, pieces of 16 elements: 24 warps of 80 registers, of which the
+// next iteration's loads take 16 while the present one is quantized (124 M x 8, 16 levels, host / device parameters: 497 / 508 us; without them
+// 24 warps 547 / 537, 28 warps 518 / 528, 32 warps 539 / 515).  Codes of 1 and 3 bits, pieces of 32: more warps instead (28 warps 500 us, 32 warps
+// 535, 24 with the second set 555 and spills).
+template <int BITS> struct LutShape {
+    static constexpr bool kTwoBuffers = BITS == 2 || BITS == 4;
+    static constexpr int kThreads = kTwoBuffers ? 768 : 896;
+};
 
-// A block's share of one row: build the table for quantizer q (n_entries per sign), then quantize the pieces begin + thread, + stride,
+// A block's share of one row: build the table for quantizer q, then quantize the pieces begin + thread, + stride,
 // ... below `end`, and with LAST the row's last one, possibly partial.
 template <int BITS, bool WAIT>
-__device__ __forceinline__ void lut_block(const LutWorker& q, uint32_t n_entries, float* s_table, const char* __restrict__ row,
+__device__ __forceinline__ void lut_block(const LutWorker& q, uint32_t* s_table, const char* __restrict__ row,
                                           uint32_t* __restrict__ prow, uint64_t d, uint64_t words_out, uint32_t worker,
                                           const RoundKeys& rk, uint64_t begin, uint64_t stride, uint64_t end, bool last) {
-    // the table: the decision for every bit pattern of the window, both signs
+    constexpr int kLutThreads = LutShape<BITS>::kThreads;
     {
-        const uint32_t base = (0u - q.base2) & 0xFFFFu;
-        for (uint32_t i = threadIdx.x; i < 2 * n_entries; i += kLutThreads) {
-            const bool neg = i >= n_entries;
-            const uint32_t c = neg ? i - n_entries : i;
-            const uint32_t pattern = (base + c) | (neg ? 0x8000u : 0u);
-            const uint32_t x = decision_x(bf16_pattern_value(pattern), q.alpha, q.levels, q.inv_width, 1u << BITS);
-            s_table[c + (neg ? kLutMaxEntries : 0)] = __uint_as_float(kSlotExpBits + x + 65535u);
+        const LutRule rule{q.alpha, 1u << BITS, q.levels, q.inv_width};
+        const uint32_t first = q.base & ~3u, n = q.top + 1 - first;             // everything below `first` is decided like zero
+        const uint32_t x0 = decision_x(0.0f, rule) + 65535u;
+        for (uint32_t i = threadIdx.x; i < first / 2; i += kLutThreads) {       // four entries at a time, both signs
+            const uint32_t at = i < first / 4 ? 4 * i : 0x8000u + 4 * i - first;
+            *reinterpret_cast<uint4*>(s_table + at) = make_uint4(x0, x0, x0, x0);
+        }
+        for (uint32_t i = threadIdx.x; i < 2 * n; i += kLutThreads) {
+            const uint32_t pattern = first + (i >= n ? i - n + 0x8000u : i);
+            s_table[pattern] = decision_x(bf16_pattern_value(pattern), rule) + 65535u;
         }
     }
     __syncthreads();
     if constexpr (WAIT) pdl_wait();          // the table came from kernel parameters
 
     constexpr int E = Piece<BITS>::kElems, PER_ITER = 32 / E;   // 32 elements per thread and iteration: four Philox blocks in flight
-    const LutCtx cx{smem_addr(s_table), q.negtop2, q.base2, (n_entries - 1) * 0x00010001u, philox_run(0u, worker, rk)};
+    const LutCtx cx{smem_addr(s_table), (q.top | 0x8000u) * 0x00010001u, q.top * 0x00010001u, philox_run(0u, worker, rk)};
     const uint64_t row_interior = (d - 1) / E, interior = end < row_interior ? end : row_interior;      // whole pieces before the row's last one
 
-    // two sets of registers take turns: the next iteration's loads are in flight while this one is quantized
     uint64_t piece = begin + threadIdx.x;
-    uint32_t a[PER_ITER][E / 2], b[PER_ITER][E / 2];
     auto fetch = [&](uint32_t (&buf)[PER_ITER][E / 2], uint64_t first) {
 #pragma unroll
         for (int k = 0; k < PER_ITER; ++k)
@@ -195,15 +173,24 @@ __device__ __forceinline__ void lut_block(const LutWorker& q, uint32_t n_entries
         for (int k = 0; k < PER_ITER; ++k)
             if (first + k * stride < interior) lut_piece<BITS, false>(buf[k], prow, first + k * stride, d, words_out, rk, cx);
     };
-    fetch(a, piece);
-    while (piece < interior) {
-        const uint64_t next = piece + PER_ITER * stride;
-        fetch(b, next);
-        quantize(a, piece);
-        if (next >= interior) break;
-        piece = next + PER_ITER * stride;
+    uint32_t a[PER_ITER][E / 2];
+    if constexpr (LutShape<BITS>::kTwoBuffers) {       // two sets of registers take turns: the next iteration's loads are in flight while this one is quantized
+        uint32_t b[PER_ITER][E / 2];
         fetch(a, piece);
-        quantize(b, next);
+        while (piece < interior) {
+            const uint64_t next = piece + PER_ITER * stride;
+            fetch(b, next);
+            quantize(a, piece);
+            if (next >= interior) break;
+            piece = next + PER_ITER * stride;
+            fetch(a, piece);
+            quantize(b, next);
+        }
+    } else {
+        for (; piece < interior; piece += PER_ITER * stride) {
+            fetch(a, piece);
+            quantize(a, piece);
+        }
     }
     if (last && threadIdx.x == 0) {
         const unsigned short* e = reinterpret_cast<const unsigned short*>(row);
@@ -220,13 +207,14 @@ __device__ __forceinline__ void lut_block(const LutWorker& q, uint32_t n_entries
 
 // Quantizers passed by value (host-side tq_params); the host has chosen the window.
 template <int BITS>
-__global__ void __launch_bounds__(kLutThreads, 1)
+__global__ void __launch_bounds__(LutShape<BITS>::kThreads, 1)
 compress_lut_kernel(const void* __restrict__ grad, uint64_t d, uint64_t grad_stride, const __grid_constant__ LutArgs args,
-                    const __grid_constant__ RoundKeys rk, uint32_t n_entries, uint32_t first_worker,
+                    const __grid_constant__ RoundKeys rk, uint32_t first_worker,
                     uint32_t* __restrict__ packed, uint64_t words_stride, uint64_t words_out) {
-    extern __shared__ __align__(16) float s_table[];          // kLutMaxEntries + n_entries: the negative half starts at entry kLutMaxEntries
+    constexpr int kLutThreads = LutShape<BITS>::kThreads;
+    extern __shared__ __align__(16) uint32_t s_table[];       // lut_bytes of the largest of the workers' last patterns
     const uint32_t wi = blockIdx.y;
-    lut_block<BITS, true>(args.q[wi], n_entries, s_table, static_cast<const char*>(grad) + static_cast<uint64_t>(wi) * grad_stride * 2,
+    lut_block<BITS, true>(args.q[wi], s_table, static_cast<const char*>(grad) + static_cast<uint64_t>(wi) * grad_stride * 2,
                     packed + static_cast<uint64_t>(wi) * words_stride, d, words_out, first_worker + wi, rk,
                     static_cast<uint64_t>(blockIdx.x) * kLutThreads, static_cast<uint64_t>(gridDim.x) * kLutThreads, ~0ull, blockIdx.x == 0);
 }
@@ -238,9 +226,9 @@ struct LutState {
     LutWorker q;
     uint32_t fits[2];                                         // bit b of the 64: a window of b + 1 binades serves the row
 };
-// The record's quantizer into s.q; returns the entries per sign, 0 if the table does not serve it.  Block-uniform; ends with a barrier.
+// The record's quantizer into s.q; says whether the table serves it.  Block-uniform; ends with a barrier.
 template <int BITS>
-__device__ __forceinline__ uint32_t lut_record(const tq_params_t& rec, LutState& s) {
+__device__ __forceinline__ bool lut_record(const tq_params_t& rec, LutState& s) {
     if (threadIdx.x < TQ_MAX_LEVELS) {
         s.q.levels[threadIdx.x] = rec.levels[threadIdx.x];
         s.q.inv_width[threadIdx.x] = rec.inv_width[threadIdx.x];
@@ -248,59 +236,58 @@ __device__ __forceinline__ uint32_t lut_record(const tq_params_t& rec, LutState&
     const float alpha = rec.alpha;                            // read beside the levels: after a barrier it would be one more trip to memory
     const bool usable = lut_usable(rec, BITS);
     __syncthreads();
-    if (!usable) return 0;
+    if (!usable) return false;
     const uint32_t top = top_pattern(alpha);
     uint32_t base = 0;
-    if (threadIdx.x < 64) {
-        const bool fits = lut_window_fits(alpha, s.q.levels, s.q.inv_width, 1u << BITS, top, kLutBinade * (threadIdx.x + 1), &base);
+    if (threadIdx.x < kLutBinades) {
+        const bool fits = lut_window_fits(LutRule{alpha, 1u << BITS, s.q.levels, s.q.inv_width}, top, kLutBinade * (threadIdx.x + 1), &base);
         const uint32_t bits = __ballot_sync(0xFFFFFFFFu, fits);
         if ((threadIdx.x & 31u) == 0) s.fits[threadIdx.x >> 5] = bits;
     }
     __syncthreads();
-    if (s.fits[1] >> 31 == 0) return 0;                       // the rule of lut_serves_record: not even the largest window
-    const uint32_t n_entries = kLutBinade * (s.fits[0] ? __ffs(static_cast<int>(s.fits[0])) : 32 + __ffs(static_cast<int>(s.fits[1])));
+    if (s.fits[1] >> 31 == 0) return false;                   // the rule of lut_serves_record: not even the largest window
+    const uint32_t n = kLutBinade * (s.fits[0] ? __ffs(static_cast<int>(s.fits[0])) : 32 + __ffs(static_cast<int>(s.fits[1])));
     if (threadIdx.x == 0) {
-        base = top >= n_entries ? top - (n_entries - 1) : 0u;
         s.q.alpha = alpha;
-        s.q.base2 = ((0u - base) & 0xFFFFu) * 0x00010001u;
-        s.q.negtop2 = (top | 0x8000u) * 0x00010001u;
+        s.q.top = top;
+        s.q.base = top >= n ? top - (n - 1) : 0u;
     }
     __syncthreads();
-    return n_entries;
+    return true;
 }
 
 template <int BITS>
-__global__ void __launch_bounds__(kLutThreads, 1)
+__global__ void __launch_bounds__(LutShape<BITS>::kThreads, 1)
 compress_lut_kernel_dev(const void* __restrict__ grad, uint64_t d, uint64_t grad_stride, const tq_params_t* params,
                         const __grid_constant__ RoundKeys rk, uint32_t first_worker, uint32_t* __restrict__ packed,
                         uint64_t words_stride, uint64_t words_out) {
-    extern __shared__ __align__(16) float s_table[];          // 2 * kLutMaxEntries
+    extern __shared__ __align__(16) uint32_t s_table[];       // kLutMostBytes
+    constexpr int kLutThreads = LutShape<BITS>::kThreads;
     __shared__ LutState s;
     const uint32_t wi = blockIdx.y;
     pdl_wait();
-    const uint32_t n_entries = lut_record<BITS>(params[wi], s);
-    if (n_entries == 0) return;
-    lut_block<BITS, false>(s.q, n_entries, s_table, static_cast<const char*>(grad) + static_cast<uint64_t>(wi) * grad_stride * 2,
+    if (!lut_record<BITS>(params[wi], s)) return;
+    lut_block<BITS, false>(s.q, s_table, static_cast<const char*>(grad) + static_cast<uint64_t>(wi) * grad_stride * 2,
                     packed + static_cast<uint64_t>(wi) * words_stride, d, words_out, first_worker + wi, rk,
                     static_cast<uint64_t>(blockIdx.x) * kLutThreads, static_cast<uint64_t>(gridDim.x) * kLutThreads, ~0ull, blockIdx.x == 0);
 }
 
 // Layer groups: a block's range of the jobs' tiles (kLutThreads pieces each), a table for every piece of a job.
 template <int BITS>
-__global__ void __launch_bounds__(kLutThreads, 1)
+__global__ void __launch_bounds__(LutShape<BITS>::kThreads, 1)
 compress_lut_kernel_segs(const void* __restrict__ grad, uint64_t grad_stride, const tq_params_t* params,
                          const __grid_constant__ RoundKeys rk, uint32_t first_worker, uint32_t* __restrict__ packed, uint64_t words_stride,
                          const __grid_constant__ TilePlan plan) {
-    extern __shared__ __align__(16) float s_table[];          // 2 * kLutMaxEntries
+    extern __shared__ __align__(16) uint32_t s_table[];       // kLutMostBytes
+    constexpr int kLutThreads = LutShape<BITS>::kThreads;
     __shared__ LutState s;
     uint64_t cur = first_tile_of_block(plan, blockIdx.x);
     const uint64_t range_end = first_tile_of_block(plan, blockIdx.x + 1);
     pdl_wait();
     while (cur < range_end) {
         const JobPiece job = next_piece(plan, cur, range_end);
-        const uint32_t n_entries = lut_record<BITS>(params[job.job], s);
-        if (n_entries != 0)
-            lut_block<BITS, false>(s.q, n_entries, s_table,
+        if (lut_record<BITS>(params[job.job], s))
+            lut_block<BITS, false>(s.q, s_table,
                                    static_cast<const char*>(grad) + (static_cast<uint64_t>(job.worker) * grad_stride + job.off) * 2,
                                    packed + static_cast<uint64_t>(job.worker) * words_stride + plan.segs.woff[job.seg], job.d,
                                    (((job.d * BITS + 31) >> 5) + 3) & ~static_cast<uint64_t>(3), first_worker + job.worker, rk,
@@ -311,28 +298,29 @@ compress_lut_kernel_segs(const void* __restrict__ grad, uint64_t grad_stride, co
 
 // ---- host --------------------------------------------------------------------------------------------
 
-// Entries per sign the worker needs, 0 if no window of at most kLutMaxEntries does.
-static uint32_t entries_needed(const tq_params_t& p, uint32_t top) {
+constexpr int lut_bytes(uint32_t top) { return static_cast<int>((0x8000u + top + 1) * sizeof(uint32_t)); }
+constexpr int kLutMostBytes = lut_bytes(kLutMostTop);
+
+// First pattern that has to be evaluated; false if no window of at most kLutBinades binades serves the quantizer.
+static bool first_pattern(const LutRule& q, uint32_t top, uint32_t* base) {
     // a window that fits stays valid when it is made larger: halve the range of sizes
-    uint32_t lo = 0, hi = kLutMaxEntries / kLutBinade, base = 0;
-    if (!lut_window_fits(p.alpha, p.levels, p.inv_width, p.num_levels, top, kLutMaxEntries, &base)) return 0;
+    uint32_t lo = 0, hi = kLutBinades;
+    if (!lut_window_fits(q, top, hi * kLutBinade, base)) return false;
     while (hi - lo > 1) {
         const uint32_t mid = (lo + hi) / 2;
-        if (lut_window_fits(p.alpha, p.levels, p.inv_width, p.num_levels, top, mid * kLutBinade, &base)) hi = mid; else lo = mid;
+        if (lut_window_fits(q, top, mid * kLutBinade, base)) hi = mid; else lo = mid;
     }
-    return hi * kLutBinade;
+    return lut_window_fits(q, top, hi * kLutBinade, base);
 }
 
 template <int BITS>
-static cudaError_t launch_lut(const CompressCall& c, const LutArgs& args, uint32_t n_entries, uint32_t per_worker) {
-    const int smem = static_cast<int>((kLutMaxEntries + n_entries) * sizeof(float));
+static cudaError_t launch_lut(const CompressCall& c, const LutArgs& args, uint32_t top, uint32_t per_worker) {
     // always the same limit: another thread may set it between this call's and the launch
-    const cudaError_t e = cudaFuncSetAttribute(compress_lut_kernel<BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * kLutMaxEntries * static_cast<int>(sizeof(float)));
+    const cudaError_t e = cudaFuncSetAttribute(compress_lut_kernel<BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize, kLutMostBytes);
     if (e != cudaSuccess) return e;
-    return launch_kernel(compress_lut_kernel<BITS>, dim3(per_worker, c.n_workers), kLutThreads, smem, c.stream, c.grad, c.d,
-                         c.grad_stride, args, round_keys(c.seed), n_entries, c.first_worker, c.packed, c.words_stride, c.words_out);
+    return launch_kernel(compress_lut_kernel<BITS>, dim3(per_worker, c.n_workers), LutShape<BITS>::kThreads, lut_bytes(top), c.stream, c.grad, c.d,
+                         c.grad_stride, args, round_keys(c.seed), c.first_worker, c.packed, c.words_stride, c.words_out);
 }
-
 
 // Blocks per row, and what the longest chain of blocks costs with them, in elements that a block quantizes in that time: a table costs
 // as much as 40000 (3.5 us), the waves follow one another, and SMs differ by 3 % of a share, which more and shorter shares
@@ -352,31 +340,30 @@ static uint64_t lut_plan(uint64_t d, uint32_t n_workers, uint32_t* per_worker) {
 
 template <int BITS>
 static cudaError_t launch_lut_dev(const CompressCall& c, uint32_t per_worker) {
-    const int smem = static_cast<int>(2 * kLutMaxEntries * sizeof(float));
-    cudaError_t e = cudaFuncSetAttribute(compress_lut_kernel_dev<BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = cudaFuncSetAttribute(compress_lut_kernel_dev<BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize, kLutMostBytes);
     if (e != cudaSuccess) return e;
-    return launch_kernel(compress_lut_kernel_dev<BITS>, dim3(per_worker, c.n_workers), kLutThreads, smem, c.stream, c.grad,
+    return launch_kernel(compress_lut_kernel_dev<BITS>, dim3(per_worker, c.n_workers), LutShape<BITS>::kThreads, kLutMostBytes, c.stream, c.grad,
                          c.d, c.grad_stride, c.params_dev, round_keys(c.seed), c.first_worker, c.packed, c.words_stride, c.words_out);
 }
 
 template <int BITS>
 static cudaError_t launch_lut_segs(const CompressCall& c, uint32_t blocks) {
     static thread_local TilePlan plan;
-    plan_tiles(&plan, c.segs, c.d, c.n_workers, static_cast<uint64_t>(kLutThreads) * Piece<BITS>::kElems, blocks);
-    const int smem = static_cast<int>(2 * kLutMaxEntries * sizeof(float));
-    const cudaError_t e = cudaFuncSetAttribute(compress_lut_kernel_segs<BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    plan_tiles(&plan, c.segs, c.d, c.n_workers, static_cast<uint64_t>(LutShape<BITS>::kThreads) * Piece<BITS>::kElems, blocks);
+    const cudaError_t e = cudaFuncSetAttribute(compress_lut_kernel_segs<BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize, kLutMostBytes);
     if (e != cudaSuccess) return e;
-    return launch_kernel(compress_lut_kernel_segs<BITS>, dim3(plan.blocks), kLutThreads, smem, c.stream, c.grad, c.grad_stride, c.params_dev,
+    return launch_kernel(compress_lut_kernel_segs<BITS>, dim3(plan.blocks), LutShape<BITS>::kThreads, kLutMostBytes, c.stream, c.grad, c.grad_stride, c.params_dev,
                          round_keys(c.seed), c.first_worker, c.packed, c.words_stride, plan);
 }
 
-// The element-wise kernels take 1.65 times as long per element (and no table; 1.43 times where the call with device parameters needs a second launch
-// for the rows that the table does not serve).  Table / element-wise, host and device parameters: 8 M 13.0 / 12.6 and 16.2 / 14.2
-// us, 10 M 12.7 / 13.6 and 16.2 / 15.3, 2 M x 8 17.0 / 21.0 and 20.9 / 22.4, 300 k x 64 (128 blocks for 148 SMs) 20.4 / 22.9 and 25.4 /
-// 24.6, 30 M 24.9 / 31.2 and 28.3 / 33.4, 124 M x 8 591 / 843 and 599 / 843.
+// The element-wise kernels take about 1.7 times as long per element and build no table.  1.78 here, because behind another kernel the table of the
+// host's parameters is built early; 1.53 with device parameters, where it is not and where a second launch looks for rows that the table
+// does not serve.  Table / element-wise, 16 levels, host and device parameters: 8 M 7.8 / 9.8 and 13.1 / 11.8 us, 12 M 9.9 / 12.6 and 14.8 / 15.9, 2 M
+// x 8 12.3 / 17.7 and 17.9 / 19.5, 300 k x 64 (128 blocks for 148 SMs) 15.7 / 20.2 and 22.6 / 22.3, 30 M 19.2 / 27.7 and 24.3 / 31.5, 124 M x 8
+// 501 / 843 and 508 / 843.
 static bool lut_pays(const CompressCall& c, uint32_t* per_worker) {
     const uint64_t cost = lut_plan(c.d, c.n_workers, per_worker), others = c.d * c.n_workers / static_cast<uint64_t>(sm_count());
-    return cost * 100 < others * (c.params_dev ? 143 : 165);
+    return cost * 100 < others * (c.params_dev ? 153 : 178);
 }
 
 cudaError_t launch_compress_lut(const CompressCall& c, bool* applied) {
@@ -413,31 +400,23 @@ cudaError_t launch_compress_lut(const CompressCall& c, bool* applied) {
         }
     }
     static thread_local LutArgs args;
-    uint32_t n_entries = 0;
+    uint32_t most = 0;
     for (uint32_t i = 0; i < c.n_workers; ++i) {
         const tq_params_t& p = c.params[i];
         if (!(p.alpha > 0.0f) || !(p.alpha <= 3.402823466e38f)) return cudaSuccess;
-        const uint32_t top = top_pattern(p.alpha);
-        const uint32_t n = entries_needed(p, top);
-        if (n == 0) return cudaSuccess;
-        if (n > n_entries) n_entries = n;
-    }
-    for (uint32_t i = 0; i < c.n_workers; ++i) {
-        const tq_params_t& p = c.params[i];
         LutWorker& q = args.q[i];
-        const uint32_t top = top_pattern(p.alpha);
-        const uint32_t base = top >= n_entries ? top - (n_entries - 1) : 0u;   // a larger window than needed stays valid
+        q.top = top_pattern(p.alpha);
+        if (q.top > kLutMostTop || !first_pattern(lut_rule(p, c.bits), q.top, &q.base)) return cudaSuccess;
+        most = q.top > most ? q.top : most;
         q.alpha = p.alpha;
-        q.base2 = ((0u - base) & 0xFFFFu) * 0x00010001u;
-        q.negtop2 = (top | 0x8000u) * 0x00010001u;
         for (int k = 0; k < TQ_MAX_LEVELS; ++k) { q.levels[k] = p.levels[k]; q.inv_width[k] = p.inv_width[k]; }
     }
     *applied = true;
     switch (c.bits) {
-        case 1: return launch_lut<1>(c, args, n_entries, per_worker);
-        case 2: return launch_lut<2>(c, args, n_entries, per_worker);
-        case 3: return launch_lut<3>(c, args, n_entries, per_worker);
-        default: return launch_lut<4>(c, args, n_entries, per_worker);
+        case 1: return launch_lut<1>(c, args, most, per_worker);
+        case 2: return launch_lut<2>(c, args, most, per_worker);
+        case 3: return launch_lut<3>(c, args, most, per_worker);
+        default: return launch_lut<4>(c, args, most, per_worker);
     }
 }
 

@@ -183,6 +183,35 @@ __device__ __forceinline__ void philox_block(uint32_t c0, const PhiloxRun& pr, c
     out[0] = x0; out[1] = x1; out[2] = x2; out[3] = x3;
 }
 
+// ---- 16-bit halves and packing ------------------------------------------------------------------------
+// c + a.lo * w.byte0 + a.hi * w.byte1: the halves of a without sign, the bytes of w without / with.  One operation of the
+// multiplier pipe, 2 cycles, where a shift or a mask and an addition are two of the integer / compare pipe, 2 cycles each.
+__device__ __forceinline__ uint32_t dot_halves(uint32_t a, uint32_t w, uint32_t c) {
+    uint32_t r; asm("dp2a.lo.u32.u32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(w), "r"(c)); return r;
+}
+__device__ __forceinline__ uint32_t dot_halves_signed(uint32_t a, uint32_t w, uint32_t c) {
+    uint32_t r; asm("dp2a.lo.u32.s32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(w), "r"(c)); return r;
+}
+// The codes in byte 2 of eight words -> their 8 * BITS packed bits, LSB first.
+template <int BITS>
+__device__ __forceinline__ uint32_t pack_byte2(const uint32_t (&v)[8]) {
+    auto four = [](uint32_t a, uint32_t b, uint32_t c, uint32_t d) {       // byte 2 of each
+        return __byte_perm(__byte_perm(a, b, 0x0062u), __byte_perm(c, d, 0x0062u), 0x5410u);
+    };
+    if constexpr (BITS <= 2) {
+        // c0 .. c3 side by side in the top byte of a product; the other partial products are disjoint bits below it
+        constexpr uint32_t K = (1u << 24) + (1u << (16 + BITS)) + (1u << (8 + 2 * BITS)) + (1u << (3 * BITS));
+        const uint32_t lo = four(v[0], v[1], v[2], v[3]) * K, hi = four(v[4], v[5], v[6], v[7]) * K;
+        if constexpr (BITS == 2) return __byte_perm(lo, hi, 0x0073u);      // 16 bits; the callers merge chunks by byte permutes
+        else return (lo >> 24) | ((hi >> 24) << 4);
+    } else {
+        const uint32_t t = four(v[0], v[2], v[4], v[6]) + (four(v[1], v[3], v[5], v[7]) << BITS);      // two codes per byte
+        if constexpr (BITS == 4) return t;
+        const uint32_t u = (t & 0x003F003Fu) | ((t >> 2) & 0x0FC00FC0u);                                // four codes per half
+        return (u & 0xFFFu) | ((u >> 4) & 0xFFF000u);
+    }
+}
+
 // ---- a block's pieces (see TilePlan) ---------------------------------------------------------------
 struct JobPiece {
     uint32_t worker, seg, job;

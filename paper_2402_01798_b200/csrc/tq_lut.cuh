@@ -6,20 +6,28 @@
 
 namespace tq {
 
-constexpr int kLutBinade = 128;          // entries per sign and binade
-constexpr int kLutMaxEntries = 8192;     // per sign: 64 binades
+constexpr uint32_t kLutBinade = 128;       // patterns per sign and binade
+constexpr uint32_t kLutBinades = 64;       // evaluated binades, at most
+constexpr uint32_t kLutMostTop = 0x61FFu;  // largest pattern with an entry: 4 * (2^15 + 0x61FF + 1) bytes of shared memory, 226 KB
+
+// What the decision depends on besides the value; the tables stay where they are.
+struct LutRule {
+    float alpha;
+    uint32_t num_levels;
+    const float* levels;
+    const float* inv_width;
+};
 
 // X = k * 2^16 + min(T, 2^16) for a gradient value g: the decision of the quantizer equation up to the
 // random draw.  One IEEE operation per step (the build disables contraction on both sides), so host and
 // device agree bit for bit.
-__host__ __device__ inline uint32_t decision_x(float g, float alpha, const float* levels, const float* inv_width,
-                                               uint32_t num_levels) {
-    const uint32_t s = num_levels - 1;
-    const float t = fminf(fmaxf(g, -alpha), alpha);          // NaN -> -alpha, +-Inf -> +-alpha
+__host__ __device__ inline uint32_t decision_x(float g, const LutRule& q) {
+    const uint32_t s = q.num_levels - 1;
+    const float t = fminf(fmaxf(g, -q.alpha), q.alpha);      // NaN -> -alpha, +-Inf -> +-alpha
     uint32_t k = 0;
     for (uint32_t j = 1; j + 1 <= s; ++j)                     // largest j <= s - 1 with l_j <= t
-        if (levels[j] <= t) k = j;
-    const float p = (t - levels[k]) * inv_width[k];
+        if (q.levels[j] <= t) k = j;
+    const float p = (t - q.levels[k]) * q.inv_width[k];
     const float tf = p * 65536.0f;
     const uint32_t T = !(tf > 0.0f) ? 0u : (tf >= 65536.0f ? 65536u : static_cast<uint32_t>(rintf(tf)));
     return k * 65536u + T;
@@ -49,26 +57,24 @@ __host__ __device__ inline uint32_t top_pattern(float alpha) {
     return p;
 }
 
-// Whether a window of n entries per sign below `top` serves the quantizer: either it reaches down to zero, or the
-// decision at +-base equals that of everything smaller (it is monotone in the value).  *base receives the window's
-// first pattern.
-__host__ __device__ inline bool lut_window_fits(float alpha, const float* levels, const float* inv_width, uint32_t num_levels,
-                                                uint32_t top, uint32_t n, uint32_t* base) {
+// Whether a window of n patterns per sign, the last one `top`, holds all that differ in their decision: either it reaches
+// down to zero, or the decision at +-base equals that of everything smaller (it is monotone in the value).  *base receives the
+// window's first pattern.
+__host__ __device__ inline bool lut_window_fits(const LutRule& q, uint32_t top, uint32_t n, uint32_t* base) {
     if (top < n) { *base = 0; return true; }
     *base = top - (n - 1);
-    return decision_x(bf16_pattern_value(*base | 0x8000u), alpha, levels, inv_width, num_levels) ==
-           decision_x(bf16_pattern_value(*base), alpha, levels, inv_width, num_levels);
+    return decision_x(bf16_pattern_value(*base | 0x8000u), q) == decision_x(bf16_pattern_value(*base), q);
 }
 
 // Device-resident parameters: a row goes through the table kernel when its record is usable and the largest window
 // serves it; the element-wise kernels evaluate the same rule and leave exactly those rows alone.
+__host__ __device__ inline LutRule lut_rule(const tq_params_t& p, uint32_t bits) { return LutRule{p.alpha, 1u << bits, p.levels, p.inv_width}; }
 __host__ __device__ inline bool lut_usable(const tq_params_t& p, uint32_t bits) {
-    return p.alpha > 0.0f && p.alpha <= 3.402823466e38f && p.bits == bits && !(p.flags & TQ_FLAG_INVALID);
+    return p.alpha > 0.0f && p.bits == bits && !(p.flags & TQ_FLAG_INVALID) && top_pattern(p.alpha) <= kLutMostTop;
 }
-__host__ __device__ inline bool lut_serves_record(const tq_params_t& p, uint32_t bits, uint32_t* top, uint32_t* base) {
-    if (!lut_usable(p, bits)) return false;
-    *top = top_pattern(p.alpha);
-    return lut_window_fits(p.alpha, p.levels, p.inv_width, 1u << bits, *top, kLutMaxEntries, base);
+__host__ __device__ inline bool lut_serves_record(const tq_params_t& p, uint32_t bits) {
+    uint32_t base;
+    return lut_usable(p, bits) && lut_window_fits(lut_rule(p, bits), top_pattern(p.alpha), kLutBinade * kLutBinades, &base);
 }
 
 }  // namespace tq

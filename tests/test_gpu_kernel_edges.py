@@ -220,6 +220,30 @@ def test_decision_table_dispatch(tq, orc, bits, d, n):
     assert np.array_equal(got[n - 1].cpu().numpy().view(np.uint32), orc.compress(g[n - 1, :d].float().cpu().numpy(), _oracle_params(orc, p), 3, n - 1))
 
 
+@pytest.mark.parametrize("bits", [1, 2, 3, 4])
+@pytest.mark.parametrize("top", [0x0200, 0x3A80, 0x3A81, 0x3A82, 0x3A83, 0x61FF, 0x6200])
+def test_decision_table_of_every_pattern(tq, orc, bits, top):
+    """The table is indexed by the bf16 pattern up to the smallest one >= alpha and filled in four entries at a time below the
+    evaluated ones: alpha at each place of a group of four, at the smallest normal numbers, and at the largest pattern that has an entry and the
+    next.  Rows hold every pattern there is but signalling NaN (which C's fmaxf, unlike the GPU's, does not drop)."""
+    d, n, L = 1_100_003, 16, 1 << bits
+    alpha = float(np.array([top << 16], np.uint32).view(np.float32)[0])
+    p = tq.tq_params_from_levels([float(np.float32(alpha) * np.float32((2 * k - (L - 1)) / (L - 1))) for k in range(L)])
+    every = torch.arange(65536, dtype=torch.int32)
+    every = torch.where((every & 0x7FFF) > 0x7F80, every | 0x40, every).to(torch.int16)
+    near = torch.randint(max(top - 1500, 0), top + 40, (d,), generator=torch.Generator().manual_seed(top), dtype=torch.int32)
+    row = torch.cat([every, (near + (torch.arange(d) % 2).int() * 0x8000).to(torch.int16)])[:d].cuda()
+    g = torch.zeros(n, (d + 15) // 16 * 16, dtype=torch.int16, device="cuda")
+    for i in range(n):
+        g[i, :d] = torch.roll(row, 1237 * i)
+    g = g.view(torch.bfloat16)
+    got = tq.tq_compress(g, [p] * n, seed=8, d=d)
+    raw = torch.frombuffer(bytearray(bytes(p) * n), dtype=torch.uint8).cuda()
+    assert torch.equal(got, tq.tq_compress_device_params(g, raw, L, tq.NONUNIFORM, seed=8, d=d))
+    for i in (0, n - 1):
+        assert np.array_equal(got[i].cpu().numpy().view(np.uint32), orc.compress(g[i, :d].float().cpu().numpy(), _oracle_params(orc, p), 8, i))
+
+
 @pytest.mark.parametrize("bits,bad", [(4, False), (3, True), (1, False)])
 def test_decision_table_of_layer_groups(tq, orc, bits, bad):
     """bf16 layer groups large enough for a table per piece: lengths from one element up, ranges that cross several jobs, one job whose
