@@ -97,35 +97,29 @@ __device__ __forceinline__ float rounds_up(float p, float rf) {
 //   y   = min(y, s/L)                          this is x = s, which the reference codes as s, like every g >= alpha
 //   Xm  = fma(y, L * 2^16, 2^23)               = 2^23 + X, rounded to nearest-even as rint does (2^23 is even)
 //   v   = bits(Xm) - r + 65535                 = 0x4B000000 + (X - r + 65535): the code is byte 2 of v
-// From Xm on the integer pipe does the work: the kernel is bound by the multiplier pipe, which Philox's wide
-// multiplies keep busy for 9 of its 16 cycles per 32 elements, and floating-point operations load that pipe too
-// (30 M x 8 fp32, 16 levels 167 -> 156 us, 4 levels 158 -> 150).  For bf16 storage the widening shares the integer pipe, and the
-// form below it (2- and 4-bit codes) stays the faster one (124 M x 8, 4 / 16 levels 498 / 511 us against 519 / 518).
+// From Xm on integers do the work.  fp32 rows: a mask or shift and one three-operand addition of the integer / compare pipe (30 M x 8,
+// 4 levels 150 us, 156 at a copy's rate).  bf16 rows are bound by the multiplier pipe, which Philox's wide multiplies keep busy for 9
+// cycles per 32 elements, and the integer pipe (2 per logic operation or byte permute): there the complement of a word of random bits,
+// 65535 - r in either half, goes through a two-way dot product (124 M x 8, 4 / 8 / 16 levels, device parameters for 4 and 8: 489 / 515 / 485
+// us; slots as floats by byte permutes, then packed subtractions and multiplications of denormals: 528 / - / 510; as for fp32: 8 levels 560.
+// For fp32 rows it is the slower form: 25.6 M x 16, 16 levels 265 -> 270).
 // sum0 / sum1 are g + alpha of the pair.
 struct UniformQ {
     float inv_step_l, c_top;      // inv_step / L, s / L
     f32x2 scale2;                 // L * 2^16, twice
-    f32x2 scale2_dn;              // L * 2^16 * 2^-100, twice (see code_uniform2_dn)
 };
 // min(y, s/L) runs on the integer/compare pipe as well.
+template <bool BF16>
 __device__ __forceinline__ void code_uniform2(float sum0, float sum1, const UniformQ& u, uint32_t rnd, uint32_t& v0, uint32_t& v1) {
     float x0, x1;
     unpair(fma2(pair(fminf(mul_sat(sum0, u.inv_step_l), u.c_top), fminf(mul_sat(sum1, u.inv_step_l), u.c_top)), u.scale2, both(kMagic)), x0, x1);
-    v0 = __float_as_uint(x0) - (rnd & 0xFFFFu) + 0xFFFFu;
-    v1 = __float_as_uint(x1) - (rnd >> 16) + 0xFFFFu;
-}
-// The same with everything scaled by 2^-100: Xm = fma(y, L * 2^16 * 2^-100, 2^-77) = 2^-77 + X * 2^-100 (rounded
-// at 2^-100 exactly as the unscaled form rounds at 1), the slot arrives as 2^-77 + r * 2^-100, and
-// (X - r) * 2^-100 * 2^-65 rounded up is ceil((X - r) / 2^16) * 2^-149: a denormal whose bit pattern is the code
-// itself, with no bias to take off (or -0 when X < r: the callers of pack8 drop the sign bit).
-constexpr uint32_t kSlotExpBits = 0x19000000u;            // 2^-77
-__device__ __forceinline__ f32x2 mul2_ru(f32x2 a, f32x2 b) {
-    f32x2 r; asm("mul.rp.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v)); return r;
-}
-__device__ __forceinline__ f32x2 code_uniform2_dn(float sum0, float sum1, const UniformQ& u, float rf0, float rf1) {
-    const f32x2 y = pair(fminf(mul_sat(sum0, u.inv_step_l), u.c_top), fminf(mul_sat(sum1, u.inv_step_l), u.c_top));
-    const f32x2 v = sub2(fma2(y, u.scale2_dn, both(6.617444900424222e-24f)), pair(rf0, rf1));
-    return mul2_ru(v, both(2.710505431213761e-20f));     // 2^-65
+    if constexpr (BF16) {
+        v0 = dot_halves(~rnd, 0x0001u, __float_as_uint(x0));
+        v1 = dot_halves(~rnd, 0x0100u, __float_as_uint(x1));
+    } else {
+        v0 = __float_as_uint(x0) - (rnd & 0xFFFFu) + 0xFFFFu;
+        v1 = __float_as_uint(x1) - (rnd >> 16) + 0xFFFFu;
+    }
 }
 
 // The same decision without the scaled inverse step (alpha so large that inv_step / L is subnormal):
@@ -224,13 +218,7 @@ __device__ __forceinline__ float code_binary(float g, float alpha, const float* 
 // Four pairs of float codes (elements 0..7 of a group, each code < 2^BITS) -> their 8*BITS packed
 // bits, LSB first.  Every partial sum is an integer below 2^24, so the fp32 arithmetic is exact.
 // Returns a word whose low 8*BITS bits are the packed codes.
-//
-// DN (2- and 4-bit codes only): the codes are denormals whose bit pattern is the code (see
-// code_uniform2_dn), sums and products of them are fixed-point arithmetic in units of 2^-149, and the
-// packed bits appear as a bit pattern without any float -> integer conversion.  Bits above the low 16 of
-// a partial result may be set (a sum of -0 terms is -0): the caller merges chunks by byte-permutes that
-// take the low 16 bits only.
-template <int BITS, bool DN>
+template <int BITS>
 __device__ __forceinline__ uint32_t pack8(const f32x2 (&c)[4]) {
     constexpr float B = static_cast<float>(1 << BITS), B2 = B * B;
     if constexpr (BITS <= 3) {
@@ -239,15 +227,12 @@ __device__ __forceinline__ uint32_t pack8(const f32x2 (&c)[4]) {
         a = fma2(a, both(B2), c[0]);
         float ev, od;
         unpair(a, ev, od);
-        if constexpr (DN) return __float_as_uint(__fmaf_rn(od, B, ev));
-        else return __float2uint_rz(__fmaf_rn(od, B, ev));
+        return __float2uint_rz(__fmaf_rn(od, B, ev));
     } else {
         float e0, o0, e1, o1;
         unpair(fma2(c[1], both(B2), c[0]), e0, o0);       // elements 0..3: 16 bits
         unpair(fma2(c[3], both(B2), c[2]), e1, o1);       // elements 4..7: 16 bits
-        if constexpr (DN)
-            return __byte_perm(__float_as_uint(__fmaf_rn(o0, B, e0)), __float_as_uint(__fmaf_rn(o1, B, e1)), 0x5410u);
-        else return __float2uint_rz(__fmaf_rn(o0, B, e0)) + (__float2uint_rz(__fmaf_rn(o1, B, e1)) << 16);
+        return __float2uint_rz(__fmaf_rn(o0, B, e0)) + (__float2uint_rz(__fmaf_rn(o1, B, e1)) << 16);
     }
 }
 
@@ -277,7 +262,7 @@ struct RunCtx {
 template <int BITS>
 __device__ __forceinline__ UniformQ uniform_q(const WorkerQ& q) {
     constexpr float L = static_cast<float>(1 << BITS);
-    return UniformQ{q.inv_step_l, (L - 1.0f) / L, both(L * 65536.0f), both(L * 65536.0f * 7.888609052210118e-31f)};
+    return UniformQ{q.inv_step_l, (L - 1.0f) / L, both(L * 65536.0f)};
 }
 
 template <int BITS, int SEARCH>
@@ -294,10 +279,9 @@ __host__ __device__ inline float scaled_inv_step(float inv_step, uint32_t num_le
     return (q >= 1.17549435e-38f && q <= 3.402823466e38f) ? q : 0.0f;
 }
 
-// the 16 random bits of slot e of a Philox block, as the float 2^23 + r (DN: 2^-77 + r * 2^-100)
-template <bool DN>
+// the 16 random bits of slot e of a Philox block, as the float 2^23 + r
 __device__ __forceinline__ float slot_as_float(const uint32_t (&rnd)[4], int e) {
-    return __uint_as_float(__byte_perm(rnd[e >> 1], DN ? kSlotExpBits : kMagicBits, (e & 1) ? 0x7432u : 0x7410u));
+    return __uint_as_float(__byte_perm(rnd[e >> 1], kMagicBits, (e & 1) ? 0x7432u : 0x7410u));
 }
 
 // The arithmetic of one run of 32 elements that are already in registers: quantize, pack, store.
@@ -308,19 +292,18 @@ __device__ __forceinline__ void quantize_run(const Raw8<BF16> (&g)[4], uint32_t*
     const uint32_t blk_lo = static_cast<uint32_t>(j0 >> 3);
     const PhiloxRun pr = philox_run(static_cast<uint32_t>(j0 >> 35), worker, rk);
     const f32x2 alpha2 = both(cx.alpha), inv_step2 = both(cx.inv_step), cell_scale2 = both(cx.cell_scale);
-    constexpr bool DN = SEARCH == kUniform && BF16 && (BITS == 2 || BITS == 4);
     uint32_t chunk[4];   // the 8*BITS packed bits of each group
 #pragma unroll
     for (int grp = 0; grp < 4; ++grp) {
         uint32_t rnd[4];
         philox_block(blk_lo + grp, pr, rk, rnd);                      // j0 >> 3 is a multiple of 4: no carry
-        if constexpr (SEARCH == kUniform && !DN) {
+        if constexpr (SEARCH == kUniform) {
             uint32_t v[8];
 #pragma unroll
             for (int h = 0; h < 4; ++h) {        // elements 2h, 2h+1 of the group
                 float sum0, sum1;
                 pair_plus_alpha<BF16>(g[grp], h, cx.alpha, sum0, sum1);
-                code_uniform2(sum0, sum1, cx.u, rnd[h], v[2 * h], v[2 * h + 1]);
+                code_uniform2<BF16>(sum0, sum1, cx.u, rnd[h], v[2 * h], v[2 * h + 1]);
             }
             chunk[grp] = pack_byte2<BITS>(v);
         } else {
@@ -328,12 +311,11 @@ __device__ __forceinline__ void quantize_run(const Raw8<BF16> (&g)[4], uint32_t*
 #pragma unroll
             for (int h = 0; h < 4; ++h) {
                 const int e = 2 * h;
-                const float rf0 = slot_as_float<DN>(rnd, e), rf1 = slot_as_float<DN>(rnd, e + 1);
-                if constexpr (is_uniform(SEARCH)) {
+                const float rf0 = slot_as_float(rnd, e), rf1 = slot_as_float(rnd, e + 1);
+                if constexpr (SEARCH == kUniformWide) {
                     float sum0, sum1;
                     pair_plus_alpha<BF16>(g[grp], h, cx.alpha, sum0, sum1);
-                    if constexpr (DN) code[h] = code_uniform2_dn(sum0, sum1, cx.u, rf0, rf1);
-                    else code[h] = code_uniform2_wide(sum0, sum1, inv_step2, cx.top, rf0, rf1);
+                    code[h] = code_uniform2_wide(sum0, sum1, inv_step2, cx.top, rf0, rf1);
                 } else {
                     const float g0 = elem<BF16>(g[grp], e), g1 = elem<BF16>(g[grp], e + 1);
                     if constexpr (SEARCH == kGrid)
@@ -344,7 +326,7 @@ __device__ __forceinline__ void quantize_run(const Raw8<BF16> (&g)[4], uint32_t*
                                         code_binary<BITS>(g1, cx.alpha, cx.s_search, reinterpret_cast<const float2*>(cx.s_cell), rf1));
                 }
             }
-            chunk[grp] = pack8<BITS, DN>(code);
+            chunk[grp] = pack8<BITS>(code);
         }
     }
 
