@@ -277,7 +277,7 @@ template <int BITS>
 __global__ void __launch_bounds__(LutShape<BITS>::kThreads, 1)
 compress_lut_kernel_segs(const void* __restrict__ grad, uint64_t grad_stride, const tq_params_t* params,
                          const __grid_constant__ RoundKeys rk, uint32_t first_worker, uint32_t* __restrict__ packed, uint64_t words_stride,
-                         const __grid_constant__ TilePlan plan) {
+                         const __grid_constant__ TilePlan plan, uint32_t start_tiles) {
     extern __shared__ __align__(16) uint32_t s_table[];       // kLutMostBytes
     constexpr int kLutThreads = LutShape<BITS>::kThreads;
     __shared__ LutState s;
@@ -285,7 +285,10 @@ compress_lut_kernel_segs(const void* __restrict__ grad, uint64_t grad_stride, co
     const uint64_t range_end = first_tile_of_block(plan, blockIdx.x + 1);
     pdl_wait();
     while (cur < range_end) {
-        const JobPiece job = next_piece(plan, cur, range_end);
+        JobPiece job = next_piece(plan, cur, range_end);
+        if (job.tile1 <= start_tiles) continue;                // nothing of the job itself
+        job.tile0 = job.tile0 > start_tiles ? job.tile0 - start_tiles : 0;
+        job.tile1 -= start_tiles;
         if (lut_record<BITS>(params[job.job], s))
             lut_block<BITS, false>(s.q, s_table,
                                    static_cast<const char*>(grad) + (static_cast<uint64_t>(job.worker) * grad_stride + job.off) * 2,
@@ -346,14 +349,21 @@ static cudaError_t launch_lut_dev(const CompressCall& c, uint32_t per_worker) {
                          c.d, c.grad_stride, c.params_dev, round_keys(c.seed), c.first_worker, c.packed, c.words_stride, c.words_out);
 }
 
+// One range per SM.  The start of a job within a range -- its record, its table, its last piece, the loads' first latency -- takes as long as 80000
+// elements and is counted with the tiles, or a range of many short jobs holds up all others (16 levels, groups of lengths up to 75 apart, started
+// for nothing / as 40000 / 80000 / 160000 elements: 25.6 M x 16 in 16 groups 291 / 274 / 264 / 267 us, 10 M x 8 in 16 92 / 72 / 65 / 68, 124 M x 8 in 16
+// 581 / 566 / 558 / 559; two ranges per SM 269, 71 and 564 at best).
+constexpr uint64_t kLutStartElems = 80000;
 template <int BITS>
 static cudaError_t launch_lut_segs(const CompressCall& c, uint32_t blocks) {
     static thread_local TilePlan plan;
-    plan_tiles(&plan, c.segs, c.d, c.n_workers, static_cast<uint64_t>(LutShape<BITS>::kThreads) * Piece<BITS>::kElems, blocks);
+    constexpr uint64_t tile = static_cast<uint64_t>(LutShape<BITS>::kThreads) * Piece<BITS>::kElems;
+    constexpr uint32_t start_tiles = static_cast<uint32_t>((kLutStartElems + tile / 2) / tile);
+    plan_tiles(&plan, c.segs, c.d, c.n_workers, tile, blocks, start_tiles);
     const cudaError_t e = cudaFuncSetAttribute(compress_lut_kernel_segs<BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize, kLutMostBytes);
     if (e != cudaSuccess) return e;
     return launch_kernel(compress_lut_kernel_segs<BITS>, dim3(plan.blocks), LutShape<BITS>::kThreads, kLutMostBytes, c.stream, c.grad, c.grad_stride, c.params_dev,
-                         round_keys(c.seed), c.first_worker, c.packed, c.words_stride, plan);
+                         round_keys(c.seed), c.first_worker, c.packed, c.words_stride, plan, start_tiles);
 }
 
 // The element-wise kernels take about 1.7 times as long per element and build no table.  1.78 here, because behind another kernel the table of the
@@ -376,11 +386,10 @@ cudaError_t launch_compress_lut(const CompressCall& c, bool* applied) {
             if (c.segs->len[s] > (1ull << 35)) return cudaSuccess;
             total += c.segs->len[s] * c.n_workers;
         }
-        // two ranges per SM; a table for every piece, of which there are at most blocks + jobs; the element-wise kernel as above
-        // (25.6 M x 16, 16 levels, 16 groups of lengths up to 75 apart: 358 us element-wise, 305 with tables, 302 / 312 in one / three
-        // ranges per SM; 25.6 M x 8, 8 levels 183 / 179 / 184)
-        const uint32_t blocks = static_cast<uint32_t>(sm_count()) * 2;
-        if ((blocks + static_cast<uint64_t>(c.n_workers) * c.segs->n) * 40000 * 100 >= total * 43) return cudaSuccess;
+        // The start of a piece against what the table saves; the element-wise kernel as above.  Table / element-wise, 16 levels, groups of lengths up to 75
+        // apart: 25.6 M x 16 in 16 264 / 361 us, 10 M x 8 in 16 65 / 80, 2 M x 64 in 5 107 / 123, 4 M x 8 in 5 29 / 34, 10 M x 8 in 40 83 / 82.
+        const uint32_t blocks = static_cast<uint32_t>(sm_count());
+        if ((blocks + static_cast<uint64_t>(c.n_workers) * c.segs->n) * kLutStartElems * 100 >= total * 48) return cudaSuccess;
         *applied = true;
         switch (c.bits) {
             case 1: return launch_lut_segs<1>(c, blocks);
