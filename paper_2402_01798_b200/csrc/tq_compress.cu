@@ -559,13 +559,19 @@ __device__ __noinline__ void compress_piece_rare(State& sh, const void* grad, ui
 
 // The block's pieces of the jobs -- workers, or (worker, segment) pairs, see TilePlan; a tile is one run per thread.
 // Rows of jobs that are marked invalid (alpha = 0) become all code 0.
-template <int BITS, bool NONUNIFORM, bool BF16>
+// BEHIND: behind the decision-table kernel, for the rows that it does not serve.
+template <int BITS, bool NONUNIFORM, bool BF16, bool BEHIND>
 __global__ void __launch_bounds__(kThreads, TQ_COMPRESS_MIN_BLOCKS)
 compress_kernel_dev(const void* __restrict__ grad, uint64_t grad_stride, const tq_params_t* params,
                     const __grid_constant__ RoundKeys rk, uint32_t first_worker, uint32_t* __restrict__ packed, uint64_t words_stride,
-                    const __grid_constant__ TilePlan plan, int table_kernel_ran) {
+                    const __grid_constant__ TilePlan plan, uint32_t n_jobs) {
     __shared__ __align__(16) BlockState<NONUNIFORM> sh;
     pdl_wait();
+    if constexpr (BEHIND) {              // nearly always nothing is left, which one look over all records shows
+        bool left = false;
+        for (uint32_t j = threadIdx.x; j < n_jobs; j += kThreads) left = left || !lut_serves_record(params[j], BITS);
+        if (!__syncthreads_or(left)) return;
+    }
     if (threadIdx.x == 0) sh.cur = first_tile_of_block(plan, blockIdx.x);
     while (true) {
         __syncthreads();                 // the previous piece has been served
@@ -579,7 +585,7 @@ compress_kernel_dev(const void* __restrict__ grad, uint64_t grad_stride, const t
         }
         __syncthreads();
         const tq_params_t& p = params[sh.piece.job];
-        if (table_kernel_ran) {          // rows the decision-table kernel served are done (same rule, evaluated by every thread)
+        if constexpr (BEHIND) {          // same rule, evaluated by every thread
             if (lut_serves_record(p, BITS)) continue;
         }
         load_worker<BITS, NONUNIFORM>(p, sh.q);
@@ -725,11 +731,12 @@ cudaError_t launch_compress(const CompressCall& c) {
 }
 
 template <int BITS>
-static cudaError_t dispatch_dev(const CompressCall& c, const TilePlan& plan, int table_kernel_ran) {
-    const auto kernel = c.nonuniform ? (c.bf16 ? compress_kernel_dev<BITS, true, true> : compress_kernel_dev<BITS, true, false>)
-                                     : (c.bf16 ? compress_kernel_dev<BITS, false, true> : compress_kernel_dev<BITS, false, false>);
+static cudaError_t dispatch_dev(const CompressCall& c, const TilePlan& plan, bool behind) {
+    const auto kernel = c.nonuniform ? (c.bf16 ? (behind ? compress_kernel_dev<BITS, true, true, true> : compress_kernel_dev<BITS, true, true, false>)
+                                               : compress_kernel_dev<BITS, true, false, false>)
+                                     : (c.bf16 ? compress_kernel_dev<BITS, false, true, false> : compress_kernel_dev<BITS, false, false, false>);
     return launch_kernel(kernel, dim3(plan.blocks), kThreads, 0, c.stream, c.grad, c.grad_stride, c.params_dev, round_keys(c.seed),
-                         c.first_worker, c.packed, c.words_stride, plan, table_kernel_ran);
+                         c.first_worker, c.packed, c.words_stride, plan, c.n_workers * plan.segs.n);
 }
 
 cudaError_t launch_compress_dev(const CompressCall& c) {
