@@ -16,11 +16,11 @@
 // whichever has room, where the result is provably the same:
 //   - floor / int conversion: add 2^23 rounding down, the integer appears in the mantissa;
 //   - threshold T = rint(p * 2^16): one fused multiply-add with 2^23;
-//   - the random slot r as the float 2^23 + r: one byte-permute; [r < T] = sat((2^23 + T) - (2^23 + r)),
-//     a saturating subtract of two exactly representable integers;
-//   - uniform codebook: interval and threshold together as the one integer X = rint(x * 2^16) = k * 2^16 + T,
-//     code = ceil((X - r) / 2^16), with the clamps of x done by saturating multiplies and a minimum;
-//   - codes are packed by exact multiply-adds, or by products and byte-permutes of integers;
+//   - interval and threshold together as the one integer X = k * 2^16 + T, code = floor((X + 65535 - r) / 2^16); for the uniform codebook
+//     X = rint(x * 2^16) at once, with the clamps of x done by saturating multiplies and a minimum;
+//   - codes are packed by byte-permutes and products of integers;
+//   - (binary search and the unscaled uniform form only) the random slot r as the float 2^23 + r: one byte-permute; [r < T] =
+//     sat((2^23 + T) - (2^23 + r)), a saturating subtract of two exactly representable integers;
 //   - table offsets are formed as denormal floats whose bit pattern IS the byte offset.
 #include <cmath>
 #include <cstring>
@@ -148,7 +148,7 @@ __device__ __forceinline__ void pair_plus_alpha(const Raw8<BF16>& g, int h, floa
     }
 }
 
-// General codebook through the lookup grid, two elements at a time.  s_grid[c] = (boundary, k_lo): k_lo
+// General codebook through the lookup grid, two elements at a time.  s_grid[c] = (boundary, 8 k_lo): k_lo
 // counts the interior levels in cells below c and `boundary` is the one interior level inside cell c
 // (NaN if none, so that not even +inf compares >= it), so
 // k = k_lo + [g >= boundary] = max{ j <= s-1 : l_j <= g }.  s_cell[k] = (l_k, 1/|Delta_k|).
@@ -157,15 +157,22 @@ __device__ __forceinline__ void pair_plus_alpha(const Raw8<BF16>& g, int h, floa
 // What follows an 8-byte lookup is scalar: to use the two halves of two lookups as pairs takes a move per value, which
 // costs an issue slot and often the multiplier pipe, more than pairing saves (25.6 M x 16, 16 levels: 355 -> 349 us, through
 // device parameters 394 -> 350 us; 250 M x 4, 8 levels 958 -> 861 us).
-__device__ __forceinline__ f32x2 code_cells2(float g0, float g1, float2 gc0, float2 gc1, const char* s_cell, float rf0, float rf1) {
-    const float k0 = __fadd_rn(gc0.y, set_ge(g0, gc0.x)), k1 = __fadd_rn(gc1.y, set_ge(g1, gc1.x));
-    const float2 q0 = *reinterpret_cast<const float2*>(s_cell + __float_as_uint(__fmul_rn(k0, __uint_as_float(8u))));   // bits = 8 * k
-    const float2 q1 = *reinterpret_cast<const float2*>(s_cell + __float_as_uint(__fmul_rn(k1, __uint_as_float(8u))));
-    const float p0 = __fmul_rn(__fsub_rn(g0, q0.x), q0.y), p1 = __fmul_rn(__fsub_rn(g1, q1.x), q1.y);
-    return pair(__fadd_rn(k0, rounds_up(p0, rf0)), __fadd_rn(k1, rounds_up(p1, rf1)));
+// The kernel is near HBM's rate with issue, multiplier, shared-memory and integer pipes all at 60-80 %, and at the GPU's power limit in
+// long runs, so every operation counts.  k appears only as the denormal 8k * 2^-149, whose bit pattern is the byte offset into s_cell and,
+// shifted, k * 2^16; T as the mantissa of 2^23 + T with p saturated by its product (T stays within 0 .. 2^16, 0 for a NaN); the
+// sum of the two and 65535 - r, from the complement of the random word, by a two-way dot product has the code in byte 2.  With k, [r < T] and the code as
+// floats: 25.6 M x 16, 16 levels, host / device parameters 329 / 335 us, now 310 / 325; 250 M x 4, 8 levels 796, now 779; 1 M x 8 12.0, 11.5.
+__device__ __forceinline__ void code_cells2(float g0, float g1, float2 gc0, float2 gc1, const char* s_cell, uint32_t rnd, uint32_t& v0, uint32_t& v1) {
+    const float eight = __uint_as_float(8u);
+    const uint32_t k0 = __float_as_uint(__fmaf_rn(set_ge(g0, gc0.x), eight, gc0.y)), k1 = __float_as_uint(__fmaf_rn(set_ge(g1, gc1.x), eight, gc1.y));
+    const float2 q0 = *reinterpret_cast<const float2*>(s_cell + k0);
+    const float2 q1 = *reinterpret_cast<const float2*>(s_cell + k1);
+    const float p0 = mul_sat(__fsub_rn(g0, q0.x), q0.y), p1 = mul_sat(__fsub_rn(g1, q1.x), q1.y);
+    v0 = dot_halves(~rnd, 0x0001u, __float_as_uint(__fmaf_rn(p0, 65536.0f, kMagic)) + (k0 << 13));
+    v1 = dot_halves(~rnd, 0x0100u, __float_as_uint(__fmaf_rn(p1, 65536.0f, kMagic)) + (k1 << 13));
 }
-__device__ __forceinline__ f32x2 code_grid2(float g0, float g1, f32x2 alpha2, float inv_2alpha, f32x2 cell_scale2,
-                                            const char* s_grid, const char* s_cell, float rf0, float rf1) {
+__device__ __forceinline__ void code_grid2(float g0, float g1, f32x2 alpha2, float inv_2alpha, f32x2 cell_scale2, const char* s_grid,
+                                           const char* s_cell, uint32_t rnd, uint32_t& v0, uint32_t& v1) {
     const f32x2 g = pair(g0, g1);
     float s0, s1;
     unpair(add2(g, alpha2), s0, s1);
@@ -175,7 +182,7 @@ __device__ __forceinline__ f32x2 code_grid2(float g0, float g1, f32x2 alpha2, fl
     unpair(cell8, c0, c1);
     const float2 gc0 = *reinterpret_cast<const float2*>(s_grid + __float_as_uint(c0));
     const float2 gc1 = *reinterpret_cast<const float2*>(s_grid + __float_as_uint(c1));
-    return code_cells2(g0, g1, gc0, gc1, s_cell, rf0, rf1);
+    code_cells2(g0, g1, gc0, gc1, s_cell, rnd, v0, v1);
 }
 
 // The same through a logarithmic grid, whose cells are the exponent and the four highest mantissa bits of |g|, 16 per binade,
@@ -191,14 +198,14 @@ __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
     uint32_t r; asm("prmt.b32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(sel)); return r;
 }
 __host__ __device__ inline uint32_t log_cell8(uint32_t bits) { return (bits >> 16) & 0x7FF8u; }
-__device__ __forceinline__ f32x2 code_log2(float g0, float g1, float alpha, uint32_t nbase2, uint32_t top2, const char* s_middle,
-                                           const char* s_cell, float rf0, float rf1) {
+__device__ __forceinline__ void code_log2(float g0, float g1, float alpha, uint32_t nbase2, uint32_t top2, const char* s_middle,
+                                          const char* s_cell, uint32_t rnd, uint32_t& v0, uint32_t& v1) {
     const float t0 = fmaxf(g0, -alpha), t1 = fmaxf(g1, -alpha);
     const uint32_t y = __byte_perm(__float_as_uint(t0), __float_as_uint(t1), 0x7632u);
     const uint32_t z = __viaddmin_s16x2_relu(y & 0x7FF87FF8u, nbase2, top2) ^ (prmt(y, y, 0xBB99u) & 0xFFF8FFF8u);
     const float2 gc0 = *reinterpret_cast<const float2*>(s_middle + static_cast<int>(prmt(z, z, 0x9910u)));
     const float2 gc1 = *reinterpret_cast<const float2*>(s_middle + static_cast<int>(prmt(z, z, 0xBB32u)));
-    return code_cells2(t0, t1, gc0, gc1, s_cell, rf0, rf1);
+    code_cells2(t0, t1, gc0, gc1, s_cell, rnd, v0, v1);
 }
 
 // General codebook by branch-free binary search (used when no grid of at most kMaxGridCells cells
@@ -297,13 +304,20 @@ __device__ __forceinline__ void quantize_run(const Raw8<BF16> (&g)[4], uint32_t*
     for (int grp = 0; grp < 4; ++grp) {
         uint32_t rnd[4];
         philox_block(blk_lo + grp, pr, rk, rnd);                      // j0 >> 3 is a multiple of 4: no carry
-        if constexpr (SEARCH == kUniform) {
-            uint32_t v[8];
+        if constexpr (SEARCH == kUniform || SEARCH == kGrid || SEARCH == kLogGrid) {
+            uint32_t v[8];                       // the codes in byte 2
 #pragma unroll
             for (int h = 0; h < 4; ++h) {        // elements 2h, 2h+1 of the group
-                float sum0, sum1;
-                pair_plus_alpha<BF16>(g[grp], h, cx.alpha, sum0, sum1);
-                code_uniform2<BF16>(sum0, sum1, cx.u, rnd[h], v[2 * h], v[2 * h + 1]);
+                if constexpr (SEARCH == kUniform) {
+                    float sum0, sum1;
+                    pair_plus_alpha<BF16>(g[grp], h, cx.alpha, sum0, sum1);
+                    code_uniform2<BF16>(sum0, sum1, cx.u, rnd[h], v[2 * h], v[2 * h + 1]);
+                } else {
+                    const float g0 = elem<BF16>(g[grp], 2 * h), g1 = elem<BF16>(g[grp], 2 * h + 1);
+                    if constexpr (SEARCH == kGrid)
+                        code_grid2(g0, g1, alpha2, cx.inv_2alpha, cell_scale2, cx.s_grid, cx.s_cell, rnd[h], v[2 * h], v[2 * h + 1]);
+                    else code_log2(g0, g1, cx.alpha, cx.log_nbase2, cx.log_top2, cx.s_grid, cx.s_cell, rnd[h], v[2 * h], v[2 * h + 1]);
+                }
             }
             chunk[grp] = pack_byte2<BITS>(v);
         } else {
@@ -318,12 +332,8 @@ __device__ __forceinline__ void quantize_run(const Raw8<BF16> (&g)[4], uint32_t*
                     code[h] = code_uniform2_wide(sum0, sum1, inv_step2, cx.top, rf0, rf1);
                 } else {
                     const float g0 = elem<BF16>(g[grp], e), g1 = elem<BF16>(g[grp], e + 1);
-                    if constexpr (SEARCH == kGrid)
-                        code[h] = code_grid2(g0, g1, alpha2, cx.inv_2alpha, cell_scale2, cx.s_grid, cx.s_cell, rf0, rf1);
-                    else if constexpr (SEARCH == kLogGrid)
-                        code[h] = code_log2(g0, g1, cx.alpha, cx.log_nbase2, cx.log_top2, cx.s_grid, cx.s_cell, rf0, rf1);
-                    else code[h] = pair(code_binary<BITS>(g0, cx.alpha, cx.s_search, reinterpret_cast<const float2*>(cx.s_cell), rf0),
-                                        code_binary<BITS>(g1, cx.alpha, cx.s_search, reinterpret_cast<const float2*>(cx.s_cell), rf1));
+                    code[h] = pair(code_binary<BITS>(g0, cx.alpha, cx.s_search, reinterpret_cast<const float2*>(cx.s_cell), rf0),
+                                   code_binary<BITS>(g1, cx.alpha, cx.s_search, reinterpret_cast<const float2*>(cx.s_cell), rf1));
                 }
             }
             chunk[grp] = pack8<BITS>(code);
@@ -424,13 +434,14 @@ __device__ __forceinline__ void build_tables(const WorkerQ& q, float2* s_grid, f
                                     : log_cell(q.levels[j], q.log_base) + q.log_cells;
         const uint32_t last = SEARCH == kGrid ? q.cells : 2 * q.log_cells - 1;
         for (uint32_t c = threadIdx.x; c <= last; c += kThreads) {
-            float below = 0.0f, boundary = __int_as_float(0x7FC00000);   // NaN: no value compares >= it
+            uint32_t below = 0;                                        // 8 times their number
+            float boundary = __int_as_float(0x7FC00000);               // NaN: no value compares >= it
 #pragma unroll
             for (int j = 1; j <= L - 2; ++j) {
-                if (lc[j] < c) below += 1.0f;
+                if (lc[j] < c) below += 8u;
                 if (lc[j] == c) boundary = q.levels[j];
             }
-            s_grid[c] = make_float2(boundary, below);
+            s_grid[c] = make_float2(boundary, __uint_as_float(below));
         }
     }
     if constexpr (!is_uniform(SEARCH)) __syncthreads();
