@@ -228,6 +228,21 @@ struct Split {
             const double k = lo + step * (lanes.lane() + 1), s = slope_at(k, log(k));
             const uint32_t rises = lanes.ballot(!(s < 0.0));
             const int c = rises ? first_bit(rises) : n;            // trial points before the first one where Q_B rises
+            if constexpr (n >= 8) {
+                // Two trial points on either side of the turn, close enough for the zero of the cubic k(slope) through the four: its error is of the
+                // order of (step / k)^4, here below 2^-40, or 2^-32.
+                if (c >= 2 && c <= n - 2 && step <= (fine ? 9.765625e-4 : 3.90625e-3) * lo) {
+                    const double sa = lanes.of(s, c - 2), sb = lanes.of(s, c - 1), sc = lanes.of(s, c), sd = lanes.of(s, c + 1);
+                    if (sa < sb && sb < sc && sc < sd) {
+                        // Neville's scheme at slope 0, places counted from the first point in steps
+                        const double ra = 1.0 / (sb - sa), rb = 1.0 / (sc - sb), rc = 1.0 / (sd - sc), rd = 1.0 / (sc - sa), re = 1.0 / (sd - sb), rf = 1.0 / (sd - sa);
+                        const double ab = -sa * ra, bc = 1.0 - sb * rb, cd = 2.0 - sc * rc;
+                        const double abc = (ab * sc - bc * sa) * rd, bcd = (bc * sd - cd * sb) * re;
+                        const double at = (abc * sd - bcd * sa) * rf;
+                        if (at >= 1.0 && at <= 2.0) return lo + step * (static_cast<double>(c - 1) + at);
+                    }
+                }
+            }
             const double new_lo = c > 0 ? lo + step * c : lo, new_hi = c < n ? lo + step * (c + 1) : hi;
             if (c > 0) s_lo = lanes.of(s, c - 1);
             if (c < n) s_hi = lanes.of(s, c);
@@ -296,6 +311,7 @@ TQ_HD inline double solve_alpha(const Lanes& lanes, const SplitGrid<Lanes>& grid
                                 int* iterations) {
     double x = m.c1 * m.ln_k;
     double least = mode == TQ_BISCALED || !(x > 0.0) ? 0.0 : -0.9;      // smallest F' that a tangent step is taken at
+    double x_before = 0.0, d_before = 0.0, inv_before = NAN;            // the iterate before, if a tangent step was taken there
     int it = 0;
     while (it < 10000 && !(x > x_cap)) {
         double slope, f;
@@ -309,9 +325,19 @@ TQ_HD inline double solve_alpha(const Lanes& lanes, const SplitGrid<Lanes>& grid
         }
         if (it == 0 && !(slope >= least)) least = 0.0;
         ++it;
-        const double d = f - x, root = f + d * slope / (1.0 - slope);      // = x + d / (1 - slope)
+        const double d = f - x, inv = 1.0 / (1.0 - slope);
+        double root = f + d * slope * inv;                               // = x + d / (1 - slope)
+        if (mode == TQ_BISCALED) {
+            // the cubic x(F - x) through this iterate and the one before, with both tangents, once it lies well inside the last step
+            const double width = d_before - d, t = -d / width;
+            if (inv_before == inv_before && fabs(t) < 0.25) {
+                const double u = 1.0 - t;
+                root = x + t * (t * (3.0 - 2.0 * t) * (x_before - x) - width * u * (inv * u - inv_before * t));
+            }
+        }
         const bool same = mode == TQ_BISCALED || least < 0.0 || d >= 0.0;
         const bool take = same && slope >= least && slope < 0.999 && x > 0.0 && root > 0.0 && finite_d(root) && !(f > x_cap) && !(root > x_cap);
+        x_before = x; d_before = d; inv_before = take ? inv : NAN;
         x = f;
         if (fabs(d) <= 1e-12) break;
         if (take) x = root;
