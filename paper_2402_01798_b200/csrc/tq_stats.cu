@@ -32,7 +32,7 @@ constexpr int kChunkBytes = 64;
 template <bool BF16> constexpr int kChunk = kChunkBytes / (BF16 ? 2 : 4);      // elements
 constexpr float kMaxFinite = 3.402823466e38f;
 
-struct alignas(64) Partial {
+struct alignas(64) Partial {                  // warp_fold reads it as eight doubles
     double sum_abs, sum_sq, sum_log2[2];
     unsigned long long n_tail[2], n_bad;
     float max_abs, pad;
@@ -594,17 +594,38 @@ __device__ __forceinline__ void hinted_piece(const JobPiece& piece, const void* 
     }
 }
 
-// What one warp makes of a job's records: the sum of |g|, and with ALL every other field too.  Same order in every warp.
+// What one warp makes of a job's records: the sum of |g|, and with ALL every other field too.  Same order in every warp.  Several records per lane
+// are asked for before the first is added: one after the other, each a trip to the L2, the 428 records of one row of 3.5 M bf16 values took
+// 4 us.
+__device__ __forceinline__ void load_pair(const void* p, double& a, double& b) {      // past the L1: other blocks may have written since
+    asm volatile("ld.volatile.global.v2.f64 {%0,%1}, [%2];" : "=d"(a), "=d"(b) : "l"(p));
+}
 template <bool ALL>
 __device__ __forceinline__ Partial warp_fold(const Partial* records, uint32_t count) {
     const uint32_t lane = threadIdx.x & 31u;
+    constexpr uint32_t kAhead = ALL ? 3 : 16;
     Partial p{};
-    for (uint32_t b = lane; b < count; b += 32) {
-        const volatile Partial* q = records + b;
-        p.sum_abs += q->sum_abs;
-        if constexpr (ALL) {
-            p.sum_sq += q->sum_sq; p.n_bad += q->n_bad; p.max_abs = fmaxf(p.max_abs, q->max_abs);
-            p.sum_log2[0] += q->sum_log2[0]; p.sum_log2[1] += q->sum_log2[1]; p.n_tail[0] += q->n_tail[0]; p.n_tail[1] += q->n_tail[1];
+    for (uint32_t first = lane; first < count; first += 32 * kAhead) {
+        double v[kAhead][ALL ? 8 : 2];
+#pragma unroll
+        for (uint32_t i = 0; i < kAhead; ++i) {
+            const uint32_t b = first + 32 * i;
+#pragma unroll
+            for (int f = 0; f < (ALL ? 8 : 2); f += 2) {
+                v[i][f] = v[i][f + 1] = 0.0;
+                if (b < count) load_pair(reinterpret_cast<const double*>(records + b) + f, v[i][f], v[i][f + 1]);
+            }
+        }
+#pragma unroll
+        for (uint32_t i = 0; i < kAhead; ++i) {
+            p.sum_abs += v[i][0];
+            if constexpr (ALL) {
+                p.sum_sq += v[i][1]; p.sum_log2[0] += v[i][2]; p.sum_log2[1] += v[i][3];
+                p.n_tail[0] += static_cast<unsigned long long>(__double_as_longlong(v[i][4]));
+                p.n_tail[1] += static_cast<unsigned long long>(__double_as_longlong(v[i][5]));
+                p.n_bad += static_cast<unsigned long long>(__double_as_longlong(v[i][6]));
+                p.max_abs = fmaxf(p.max_abs, __int_as_float(__double2loint(v[i][7])));
+            }
         }
     }
     p.sum_abs = __shfl_sync(0xFFFFFFFFu, warp_sum(p.sum_abs), 0);
