@@ -126,6 +126,21 @@ def test_aggregation_forms(tq, orc, bits, n, d):
     assert tq.tq_wait_expired_count() == 0
 
 
+@pytest.mark.parametrize("n", [1, 2, 3, 4, 5])
+@pytest.mark.parametrize("weighted", [False, True])
+def test_first_two_workers_of_two_bit_rows(tq, orc, n, weighted):
+    """The bulk kernel looks up the sum of the first two workers' values at once: one worker, exactly two, short and full steps of four.  The
+    additions are those of the oracle, so the results are equal; host and device parameters."""
+    d, r = 300 * 4096 + 21, random.Random(n)
+    ps = [tq.tq_params_from_levels(sorted([-1.0 - i, r.uniform(-0.9, -0.1), r.uniform(0.0, 0.9), 1.0 + i])) for i in range(n)]
+    w = [r.uniform(0.1, 0.9) for _ in range(n)] if weighted else None
+    packed = torch.randint(-2 ** 31, 2 ** 31, (n, tq.tq_packed_words(d, 2)), dtype=torch.int64, generator=torch.Generator().manual_seed(n)).to(torch.int32).cuda()
+    want = orc.decompress_aggregate(packed.cpu().numpy().view(np.uint32), d, [_oracle_params(orc, p) for p in ps], w)
+    assert np.array_equal(tq.tq_decompress_aggregate(packed, d, ps, weights=w).cpu().numpy(), want)
+    raw = torch.frombuffer(bytearray(b"".join(bytes(p) for p in ps)), dtype=torch.uint8).cuda()
+    assert np.array_equal(tq.tq_decompress_aggregate_device_params(packed, d, raw, 4, weights=w).cpu().numpy(), want)
+
+
 @pytest.mark.parametrize("bits,n,momentum", [(3, 2, 0.9), (4, 1, 0.0), (4, 33, 0.9)])
 @pytest.mark.parametrize("d", [4095 * 4096, 4096 * 4096 - 2047, 4096 * 4096 + 2049])
 def test_fused_update_of_long_rows(tq, bits, n, momentum, d):
