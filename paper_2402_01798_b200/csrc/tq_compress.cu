@@ -414,8 +414,10 @@ __device__ __forceinline__ void compress_last_run(const char* row, uint32_t* pro
 #endif
 
 // Per-block set-up of the shared tables for quantizer q (ends with a block barrier unless the codebook is uniform).
-// s_grid must hold kMaxGridCells + 1 entries when SEARCH is a grid.
-template <int BITS, int SEARCH>
+// s_grid must hold kMaxGridCells + 1 entries when SEARCH is a grid.  LANES: the form for quantizers in device memory, whose tables
+// nothing hides; host parameters' are built while the kernel before still runs, and with that form their main loop gets other registers
+// (25.6 M x 16, 16 levels: 310 -> 322 us).
+template <int BITS, int SEARCH, bool LANES>
 __device__ __forceinline__ void build_tables(const WorkerQ& q, float2* s_grid, float2* s_cell, float* s_search) {
     constexpr int L = 1 << BITS;
     if constexpr (!is_uniform(SEARCH)) {
@@ -425,7 +427,30 @@ __device__ __forceinline__ void build_tables(const WorkerQ& q, float2* s_grid, f
         if (threadIdx.x < 2 * TQ_MAX_LEVELS)
             s_search[threadIdx.x] = (threadIdx.x >= 1 && threadIdx.x <= L - 2) ? q.levels[threadIdx.x] : __int_as_float(0x7F800000);
     }
-    if constexpr (SEARCH == kGrid || SEARCH == kLogGrid) {
+    constexpr bool kCells = SEARCH == kGrid || SEARCH == kLogGrid;
+    if constexpr (kCells && LANES) {
+        // A lane for each interior level l_1 .. l_{s-1} (their cells are distinct and in order, or the grid would not have been chosen); a warp fills
+        // in 32 cells at a time, most of which hold none (each thread comparing its cells with all levels took 1 us of a call of 1 M x 8, 16
+        // levels).
+        const uint32_t lane = threadIdx.x & 31u;
+        const bool interior = lane >= 1 && lane <= L - 2;
+        const float level = lane < L ? q.levels[lane] : 0.0f;
+        const uint32_t cell = SEARCH == kGrid ? __float_as_uint(grid_cell(level, q.alpha, q.inv_2alpha, q.cell_scale)) : log_cell(level, q.log_base) + q.log_cells;
+        const uint32_t last = SEARCH == kGrid ? q.cells : 2 * q.log_cells - 1;
+        for (uint32_t c0 = threadIdx.x - lane; c0 <= last; c0 += kThreads) {
+            const uint32_t c = c0 + lane;
+            uint32_t below = __popc(__ballot_sync(0xFFFFFFFFu, interior && cell < c0));
+            float boundary = __int_as_float(0x7FC00000);               // NaN: no value compares >= it
+            for (uint32_t here = __ballot_sync(0xFFFFFFFFu, interior && cell - c0 < 32u); here != 0; here &= here - 1) {
+                const int j = __ffs(static_cast<int>(here)) - 1;
+                const uint32_t at = __shfl_sync(0xFFFFFFFFu, cell, j);
+                const float l = __shfl_sync(0xFFFFFFFFu, level, j);
+                if (at < c) ++below;
+                if (at == c) boundary = l;
+            }
+            if (c <= last) s_grid[c] = make_float2(boundary, __uint_as_float(8 * below));
+        }
+    } else if constexpr (kCells) {
         // cells of the interior levels l_1 .. l_{s-1} (distinct, or the grid would not have been chosen)
         uint32_t lc[L];
 #pragma unroll
@@ -461,7 +486,7 @@ compress_kernel(const void* __restrict__ grad, uint64_t d, uint64_t grad_stride,
     const uint32_t worker = first_worker + blockIdx.y;
     const char* row = static_cast<const char*>(grad) + static_cast<uint64_t>(blockIdx.y) * grad_stride * esz;
     uint32_t* prow = packed + static_cast<uint64_t>(blockIdx.y) * words_stride;
-    build_tables<BITS, SEARCH>(q, s_grid, s_cell, s_search);          // from kernel parameters: before the wait
+    build_tables<BITS, SEARCH, false>(q, s_grid, s_cell, s_search);          // from kernel parameters: before the wait
     pdl_wait();
     const RunCtx cx = run_ctx<BITS, SEARCH>(q, s_grid, s_cell, s_search);
     const uint64_t whole = (d - 1) >> 5, stride = static_cast<uint64_t>(gridDim.x) * kThreads;     // runs before the row's last one are whole
@@ -533,7 +558,7 @@ struct BlockState {
     float search[2 * TQ_MAX_LEVELS];
     WorkerQ q;
     JobPiece piece;
-    uint64_t cur;
+    uint64_t cur, end;
 };
 
 // The piece in sh.piece.
@@ -542,7 +567,7 @@ __device__ __forceinline__ void compress_piece(State& sh, const void* __restrict
                                                uint32_t first_worker, uint32_t* __restrict__ packed, uint64_t words_stride,
                                                const TilePlan& plan) {
     constexpr size_t esz = BF16 ? 2 : 4;
-    build_tables<BITS, SEARCH>(sh.q, sh.grid, sh.cell, sh.search);
+    build_tables<BITS, SEARCH, true>(sh.q, sh.grid, sh.cell, sh.search);
     const RunCtx cx = run_ctx<BITS, SEARCH>(sh.q, sh.grid, sh.cell, sh.search);
     const char* row = static_cast<const char*>(grad) + (static_cast<uint64_t>(sh.piece.worker) * grad_stride + sh.piece.off) * esz;
     uint32_t* prow = packed + static_cast<uint64_t>(sh.piece.worker) * words_stride + plan.segs.woff[sh.piece.seg];
@@ -577,42 +602,44 @@ compress_kernel_dev(const void* __restrict__ grad, uint64_t grad_stride, const t
                     const __grid_constant__ RoundKeys rk, uint32_t first_worker, uint32_t* __restrict__ packed, uint64_t words_stride,
                     const __grid_constant__ TilePlan plan, uint32_t n_jobs) {
     __shared__ __align__(16) BlockState<NONUNIFORM> sh;
+    if (threadIdx.x == 0) {                                    // the first piece, before the wait; no block is empty
+        uint64_t cur = first_tile_of_block(plan, blockIdx.x);
+        sh.end = first_tile_of_block(plan, blockIdx.x + 1);
+        sh.piece = next_piece(plan, cur, sh.end);
+        sh.cur = cur;
+    }
     pdl_wait();
     if constexpr (BEHIND) {              // nearly always nothing is left, which one look over all records shows
         bool left = false;
         for (uint32_t j = threadIdx.x; j < n_jobs; j += kThreads) left = left || !lut_serves_record(params[j], BITS);
         if (!__syncthreads_or(left)) return;
     }
-    if (threadIdx.x == 0) sh.cur = first_tile_of_block(plan, blockIdx.x);
     while (true) {
-        __syncthreads();                 // the previous piece has been served
-        const uint64_t range_end = first_tile_of_block(plan, blockIdx.x + 1);
-        if (sh.cur >= range_end) return;
-        __syncthreads();
+        __syncthreads();                 // the piece is known
+        const tq_params_t& p = params[sh.piece.job];
+        if (!BEHIND || !lut_serves_record(p, BITS)) {        // same rule, evaluated by every thread
+            load_worker<BITS, NONUNIFORM>(p, sh.q);
+            if (!(sh.q.alpha > 0.0f)) {
+                uint32_t* prow = packed + static_cast<uint64_t>(sh.piece.worker) * words_stride + plan.segs.woff[sh.piece.seg];
+                const uint64_t words_out = (((sh.piece.d * BITS + 31) >> 5) + 3) & ~static_cast<uint64_t>(3);
+                const uint64_t w1 = sh.piece.last ? words_out : sh.piece.tile1 * kThreads * BITS;
+                for (uint64_t w = sh.piece.tile0 * kThreads * BITS + threadIdx.x; w < w1; w += kThreads) prow[w] = 0u;
+            } else if (NONUNIFORM && sh.q.cells == 0 && sh.q.log_cells != 0) {
+                compress_piece_rare<BITS, kLogGrid, BF16>(sh, grad, grad_stride, rk, first_worker, packed, words_stride, plan);
+            } else if (NONUNIFORM && sh.q.cells == 0) {
+                compress_piece_rare<BITS, kBinary, BF16>(sh, grad, grad_stride, rk, first_worker, packed, words_stride, plan);
+            } else if (!NONUNIFORM && sh.q.inv_step_l == 0.0f) {
+                compress_piece_rare<BITS, kUniformWide, BF16>(sh, grad, grad_stride, rk, first_worker, packed, words_stride, plan);
+            } else {
+                compress_piece<BITS, NONUNIFORM ? kGrid : kUniform, BF16>(sh, grad, grad_stride, rk, first_worker, packed, words_stride, plan);
+            }
+        }
+        if (sh.cur >= sh.end) return;
+        __syncthreads();                 // the piece has been served
         if (threadIdx.x == 0) {
             uint64_t cur = sh.cur;
-            sh.piece = next_piece(plan, cur, range_end);
+            sh.piece = next_piece(plan, cur, sh.end);
             sh.cur = cur;
-        }
-        __syncthreads();
-        const tq_params_t& p = params[sh.piece.job];
-        if constexpr (BEHIND) {          // same rule, evaluated by every thread
-            if (lut_serves_record(p, BITS)) continue;
-        }
-        load_worker<BITS, NONUNIFORM>(p, sh.q);
-        if (!(sh.q.alpha > 0.0f)) {
-            uint32_t* prow = packed + static_cast<uint64_t>(sh.piece.worker) * words_stride + plan.segs.woff[sh.piece.seg];
-            const uint64_t words_out = (((sh.piece.d * BITS + 31) >> 5) + 3) & ~static_cast<uint64_t>(3);
-            const uint64_t w1 = sh.piece.last ? words_out : sh.piece.tile1 * kThreads * BITS;
-            for (uint64_t w = sh.piece.tile0 * kThreads * BITS + threadIdx.x; w < w1; w += kThreads) prow[w] = 0u;
-        } else if (NONUNIFORM && sh.q.cells == 0 && sh.q.log_cells != 0) {
-            compress_piece_rare<BITS, kLogGrid, BF16>(sh, grad, grad_stride, rk, first_worker, packed, words_stride, plan);
-        } else if (NONUNIFORM && sh.q.cells == 0) {
-            compress_piece_rare<BITS, kBinary, BF16>(sh, grad, grad_stride, rk, first_worker, packed, words_stride, plan);
-        } else if (!NONUNIFORM && sh.q.inv_step_l == 0.0f) {
-            compress_piece_rare<BITS, kUniformWide, BF16>(sh, grad, grad_stride, rk, first_worker, packed, words_stride, plan);
-        } else {
-            compress_piece<BITS, NONUNIFORM ? kGrid : kUniform, BF16>(sh, grad, grad_stride, rk, first_worker, packed, words_stride, plan);
         }
     }
 }
