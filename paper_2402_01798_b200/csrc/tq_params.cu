@@ -16,8 +16,9 @@
 // x = ln(a / g_min), in which a boxed alpha equation costs one exp and one log; it is solved by Newton
 // steps (4 to 8 evaluations); and everything that exists once per level or per trial point (levels, inverse
 // widths, the split of the two-step quantizer) is spread over the lanes of the warp.  Measured on B200 for
-// one worker, uniform, 4 levels / 8 workers, 16-level two-step quantizer: 5.3 us / 24.5 us, against
-// 21.1 us / 3590 us with one thread per worker, two pow per evaluation and Aitken steps.  The two-step quantizer's
+// one worker, uniform, 4 levels / 8 workers, 16-level two-step quantizer: 4.5 us / 19.1 us (18.3 with the split as the first cubic
+// through four trial points gives it, which is up to 2^-24 off), against 21.1 us / 3590 us with one thread per worker, two pow per evaluation
+// and Aitken steps.  The two-step quantizer's
 // trial points are the same for every alpha, so their powers k^-gamma are taken once (29.1 us with an exp
 // and a division per point and alpha; on the host, where one thread does all of them, 22 -> 6.6 us per record).
 #include <cmath>
@@ -105,6 +106,7 @@ struct TailModel {
 };
 
 constexpr int kSplitGrid = 128;
+constexpr double kSplitClose = 1.4901161193847656e-08;      // 2^-26: see close_in
 constexpr double kSplitFirst = 9.094947017729282e-13, kSplitLnFirst = -27.72588722239781;   // 2^-40: the grid's first point, in place of 0
 // k^-gamma at the grid points of one lane, k = j / 128 with j = t * kLanes + lane + 1: the same for every alpha, and for every
 // record of one gamma.
@@ -170,8 +172,8 @@ struct Split {
     // Q_B(a, 0) = Q_B(a, 1) = Q_U(a), so the minimum is a point where Q_B turns from falling to rising.  Every
     // such turn between neighbours of a 128-point grid is closed in on; the turn with the smallest Q_B wins.  No turn:
     // the minimum is an end.  Where the density jumps (k a = g_min) the turn may be a kink, which is tested for by itself.
-    // Q_B is flat at a smooth turn, so an error of 2^-34 there does not show in its last bit: the alpha iteration asks
-    // for no more.
+    // Q_B is flat at a smooth turn: an error of 2^-26 there enters Q_B by its square, and the alpha iteration asks for no more (alpha, exponents 2.2 to 4.5,
+    // against 64-bit significands: off by 2^-52 in the middle of 3000 cases and by up to the 2^-40 at which it stops).
     template <class Lanes>
     TQ_HD double best(const Lanes& lanes, const SplitGrid<Lanes>& grid, bool fine, double* q_best, double* ln_slope) const {
         constexpr int n = Lanes::kLanes;
@@ -208,9 +210,11 @@ struct Split {
         *q_best = best_q;
         return best_k;
     }
-    // Q_B falls at lo and does not at hi: the lanes' trial points cut the bracket into kLanes + 1 parts each time until it is
-    // 2^-17 wide (relative).  The slope is then a straight line in it, and its zero is off by the square of that width, 2^-34;
-    // `fine` adds a Newton step with the slope of that line, which multiplies the error by 2^-17 once more.
+    // Q_B falls at lo and does not at hi: the lanes' trial points cut the bracket into kLanes + 1 parts each time.  A warp's cubic through four of
+    // them ends that; otherwise it goes on until the bracket is 2^-17 wide (relative), where the slope is close to a straight line whose zero
+    // is off by the square of that width times a factor that grows where the slope bends; `fine` adds a Newton step with the slope of that line.
+    // Against 64-bit significands, 18000 cases of exponents 2.05 to 10, alpha given or solved for, levels are off by 2^-48 to 2^-53 in the
+    // middle of the cases and by up to 2^-33 (the rounding of the slope) either way to the end, the coarse split by up to 2^-28.
     template <class Lanes>
     TQ_HD double close_in(const Lanes& lanes, double lo, double hi, bool fine, bool* at_kink) const {
         constexpr int n = Lanes::kLanes;
@@ -229,9 +233,11 @@ struct Split {
             const uint32_t rises = lanes.ballot(!(s < 0.0));
             const int c = rises ? first_bit(rises) : n;            // trial points before the first one where Q_B rises
             if constexpr (n >= 8) {
-                // Two trial points on either side of the turn, close enough for the zero of the cubic k(slope) through the four: its error is of the
-                // order of (step / k)^4, here below 2^-40, or 2^-32.
-                if (c >= 2 && c <= n - 2 && step <= (fine ? 9.765625e-4 : 3.90625e-3) * lo) {
+                // Two trial points on either side of the turn: the zero of the cubic k(slope) through the four, if they are close enough for it.  How
+                // close that is depends on where the slope bends (k near 0 or 1, large exponents): with r2 and r3 the second and third
+                // differences over the first, the cubic is off by about the 3/2 power of max(r2^2, r3), in steps.  `fine` goes on from there by the slope
+                // at that point, with its first and second derivative from the differences.
+                if (c >= 2 && c <= n - 2) {
                     const double sa = lanes.of(s, c - 2), sb = lanes.of(s, c - 1), sc = lanes.of(s, c), sd = lanes.of(s, c + 1);
                     if (sa < sb && sb < sc && sc < sd) {
                         // Neville's scheme at slope 0, places counted from the first point in steps
@@ -239,7 +245,19 @@ struct Split {
                         const double ab = -sa * ra, bc = 1.0 - sb * rb, cd = 2.0 - sc * rc;
                         const double abc = (ab * sc - bc * sa) * rd, bcd = (bc * sd - cd * sb) * re;
                         const double at = (abc * sd - bcd * sa) * rf;
-                        if (at >= 1.0 && at <= 2.0) return lo + step * (static_cast<double>(c - 1) + at);
+                        const double before = (sc - sb - (sb - sa)) * rb, after = (sd - sc - (sc - sb)) * rb;
+                        const double bend = fmax(fmax(before * before, after * after), fabs(after - before)), most = kSplitClose * lo;
+                        if (at >= 1.0 && at <= 2.0 && bend * bend * bend * (step * step) <= most * most) {
+                            double k = lo + step * (static_cast<double>(c - 1) + at);
+                            if (fine) {
+                                const double off = at - 1.5, mean = 0.5 * (before + after), third = after - before;
+                                const double per_slope = rb / (1.0 + off * mean + (0.5 * off * off - 1.0 / 24.0) * third);
+                                const double by = slope_at(k, log(k)) * per_slope;                  // steps
+                                const double better = k - step * (by + 0.5 * by * by * (mean + off * third));
+                                if (better > lo && better < hi) k = better;
+                            }
+                            return k;
+                        }
                     }
                 }
             }

@@ -45,6 +45,71 @@ def test_params_device_record_counts(tq, mode, n):
         assert np.allclose(list(got[i].levels), list(want.levels), rtol=5e-7, atol=0)
 
 
+def _two_step_levels(g_min, rho, gamma, alpha, L):
+    """The two-step quantizer's upper levels below alpha, one row per record, with 64-bit significands: k* is where Q_B turns on either side of
+    the best of 2048 grid points, closed in on by halving.  Second result: records whose k* is beyond doubt (one best turn,
+    not beside the jump of the density)."""
+    def masses(k, a, rho, gamma):
+        inside = lambda t: np.where(t <= 1, (1 - 2 * rho) * t, 1 - 2 * rho * np.maximum(t, 1) ** (1 - gamma))
+        u = inside(k * a)
+        return u, np.maximum(inside(a) - u, 0)
+
+    a, rho, gamma = (alpha / g_min)[:, None], rho[:, None], gamma[:, None]
+    k = np.arange(1, 2048)[None, :] / 2048
+    u, w = masses(k, a, rho, gamma)
+    q = np.cbrt(w * (1 - k) ** 2) + np.cbrt(u * k * k)
+    best = q.argmin(1)
+    low = np.zeros(q.shape, bool)
+    low[:, 1:-1] = (q[:, 1:-1] <= q[:, :-2]) & (q[:, 1:-1] <= q[:, 2:])
+    other = np.where(low & (np.abs(np.arange(2047)[None, :] - best[:, None]) > 2), q, np.inf).min(1)
+    sure = (a[:, 0] > 1.1) & (best > 1) & (best < 2045) & (other > q.min(1) * (1 + 1e-9))
+
+    a, rho, gamma, g_min = (v.astype(np.longdouble) for v in (a, rho, gamma, g_min[:, None]))
+
+    def rises(k):
+        u, w = masses(k, a, rho, gamma)
+        du = np.where(k * a <= 1, (1 - 2 * rho) * a, 2 * rho * (gamma - 1) * a ** (1 - gamma) * k ** -gamma)
+        return w * w * (1 - k) * (du * k + 2 * u) ** 3 >= u * u * k * (du * (1 - k) + 2 * w) ** 3
+
+    lo, hi = np.maximum(best, 1)[:, None].astype(np.longdouble) / 2048, (best[:, None] + 2).astype(np.longdouble) / 2048
+    sure &= (~rises(lo) & rises(hi))[:, 0]
+    for _ in range(64):
+        mid = (lo + hi) / 2
+        up = rises(mid)
+        lo, hi = np.where(up, lo, mid), np.where(up, mid, hi)
+    k, s = (lo + hi) / 2, L - 1
+    u, w = masses(k, a, rho, gamma)
+    beta = k * a
+    c_in, c_out = np.cbrt(u / beta), np.cbrt(w / (a - beta))
+    denom = 2 * a * (c_out * (1 - k) + c_in * k)
+    c, lam_in, lam_out = np.arange(L // 2, s)[None, :] - np.longdouble(s) / 2, s * c_in / denom, s * c_out / denom
+    return g_min * np.where(c <= lam_in * beta, c / lam_in, beta + (c - lam_in * beta) / lam_out), sure
+
+
+@pytest.mark.parametrize("alpha", [None, 2.5e-3, 2e-2])
+@pytest.mark.parametrize("L", [4, 8, 16])
+def test_two_step_levels_are_rounded_once(tq, alpha, L):
+    """Only the warp's form cuts the split's bracket 33-fold at a time.  Its levels are those of the exact split, rounded once to fp32, for
+    exponents up to 10 and splits close to either end, alpha solved for or given.  In double precision the slope's own rounding moves a level by
+    up to 2^-33 of itself, so those that stand closer than 2^-32 to the middle between two fp32 numbers may go either way."""
+    n, d, r = 4096, 1_000_003, np.random.default_rng(L)
+    tail, g_min, gamma = (d * 2 * r.uniform(0.005, 0.24, n)).astype(np.int64), np.exp(r.uniform(-9, -6.5, n)).astype(np.float32), r.uniform(2.05, 10, n)
+    stats = [tq.Stats(d=d, n_tail=int(t), g_min=float(m), sum_log_tail=float(t / (g - 1)), max_abs=float(m) * 1e4) for t, m, g in zip(tail, g_min, gamma)]
+    gamma = 1 + tail / np.array([s.sum_log_tail for s in stats])          # as the library reads it back from the record
+    raw = torch.from_numpy(np.frombuffer(b"".join(bytes(s) for s in stats), dtype=np.uint8).copy()).cuda()
+    rule = {} if alpha is None else dict(alpha_rule=tq.ALPHA_USER, alpha_user=alpha)
+    got = tq.params_to_host(tq.tq_params_device(raw, n, L, tq.BISCALED, **rule))
+    ok = np.array([p.flags & tq.FLAG_INVALID == 0 and p.alpha > 0 for p in got])
+    top = np.array([p.alpha if v else 1.0 for p, v in zip(got, ok)], np.float32)
+    want, sure = _two_step_levels(g_min.astype(np.float64), tail / (2.0 * d), gamma, top.astype(np.float64), L)
+    sure &= ok
+    assert sure.sum() > n // 8
+    levels = np.array([list(p.levels)[L // 2:L - 1] for p in got], np.float32)
+    lo, hi = (want * (1 - np.longdouble(2) ** -32)).astype(np.float32), (want * (1 + np.longdouble(2) ** -32)).astype(np.float32)
+    wrong = sure[:, None] & (levels != lo) & (levels != hi)
+    assert not wrong.any(), (int(wrong.sum()), int(sure.sum()), [(gamma[i], float(top[i])) for i in np.flatnonzero(wrong.any(1))[:4]])
+
+
 @pytest.fixture(scope="module")
 def orc():
     import oracle
