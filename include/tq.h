@@ -292,7 +292,8 @@ tq_status tq_decompress_aggregate_apply(const uint32_t* packed_dev, size_t words
  *   of alpha or a level.
  * tq_compress_device_params / tq_decompress_aggregate_device_params: as tq_compress /
  *   tq_decompress_aggregate with params_dev[n_workers] in device memory; bits and mode are not read
- *   from the records but given by the caller (num_levels, mode).
+ *   from the records but given by the caller (num_levels, mode).  Long bf16 rows with table codebooks whose alpha
+ *   is 2^69 or more take about four times as long here as with tq_compress.
  * All three only enqueue work on `stream`, so a round made of tq_stats_hinted (or tq_stats) and these three can be
  * captured into a CUDA graph and replayed; call each once outside the capture first (the first launch of some kernels
  * sets a function attribute).  Errors: INVALID_ARG, DOMAIN (alpha_user <= 0), ALIGNMENT, BUFFER_TOO_SMALL, CUDA.

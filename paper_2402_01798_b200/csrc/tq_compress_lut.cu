@@ -35,7 +35,7 @@ namespace tq {
 
 struct LutWorker {
     float alpha;
-    uint32_t top, base;   // the largest pattern, the smallest one that is evaluated
+    uint32_t top, base;   // the largest pattern, the smallest one that is evaluated (without lut_lift of alpha's pattern)
     float levels[TQ_MAX_LEVELS];
     float inv_width[TQ_MAX_LEVELS];
 };
@@ -52,10 +52,15 @@ __device__ __forceinline__ uint32_t min_bf16x2(uint32_t a, uint32_t b) {
     uint32_t r; asm("min.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b)); return r;
 }
 
+__device__ __forceinline__ uint32_t mul_bf16x2(uint32_t a, uint32_t b) {
+    uint32_t r; asm("mul.rn.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b)); return r;
+}
+
 struct LutCtx {
     uint32_t table;          // shared-memory address of entry 0
     uint32_t negtop2, top2;  // the bf16 values -P_top and P_top in both halves
     PhiloxRun pr;
+    uint32_t factor2;        // LIFT: 1 or 2^-64 in both halves
 };
 
 __device__ __forceinline__ uint32_t lds_u32(uint32_t addr) {
@@ -66,8 +71,9 @@ __device__ __forceinline__ uint32_t lds_u32(uint32_t addr) {
 // warp's load covers one contiguous kilobyte), and packing to whole 32-bit words.
 template <int BITS> struct Piece { static constexpr int kElems = (BITS == 2 || BITS == 4) ? 16 : 32; };
 
-// One piece whose words are in registers: quantize, pack, store.  TAIL = the row's last piece, possibly partial.
-template <int BITS, bool TAIL>
+// One piece whose words are in registers: quantize, pack, store.  LIFT = alpha may be 2^69 or more (see lut_lift).  TAIL = the row's last piece,
+// possibly partial.
+template <int BITS, bool LIFT, bool TAIL>
 __device__ __forceinline__ void lut_piece(const uint32_t (&g)[Piece<BITS>::kElems / 2], uint32_t* prow, uint64_t piece, uint64_t d,
                                           uint64_t words_out, const RoundKeys& rk, const LutCtx& cx) {
     constexpr int E = Piece<BITS>::kElems, GROUPS = E / 8, WORDS = E * BITS / 32;
@@ -80,7 +86,8 @@ __device__ __forceinline__ void lut_piece(const uint32_t (&g)[Piece<BITS>::kElem
         philox_block(blk_lo + grp, cx.pr, rk, rnd);           // j0 >> 3 is a multiple of GROUPS: no carry
 #pragma unroll
         for (int h = 0; h < 4; ++h) {                          // elements 2h, 2h+1 of the group
-            const uint32_t w = min_bf16x2(max_bf16x2(g[4 * grp + h], cx.negtop2), cx.top2);
+            const uint32_t in = LIFT ? mul_bf16x2(g[4 * grp + h], cx.factor2) : g[4 * grp + h];
+            const uint32_t w = min_bf16x2(max_bf16x2(in, cx.negtop2), cx.top2);
             v[2 * h] = dot_halves_signed(rnd[h], 0x00FFu, lds_u32(dot_halves(w, 0x0004u, cx.table)));           // X + 65535 - r
             v[2 * h + 1] = dot_halves_signed(rnd[h], 0xFF00u, lds_u32(dot_halves(w, 0x0400u, cx.table)));
             if constexpr (TAIL) {                              // padding bits are zero
@@ -137,11 +144,12 @@ template <int BITS> struct LutShape {
 
 // A block's share of one row: build the table for quantizer q, then quantize the pieces begin + thread, + stride,
 // ... below `end`, and with LAST the row's last one, possibly partial.
-template <int BITS, bool WAIT>
+template <int BITS, bool WAIT, bool LIFT = false>
 __device__ __forceinline__ void lut_block(const LutWorker& q, uint32_t* s_table, const char* __restrict__ row,
                                           uint32_t* __restrict__ prow, uint64_t d, uint64_t words_out, uint32_t worker,
                                           const RoundKeys& rk, uint64_t begin, uint64_t stride, uint64_t end, bool last) {
     constexpr int kLutThreads = LutShape<BITS>::kThreads;
+    const uint32_t lift = LIFT ? lut_lift(top_pattern(q.alpha)) : 0u;
     {
         const LutRule rule{q.alpha, 1u << BITS, q.levels, q.inv_width};
         const uint32_t first = q.base & ~3u, n = q.top + 1 - first;             // everything below `first` is decided like zero
@@ -152,14 +160,14 @@ __device__ __forceinline__ void lut_block(const LutWorker& q, uint32_t* s_table,
         }
         for (uint32_t i = threadIdx.x; i < 2 * n; i += kLutThreads) {
             const uint32_t pattern = first + (i >= n ? i - n + 0x8000u : i);
-            s_table[pattern] = decision_x(bf16_pattern_value(pattern), rule) + 65535u;
+            s_table[pattern] = decision_x(bf16_pattern_value(pattern + lift), rule) + 65535u;
         }
     }
     __syncthreads();
     if constexpr (WAIT) pdl_wait();          // the table came from kernel parameters
 
     constexpr int E = Piece<BITS>::kElems, PER_ITER = 32 / E;   // 32 elements per thread and iteration: four Philox blocks in flight
-    const LutCtx cx{smem_addr(s_table), (q.top | 0x8000u) * 0x00010001u, q.top * 0x00010001u, philox_run(0u, worker, rk)};
+    const LutCtx cx{smem_addr(s_table), (q.top | 0x8000u) * 0x00010001u, q.top * 0x00010001u, philox_run(0u, worker, rk), lift ? 0x1F801F80u : 0x3F803F80u};
     const uint64_t row_interior = (d - 1) / E, interior = end < row_interior ? end : row_interior;      // whole pieces before the row's last one
 
     uint64_t piece = begin + threadIdx.x;
@@ -171,7 +179,7 @@ __device__ __forceinline__ void lut_block(const LutWorker& q, uint32_t* s_table,
     auto quantize = [&](const uint32_t (&buf)[PER_ITER][E / 2], uint64_t first) {
 #pragma unroll
         for (int k = 0; k < PER_ITER; ++k)
-            if (first + k * stride < interior) lut_piece<BITS, false>(buf[k], prow, first + k * stride, d, words_out, rk, cx);
+            if (first + k * stride < interior) lut_piece<BITS, LIFT, false>(buf[k], prow, first + k * stride, d, words_out, rk, cx);
     };
     uint32_t a[PER_ITER][E / 2];
     if constexpr (LutShape<BITS>::kTwoBuffers) {       // two sets of registers take turns: the next iteration's loads are in flight while this one is quantized
@@ -201,12 +209,12 @@ __device__ __forceinline__ void lut_block(const LutWorker& q, uint32_t* s_table,
             const uint32_t lo = j < d ? ldg16(e + j) : 0u, hi = j + 1 < d ? ldg16(e + j + 1) : 0u;
             t[i] = lo | (hi << 16);
         }
-        lut_piece<BITS, true>(t, prow, row_interior, d, words_out, rk, cx);
+        lut_piece<BITS, LIFT, true>(t, prow, row_interior, d, words_out, rk, cx);
     }
 }
 
-// Quantizers passed by value (host-side tq_params); the host has chosen the window.
-template <int BITS>
+// Quantizers passed by value (host-side tq_params); the host has chosen the window.  LIFT: for calls with at least one such row.
+template <int BITS, bool LIFT>
 __global__ void __launch_bounds__(LutShape<BITS>::kThreads, 1)
 compress_lut_kernel(const void* __restrict__ grad, uint64_t d, uint64_t grad_stride, const __grid_constant__ LutArgs args,
                     const __grid_constant__ RoundKeys rk, uint32_t first_worker,
@@ -214,7 +222,7 @@ compress_lut_kernel(const void* __restrict__ grad, uint64_t d, uint64_t grad_str
     constexpr int kLutThreads = LutShape<BITS>::kThreads;
     extern __shared__ __align__(16) uint32_t s_table[];       // lut_bytes of the largest of the workers' last patterns
     const uint32_t wi = blockIdx.y;
-    lut_block<BITS, true>(args.q[wi], s_table, static_cast<const char*>(grad) + static_cast<uint64_t>(wi) * grad_stride * 2,
+    lut_block<BITS, true, LIFT>(args.q[wi], s_table, static_cast<const char*>(grad) + static_cast<uint64_t>(wi) * grad_stride * 2,
                     packed + static_cast<uint64_t>(wi) * words_stride, d, words_out, first_worker + wi, rk,
                     static_cast<uint64_t>(blockIdx.x) * kLutThreads, static_cast<uint64_t>(gridDim.x) * kLutThreads, ~0ull, blockIdx.x == 0);
 }
@@ -316,13 +324,17 @@ static bool first_pattern(const LutRule& q, uint32_t top, uint32_t* base) {
     return lut_window_fits(q, top, hi * kLutBinade, base);
 }
 
-template <int BITS>
-static cudaError_t launch_lut(const CompressCall& c, const LutArgs& args, uint32_t top, uint32_t per_worker) {
+template <int BITS, bool LIFT>
+static cudaError_t launch_lut_form(const CompressCall& c, const LutArgs& args, uint32_t top, uint32_t per_worker) {
     // always the same limit: another thread may set it between this call's and the launch
-    const cudaError_t e = cudaFuncSetAttribute(compress_lut_kernel<BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize, kLutMostBytes);
+    const cudaError_t e = cudaFuncSetAttribute(compress_lut_kernel<BITS, LIFT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kLutMostBytes);
     if (e != cudaSuccess) return e;
-    return launch_kernel(compress_lut_kernel<BITS>, dim3(per_worker, c.n_workers), LutShape<BITS>::kThreads, lut_bytes(top), c.stream, c.grad, c.d,
+    return launch_kernel(compress_lut_kernel<BITS, LIFT>, dim3(per_worker, c.n_workers), LutShape<BITS>::kThreads, lut_bytes(top), c.stream, c.grad, c.d,
                          c.grad_stride, args, round_keys(c.seed), c.first_worker, c.packed, c.words_stride, c.words_out);
+}
+template <int BITS>
+static cudaError_t launch_lut(const CompressCall& c, const LutArgs& args, uint32_t top, uint32_t per_worker, bool lift) {
+    return lift ? launch_lut_form<BITS, true>(c, args, top, per_worker) : launch_lut_form<BITS, false>(c, args, top, per_worker);
 }
 
 // Blocks per row, and what the longest chain of blocks costs with them, in elements that a block quantizes in that time: a table costs
@@ -410,22 +422,27 @@ cudaError_t launch_compress_lut(const CompressCall& c, bool* applied) {
     }
     static thread_local LutArgs args;
     uint32_t most = 0;
+    bool lift = false;
     for (uint32_t i = 0; i < c.n_workers; ++i) {
         const tq_params_t& p = c.params[i];
         if (!(p.alpha > 0.0f) || !(p.alpha <= 3.402823466e38f)) return cudaSuccess;
         LutWorker& q = args.q[i];
         q.top = top_pattern(p.alpha);
-        if (q.top > kLutMostTop || !first_pattern(lut_rule(p, c.bits), q.top, &q.base)) return cudaSuccess;
+        if (!first_pattern(lut_rule(p, c.bits), q.top, &q.base)) return cudaSuccess;
+        const uint32_t low = lut_lift(q.top);
+        lift = lift || low != 0;
+        q.top -= low;
+        q.base -= low;
         most = q.top > most ? q.top : most;
         q.alpha = p.alpha;
         for (int k = 0; k < TQ_MAX_LEVELS; ++k) { q.levels[k] = p.levels[k]; q.inv_width[k] = p.inv_width[k]; }
     }
     *applied = true;
     switch (c.bits) {
-        case 1: return launch_lut<1>(c, args, most, per_worker);
-        case 2: return launch_lut<2>(c, args, most, per_worker);
-        case 3: return launch_lut<3>(c, args, most, per_worker);
-        default: return launch_lut<4>(c, args, most, per_worker);
+        case 1: return launch_lut<1>(c, args, most, per_worker, lift);
+        case 2: return launch_lut<2>(c, args, most, per_worker, lift);
+        case 3: return launch_lut<3>(c, args, most, per_worker, lift);
+        default: return launch_lut<4>(c, args, most, per_worker, lift);
     }
 }
 

@@ -10,6 +10,12 @@ constexpr uint32_t kLutBinade = 128;       // patterns per sign and binade
 constexpr uint32_t kLutBinades = 64;       // evaluated binades, at most
 constexpr uint32_t kLutMostTop = 0x61FFu;  // largest pattern with an entry: 4 * (2^15 + 0x61FF + 1) bytes of shared memory, 226 KB
 
+// A row whose alpha has a larger pattern (2^69 and more) is served as 2^-64 times its values, whose patterns are this much lower: what
+// that takes below the normal numbers lies far below the evaluated patterns, which are decided like zero.  Host parameters only: with device
+// parameters, where the host cannot choose the kernel, such rows are left to the element-wise kernels (the factor in the common kernel: 124 M x 8
+// 522 -> 532 us with 16 levels, 525 -> 604 with 4; the lifted form beside it, inlined or in a function: 506 -> 532 and 574).
+__host__ __device__ inline uint32_t lut_lift(uint32_t top) { return top > kLutMostTop ? kLutBinade * kLutBinades : 0u; }
+
 // What the decision depends on besides the value; the tables stay where they are.
 struct LutRule {
     float alpha;

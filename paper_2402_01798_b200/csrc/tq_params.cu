@@ -16,9 +16,8 @@
 // x = ln(a / g_min), in which a boxed alpha equation costs one exp and one log; it is solved by Newton
 // steps (4 to 8 evaluations); and everything that exists once per level or per trial point (levels, inverse
 // widths, the split of the two-step quantizer) is spread over the lanes of the warp.  Measured on B200 for
-// one worker, uniform, 4 levels / 8 workers, 16-level two-step quantizer: 4.5 us / 19.1 us (18.3 with the split as the first cubic
-// through four trial points gives it, which is up to 2^-24 off), against 21.1 us / 3590 us with one thread per worker, two pow per evaluation
-// and Aitken steps.  The two-step quantizer's
+// one worker, uniform, 4 levels / 8 workers, 16-level two-step quantizer: 4.5 us / 18.1 us, against
+// 21.1 us / 3590 us with one thread per worker, two pow per evaluation and Aitken steps.  The two-step quantizer's
 // trial points are the same for every alpha, so their powers k^-gamma are taken once (29.1 us with an exp
 // and a division per point and alpha; on the host, where one thread does all of them, 22 -> 6.6 us per record).
 #include <cmath>

@@ -301,11 +301,11 @@ def test_decision_table_dispatch(tq, orc, bits, d, n):
 
 
 @pytest.mark.parametrize("bits", [1, 2, 3, 4])
-@pytest.mark.parametrize("top", [0x0200, 0x3A80, 0x3A81, 0x3A82, 0x3A83, 0x61FF, 0x6200])
+@pytest.mark.parametrize("top", [0x0200, 0x3A80, 0x3A81, 0x3A82, 0x3A83, 0x61FF, 0x6200, 0x6203, 0x7EFF])
 def test_decision_table_of_every_pattern(tq, orc, bits, top):
     """The table is indexed by the bf16 pattern up to the smallest one >= alpha and filled in four entries at a time below the
-    evaluated ones: alpha at each place of a group of four, at the smallest normal numbers, and at the largest pattern that has an entry and the
-    next.  Rows hold every pattern there is but signalling NaN (which C's fmaxf, unlike the GPU's, does not drop)."""
+    evaluated ones: alpha at each place of a group of four, at the smallest normal numbers, at the largest pattern that has an entry, at the
+    next, from which on values enter with a factor, and near the largest of all.  Rows hold every pattern there is but signalling NaN (which C's fmaxf, unlike the GPU's, does not drop)."""
     d, n, L = 1_100_003, 16, 1 << bits
     alpha = float(np.array([top << 16], np.uint32).view(np.float32)[0])
     p = tq.tq_params_from_levels([float(np.float32(alpha) * np.float32((2 * k - (L - 1)) / (L - 1))) for k in range(L)])
@@ -322,6 +322,47 @@ def test_decision_table_of_every_pattern(tq, orc, bits, top):
     assert torch.equal(got, tq.tq_compress_device_params(g, raw, L, tq.NONUNIFORM, seed=8, d=d))
     for i in (0, n - 1):
         assert np.array_equal(got[i].cpu().numpy().view(np.uint32), orc.compress(g[i, :d].float().cpu().numpy(), _oracle_params(orc, p), 8, i))
+
+
+def _kernels(call):
+    """Names of the kernels that a call launches."""
+    from torch.profiler import ProfilerActivity, profile
+    call()
+    torch.cuda.synchronize()
+    with profile(activities=[ProfilerActivity.CUDA]) as seen:
+        call()
+        torch.cuda.synchronize()
+    return " ".join(e.key for e in seen.key_averages())
+
+
+def _one_book(tq, L, alpha):
+    mags = np.geomspace(alpha * 1e-3, alpha, L // 2).astype(np.float32) if L > 2 else np.array([alpha], np.float32)
+    return tq.tq_params_from_levels([float(x) for x in np.concatenate([-mags[::-1], mags])])
+
+
+@pytest.mark.parametrize("alphas", [(3e-3, 3e-3), (3e-3, 1e20), (3e-3, 1e25), (1e25, 1e37)])
+def test_decision_table_serves_every_alpha(tq, alphas):
+    """Rows with an alpha beyond the table's patterns (2^69) neither leave the table themselves nor take the call's other rows with them."""
+    d = 6_000_001
+    g = torch.zeros(2, (d + 31) // 32 * 32, dtype=torch.bfloat16, device="cuda")
+    ps, out = [_one_book(tq, 16, a) for a in alphas], torch.empty(2, tq.tq_packed_words(d, 4), dtype=torch.int32, device="cuda")
+    names = _kernels(lambda: tq.tq_compress(g, ps, seed=5, d=d, packed=out))
+    assert "compress_lut_kernel" in names and "compress_kernel" not in names, names
+
+
+@pytest.mark.parametrize("bits", [1, 2, 3, 4])
+@pytest.mark.parametrize("alpha", [3e-3, 1e30])
+def test_decision_table_and_signalling_nan(tq, bits, alpha):
+    """The oracle treats signalling NaN otherwise (see above): the table's codes for every pattern are those of the element-wise kernel, which
+    serves a call of the first 65536 elements alone."""
+    d, n = 17_000_016, 1
+    p = _one_book(tq, 1 << bits, alpha)
+    g = torch.arange(d, device="cuda").to(torch.int16).view(torch.bfloat16).view(1, d)
+    few = tq.tq_compress(g[:, :65536], [p], seed=8, d=65536)
+    words = few.shape[1] // 4 * 4
+    assert torch.equal(tq.tq_compress(g, [p], seed=8, d=d)[:, :words], few[:, :words])
+    raw = torch.frombuffer(bytearray(bytes(p)), dtype=torch.uint8).cuda()
+    assert torch.equal(tq.tq_compress_device_params(g, raw, 1 << bits, tq.NONUNIFORM, seed=8, d=d)[:, :words], few[:, :words])
 
 
 @pytest.mark.parametrize("bits,bad", [(4, False), (3, True), (1, False)])
