@@ -441,15 +441,12 @@ def test_two_pass_threshold_is_one_number(tq):
 
 
 def test_decision_tables_of_two_threads(tq):
-    """Two threads compress bf16 rows whose quantizers need tables of different sizes, each on its own stream: every call is accepted
-    and gives what it gives alone."""
+    """Two threads compress bf16 rows whose quantizers need tables of different sizes (they reach up to alpha's pattern: 1e-30 and 1e20), each
+    on its own stream: every call is accepted and gives what it gives alone."""
     d = 17_000_000
-    g = (torch.randn(1, d, device="cuda", generator=torch.Generator(device="cuda").manual_seed(1)) * 1e-3).to(torch.bfloat16)
-    books = []
-    for inner in (1e-3, 1e-12):                                  # two binades of entries, thirty-odd
-        mags = np.geomspace(inner, 3e-3, 8).astype(np.float32)
-        books.append([tq.tq_params_from_levels([float(x) for x in np.concatenate([-mags[::-1], mags])])])
-    want = [tq.tq_compress(g, p, seed=5, d=d) for p in books]
+    x = torch.randn(1, d, device="cuda", generator=torch.Generator(device="cuda").manual_seed(1))
+    rows, books = [(x * a / 3).to(torch.bfloat16) for a in (1e-30, 1e20)], [[_one_book(tq, 16, a)] for a in (1e-30, 1e20)]
+    want = [tq.tq_compress(g, p, seed=5, d=d) for g, p in zip(rows, books)]
     torch.cuda.synchronize()
     failed = []
 
@@ -458,7 +455,7 @@ def test_decision_tables_of_two_threads(tq):
             stream, out = torch.cuda.Stream(), torch.empty_like(want[k])
             with torch.cuda.stream(stream):
                 for _ in range(2000):
-                    tq.tq_compress(g, books[k], seed=5, d=d, packed=out)
+                    tq.tq_compress(rows[k], books[k], seed=5, d=d, packed=out)
                 stream.synchronize()
                 assert torch.equal(out, want[k])
         except BaseException as e:

@@ -210,11 +210,9 @@ def test_compress_bit_exact_ragged_sizes(tq, orc, bits, mode, dtype):
 @pytest.mark.parametrize("bits", [1, 2, 3, 4])
 @pytest.mark.parametrize("mode", [0, 1])
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
-def test_compress_tiled_copy_path_ragged_sizes(tq, orc, bits, mode, dtype):
-    """Table-mode bf16 rows of 65536 elements and more go through the kernel that brings the gradient in by
-    tiled copies (tiles of 8192 elements; fp32 rows and uniform mode keep the direct kernel and run here too):
-    whole tiles, one run more or less, a partial last run, a last tile with a single run, several workers
-    with a padded row stride; salted with NaN, Inf, levels."""
+def test_compress_ragged_sizes_around_tiles(tq, orc, bits, mode, dtype):
+    """Element-wise kernels at sizes around multiples of a block's 8192 elements: whole tiles, one run more or less, a
+    partial last run, a last tile with a single run, several workers with a padded row stride; salted with NaN, Inf, levels."""
     L = 1 << bits
     for d, n in ((65_536, 2), (65_537, 1), (65_568, 3), (73_728, 1), (73_729, 2), (81_919, 1), (200_003, 3)):
         g = heavy_tailed(d, n, dtype, seed=7 * bits + d)
@@ -241,19 +239,20 @@ def test_compress_tiled_copy_path_ragged_sizes(tq, orc, bits, mode, dtype):
 @pytest.mark.parametrize("bits", [1, 2, 3, 4])
 @pytest.mark.parametrize("mode", [0, 1])
 def test_compress_decision_table_path_ragged_sizes(tq, orc, bits, mode):
-    """bf16 rows of 2^18 elements and more take the kernel that reads the decision (interval and threshold)
-    from a per-block table indexed by the element's bit pattern: whole tiles, one element more, a partial
-    last run, several workers with a padded stride and different quantizers; salted with NaN of both signs,
+    """48 bf16 rows of 2^18 elements and more take the kernel that reads the decision (interval and threshold)
+    from a per-block table indexed by the element's bit pattern (mode 1; uniform mode keeps its arithmetic): whole tiles, one element more, a partial
+    last run, a padded stride and different quantizers; salted with NaN of both signs,
     Inf, +-alpha, zeros, subnormals and the levels themselves."""
-    L = 1 << bits
-    for d, n in ((262_144, 2), (262_145, 1), (262_176, 3), (270_337, 2), (300_003, 3)):
+    L, n = 1 << bits, 48
+    for d in (262_144, 262_145, 262_176, 270_337, 300_003):
         g = heavy_tailed(d, n, torch.bfloat16, seed=13 * bits + d)
         ps = []
-        for i in range(n):
+        for i in range(3):
             s = orc.stats(host_f32(orc, g[i, :d]), g_min=5e-4)
             ls = tq.Stats(d=s.d, n_tail=max(s.n_tail, 100), n_nonfinite=0, sum_abs=s.sum_abs, sum_sq=s.sum_sq,
                           sum_log_tail=max(s.sum_log_tail, 50.0), max_abs=max(s.max_abs, 0.05), g_min=5e-4)
             ps.append(tq.tq_params(ls, L, mode, 3.0 + 0.25 * i))
+        ps *= n // 3
         salt_special_values(g, d, ps[0])
         g[:, 5] = -float("nan")
         g.view(torch.int16)[:, 6] = 0x7FFF                                               # NaN with the largest payload
@@ -265,17 +264,17 @@ def test_compress_decision_table_path_ragged_sizes(tq, orc, bits, mode):
         packed = torch.full((n, words + 8), 0x5A5A5A5A, dtype=torch.int32, device="cuda")
         tq.tq_compress(g, ps, seed, first, d=d, packed=packed)
         got = packed.cpu().numpy().view(np.uint32)
-        for i in range(n):
+        for i in (0, 1, 2, 23, n - 1):
             want = orc.compress(host_f32(orc, g[i, :d]), to_oracle_params(orc, ps[i]), seed, first + i)
             assert np.array_equal(got[i, :words], want), (d, i)
             assert np.all(got[i, words:] == 0x5A5A5A5A)
 
 
 def test_compress_decision_table_windows_and_fallback(tq, orc):
-    """The table covers a window of 16, 32 or 64 binades below alpha.  Codebooks whose scale puts the window
+    """The table evaluates up to 64 binades below alpha.  Codebooks whose scale puts these
     at the bottom of the exponent range, at its top, and whose central levels are too small for any window
-    (the element-wise kernel then runs) all give the oracle's codes; so does alpha = max|g| (no truncation)."""
-    d = 262_144 + 77
+    (the element-wise kernel then runs) all give the oracle's codes; so does alpha = max|g| (no truncation).  48 rows: enough for a table."""
+    d, n = 262_144 + 77, 48
     books = [
         np.array([-1e-36, -3e-37, 2e-37, 1e-36], dtype=F32),                    # window reaches zero
         np.array([-3e30, -1e30, -1e29, 1e28, 2e29, 5e29, 2e30, 3e30], dtype=F32),   # window high in the exponent range
@@ -285,43 +284,48 @@ def test_compress_decision_table_windows_and_fallback(tq, orc):
     ]
     for lv in books:
         p = tq.tq_params_from_levels([float(x) for x in lv])
-        g = heavy_tailed(d, 2, torch.bfloat16, seed=len(lv), scale=float(lv[-1]) / 8)
+        g = heavy_tailed(d, n, torch.bfloat16, seed=len(lv), scale=float(lv[-1]) / 8)
         salt_special_values(g, d, p)
-        got = tq.tq_compress(g, [p, p], seed=5, first_worker=1, d=d).cpu().numpy().view(np.uint32)
-        for i in range(2):
+        got = tq.tq_compress(g, [p] * n, seed=5, first_worker=1, d=d).cpu().numpy().view(np.uint32)
+        for i in (0, 1, n - 1):
             want = orc.compress(host_f32(orc, g[i, :d]), to_oracle_params(orc, p), 5, 1 + i)
             assert np.array_equal(got[i], want), lv
-    g = heavy_tailed(d, 2, torch.bfloat16, seed=3)
+    g = heavy_tailed(d, n, torch.bfloat16, seed=3)
     st = tq.stats_to_host(tq.tq_stats(g, d))
     for mode in (tq.UNIFORM, tq.NONUNIFORM):
         ps = [tq.tq_params(s, 16, mode, 3.0, tq.ALPHA_MAXABS) for s in st]
         got = tq.tq_compress(g, ps, seed=6, d=d).cpu().numpy().view(np.uint32)
-        for i in range(2):
+        for i in (0, 1, n - 1):
             assert np.array_equal(got[i], orc.compress(host_f32(orc, g[i, :d]), to_oracle_params(orc, ps[i]), 6, i))
 
 
-def test_compress_decision_table_many_workers_mixed_windows(tq, orc):
-    """64 workers in one launch whose codebooks need windows of different sizes (scales from 1e-20 to 1e30, centres
-    from close to alpha to 40 binades below it): the launch uses the largest window, every row still matches."""
+@pytest.mark.parametrize("largest", [30, 20])
+def test_compress_decision_table_many_workers_mixed_windows(tq, orc, largest):
+    """64 workers in one launch whose codebooks need tables of different sizes (scales from 1e-20 on, centres from close to alpha to 40 binades
+    below it): the launch takes the shared memory of the largest, every row still matches.  Up to 1e30: some rows have an alpha beyond the
+    table's patterns (2^69), which host parameters serve by a factor and device parameters by the element-wise kernel.  Up to 1e20: none."""
     d, n, L = 262_144 + 33, 64, 8
     rng = np.random.default_rng(7)
     ps, scales = [], []
     for i in range(n):
-        a = float(10.0 ** rng.uniform(-20, 30))
+        a = float(10.0 ** rng.uniform(-20, largest))
         inner = float(10.0 ** rng.uniform(-12, -0.3))
         mags = np.geomspace(a * inner, a, L // 2).astype(F32)
         ps.append(tq.tq_params_from_levels([float(x) for x in np.concatenate([-mags[::-1], mags])]))
         scales.append(a)
+    assert (max(scales) > 2.0 ** 69) == (largest == 30) and max(scales) / min(scales) > 1e30
     from paper_2402_01798_b200 import inputs
     stride = inputs.worker_stride(d, torch.bfloat16)
     g = torch.zeros((n, stride), dtype=torch.bfloat16, device="cuda")
     for i in range(n):
         inputs.powerlaw_gradient(d, 3.0, scales[i] / 30, 900 + i, "cuda", torch.bfloat16, out=g[i, :d])
     g[:, 11] = float("nan"); g[:, 12] = float("inf"); g[:, 13] = -float("inf"); g[:, 14] = 0.0
+    raw = torch.frombuffer(bytearray(b"".join(bytes(p) for p in ps)), dtype=torch.uint8).cuda()
     got = tq.tq_compress(g, ps, seed=99, first_worker=0, d=d).cpu().numpy().view(np.uint32)
-    for i in range(0, n, 3):
+    dev = tq.tq_compress_device_params(g, raw, L, tq.NONUNIFORM, seed=99, first_worker=0, d=d).cpu().numpy().view(np.uint32)
+    for i in range(n):
         want = orc.compress(host_f32(orc, g[i, :d]), to_oracle_params(orc, ps[i]), 99, i)
-        assert np.array_equal(got[i], want), (i, scales[i])
+        assert np.array_equal(got[i], want) and np.array_equal(dev[i], want), (i, scales[i])
 
 
 @pytest.mark.parametrize("bits,mode", [(2, 0), (3, 1), (4, 1), (4, 0)])
