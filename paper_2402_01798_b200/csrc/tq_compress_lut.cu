@@ -382,10 +382,14 @@ static cudaError_t launch_lut_segs(const CompressCall& c, uint32_t blocks) {
 // host's parameters is built early; 1.53 with device parameters, where it is not and where a second launch looks for rows that the table
 // does not serve.  Table / element-wise, 16 levels, host and device parameters: 8 M 7.8 / 9.8 and 13.1 / 11.8 us, 12 M 9.9 / 12.6 and 14.8 / 15.9, 2 M
 // x 8 12.3 / 17.7 and 17.9 / 19.5, 300 k x 64 (128 blocks for 148 SMs) 15.7 / 20.2 and 22.6 / 22.3, 30 M 19.2 / 27.7 and 24.3 / 31.5, 124 M x 8
-// 501 / 843 and 508 / 843.
+// 501 / 843 and 508 / 843.  Codes of 1 and 3 bits from 1.65 on where a thread has
+// more than two of their long pieces: host parameters often come to an idle GPU (the records have just been waited for), where nothing hides the table.
+// Call and wait on an idle GPU, 8 levels, table / element-wise: 8 M 19.5 / 20.3 us, 9 M 21.5 / 20.4, 562500 x 16 24.3 / 21.9, 10 M 21.6 / 21.8,
+// 625 k x 16 24.0 / 25.5; 16 levels 9 M 19.5 / 21.5, 562500 x 16 23.0 / 23.0.
 static bool lut_pays(const CompressCall& c, uint32_t* per_worker) {
     const uint64_t cost = lut_plan(c.d, c.n_workers, per_worker), others = c.d * c.n_workers / static_cast<uint64_t>(sm_count());
-    return cost * 100 < others * (c.params_dev ? 153 : 178);
+    const bool late = c.bits % 2 != 0 && c.d / *per_worker > 2ull * LutShape<3>::kThreads * Piece<3>::kElems;      // 1 and 3 bits: the same shape
+    return cost * 100 < others * (c.params_dev ? 153 : late ? 165 : 178);
 }
 
 cudaError_t launch_compress_lut(const CompressCall& c, bool* applied) {

@@ -340,6 +340,16 @@ def _one_book(tq, L, alpha):
     return tq.tq_params_from_levels([float(x) for x in np.concatenate([-mags[::-1], mags])])
 
 
+@pytest.mark.parametrize("L,d,n,table", [(8, 8_200_000, 1, True), (8, 9_000_000, 1, False), (2, 562_500, 16, False), (8, 10_500_000, 1, True), (8, 656_250, 16, True), (16, 9_000_000, 1, True), (4, 562_500, 16, True)])
+def test_decision_table_from_where_it_pays_on_an_idle_gpu(tq, L, d, n, table):
+    """With host parameters nothing may be running that hides the table: codes of 1 and 3 bits, whose threads then take a third long piece, use it
+    from a little later on."""
+    g = torch.zeros(n, (d + 31) // 32 * 32, dtype=torch.bfloat16, device="cuda")
+    ps, out = [_one_book(tq, L, 3e-3)] * n, torch.empty(n, tq.tq_packed_words(d, {2: 1, 4: 2, 8: 3, 16: 4}[L]), dtype=torch.int32, device="cuda")
+    names = _kernels(lambda: tq.tq_compress(g, ps, seed=5, d=d, packed=out))
+    assert ("compress_lut_kernel" in names) == table, names
+
+
 @pytest.mark.parametrize("alphas", [(3e-3, 3e-3), (3e-3, 1e20), (3e-3, 1e25), (1e25, 1e37)])
 def test_decision_table_serves_every_alpha(tq, alphas):
     """Rows with an alpha beyond the table's patterns (2^69) neither leave the table themselves nor take the call's other rows with them."""
