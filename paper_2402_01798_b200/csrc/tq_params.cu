@@ -105,7 +105,7 @@ struct TailModel {
 };
 
 constexpr int kSplitGrid = 128;
-constexpr double kSplitClose = 1.4901161193847656e-08;      // 2^-26: see close_in
+constexpr double kSplitFine = 1.4901161193847656e-08, kSplitCoarse = 2.384185791015625e-07;      // 2^-26, 2^-22: see close_in
 constexpr double kSplitFirst = 9.094947017729282e-13, kSplitLnFirst = -27.72588722239781;   // 2^-40: the grid's first point, in place of 0
 // k^-gamma at the grid points of one lane, k = j / 128 with j = t * kLanes + lane + 1: the same for every alpha, and for every
 // record of one gamma.
@@ -171,8 +171,9 @@ struct Split {
     // Q_B(a, 0) = Q_B(a, 1) = Q_U(a), so the minimum is a point where Q_B turns from falling to rising.  Every
     // such turn between neighbours of a 128-point grid is closed in on; the turn with the smallest Q_B wins.  No turn:
     // the minimum is an end.  Where the density jumps (k a = g_min) the turn may be a kink, which is tested for by itself.
-    // Q_B is flat at a smooth turn: an error of 2^-26 there enters Q_B by its square, and the alpha iteration asks for no more (alpha, exponents 2.2 to 4.5,
-    // against 64-bit significands: off by 2^-52 in the middle of 3000 cases and by up to the 2^-40 at which it stops).
+    // Q_B is flat at a smooth turn: an error of 2^-24 there enters Q_B by its square, and the alpha iteration asks for no more (alpha, exponents 2.2 to 4.5,
+    // against 64-bit significands: off by 2^-52 in the middle of 12000 cases, by 2^-45 in a tenth and by up to the 2^-40 at which it stops; with
+    // the bracket closed in to the end 2^-50, 2^-44 and 2^-40).
     template <class Lanes>
     TQ_HD double best(const Lanes& lanes, const SplitGrid<Lanes>& grid, bool fine, double* q_best, double* ln_slope) const {
         constexpr int n = Lanes::kLanes;
@@ -213,7 +214,7 @@ struct Split {
     // them ends that; otherwise it goes on until the bracket is 2^-17 wide (relative), where the slope is close to a straight line whose zero
     // is off by the square of that width times a factor that grows where the slope bends; `fine` adds a Newton step with the slope of that line.
     // Against 64-bit significands, 18000 cases of exponents 2.05 to 10, alpha given or solved for, levels are off by 2^-48 to 2^-53 in the
-    // middle of the cases and by up to 2^-33 (the rounding of the slope) either way to the end, the coarse split by up to 2^-28.
+    // middle of the cases and by up to 2^-33 (the rounding of the slope) either way to the end, the coarse split by up to 2^-24.
     template <class Lanes>
     TQ_HD double close_in(const Lanes& lanes, double lo, double hi, bool fine, bool* at_kink) const {
         constexpr int n = Lanes::kLanes;
@@ -234,8 +235,8 @@ struct Split {
             if constexpr (n >= 8) {
                 // Two trial points on either side of the turn: the zero of the cubic k(slope) through the four, if they are close enough for it.  How
                 // close that is depends on where the slope bends (k near 0 or 1, large exponents): with r2 and r3 the second and third
-                // differences over the first, the cubic is off by about the 3/2 power of max(r2^2, r3), in steps.  `fine` goes on from there by the slope
-                // at that point, with its first and second derivative from the differences.
+                // differences over the first, the cubic is off by less than a quarter of the 3/2 power of max(r2^2, r3), in steps.  `fine` goes
+                // on from there by the slope at that point, with its first and second derivative from the differences.
                 if (c >= 2 && c <= n - 2) {
                     const double sa = lanes.of(s, c - 2), sb = lanes.of(s, c - 1), sc = lanes.of(s, c), sd = lanes.of(s, c + 1);
                     if (sa < sb && sb < sc && sc < sd) {
@@ -245,7 +246,7 @@ struct Split {
                         const double abc = (ab * sc - bc * sa) * rd, bcd = (bc * sd - cd * sb) * re;
                         const double at = (abc * sd - bcd * sa) * rf;
                         const double before = (sc - sb - (sb - sa)) * rb, after = (sd - sc - (sc - sb)) * rb;
-                        const double bend = fmax(fmax(before * before, after * after), fabs(after - before)), most = kSplitClose * lo;
+                        const double bend = fmax(fmax(before * before, after * after), fabs(after - before)), most = (fine ? kSplitFine : kSplitCoarse) * lo;
                         if (at >= 1.0 && at <= 2.0 && bend * bend * bend * (step * step) <= most * most) {
                             double k = lo + step * (static_cast<double>(c - 1) + at);
                             if (fine) {
