@@ -161,7 +161,7 @@ __device__ __forceinline__ void pair_plus_alpha(const Raw8<BF16>& g, int h, floa
 // long runs, so every operation counts.  k appears only as the denormal 8k * 2^-149, whose bit pattern is the byte offset into s_cell and,
 // shifted, k * 2^16; T as the mantissa of 2^23 + T with p saturated by its product (T stays within 0 .. 2^16, 0 for a NaN); the
 // sum of the two and 65535 - r, from the complement of the random word, by a two-way dot product has the code in byte 2.  With k, [r < T] and the code as
-// floats: 25.6 M x 16, 16 levels, host / device parameters 329 / 335 us, now 310 / 325; 250 M x 4, 8 levels 796, now 779; 1 M x 8 12.0, 11.5.
+// floats: 25.6 M x 16, 16 levels, host / device parameters 329 / 335 us, now 310 / 322; 250 M x 4, 8 levels 796, now 779; 1 M x 8 12.0, 11.5.
 __device__ __forceinline__ void code_cells2(float g0, float g1, float2 gc0, float2 gc1, const char* s_cell, uint32_t rnd, uint32_t& v0, uint32_t& v1) {
     const float eight = __uint_as_float(8u);
     const uint32_t k0 = __float_as_uint(__fmaf_rn(set_ge(g0, gc0.x), eight, gc0.y)), k1 = __float_as_uint(__fmaf_rn(set_ge(g1, gc1.x), eight, gc1.y));

@@ -23,7 +23,7 @@
 // halves (one operation of the multiplier pipe, 2 cycles) makes the address, table + 4 * pattern, from either half of a word, and
 // X + 65535 - r from either half of a word of random bits.  The code is then byte 2 of the difference, and codes are packed by
 // byte permutes.  124 M x 8, 16 levels, against an index of clamped binades with the sign moved beside it and r made into a
-// float by a byte permute (14.3 instructions per element, now 12.2; integer pipe 14.8 cycles): 601 -> 515 us through device
+// float by a byte permute (14.3 instructions per element, now 12.2; integer pipe 14.8 cycles): 601 -> 508 us through device
 // parameters, 591 -> 497 with the host's; 4 levels 600 -> 504.
 #include <cmath>
 
@@ -337,17 +337,22 @@ static cudaError_t launch_lut(const CompressCall& c, const LutArgs& args, uint32
     return lift ? launch_lut_form<BITS, true>(c, args, top, per_worker) : launch_lut_form<BITS, false>(c, args, top, per_worker);
 }
 
-// Blocks per row, and what the longest chain of blocks costs with them, in elements that a block quantizes in that time: a table costs
-// as much as 40000 (3.5 us), the waves follow one another, and SMs differ by 3 % of a share, which more and shorter shares
-// even out (124 M x 8, 36 / 55 / 74 blocks a row: 604 / 608 / 611 us); rows that do not divide the SMs waste less in several (37 blocks
-// a row, 296 in all, two for each SM: 591 us).
-static uint64_t lut_plan(uint64_t d, uint32_t n_workers, uint32_t* per_worker) {
+// Blocks per row, and what the longest chain of blocks costs with them, in elements that a block quantizes in that time.  The waves follow one
+// another, each with its tables: 30 M x 1 in 1 / 2 / 3 / 4 / 8 waves 19.0 / 22.9 / 26.7 / 30.6 / 45.2 us with 16 levels, 19.0 / 21.2 / 24.6 / 27.8 / 40.9
+// with 8, 3.8 and 3.1 us a table or 50000 and 40000 elements.  Rows that do not divide the SMs waste less in several waves (124 M x 8, 16 levels,
+// 18 / 36 / 37 / 55 / 74 blocks a row: 527 / 531 / 518 / 527 / 527 us; 25.6 M x 16, 9 / 18 / 27 / 37 / 46: 212 / 217 / 221 / 220 / 226).  With codes of 1
+// and 3 bits more and shorter shares also even out SMs of different speed, 3 % of a share, at the largest sizes (8 levels, 193 M x 2 in 1 / 2 waves
+// 250 / 232 us, 46 M x 11 in 1 / 3 317 / 306); with 2 and 4 bits they do not (16 levels 210 / 210 and 280 / 280).
+static uint64_t lut_plan(const CompressCall& c, uint32_t* per_worker) {
+    const bool two_buffers = c.bits % 2 == 0;
+    const uint64_t d = c.d, n_workers = c.n_workers, table = two_buffers ? 50000 : 40000;
     const uint64_t sms = static_cast<uint64_t>(sm_count());
     uint64_t best = ~0ull;
     for (uint64_t shares = 1; shares <= 8; ++shares) {
         uint64_t p = sms * shares / n_workers;
         if (p == 0) p = 1;
-        const uint64_t waves = (p * n_workers + sms - 1) / sms, share = d / p + 1, cost = waves * (40000 + share) + share / 32;
+        const uint64_t waves = (p * n_workers + sms - 1) / sms, share = d / p + 1;
+        const uint64_t cost = waves * (table + share) + (two_buffers ? 0 : share / 32);
         if (cost < best) { best = cost; *per_worker = static_cast<uint32_t>(p); }
     }
     return best;
@@ -378,17 +383,18 @@ static cudaError_t launch_lut_segs(const CompressCall& c, uint32_t blocks) {
                          round_keys(c.seed), c.first_worker, c.packed, c.words_stride, plan, start_tiles);
 }
 
-// The element-wise kernels take about 1.7 times as long per element and build no table.  1.78 here, because behind another kernel the table of the
-// host's parameters is built early; 1.53 with device parameters, where it is not and where a second launch looks for rows that the table
-// does not serve.  Table / element-wise, 16 levels, host and device parameters: 8 M 7.8 / 9.8 and 13.1 / 11.8 us, 12 M 9.9 / 12.6 and 14.8 / 15.9, 2 M
-// x 8 12.3 / 17.7 and 17.9 / 19.5, 300 k x 64 (128 blocks for 148 SMs) 15.7 / 20.2 and 22.6 / 22.3, 30 M 19.2 / 27.7 and 24.3 / 31.5, 124 M x 8
-// 501 / 843 and 508 / 843.  Codes of 1 and 3 bits from 1.65 on where a thread has
-// more than two of their long pieces: host parameters often come to an idle GPU (the records have just been waited for), where nothing hides the table.
-// Call and wait on an idle GPU, 8 levels, table / element-wise: 8 M 19.5 / 20.3 us, 9 M 21.5 / 20.4, 562500 x 16 24.3 / 21.9, 10 M 21.6 / 21.8,
-// 625 k x 16 24.0 / 25.5; 16 levels 9 M 19.5 / 21.5, 562500 x 16 23.0 / 23.0.
+// The element-wise kernels take about 1.7 times as long per element and build no table.  With host parameters the line is higher than that, because
+// behind another kernel the table is built early; with device parameters lower, because there it is not and a second launch looks for rows
+// that the table does not serve.  In both cases from about 8 M (12 M) elements that divide the SMs evenly.  Table / element-wise, 16 levels, host
+// and device parameters: 8 M 7.5 / 9.6 and 11.3 / 11.4 us, 12.5 M 9.8 / 12.7 and 13.3 / 15.7, 2 M x 8 11.8 / 17.5 and 16.2 / 19.3, 250 k x 64 (128
+// blocks for 148 SMs) 18.4 / 20.1 with device parameters, 24 M 15.4 / 22.1 and 19.2 / 23.9, 124 M x 8 501 / 843 and 508 / 843.  Codes of 1 and 3
+// bits with host parameters from 1.65 on where a thread has more than two of their long pieces: such parameters often come to an idle GPU (the
+// records have just been waited for), where nothing hides the table.  Call and wait on an idle GPU, 8 levels, table / element-wise: 8 M 19.5 / 20.3 us,
+// 9 M 21.5 / 20.4, 562500 x 16 24.3 / 21.9, 10 M 21.6 / 21.8, 625 k x 16 24.0 / 25.5; 16 levels 9 M 19.5 / 21.5, 562500 x 16 23.0 / 23.0.
 static bool lut_pays(const CompressCall& c, uint32_t* per_worker) {
-    const uint64_t cost = lut_plan(c.d, c.n_workers, per_worker), others = c.d * c.n_workers / static_cast<uint64_t>(sm_count());
-    const bool late = c.bits % 2 != 0 && c.d / *per_worker > 2ull * LutShape<3>::kThreads * Piece<3>::kElems;      // 1 and 3 bits: the same shape
+    const uint64_t cost = lut_plan(c, per_worker), others = c.d * c.n_workers / static_cast<uint64_t>(sm_count());
+    if (c.bits % 2 == 0) return cost * 100 < others * (c.params_dev ? 162 : 194);
+    const bool late = c.d / *per_worker > 2ull * LutShape<3>::kThreads * Piece<3>::kElems;      // 1 and 3 bits: the same shape
     return cost * 100 < others * (c.params_dev ? 153 : late ? 165 : 178);
 }
 
