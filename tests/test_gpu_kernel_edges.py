@@ -324,15 +324,16 @@ def test_decision_table_of_every_pattern(tq, orc, bits, top):
         assert np.array_equal(got[i].cpu().numpy().view(np.uint32), orc.compress(g[i, :d].float().cpu().numpy(), _oracle_params(orc, p), 8, i))
 
 
-def _kernels(call):
-    """Names of the kernels that a call launches."""
-    from torch.profiler import ProfilerActivity, profile
-    call()
+def _kernels(call, path):
+    """The kernels that a call launches: the nodes of a graph captured from it, as text."""
+    call()                                                       # the first launch of some kernels sets a function attribute
     torch.cuda.synchronize()
-    with profile(activities=[ProfilerActivity.CUDA]) as seen:
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    graph.enable_debug_mode()
+    with torch.cuda.graph(graph):
         call()
-        torch.cuda.synchronize()
-    return " ".join(e.key for e in seen.key_averages())
+    graph.debug_dump(str(path))
+    return path.read_text()
 
 
 def _one_book(tq, L, alpha):
@@ -341,22 +342,22 @@ def _one_book(tq, L, alpha):
 
 
 @pytest.mark.parametrize("L,d,n,table", [(8, 8_200_000, 1, True), (8, 9_000_000, 1, False), (2, 562_500, 16, False), (8, 10_500_000, 1, True), (8, 656_250, 16, True), (16, 9_000_000, 1, True), (4, 562_500, 16, True)])
-def test_decision_table_from_where_it_pays_on_an_idle_gpu(tq, L, d, n, table):
+def test_decision_table_from_where_it_pays_on_an_idle_gpu(tq, tmp_path, L, d, n, table):
     """With host parameters nothing may be running that hides the table: codes of 1 and 3 bits, whose threads then take a third long piece, use it
     from a little later on."""
     g = torch.zeros(n, (d + 31) // 32 * 32, dtype=torch.bfloat16, device="cuda")
     ps, out = [_one_book(tq, L, 3e-3)] * n, torch.empty(n, tq.tq_packed_words(d, {2: 1, 4: 2, 8: 3, 16: 4}[L]), dtype=torch.int32, device="cuda")
-    names = _kernels(lambda: tq.tq_compress(g, ps, seed=5, d=d, packed=out))
-    assert ("compress_lut_kernel" in names) == table, names
+    names = _kernels(lambda: tq.tq_compress(g, ps, seed=5, d=d, packed=out), tmp_path / "graph.dot")
+    assert ("compress_lut_kernel" in names) == table and ("compress_kernel" in names) == (not table), names
 
 
 @pytest.mark.parametrize("alphas", [(3e-3, 3e-3), (3e-3, 1e20), (3e-3, 1e25), (1e25, 1e37)])
-def test_decision_table_serves_every_alpha(tq, alphas):
+def test_decision_table_serves_every_alpha(tq, tmp_path, alphas):
     """Rows with an alpha beyond the table's patterns (2^69) neither leave the table themselves nor take the call's other rows with them."""
     d = 6_000_001
     g = torch.zeros(2, (d + 31) // 32 * 32, dtype=torch.bfloat16, device="cuda")
     ps, out = [_one_book(tq, 16, a) for a in alphas], torch.empty(2, tq.tq_packed_words(d, 4), dtype=torch.int32, device="cuda")
-    names = _kernels(lambda: tq.tq_compress(g, ps, seed=5, d=d, packed=out))
+    names = _kernels(lambda: tq.tq_compress(g, ps, seed=5, d=d, packed=out), tmp_path / "graph.dot")
     assert "compress_lut_kernel" in names and "compress_kernel" not in names, names
 
 
