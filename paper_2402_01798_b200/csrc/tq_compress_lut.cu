@@ -26,6 +26,7 @@
 // float by a byte permute (14.3 instructions per element, now 12.2; integer pipe 14.8 cycles): 601 -> 508 us through device
 // parameters, 591 -> 497 with the host's; 4 levels 600 -> 504.
 #include <cmath>
+#include <type_traits>
 
 #include "tq_device.cuh"
 #include "tq_launch.h"
@@ -147,7 +148,7 @@ template <int BITS> struct LutShape {
 template <int BITS, bool WAIT, bool LIFT = false>
 __device__ __forceinline__ void lut_block(const LutWorker& q, uint32_t* s_table, const char* __restrict__ row,
                                           uint32_t* __restrict__ prow, uint64_t d, uint64_t words_out, uint32_t worker,
-                                          const RoundKeys& rk, uint64_t begin, uint64_t stride, uint64_t end, bool last) {
+                                          const RoundKeys& rk, uint64_t begin, uint64_t stride, uint64_t end, bool last, std::bool_constant<LIFT> = {}) {
     constexpr int kLutThreads = LutShape<BITS>::kThreads;
     const uint32_t lift = LIFT ? lut_lift(top_pattern(q.alpha)) : 0u;
     {
@@ -222,9 +223,9 @@ compress_lut_kernel(const void* __restrict__ grad, uint64_t d, uint64_t grad_str
     constexpr int kLutThreads = LutShape<BITS>::kThreads;
     extern __shared__ __align__(16) uint32_t s_table[];       // lut_bytes of the largest of the workers' last patterns
     const uint32_t wi = blockIdx.y;
-    lut_block<BITS, true, LIFT>(args.q[wi], s_table, static_cast<const char*>(grad) + static_cast<uint64_t>(wi) * grad_stride * 2,
+    lut_block<BITS, true>(args.q[wi], s_table, static_cast<const char*>(grad) + static_cast<uint64_t>(wi) * grad_stride * 2,
                     packed + static_cast<uint64_t>(wi) * words_stride, d, words_out, first_worker + wi, rk,
-                    static_cast<uint64_t>(blockIdx.x) * kLutThreads, static_cast<uint64_t>(gridDim.x) * kLutThreads, ~0ull, blockIdx.x == 0);
+                    static_cast<uint64_t>(blockIdx.x) * kLutThreads, static_cast<uint64_t>(gridDim.x) * kLutThreads, ~0ull, blockIdx.x == 0, std::bool_constant<LIFT>{});
 }
 
 // Quantizers read from device memory (tq_params_device).  Every block decides by lut_serves_record whether the
