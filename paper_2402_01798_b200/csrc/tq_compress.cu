@@ -414,9 +414,11 @@ __device__ __forceinline__ void compress_last_run(const char* row, uint32_t* pro
 #endif
 
 // Per-block set-up of the shared tables for quantizer q (ends with a block barrier unless the codebook is uniform).
-// s_grid must hold kMaxGridCells + 1 entries when SEARCH is a grid.  LANES: the form for quantizers in device memory, whose tables
-// nothing hides; host parameters' are built while the kernel before still runs, and with that form their main loop gets other registers
-// (25.6 M x 16, 16 levels: 310 -> 322 us).
+// s_grid must hold kMaxGridCells + 1 entries when SEARCH is a grid.  LANES: a lane per level, for fp32 rows with 16 levels in device memory, where fourteen
+// comparisons per cell show in the start of a row (3.5 M x 1 7.25 -> 7.11 us, 2 M x 4 11.56 -> 11.38, 250 M x 4 984 -> 979).  Elsewhere it is the slower form: bf16
+// rows and fewer levels (64 x 547 k bf16 in 16 groups, 16 / 8 / 4 levels 49.2 / 46.2 / 45.7 us, with it 51.1 / 48.1 / 46.3; 1 M x 1 fp32, 8 levels 3.9, with it
+// 4.3), and the host's parameters, whose tables are built while the kernel before still runs and whose main loop gets other registers (25.6 M x 16, 16
+// levels: 310 -> 322 us).
 template <int BITS, int SEARCH, bool LANES>
 __device__ __forceinline__ void build_tables(const WorkerQ& q, float2* s_grid, float2* s_cell, float* s_search) {
     constexpr int L = 1 << BITS;
@@ -430,8 +432,7 @@ __device__ __forceinline__ void build_tables(const WorkerQ& q, float2* s_grid, f
     constexpr bool kCells = SEARCH == kGrid || SEARCH == kLogGrid;
     if constexpr (kCells && LANES) {
         // A lane for each interior level l_1 .. l_{s-1} (their cells are distinct and in order, or the grid would not have been chosen); a warp fills
-        // in 32 cells at a time, most of which hold none (each thread comparing its cells with all levels took 1 us of a call of 1 M x 8, 16
-        // levels).
+        // in 32 cells at a time, most of which hold none.
         const uint32_t lane = threadIdx.x & 31u;
         const bool interior = lane >= 1 && lane <= L - 2;
         const float level = lane < L ? q.levels[lane] : 0.0f;
@@ -567,7 +568,7 @@ __device__ __forceinline__ void compress_piece(State& sh, const void* __restrict
                                                uint32_t first_worker, uint32_t* __restrict__ packed, uint64_t words_stride,
                                                const TilePlan& plan) {
     constexpr size_t esz = BF16 ? 2 : 4;
-    build_tables<BITS, SEARCH, true>(sh.q, sh.grid, sh.cell, sh.search);
+    build_tables<BITS, SEARCH, !BF16 && BITS == 4>(sh.q, sh.grid, sh.cell, sh.search);
     const RunCtx cx = run_ctx<BITS, SEARCH>(sh.q, sh.grid, sh.cell, sh.search);
     const char* row = static_cast<const char*>(grad) + (static_cast<uint64_t>(sh.piece.worker) * grad_stride + sh.piece.off) * esz;
     uint32_t* prow = packed + static_cast<uint64_t>(sh.piece.worker) * words_stride + plan.segs.woff[sh.piece.seg];
